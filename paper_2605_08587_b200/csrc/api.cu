@@ -447,6 +447,22 @@ static kla_status check_decode(const kla_desc *d, const void *q, const void *k, 
     return KLA_OK;
 }
 
+static DecodeParams decode_params(const kla_desc *desc, int32_t n_steps, const void *q, const void *k, const void *v, const float *log_alpha,
+                                  const float *eta, float eps, float *state, void *out, int diag)
+{
+    DecodeParams p;
+    p.q = q; p.k = k; p.v = v;
+    p.log_alpha = log_alpha; p.eta = eta;
+    p.state = state; p.out = out;
+    p.BH = desc->B * desc->H;
+    p.eps = eps;
+    p.coeff_eta = (desc->flags & KLA_FLAG_COEFF_ETA) ? 1 : 0;
+    p.qnorm = (desc->flags & KLA_FLAG_QNORM) ? 1 : 0;
+    p.diag = diag;
+    p.n_steps = n_steps;
+    return p;
+}
+
 kla_status kla_decode_steps(const kla_desc *desc, int32_t n_steps, const void *q, const void *k,
                             const void *v, const float *log_alpha, const float *eta, float eps,
                             float *state_inout, void *out)
@@ -457,27 +473,11 @@ kla_status kla_decode_steps(const kla_desc *desc, int32_t n_steps, const void *q
     st = check_arch();
     if (st != KLA_OK) return st;
     const size_t bh = (size_t)desc->B * desc->H;
-    const size_t io_sz = desc->io_dtype == KLA_BF16 ? 2 : 4, out_sz = desc->out_dtype == KLA_BF16 ? 2 : 4;
     // per-step strides must keep the 16-byte alignment of the gate arrays
     if (n_steps > 1 && ((bh * sizeof(float)) & 15u)) return KLA_ERR_ALIGN;
-    for (int32_t s = 0; s < n_steps; ++s) {
-        DecodeParams p;
-        p.q = (const char *)q + (size_t)s * bh * desc->d_k * io_sz;
-        p.k = (const char *)k + (size_t)s * bh * desc->d_k * io_sz;
-        p.v = (const char *)v + (size_t)s * bh * desc->d_v * io_sz;
-        p.log_alpha = log_alpha + (size_t)s * bh;
-        p.eta = eta + (size_t)s * bh;
-        p.state = state_inout;
-        p.out = (char *)out + (size_t)s * bh * desc->d_v * out_sz;
-        p.BH = (int32_t)bh;
-        p.eps = eps;
-        p.inputs_ready = s > 0 ? 1 : 0;
-        p.coeff_eta = (desc->flags & KLA_FLAG_COEFF_ETA) ? 1 : 0;
-        p.qnorm = (desc->flags & KLA_FLAG_QNORM) ? 1 : 0;
-        if (launch_decode(p, desc->d_k, desc->io_dtype, desc->out_dtype, (cudaStream_t)desc->stream) != cudaSuccess)
-            return KLA_ERR_LAUNCH;
-    }
-    return KLA_OK;
+    if (n_steps == 0) return KLA_OK;
+    return launch_decode(decode_params(desc, n_steps, q, k, v, log_alpha, eta, eps, state_inout, out, 0), desc->d_k, desc->io_dtype,
+                         desc->out_dtype, (cudaStream_t)desc->stream) == cudaSuccess ? KLA_OK : KLA_ERR_LAUNCH;
 }
 
 kla_status kla_decode_step(const kla_desc *desc, const void *q, const void *k, const void *v,
@@ -519,10 +519,8 @@ kla_status kla_dg_decode_step(const kla_desc *desc, const void *q, const void *k
     if (st != KLA_OK) return st;
     st = check_arch();
     if (st != KLA_OK) return st;
-    // one token per sequence; every warp reads its columns of the state before it writes them, so the update is in place
-    return launch_dg_scan(q, k, v, log_alpha, eta, state_inout, out, state_inout, nullptr, 1, desc->H, desc->B, desc->d_k, eps,
-                          (desc->flags & KLA_FLAG_COEFF_ETA) ? 1 : 0, (desc->flags & KLA_FLAG_QNORM) ? 1 : 0, desc->io_dtype,
-                          desc->out_dtype, (cudaStream_t)desc->stream) == cudaSuccess ? KLA_OK : KLA_ERR_LAUNCH;
+    return launch_decode(decode_params(desc, 1, q, k, v, log_alpha, eta, eps, state_inout, out, 1), desc->d_k, desc->io_dtype,
+                         desc->out_dtype, (cudaStream_t)desc->stream) == cudaSuccess ? KLA_OK : KLA_ERR_LAUNCH;
 }
 
 size_t kla_bwd_workspace_bytes(const kla_desc *desc)

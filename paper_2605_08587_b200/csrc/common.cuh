@@ -51,10 +51,9 @@ struct DecodeParams {
     void *out;
     int32_t BH;
     float eps;
-    // 1: q, k, v, log_alpha, eta were complete before the previous kernel on the stream started (later steps of
-    // kla_decode_steps), so they may be read while that kernel drains; 0: they may be its outputs
-    int32_t inputs_ready;
     int32_t coeff_eta, qnorm;   // as in ChunkParams
+    int32_t diag;               // log_alpha is [BH, d]: one decay per row of the state
+    int32_t n_steps;            // consecutive tokens: step s reads rows s BH .. of q, k, v, log_alpha, eta
 };
 
 // Launchers implemented in the kernel translation units.  Each returns cudaGetLastError().
@@ -126,6 +125,24 @@ __device__ __forceinline__ float4 load4(const __nv_bfloat16 *p)
     float2 fa = __bfloat1622float2(a), fb = __bfloat1622float2(b);
     return make_float4(fa.x, fa.y, fb.x, fb.y);
 }
+// Four consecutive elements as loaded, converted on use.
+template <typename IO>
+struct Vec4 {
+    float4 r;
+    __device__ __forceinline__ void load(const float *p) { r = load4(p); }
+    __device__ __forceinline__ float4 get() const { return r; }
+};
+template <>
+struct Vec4<__nv_bfloat16> {
+    uint2 r;
+    __device__ __forceinline__ void load(const __nv_bfloat16 *p) { r = *reinterpret_cast<const uint2 *>(p); }
+    __device__ __forceinline__ float4 get() const
+    {
+        const float2 a = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162 *>(&r.x)), b = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162 *>(&r.y));
+        return make_float4(a.x, a.y, b.x, b.y);
+    }
+};
+
 __device__ __forceinline__ void store4(float *p, float4 x) { *reinterpret_cast<float4 *>(p) = x; }
 __device__ __forceinline__ void store4(__nv_bfloat16 *p, float4 x)
 {
