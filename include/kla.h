@@ -60,7 +60,7 @@ typedef enum { KLA_F32 = 0, KLA_BF16 = 1 } kla_dtype;
 
 /* desc->flags */
 #define KLA_FLAG_NONE 0
-/* Force the CUDA-core fp32 chunk kernel even where the tensor-core kernel applies (used to
+/* Force the fp32 kernel on CUDA cores (a scan over blocks of four tokens) even where the tensor-core kernel applies (used to
  * cross-check the two device paths against each other and against the oracle). */
 #define KLA_FLAG_FORCE_SIMT 1
 /* Layer-edge variants named by the paper; both default to off (the recurrence at the top of this file). */
@@ -264,7 +264,7 @@ kla_status kla_decode_steps(const kla_desc *desc, int32_t n_steps, const void *q
  * and the residual, the coefficient of Eq. 3, the write and the read-out are unchanged.  Arguments as kla_chunk_fwd /
  * kla_decode_step except
  *   log_alpha   [B, T, H, d_k] fp32 (decode: [B, H, d_k])
- * and no chunk length, workspace or segment flags: the recurrence is evaluated token by token on CUDA cores, in fp32,
+ * and no chunk length, workspace or segment flags: the recurrence is evaluated four tokens at a time on CUDA cores, in fp32,
  * with the state of every (sequence, head) in registers (the chunkwise form with elementwise decay products is not
  * built).  Packed input (cu_seqlens), KLA_FLAG_COEFF_ETA and KLA_FLAG_QNORM are supported; fp32 or bf16 q, k, v.
  */

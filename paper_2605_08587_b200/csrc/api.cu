@@ -204,6 +204,22 @@ size_t kla_chunk_fwd_plan_word_offset(const kla_desc *desc, int32_t chunk)
 
 }  // extern "C"
 
+static TokenScanParams token_scan_params(const kla_desc *desc, const void *q, const void *k, const void *v, const float *log_alpha,
+                                         const float *eta, float eps, const float *init_state, void *out, float *final_state)
+{
+    TokenScanParams t;
+    t.q = q; t.k = k; t.v = v;
+    t.log_alpha = log_alpha; t.eta = eta;
+    t.init_state = init_state; t.out = out; t.final_state = final_state;
+    t.cu_seqlens = desc->cu_seqlens;
+    t.T = desc->T; t.H = desc->H; t.n_seq = desc->n_seq;
+    t.eps = eps;
+    t.coeff_eta = (desc->flags & KLA_FLAG_COEFF_ETA) ? 1 : 0;
+    t.qnorm = (desc->flags & KLA_FLAG_QNORM) ? 1 : 0;
+    t.diag = 0;
+    return t;
+}
+
 // The chunk forward proper.  `marks`: null, or five events recorded on the stream around the set-up kernels, segment
 // pass 1, the chaining of the segment maps and the main pass (kla_chunk_fwd_timed).
 static kla_status chunk_fwd_impl(const kla_desc *desc, const void *q, const void *k, const void *v,
@@ -311,7 +327,8 @@ static kla_status chunk_fwd_impl(const kla_desc *desc, const void *q, const void
     }
     else {
         mark(1); mark(2); mark(3);
-        err = launch_chunk_simt(p, desc->d_k, chunk, desc->io_dtype, desc->out_dtype, stream);
+        TokenScanParams t = token_scan_params(desc, q, k, v, log_alpha, eta, eps, init_state, out, final_state);
+        err = launch_token_scan(t, desc->d_k, desc->io_dtype, desc->out_dtype, stream);
     }
     mark(4);
     return err == cudaSuccess ? KLA_OK : KLA_ERR_LAUNCH;
@@ -506,9 +523,9 @@ kla_status kla_dg_fwd(const kla_desc *desc, const void *q, const void *k, const 
         }
         return KLA_OK;
     }
-    return launch_dg_scan(q, k, v, log_alpha, eta, init_state, out, final_state, desc->cu_seqlens, desc->T, desc->H, desc->n_seq,
-                          desc->d_k, eps, (desc->flags & KLA_FLAG_COEFF_ETA) ? 1 : 0, (desc->flags & KLA_FLAG_QNORM) ? 1 : 0,
-                          desc->io_dtype, desc->out_dtype, stream) == cudaSuccess ? KLA_OK : KLA_ERR_LAUNCH;
+    TokenScanParams t = token_scan_params(desc, q, k, v, log_alpha, eta, eps, init_state, out, final_state);
+    t.diag = 1;
+    return launch_token_scan(t, desc->d_k, desc->io_dtype, desc->out_dtype, stream) == cudaSuccess ? KLA_OK : KLA_ERR_LAUNCH;
 }
 
 kla_status kla_dg_decode_step(const kla_desc *desc, const void *q, const void *k, const void *v,

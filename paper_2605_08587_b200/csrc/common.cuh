@@ -59,8 +59,6 @@ struct DecodeParams {
 // Launchers implemented in the kernel translation units.  Each returns cudaGetLastError().
 cudaError_t launch_decode(const DecodeParams &p, int d, int io_dtype, int out_dtype,
                           cudaStream_t stream);
-cudaError_t launch_chunk_simt(const ChunkParams &p, int d, int chunk, int io_dtype, int out_dtype,
-                              cudaStream_t stream);
 cudaError_t launch_chunk_tc(const ChunkParams &p, int d, int io_dtype, int out_dtype,
                             cudaStream_t stream);
 // Head dimension 128, the two slices of a head as a cluster of two CTAs (chunk_wy.cu); called by launch_chunk_tc.
@@ -85,10 +83,21 @@ cudaError_t launch_packed_units(const int32_t *cu_seqlens, int n_seq, int seg_le
 // (`skip_if_one`: null, or a device word; the kernel does nothing when it holds 1)
 cudaError_t launch_seg_combine(const float *init_state, const float *map, const float *local, float *start, int B, int H,
                                int G, int d, const int32_t *skip_if_one, cudaStream_t stream);
-// Diagonal-gated recurrence, token by token on CUDA cores (dg_scan.cu); log_alpha [n_tok, H, d].
-cudaError_t launch_dg_scan(const void *q, const void *k, const void *v, const float *log_alpha, const float *eta,
-                           const float *init_state, void *out, float *final_state, const int32_t *cu_seqlens, int T, int H,
-                           int n_seq, int d, float eps, int coeff_eta, int qnorm, int io_dtype, int out_dtype, cudaStream_t stream);
+// The recurrence in fp32 on CUDA cores, four tokens at a time (token_scan.cu): diagonal gates, fp32 inputs.
+struct TokenScanParams {
+    const void *q, *k, *v;
+    const float *log_alpha;     // [rows], diag: [rows, D]
+    const float *eta;           // [rows]
+    const float *init_state;    // [n_seq, H, D, D] or null
+    void *out;                  // [rows, D]
+    float *final_state;         // [n_seq, H, D, D] or null (may alias init_state: every warp reads its columns first)
+    const int32_t *cu_seqlens;  // null: fixed length T
+    int32_t T, H, n_seq;
+    float eps;
+    int32_t coeff_eta, qnorm;   // as in ChunkParams
+    int32_t diag;               // one decay per row of the state
+};
+cudaError_t launch_token_scan(const TokenScanParams &p, int d, int io_dtype, int out_dtype, cudaStream_t stream);
 // Reverse-mode derivative of the recurrence, token by token on CUDA cores (bwd_scan.cu); gradients in fp32.
 size_t bwd_workspace_bytes(int n_seq, long long n_tok, int H, int d);
 cudaError_t launch_bwd_scan(const void *q, const void *k, const void *v, const float *log_alpha, const float *eta,

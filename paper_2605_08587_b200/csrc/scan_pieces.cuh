@@ -1,4 +1,4 @@
-// Warp-level pieces shared by the token-by-token kernels (dg_scan.cu, bwd_scan.cu): one warp owns WC columns of a
+// Warp-level pieces shared by the token-by-token kernels (token_scan.cu, bwd_scan.cu): one warp owns WC columns of a
 // d x d state, lane l holds rows l, l + 32, ... of those columns in registers.
 #pragma once
 #include "common.cuh"
