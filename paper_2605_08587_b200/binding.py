@@ -2,7 +2,8 @@
 
 PyTorch supplies device memory and the current stream; every arithmetic step of the path runs in
 the library's CUDA kernels.  There is no fallback: a missing library raises at import of the
-symbols, and a non-zero status raises `KlaError`.
+symbols, and a non-zero status raises `KlaError`.  The forward and decode calls marshal in native code (csrc/host.cpp, `_host`):
+through ctypes they took 16 us of host time, more than a decode step takes on the device.
 """
 import ctypes
 import os
@@ -44,6 +45,7 @@ class KlaDesc(ctypes.Structure):
 
 
 _lib = None
+_host = None   # native marshalling (csrc/host.cpp), imported by load()
 
 
 def load():
@@ -88,6 +90,10 @@ def load():
     lib.kla_status_str.argtypes = [ctypes.c_int]
     lib.kla_launch_count.restype = ctypes.c_uint64
     lib.kla_launch_count.argtypes = []
+    global _host
+    from . import _host as host   # linked against the library above
+    host.init(KlaError, _status_for)
+    _host = host
     _lib = lib
     return lib
 
@@ -127,7 +133,9 @@ _own_status = {}   # device index -> int32[1] the binding passes as status word 
 
 
 def _status_for(dev):
-    i = torch.device(dev).index
+    if dev in _own_status:
+        return _own_status[dev]
+    i = dev if isinstance(dev, int) else torch.device(dev).index
     i = torch.cuda.current_device() if i is None else i
     if i not in _own_status:
         _own_status[i] = torch.zeros(1, dtype=torch.int32, device="cuda:%d" % i)
@@ -168,7 +176,12 @@ def kla_chunk_fwd(q, k, v, log_alpha, eta, eps, chunk=64, init_state=None, out=N
     `pass_ms`: a list; if given the call goes through kla_chunk_fwd_timed (which waits for the stream) and the four
     per-pass device times in ms (set-up, segment pass 1, chaining, main pass) are appended to it.
     """
-    lib = load()
+    lib = _lib or load()
+    if pass_ms is None and plan_word is None:
+        if cu_seqlens is not None and host_seqlens is None:
+            host_seqlens = cu_seqlens.cpu()
+        return _host.forward(q, k, v, log_alpha, eta, eps, chunk, init_state, out, final_state, cu_seqlens, host_seqlens, out_dtype,
+                             flags, want_final_state, status_word, 0)
     B, T, H, d_k = q.shape
     d_v = v.shape[-1]
     if tuple(k.shape) != (B, T, H, d_k) or tuple(v.shape) != (B, T, H, d_v):
@@ -291,72 +304,32 @@ def kla_state_chain(phi, n, init_state=None):
     return start
 
 
-def _decode_desc(q, v, out, B, H, d_k, d_v, flags=0):
-    return KlaDesc(B=B, T=1, H=H, d_k=d_k, d_v=d_v, n_seq=B, cu_seqlens=None, host_seqlens=None,
-                   io_dtype=_dt(q), out_dtype=_dt(out), flags=flags, workspace=None, workspace_bytes=0,
-                   status_word=None, stream=_stream(q.device))
-
-
 def kla_decode_step(q, k, v, log_alpha, eta, eps, state_inout, out=None, out_dtype=None, flags=KLA_FLAG_NONE):
     """One decode step (include/kla.h: kla_decode_step).  q, k [B, H, d_k]; v [B, H, d_v];
     log_alpha, eta [B, H] fp32; state_inout [B, H, d_k, d_v] fp32, updated in place."""
-    lib = load()
-    B, H, d_k = q.shape
-    d_v = v.shape[-1]
-    if out is None:
-        out = torch.empty((B, H, d_v), device=q.device, dtype=out_dtype or q.dtype)
-    desc = _decode_desc(q, v, out, B, H, d_k, d_v, flags)
-    with torch.cuda.device(q.device):
-        code = lib.kla_decode_step(ctypes.byref(desc), _dev(q, "q"), _dev(k, "k"), _dev(v, "v"),
-                                   _dev(log_alpha, "log_alpha", torch.float32), _dev(eta, "eta", torch.float32),
-                                   float(eps), _dev(state_inout, "state_inout", torch.float32), _dev(out, "out"))
-    _check(code)
-    return out
+    if _host is None:
+        load()
+    return _host.decode(q, k, v, log_alpha, eta, eps, state_inout, out, out_dtype, flags, 0)
 
 
 def kla_decode_steps(q, k, v, log_alpha, eta, eps, state_inout, out=None, out_dtype=None, flags=KLA_FLAG_NONE):
     """n consecutive decode steps (include/kla.h: kla_decode_steps).  q, k [n, B, H, d_k];
     v [n, B, H, d_v]; log_alpha, eta [n, B, H]; state carried in place; out [n, B, H, d_v]."""
-    lib = load()
-    n, B, H, d_k = q.shape
-    d_v = v.shape[-1]
-    if out is None:
-        out = torch.empty((n, B, H, d_v), device=q.device, dtype=out_dtype or q.dtype)
-    desc = _decode_desc(q, v, out, B, H, d_k, d_v, flags)
-    with torch.cuda.device(q.device):
-        code = lib.kla_decode_steps(ctypes.byref(desc), n, _dev(q, "q"), _dev(k, "k"), _dev(v, "v"),
-                                    _dev(log_alpha, "log_alpha", torch.float32), _dev(eta, "eta", torch.float32),
-                                    float(eps), _dev(state_inout, "state_inout", torch.float32), _dev(out, "out"))
-    _check(code)
-    return out
+    if _host is None:
+        load()
+    return _host.decode(q, k, v, log_alpha, eta, eps, state_inout, out, out_dtype, flags, 1)
 
 
 def kla_dg_fwd(q, k, v, log_alpha, eta, eps, init_state=None, out=None, final_state=None, cu_seqlens=None, host_seqlens=None,
                out_dtype=None, flags=KLA_FLAG_NONE, want_final_state=True):
     """Diagonal-gated forward (include/kla.h: kla_dg_fwd): as kla_chunk_fwd with log_alpha [B, T, H, d_k], one decay per
     row of the state.  Returns (out, final_state)."""
-    lib = load()
-    B, T, H, d_k = q.shape
-    d_v = v.shape[-1]
-    if tuple(log_alpha.shape) != (B, T, H, d_k) or tuple(eta.shape) != (B, T, H):
-        raise ValueError("log_alpha must be [B, T, H, d_k] and eta [B, T, H]")
-    n_seq, hs = B, None
-    if cu_seqlens is not None:
-        hs = (cu_seqlens.cpu() if host_seqlens is None else host_seqlens).contiguous()
-        n_seq = cu_seqlens.numel() - 1
-    if out is None:
-        out = torch.empty((B, T, H, d_v), device=q.device, dtype=out_dtype or q.dtype)
-    if final_state is None and want_final_state:
-        final_state = torch.empty((n_seq, H, d_k, d_v), device=q.device, dtype=torch.float32)
-    desc = KlaDesc(B=B, T=T, H=H, d_k=d_k, d_v=d_v, n_seq=n_seq, cu_seqlens=_dev(cu_seqlens, "cu_seqlens"),
-                   host_seqlens=hs.data_ptr() if hs is not None else None, io_dtype=_dt(q), out_dtype=_dt(out), flags=flags,
-                   workspace=None, workspace_bytes=0, status_word=None, stream=_stream(q.device))
-    with torch.cuda.device(q.device):
-        code = lib.kla_dg_fwd(ctypes.byref(desc), _dev(q, "q"), _dev(k, "k"), _dev(v, "v"), _dev(log_alpha, "log_alpha", torch.float32),
-                              _dev(eta, "eta", torch.float32), float(eps), _dev(init_state, "init_state", torch.float32),
-                              _dev(out, "out"), _dev(final_state, "final_state", torch.float32))
-    _check(code)
-    return out, final_state
+    if _host is None:
+        load()
+    if cu_seqlens is not None and host_seqlens is None:
+        host_seqlens = cu_seqlens.cpu()
+    return _host.forward(q, k, v, log_alpha, eta, eps, 64, init_state, out, final_state, cu_seqlens, host_seqlens, out_dtype, flags,
+                         want_final_state, None, 1)
 
 
 def kla_bwd(q, k, v, log_alpha, eta, eps, d_out, init_state=None, d_final_state=None, cu_seqlens=None, host_seqlens=None,
@@ -399,15 +372,6 @@ def kla_bwd(q, k, v, log_alpha, eta, eps, d_out, init_state=None, d_final_state=
 
 def kla_dg_decode_step(q, k, v, log_alpha, eta, eps, state_inout, out=None, out_dtype=None, flags=KLA_FLAG_NONE):
     """One diagonal-gated decode step (include/kla.h: kla_dg_decode_step): log_alpha [B, H, d_k]; state updated in place."""
-    lib = load()
-    B, H, d_k = q.shape
-    d_v = v.shape[-1]
-    if out is None:
-        out = torch.empty((B, H, d_v), device=q.device, dtype=out_dtype or q.dtype)
-    desc = _decode_desc(q, v, out, B, H, d_k, d_v, flags)
-    with torch.cuda.device(q.device):
-        code = lib.kla_dg_decode_step(ctypes.byref(desc), _dev(q, "q"), _dev(k, "k"), _dev(v, "v"),
-                                      _dev(log_alpha, "log_alpha", torch.float32), _dev(eta, "eta", torch.float32), float(eps),
-                                      _dev(state_inout, "state_inout", torch.float32), _dev(out, "out"))
-    _check(code)
-    return out
+    if _host is None:
+        load()
+    return _host.decode(q, k, v, log_alpha, eta, eps, state_inout, out, out_dtype, flags, 2)
