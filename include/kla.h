@@ -292,11 +292,13 @@ kla_status kla_dg_decode_step(const kla_desc *desc, const void *q, const void *k
  *   d_final_state  [n_seq, H, d_k, d_v] fp32, dL/dfinal_state, or NULL for zeros
  *   dq, dk         [B, T, H, d_k] fp32; dv [B, T, H, d_v] fp32; dlog_alpha, deta [B, T, H] fp32: fully overwritten
  *   dinit_state    [n_seq, H, d_k, d_v] fp32, dL/dinit_state, or NULL to skip; an empty sequence gets d_final_state
- * All arithmetic is fp32 on CUDA cores.  The forward states are not an input: they are recomputed (a state is kept every
- * 16 tokens on a forward sweep, the ones in between are re-run when the reverse sweep reaches them), which needs
- * desc->workspace of kla_bwd_workspace_bytes(desc) bytes: (B T / 16 + n_seq) x H x d_k x d_v fp32 for the kept states,
- * 16 x 64 x d_k fp32 of scratch per resident thread block (at most one per SM) and 256 bytes (host function; it reads
- * the current device's SM count when a device is present; 0 for an invalid descriptor).  Errors as kla_chunk_fwd.
+ * The arithmetic is that of fp32.  bf16 inputs: chunk by chunk (64 tokens) on the tensor cores, every derived operand as three
+ * bf16 values (24 significand bits), fp32 accumulation.  fp32 inputs: token by token on CUDA cores.  The forward states are not
+ * an input: they are recomputed, which needs desc->workspace of kla_bwd_workspace_bytes(desc) bytes, the larger of
+ *   (B T / 64 + n_seq) x H x (24 KB + 512 d_k + 8 d_k d_v + 2 KB) plus 4 bytes per sequence (bf16), and
+ *   (B T / 16 + n_seq) x H x d_k x d_v fp32, 16 x 64 x d_k fp32 per resident thread block (at most one per SM), 256 bytes (fp32)
+ * (host function; it reads the current device's SM count when a device is present; 0 for an invalid descriptor).  Errors as
+ * kla_chunk_fwd.
  */
 size_t kla_bwd_workspace_bytes(const kla_desc *desc);
 kla_status kla_bwd(const kla_desc *desc, const void *q, const void *k, const void *v,

@@ -543,7 +543,11 @@ kla_status kla_dg_decode_step(const kla_desc *desc, const void *q, const void *k
 size_t kla_bwd_workspace_bytes(const kla_desc *desc)
 {
     if (check_common(desc) != KLA_OK || desc->n_seq < 1) return 0;
-    return bwd_workspace_bytes(desc->n_seq, (long long)desc->B * desc->T, desc->H, desc->d_k);
+    // (one size for both kernels, whichever the dtype selects)
+    const long long n_tok = (long long)desc->B * desc->T;
+    const size_t a = bwd_scan_workspace_bytes(desc->n_seq, n_tok, desc->H, desc->d_k);
+    const size_t b = bwd_chunk_workspace_bytes(desc->n_seq, n_tok, desc->H, desc->d_k);
+    return a > b ? a : b;
 }
 
 kla_status kla_bwd(const kla_desc *desc, const void *q, const void *k, const void *v,
@@ -564,10 +568,20 @@ kla_status kla_bwd(const kla_desc *desc, const void *q, const void *k, const voi
     st = check_arch();
     if (st != KLA_OK) return st;
     cudaStream_t stream = (cudaStream_t)desc->stream;
-    return launch_bwd_scan(q, k, v, log_alpha, eta, init_state, d_out, d_final_state, dq, dk, dv, dlog_alpha, deta, dinit_state,
-                           desc->workspace, desc->cu_seqlens, desc->T, (long long)desc->B * desc->T, desc->H, desc->n_seq,
-                           desc->d_k, eps, (desc->flags & KLA_FLAG_COEFF_ETA) ? 1 : 0, (desc->flags & KLA_FLAG_QNORM) ? 1 : 0,
-                           desc->io_dtype, stream) == cudaSuccess ? KLA_OK : KLA_ERR_LAUNCH;
+    BwdArgs a;
+    a.q = q; a.k = k; a.v = v; a.dout = d_out;
+    a.log_alpha = log_alpha; a.eta = eta;
+    a.init_state = init_state; a.dfinal = d_final_state;
+    a.dq = dq; a.dk = dk; a.dv = dv; a.dlog_alpha = dlog_alpha; a.deta = deta; a.dinit = dinit_state;
+    a.workspace = desc->workspace;
+    a.cu_seqlens = desc->cu_seqlens;
+    a.T = desc->T; a.H = desc->H; a.n_seq = desc->n_seq; a.d = desc->d_k;
+    a.n_tok = (long long)desc->B * desc->T;
+    a.eps = eps;
+    a.coeff_eta = (desc->flags & KLA_FLAG_COEFF_ETA) ? 1 : 0;
+    a.qnorm = (desc->flags & KLA_FLAG_QNORM) ? 1 : 0;
+    const cudaError_t err = desc->io_dtype == KLA_BF16 ? launch_bwd_chunk(a, stream) : launch_bwd_scan(a, stream);
+    return err == cudaSuccess ? KLA_OK : KLA_ERR_LAUNCH;
 }
 
 const char *kla_status_str(kla_status s)

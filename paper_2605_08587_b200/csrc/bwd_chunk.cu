@@ -1,0 +1,1080 @@
+// Reverse-mode derivative of the KLA recurrence, chunkwise (bf16 inputs).  The paper prints no backward; this is the derivative
+// of its chunk algebra (Eqs. 7-9), which is the derivative of the recurrence of Algorithm 1 left up to the order of the sums.
+//
+// One chunk of 64 tokens, g the chunk-local running sum of log alpha, Gam = diag(exp g_i), D = diag(exp(g_C - g_j)), gC = exp g_C,
+// A_ij = exp(g_i - g_j), X = A^- o K K^T, P = A o Q K^T, B = diag(beta), T = (I + B X)^-1:
+//
+//     forward     R = V - Gam K S_0,  U = T B R,  O = Gam Q S_0 + P U,  S_1 = gC S_0 + K^T D U
+//     backward    dU = P^T dO + D K G_1,  w = T^T dU,  lam = B w (= dV),  G_0 = gC G_1 + (Gam Q)^T dO - (Gam K)^T lam
+//     gradients   dQ = Gam dO S_0^T + F K,               F = A o (dO U^T), lower triangle
+//                 dK = E K - Gam lam S_0^T               E = -A o (lam U^T), strictly lower   ("row" side: k_i as a query)
+//                    + E^T K + F^T Q + D U G_1^T                                              ("column" side: k_j as a key)
+//                    - 2 k dbeta beta / n,  deta = dbeta / n (Eq. 3),  dbeta_i = sum (U / beta)_i o w_i
+//     decay       exp(g_i) multiplies q_i and the row side of k_i, exp(-g_j) the column side of k_j, so
+//                 dg_i = q_i . dq_i + k_i . dk_i(row) - k_i . dk_i(column), dg_C += <G_1, S_1>, dlog_alpha_t = sum_{i >= t} dg_i
+//
+// (G = dL/dS.)  Three launches:
+//   1. prepare   one block per (chunk, head): decays, beta, T (as operand planes), P^T dO, per-token scalars;
+//   2. chains    one block per (sequence, head, 64 columns) and direction: the recurrences over S and over G, each leaving the
+//                state at every chunk (and U, respectively dV) in the workspace; the two do not depend on each other;
+//   3. gradients one block per (chunk, head): everything that is left, in parallel over chunks.
+// Token by token on CUDA cores (bwd_scan.cu, which stays for fp32 inputs) the layer shape took 8.1 ms.
+//
+// beta = 0 (eta = 0) would make U = B (...) carry no trace of the residual e = U / beta that dbeta needs; such a beta is taken
+// as 1e-30, where every gradient has its limit to the last bit.
+#include "common.cuh"
+#include "mma_pieces.cuh"
+#include "scan_pieces.cuh"
+
+namespace kla {
+
+namespace {
+
+using namespace wmm;
+
+constexpr int C = 64;        // chunk length
+constexpr int LDT = 68;      // row stride (floats) of the fp32 solve matrix
+constexpr int LDM = 40;      // row stride of the solve scratch
+constexpr int T_BYTES = 3 * 8192;   // three planes of a 64 x 64 operand
+
+// Per-token scalars of one chunk, as the kernels hand them on.
+struct Scal {
+    float beta[C];   // Eq. 3 (or eta), tokens past the end: 0; never 0 otherwise
+    float gam[C];    // exp(g_i)
+    float dec[C];    // exp(g_C - g_i)
+    float g2h[C], g2l[C];   // log2(e) g_i = g2h + g2l (differences of large sums keep their fp32 digits)
+    float nrm[C];    // ||k||^2 + eps
+    float qinv[C];   // 1 / ||q|| with the normalised read-out, else 1
+    float dn[C];     // used by the gradients: dk_i += dn_i k_i through the norm in Eq. 3
+};
+
+struct BwdChunkParams {
+    const __nv_bfloat16 *q, *k, *v, *dout;
+    const float *log_alpha, *eta;
+    const float *init_state, *dfinal;
+    float *dq, *dk, *dv, *dlog_alpha, *deta, *dinit;
+    const int32_t *cu_seqlens;   // null: fixed length T
+    const int32_t *order;        // packed input: sequences longest first (or null)
+    int32_t T, H, n_seq;
+    float eps;
+    int32_t coeff_eta, qnorm;
+    // workspace, one entry per (slot, head); a slot is a chunk: n ceil(T / 64) + c, packed tok0 / 64 + n + c
+    unsigned char *tpl;   // T as three operand planes, 64 x 64 each, sw128 layout
+    float *pdo;           // (P^T dO)^T  [D][64]
+    float *u;             // U           [64][D]
+    float *s0, *g1;       // S_0^T, G_1^T  [d_v][d_k]
+    Scal *scal;
+    int32_t n_slots;
+};
+
+struct Where {
+    int n, c, tok0, len;   // sequence, chunk of it, its first token, its length
+};
+__device__ __forceinline__ int slot_of(const BwdChunkParams &p, int n, int tok0, int c)
+{
+    return p.cu_seqlens ? tok0 / C + n + c : n * ((p.T + C - 1) / C) + c;
+}
+// The chunk of a slot; c beyond the sequence's chunks: the slot is empty.
+__device__ __forceinline__ Where locate(const BwdChunkParams &p, int slot)
+{
+    Where w;
+    if (!p.cu_seqlens) {
+        const int cps = (p.T + C - 1) / C;
+        w.n = slot / cps;
+        w.c = slot - w.n * cps;
+        w.tok0 = w.n * p.T;
+        w.len = p.T;
+        return w;
+    }
+    int lo = 0, hi = p.n_seq - 1;   // last n with cu[n] / 64 + n <= slot (strictly increasing in n)
+    while (lo < hi) {
+        const int mid = (lo + hi + 1) >> 1;
+        if (p.cu_seqlens[mid] / C + mid <= slot) lo = mid;
+        else hi = mid - 1;
+    }
+    w.n = lo;
+    w.tok0 = p.cu_seqlens[lo];
+    w.len = p.cu_seqlens[lo + 1] - w.tok0;
+    w.c = slot - (w.tok0 / C + lo);
+    return w;
+}
+
+// Rows t0 .. t0 + 63 (of which `rows` exist, the others become zero) of a [token][H][D] array, columns col .. col + 64 NB - 1
+// of head h, into NB consecutive 64 x 64 tiles; all NTH threads.
+template <int NB, int D, int NTH>
+__device__ __forceinline__ void load_tile(uint32_t dst, const __nv_bfloat16 *src, size_t t0, int rows, int H, int h, int col, int tid)
+{
+#pragma unroll
+    for (int e = tid; e < NB * C * 8; e += NTH) {
+        const int r = e / (NB * 8), ch = e % (NB * 8);
+        const int rr = r < rows ? r : 0;
+        cp16(dst + (ch >> 3) * 8192 + sw128(r, ch & 7), src + ((t0 + rr) * H + h) * D + col + ch * 8, r < rows);
+    }
+}
+
+// ---- 1. prepare -----------------------------------------------------------------------------------------------------------
+// One level of the blocked inverse of I + B X (see chunk_tc.cu): for every pair of adjacent inverted BS x BS diagonal blocks the
+// block below the diagonal becomes T_10 = -T_11 (B_1 X_10 T_00).  256 threads, 1 x 4 results each.
+template <int BS>
+__device__ __forceinline__ void merge_level(float *tl, float *mm, const float *bet, int pt)
+{
+    constexpr int QPR = BS / 4;
+    const bool act = pt < 8 * BS;
+    const int R = pt / QPR, c4 = (pt % QPR) * 4;
+    const int pr = R / BS, r = R % BS;
+    const int rb = (2 * pr + 1) * BS, cb = 2 * pr * BS;
+    if (act) {
+        const float *Ap = tl + (rb + r) * LDT + cb, *Bp = tl + cb * LDT + cb + c4;
+        float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll 2
+        for (int k = 0; k < BS; k += 4) {
+            const float4 a = load4(Ap + k);
+            const float av[4] = {a.x, a.y, a.z, a.w};
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const float4 b = load4(Bp + (k + u) * LDT);
+                acc.x += av[u] * b.x; acc.y += av[u] * b.y; acc.z += av[u] * b.z; acc.w += av[u] * b.w;
+            }
+        }
+        const float s = bet[rb + r];
+        store4(&mm[R * LDM + c4], make_float4(s * acc.x, s * acc.y, s * acc.z, s * acc.w));
+    }
+    __syncthreads();
+    if (act) {
+        const float *Ap = tl + (rb + r) * LDT + rb, *Bp = mm + (pr * BS) * LDM + c4;
+        float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll 2
+        for (int k = 0; k <= r; k += 4) {   // T_11 is lower triangular
+            const float4 a = load4(Ap + k);
+            const float av[4] = {a.x, a.y, a.z, a.w};
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const float4 b = load4(Bp + (k + u) * LDM);
+                acc.x += av[u] * b.x; acc.y += av[u] * b.y; acc.z += av[u] * b.z; acc.w += av[u] * b.w;
+            }
+        }
+        store4(&tl[(rb + r) * LDT + cb + c4], make_float4(-acc.x, -acc.y, -acc.z, -acc.w));
+    }
+    __syncthreads();
+}
+
+template <int D>
+struct PrepSmem {
+    alignas(1024) unsigned char k[D / 64 * 8192], q[D / 64 * 8192], dout[D / 64 * 8192];
+    alignas(1024) unsigned char p[T_BYTES];   // P, three planes
+    alignas(16) float tl[C * LDT];            // X, overwritten by T
+    alignas(16) float mm[32 * LDM];
+    Scal s;
+    float eta[C];
+};
+
+template <int D>
+__global__ void __launch_bounds__(256, 2) kla_bwd_prepare_kernel(BwdChunkParams p)
+{
+    extern __shared__ unsigned char smem_dyn[];
+    using Smem = PrepSmem<D>;
+    Smem &sm = *reinterpret_cast<Smem *>((reinterpret_cast<uintptr_t>(smem_dyn) + 1023) & ~(uintptr_t)1023);
+    constexpr int NB = D / 64;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int slot = blockIdx.x / p.H, h = blockIdx.x % p.H;
+    const Where w = locate(p, slot);
+    if (w.c * C >= w.len) return;
+    const int rows = min(C, w.len - w.c * C);
+    const size_t t0 = (size_t)w.tok0 + w.c * C;
+    load_tile<NB, D, 256>(smem_u32(sm.k), p.k, t0, rows, p.H, h, 0, tid);
+    load_tile<NB, D, 256>(smem_u32(sm.q), p.q, t0, rows, p.H, h, 0, tid);
+    cp_commit();
+    load_tile<NB, D, 256>(smem_u32(sm.dout), p.dout, t0, rows, p.H, h, 0, tid);
+    cp_commit();
+
+    if (warp == 0) {   // decay sums in fp64 (tokens 2 lane, 2 lane + 1)
+        const int a = 2 * lane;
+        const double x0 = a < rows ? (double)p.log_alpha[(t0 + a) * p.H + h] : 0.0;
+        const double x1 = a + 1 < rows ? (double)p.log_alpha[(t0 + a + 1) * p.H + h] : 0.0;
+        double incl = x0 + x1;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const double y = __shfl_up_sync(0xffffffffu, incl, o);
+            if (lane >= o) incl += y;
+        }
+        const double gc = __shfl_sync(0xffffffffu, incl, 31);
+        const double g[2] = {incl - x1, incl};
+#pragma unroll
+        for (int u = 0; u < 2; ++u) {
+            sm.s.gam[a + u] = expf((float)g[u]);
+            sm.s.dec[a + u] = expf((float)(gc - g[u]));
+            const double g2 = g[u] * 1.4426950408889634074;
+            sm.s.g2h[a + u] = (float)g2;
+            sm.s.g2l[a + u] = (float)(g2 - (double)(float)g2);
+        }
+    } else if (warp < 3) {
+        const int i = (warp - 1) * 32 + lane;
+        sm.eta[i] = i < rows ? p.eta[(t0 + i) * p.H + h] : 0.f;
+        sm.s.qinv[i] = 1.f;
+        sm.s.dn[i] = 0.f;
+    }
+    for (int e = tid; e < C * LDT; e += 256) sm.tl[e] = 0.f;
+    cp_wait<1>();
+    __syncthreads();
+    if (p.qnorm && tid < C) {
+        float n = 0.f;
+        for (int e = 0; e < NB * 8; ++e) {
+            const uint4 raw = *reinterpret_cast<const uint4 *>(sm.q + (e >> 3) * 8192 + sw128(tid, e & 7));
+            const uint32_t x[4] = {raw.x, raw.y, raw.z, raw.w};
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                const float2 f = unpack(x[u]);
+                n += f.x * f.x + f.y * f.y;
+            }
+        }
+        sm.s.qinv[tid] = tid < rows ? 1.f / sqrtf(n) : 0.f;
+    }
+
+    // K K^T (warps 0..3) and Q K^T (warps 4..7): 16 rows each, columns up to the diagonal block
+    const int mt = warp & 3, i0 = mt * 16;
+    float acc[8][4];
+#pragma unroll
+    for (int t = 0; t < 8; ++t)
+#pragma unroll
+        for (int e = 0; e < 4; ++e) acc[t][e] = 0.f;
+    {
+        const uint32_t at = smem_u32(warp < 4 ? sm.k : sm.q), bt = smem_u32(sm.k);
+#pragma unroll
+        for (int ks = 0; ks < D / 16; ++ks) {
+            const uint32_t off = (ks >> 2) * 8192;
+            uint32_t a[4];
+            frag_a(a, at + off, i0, (ks & 3) * 16, lane);
+#pragma unroll
+            for (int np = 0; np < 4; ++np) {
+                if (np <= mt) {
+                    uint32_t b[4];
+                    frag_b(b, bt + off, (ks & 3) * 16, np * 16, lane);
+                    mma(acc[2 * np], a, b[0], b[1]);
+                    mma(acc[2 * np + 1], a, b[2], b[3]);
+                }
+            }
+        }
+    }
+    // accumulator element (t, e): row i0 + lane / 4 (+ 8 for e >= 2), column 8 t + 2 (lane % 4) + (e & 1)
+    const int r0 = i0 + (lane >> 2), cq = 2 * (lane & 3);
+    if (warp < 4) {
+#pragma unroll
+        for (int t = 0; t < 8; ++t)
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                const int i = r0 + (e >> 1) * 8, j = 8 * t + cq + (e & 1);
+                if (i == j) {   // ||k_i||^2
+                    const float n = acc[t][e] + p.eps;
+                    float b = i < rows ? (p.coeff_eta ? sm.eta[i] : sm.eta[i] / n) : 0.f;
+                    if (i < rows && fabsf(b) < 1e-30f) b = 1e-30f;
+                    sm.s.nrm[i] = n;
+                    sm.s.beta[i] = b;
+                }
+            }
+    }
+    __syncthreads();   // scalars are complete
+    if (warp < 4) {
+#pragma unroll
+        for (int t = 0; t < 8; ++t)
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                const int i = r0 + (e >> 1) * 8, j = 8 * t + cq + (e & 1);
+                if (j < i) sm.tl[i * LDT + j] = exp2f((sm.s.g2h[i] - sm.s.g2h[j]) + (sm.s.g2l[i] - sm.s.g2l[j])) * acc[t][e];
+            }
+    } else {
+#pragma unroll
+        for (int t = 0; t < 8; ++t)
+#pragma unroll
+            for (int e = 0; e < 4; e += 2) {
+                const int i = r0 + (e >> 1) * 8, j = 8 * t + cq;
+                const float hi = sm.s.g2h[i], li = sm.s.g2l[i], qi = sm.s.qinv[i];
+                const float x = j <= i ? qi * exp2f((hi - sm.s.g2h[j]) + (li - sm.s.g2l[j])) * acc[t][e] : 0.f;
+                const float y = j + 1 <= i ? qi * exp2f((hi - sm.s.g2h[j + 1]) + (li - sm.s.g2l[j + 1])) * acc[t][e + 1] : 0.f;
+                uint32_t a, b, c;
+                split3(x, y, a, b, c);
+                const uint32_t off = sw128(i, t) + 4 * (lane & 3);
+                *reinterpret_cast<uint32_t *>(sm.p + off) = a;
+                *reinterpret_cast<uint32_t *>(sm.p + 8192 + off) = b;
+                *reinterpret_cast<uint32_t *>(sm.p + 16384 + off) = c;
+            }
+    }
+    cp_wait<0>();
+    __syncthreads();
+    const size_t ch = (size_t)slot * p.H + h;
+    if (tid < sizeof(Scal) / 16) reinterpret_cast<float4 *>(p.scal + ch)[tid] = reinterpret_cast<const float4 *>(&sm.s)[tid];
+
+    // (P^T dO)^T = dO^T P: 16 rows (columns of V) per warp
+    if (warp * 16 < D) {
+        float o[8][4];
+#pragma unroll
+        for (int t = 0; t < 8; ++t)
+#pragma unroll
+            for (int e = 0; e < 4; ++e) o[t][e] = 0.f;
+        const uint32_t at = smem_u32(sm.dout) + (warp >> 2) * 8192, bt = smem_u32(sm.p);
+#pragma unroll
+        for (int ks = 0; ks < 4; ++ks) {
+            uint32_t a[4];
+            frag_at(a, at, (warp & 3) * 16, ks * 16, lane);
+#pragma unroll
+            for (int pl = 0; pl < 3; ++pl)
+#pragma unroll
+                for (int np = 0; np <= ks; ++np) {
+                    uint32_t b[4];
+                    frag_bt(b, bt + pl * 8192, ks * 16, np * 16, lane);
+                    mma(o[2 * np], a, b[0], b[1]);
+                    mma(o[2 * np + 1], a, b[2], b[3]);
+                }
+        }
+        float *dst = p.pdo + ch * D * C + (size_t)(warp * 16 + (lane >> 2)) * C + cq;
+#pragma unroll
+        for (int t = 0; t < 8; ++t) {
+            store2(dst + 8 * t, o[t][0], o[t][1]);
+            store2(dst + 8 * C + 8 * t, o[t][2], o[t][3]);
+        }
+    }
+
+    // T = (I + B X)^-1: 8 x 8 diagonal blocks by substitution (column tid % 8 of block tid / 8), then block merges
+    const float *bet = sm.s.beta;
+    float x[8];
+    if (tid < 64) {
+        const int blk = tid >> 3, j = tid & 7;
+        const float *Lb = sm.tl + (blk * 8) * LDT + blk * 8;
+#pragma unroll
+        for (int r = 0; r < 8; ++r) {
+            float s = 0.f;
+#pragma unroll
+            for (int m = 0; m < r; ++m) s += Lb[r * LDT + m] * x[m];
+            x[r] = (r == j) ? 1.f : ((r > j) ? -bet[blk * 8 + r] * s : 0.f);
+        }
+    }
+    __syncthreads();
+    if (tid < 64) {
+        const int blk = tid >> 3, j = tid & 7;
+#pragma unroll
+        for (int r = 0; r < 8; ++r) sm.tl[(blk * 8 + r) * LDT + blk * 8 + j] = x[r];
+    }
+    __syncthreads();
+    merge_level<8>(sm.tl, sm.mm, bet, tid);
+    merge_level<16>(sm.tl, sm.mm, bet, tid);
+    merge_level<32>(sm.tl, sm.mm, bet, tid);
+    // T as three operand planes: 8 columns per item
+    unsigned char *tp = p.tpl + ch * T_BYTES;
+#pragma unroll
+    for (int e = tid; e < C * 8; e += 256) {
+        const int r = e >> 3, c8 = e & 7;
+        uint32_t hh[4], mm[4], ll[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) split3(sm.tl[r * LDT + c8 * 8 + 2 * u], sm.tl[r * LDT + c8 * 8 + 2 * u + 1], hh[u], mm[u], ll[u]);
+        const uint32_t off = sw128(r, c8);
+        *reinterpret_cast<uint4 *>(tp + off) = make_uint4(hh[0], hh[1], hh[2], hh[3]);
+        *reinterpret_cast<uint4 *>(tp + 8192 + off) = make_uint4(mm[0], mm[1], mm[2], mm[3]);
+        *reinterpret_cast<uint4 *>(tp + 16384 + off) = make_uint4(ll[0], ll[1], ll[2], ll[3]);
+    }
+}
+
+// ---- 2. chains ------------------------------------------------------------------------------------------------------------
+// Four warps, 16 columns of d_v each; the transposed state (16 x D) stays in registers as accumulator tiles, is split into
+// operand planes on the fly and never leaves the warp.  K is fetched a chunk ahead into the other of two buffers; what a chunk
+// uses last (T, V, respectively T, Q, dO) has one buffer and is fetched as soon as every warp has passed it.
+// What bounds it: the warp-level tensor pipe, 504 (forward) and 696 (backward) instructions per chunk and warp at D = 128.
+// Both directions are one launch so that an SM holds a block of each and one fills the other's latencies.
+template <int D>
+struct ChainSmem {
+    alignas(1024) unsigned char k[2][D / 64 * 8192];
+    alignas(1024) unsigned char t[T_BYTES];
+    alignas(1024) unsigned char vd[8192];            // V (forward), dO (backward): this block's 64 columns
+    alignas(1024) unsigned char q[D / 64 * 8192];    // backward only
+    Scal s[2];
+};
+
+// acc[token tile] = (16 x D state) (64 x D tile)^T: columns are tokens
+template <int D>
+__device__ __forceinline__ void state_times_tile(float (&acc)[8][4], const float (&S)[D / 8][4], uint32_t kt, int lane)
+{
+#pragma unroll
+    for (int t = 0; t < 8; ++t)
+#pragma unroll
+        for (int e = 0; e < 4; ++e) acc[t][e] = 0.f;
+#pragma unroll
+    for (int ks = 0; ks < D / 16; ++ks) {
+        uint32_t a[3][4], b[4][4];
+        split_a(S[2 * ks], S[2 * ks + 1], a[0], a[1], a[2]);
+#pragma unroll
+        for (int np = 0; np < 4; ++np) frag_b(b[np], kt + (ks >> 2) * 8192, (ks & 3) * 16, np * 16, lane);
+#pragma unroll
+        for (int pl = 0; pl < 3; ++pl)
+#pragma unroll
+            for (int np = 0; np < 4; ++np) {
+                mma(acc[2 * np], a[pl], b[np][0], b[np][1]);
+                mma(acc[2 * np + 1], a[pl], b[np][2], b[np][3]);
+            }
+    }
+}
+// S += (16 tokens of a 16 x 64 factor, three planes) (tile)[those tokens][D]
+template <int D>
+__device__ __forceinline__ void state_update(float (&S)[D / 8][4], const uint32_t (&a)[3][4], uint32_t tile, int ks, int lane)
+{
+#pragma unroll
+    for (int np = 0; np < D / 16; np += 2) {
+        uint32_t b[2][4];
+        frag_bt(b[0], tile + (np >> 2) * 8192, ks * 16, (np & 3) * 16, lane);
+        frag_bt(b[1], tile + (np >> 2) * 8192, ks * 16, (np & 3) * 16 + 16, lane);
+#pragma unroll
+        for (int pl = 0; pl < 3; ++pl)
+#pragma unroll
+            for (int u = 0; u < 2; ++u) {
+                mma(S[2 * (np + u)], a[pl], b[u][0], b[u][1]);
+                mma(S[2 * (np + u) + 1], a[pl], b[u][2], b[u][3]);
+            }
+    }
+}
+// three-plane x three-plane product on two tiles, terms down to 2^-24
+__device__ __forceinline__ void mma6(float (&c0)[4], float (&c1)[4], const uint32_t (&a)[3][4], const uint32_t (&b)[3][4])
+{
+    constexpr int PA[6] = {0, 0, 1, 0, 2, 1}, PB[6] = {0, 1, 0, 2, 0, 1};
+#pragma unroll
+    for (int t = 0; t < 6; ++t) {
+        mma(c0, a[PA[t]], b[PB[t]][0], b[PB[t]][1]);
+        mma(c1, a[PA[t]], b[PB[t]][2], b[PB[t]][3]);
+    }
+}
+
+template <int D, bool BWD>
+__device__ __forceinline__ void chain(const BwdChunkParams &p, ChainSmem<D> &sm, int unit)
+{
+    constexpr int NB = D / 64;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int sl = unit % NB, h = (unit / NB) % p.H;
+    int n = unit / (NB * p.H);
+    if (p.order) n = p.order[n];
+    int tok0, len;
+    if (p.cu_seqlens) {
+        tok0 = p.cu_seqlens[n];
+        len = p.cu_seqlens[n + 1] - tok0;
+    } else {
+        tok0 = n * p.T;
+        len = p.T;
+    }
+    const int nc = (len + C - 1) / C;
+    const int r = lane >> 2, cq = 2 * (lane & 3);
+    const int col = sl * 64 + warp * 16 + r;   // columns col, col + 8 of d_v
+    // element (t, e) of a state tile: column col (+ 8 for e >= 2), row 8 t + cq + (e & 1)
+    float S[D / 8][4];
+    {
+        const float *src = BWD ? p.dfinal : p.init_state;
+        const size_t base = ((size_t)n * p.H + h) * D * D + col;
+#pragma unroll
+        for (int t = 0; t < D / 8; ++t)
+#pragma unroll
+            for (int e = 0; e < 4; ++e) S[t][e] = src ? src[base + (size_t)(8 * t + cq + (e & 1)) * D + (e >> 1) * 8] : 0.f;
+    }
+    const size_t ch0 = (size_t)slot_of(p, n, tok0, 0) * p.H + h;   // chunk c: + c H
+    auto rows_of = [&](int c) { return min(C, len - c * C); };
+    auto load_k = [&](int c) {
+        load_tile<NB, D, 128>(smem_u32(sm.k[c & 1]), p.k, (size_t)tok0 + c * C, rows_of(c), p.H, h, 0, tid);
+        cp16(smem_u32(&sm.s[c & 1]) + tid * 16, reinterpret_cast<const char *>(p.scal + ch0 + (size_t)c * p.H) + tid * 16, true);
+    };
+    auto load_t = [&](int c) {
+        const unsigned char *src = p.tpl + (ch0 + (size_t)c * p.H) * T_BYTES;
+#pragma unroll
+        for (int e = tid; e < T_BYTES / 16; e += 128) cp16(smem_u32(sm.t) + e * 16, src + e * 16, true);
+    };
+    auto load_vd = [&](int c) {
+        load_tile<1, D, 128>(smem_u32(sm.vd), BWD ? p.dout : p.v, (size_t)tok0 + c * C, rows_of(c), p.H, h, sl * 64, tid);
+    };
+    const int step = BWD ? -1 : 1;
+    int c = BWD ? nc - 1 : 0;
+    if (nc > 0) {
+        load_k(c);
+        load_t(c);
+        if (!BWD) load_vd(c);
+        cp_commit();
+    }
+    for (int it = 0; it < nc; ++it, c += step) {
+        const Scal &s = sm.s[c & 1];
+        const size_t ch = ch0 + (size_t)c * p.H;
+        const uint32_t kt = smem_u32(sm.k[c & 1]), tt = smem_u32(sm.t);
+        cp_wait<0>();
+        __syncthreads();
+        if (BWD) {
+            load_vd(c);
+            load_tile<NB, D, 128>(smem_u32(sm.q), p.q, (size_t)tok0 + c * C, rows_of(c), p.H, h, 0, tid);
+            cp_commit();
+        }
+        if (it + 1 < nc) load_k(c + step);
+        cp_commit();
+        // the state at this end of the chunk, transposed
+        {
+            float *dst = (BWD ? p.g1 : p.s0) + ch * D * D + (size_t)col * D + cq;
+#pragma unroll
+            for (int t = 0; t < D / 8; ++t) {
+                store2(dst + 8 * t, S[t][0], S[t][1]);
+                store2(dst + 8 * D + 8 * t, S[t][2], S[t][3]);
+            }
+        }
+        float2 pd[BWD ? 8 : 1][2];
+        if constexpr (BWD) {
+            const float *src = p.pdo + ch * D * C + (size_t)col * C + cq;
+#pragma unroll
+            for (int t = 0; t < 8; ++t) {
+                pd[t][0] = *reinterpret_cast<const float2 *>(src + 8 * t);
+                pd[t][1] = *reinterpret_cast<const float2 *>(src + 8 * C + 8 * t);
+            }
+        }
+        float x[8][4], y[8][4];
+        state_times_tile<D>(x, S, kt, lane);   // (K S_0)^T or (K G_1)^T
+        if constexpr (BWD) {   // dU = D K G_1 + P^T dO
+#pragma unroll
+            for (int t = 0; t < 8; ++t) {
+                const float2 d = *reinterpret_cast<const float2 *>(&s.dec[8 * t + cq]);
+                x[t][0] = d.x * x[t][0] + pd[t][0].x;
+                x[t][1] = d.y * x[t][1] + pd[t][0].y;
+                x[t][2] = d.x * x[t][2] + pd[t][1].x;
+                x[t][3] = d.y * x[t][3] + pd[t][1].y;
+            }
+        } else {   // B (V - Gam K S_0)
+#pragma unroll
+            for (int tp = 0; tp < 4; ++tp) {
+                uint32_t vv[4];
+                ldsm4t(vv, smem_u32(sm.vd) + sw128(tp * 16 + (lane & 7) + (lane >> 4) * 8, warp * 2 + ((lane >> 3) & 1)));
+#pragma unroll
+                for (int u = 0; u < 2; ++u) {
+                    const int t = 2 * tp + u;
+                    const float2 b = *reinterpret_cast<const float2 *>(&s.beta[8 * t + cq]), g = *reinterpret_cast<const float2 *>(&s.gam[8 * t + cq]);
+                    const float2 v0 = unpack(vv[2 * u]), v1 = unpack(vv[2 * u + 1]);
+                    x[t][0] = b.x * (v0.x - g.x * x[t][0]);
+                    x[t][1] = b.y * (v0.y - g.y * x[t][1]);
+                    x[t][2] = b.x * (v1.x - g.x * x[t][2]);
+                    x[t][3] = b.y * (v1.y - g.y * x[t][3]);
+                }
+            }
+        }
+        // U^T = rhs^T T^T (T_ij, j <= i) or w^T = dU^T T
+#pragma unroll
+        for (int t = 0; t < 8; ++t)
+#pragma unroll
+            for (int e = 0; e < 4; ++e) y[t][e] = 0.f;
+#pragma unroll
+        for (int ks = 0; ks < 4; ++ks) {
+            uint32_t a[3][4];
+            split_a(x[2 * ks], x[2 * ks + 1], a[0], a[1], a[2]);
+#pragma unroll
+            for (int np = BWD ? 0 : ks; np <= (BWD ? ks : 3); ++np) {
+                uint32_t b[3][4];
+#pragma unroll
+                for (int pl = 0; pl < 3; ++pl) {
+                    if (BWD) frag_bt(b[pl], tt + pl * 8192, ks * 16, np * 16, lane);
+                    else frag_b(b[pl], tt + pl * 8192, ks * 16, np * 16, lane);
+                }
+                mma6(y[2 * np], y[2 * np + 1], a, b);
+            }
+        }
+        if (BWD) cp_wait<1>();   // Q and dO have landed
+        __syncthreads();         // every warp is done with T (and V)
+        if (it + 1 < nc) {
+            load_t(c + step);
+            if (!BWD) load_vd(c + step);
+        }
+        cp_commit();
+        const int rows = rows_of(c);
+        const float gc = s.gam[C - 1];
+        if constexpr (BWD) {   // lam = B w
+            float *dst = p.dv + (((size_t)tok0 + c * C + cq) * p.H + h) * D + col;
+            const size_t row = (size_t)p.H * D;
+#pragma unroll
+            for (int t = 0; t < 8; ++t) {
+                const float2 b = *reinterpret_cast<const float2 *>(&s.beta[8 * t + cq]), g = *reinterpret_cast<const float2 *>(&s.gam[8 * t + cq]);
+                y[t][0] *= b.x; y[t][1] *= b.y; y[t][2] *= b.x; y[t][3] *= b.y;
+                if (8 * t + cq < rows) {
+                    dst[(8 * t) * row] = y[t][0];
+                    dst[(8 * t) * row + 8] = y[t][2];
+                }
+                if (8 * t + cq + 1 < rows) {
+                    dst[(8 * t + 1) * row] = y[t][1];
+                    dst[(8 * t + 1) * row + 8] = y[t][3];
+                }
+                y[t][0] *= -g.x; y[t][1] *= -g.y; y[t][2] *= -g.x; y[t][3] *= -g.y;
+            }
+        } else {
+            float *dst = p.u + ch * C * D + (size_t)cq * D + col;
+#pragma unroll
+            for (int t = 0; t < 8; ++t) {
+                const float2 d = *reinterpret_cast<const float2 *>(&s.dec[8 * t + cq]);
+                dst[(8 * t) * D] = y[t][0];
+                dst[(8 * t) * D + 8] = y[t][2];
+                dst[(8 * t + 1) * D] = y[t][1];
+                dst[(8 * t + 1) * D + 8] = y[t][3];
+                y[t][0] *= d.x; y[t][1] *= d.y; y[t][2] *= d.x; y[t][3] *= d.y;
+            }
+        }
+#pragma unroll
+        for (int t = 0; t < D / 8; ++t)
+#pragma unroll
+            for (int e = 0; e < 4; ++e) S[t][e] *= gc;
+#pragma unroll
+        for (int ks = 0; ks < 4; ++ks) {   // += (D U)^T K, or -= (Gam lam)^T K
+            uint32_t a[3][4];
+            split_a(y[2 * ks], y[2 * ks + 1], a[0], a[1], a[2]);
+            state_update<D>(S, a, kt, ks, lane);
+        }
+        if constexpr (BWD) {
+#pragma unroll
+            for (int ks = 0; ks < 4; ++ks) {   // += dO^T (Gam Q): the decay goes with dO, in registers
+                uint32_t d[4], a[3][4];
+                frag_at(d, smem_u32(sm.vd), warp * 16, ks * 16, lane);
+                // registers: (row r, tokens cq, cq + 1), (row r + 8, ...), then tokens + 8
+#pragma unroll
+                for (int e = 0; e < 4; ++e) {
+                    const int tk = ks * 16 + cq + (e >> 1) * 8;
+                    const float2 f = unpack(d[e]), g = *reinterpret_cast<const float2 *>(&s.gam[tk]), qi = *reinterpret_cast<const float2 *>(&s.qinv[tk]);
+                    split3(f.x * (g.x * qi.x), f.y * (g.y * qi.y), a[0][e], a[1][e], a[2][e]);
+                }
+                state_update<D>(S, a, smem_u32(sm.q), ks, lane);
+            }
+        }
+    }
+    if (BWD && p.dinit) {
+        float *dst = p.dinit + ((size_t)n * p.H + h) * D * D + col;
+#pragma unroll
+        for (int t = 0; t < D / 8; ++t)
+#pragma unroll
+            for (int e = 0; e < 4; ++e) dst[(size_t)(8 * t + cq + (e & 1)) * D + (e >> 1) * 8] = S[t][e];
+    }
+}
+
+template <int D>
+__global__ void __launch_bounds__(128, 2) kla_bwd_chain_kernel(BwdChunkParams p, int n_units)
+{
+    extern __shared__ unsigned char smem_dyn[];
+    ChainSmem<D> &sm = *reinterpret_cast<ChainSmem<D> *>((reinterpret_cast<uintptr_t>(smem_dyn) + 1023) & ~(uintptr_t)1023);
+    // the backward chains, the longer ones, first
+    if ((int)blockIdx.x < n_units) chain<D, true>(p, sm, blockIdx.x);
+    else chain<D, false>(p, sm, blockIdx.x - n_units);
+}
+
+// ---- 3. gradients ---------------------------------------------------------------------------------------------------------
+// One block of eight warps per (chunk, head).  Output columns (d_k) are taken in halves of 64: the operand planes of S_0, then
+// of G_1, of one half share a buffer.  A warp owns 16 tokens x 32 columns; operands that two products have in common are
+// loaded once for both.  Global loads of the next operand are requested before the products of the one at hand.
+template <int D>
+struct GradSmem {
+    unsigned char dout[D / 64 * 8192];            // [token][d_v]
+    unsigned char u[D / 64 * T_BYTES];            // planes, [token][d_v] (plane pl, block b at (pl NB + b) 8192)
+    unsigned char lam[D / 64 * T_BYTES];
+    unsigned char f[T_BYTES], e[T_BYTES];         // planes, [i][j]; only blocks on and below the diagonal are used
+    unsigned char sg[3 * D * 128];                // S_0^T or G_1^T, planes, [d_v][64 of d_k]
+    unsigned char k[8192], q[8192];               // [token][64 of d_k]
+    Scal s;
+    float red[2][64];                             // dg_i, the parts of the two column halves of the warps
+    float gs[8];                                  // <G_1, S_1> of the warps
+};
+
+template <int D>
+__global__ void __launch_bounds__(256, 1) kla_bwd_grad_kernel(BwdChunkParams p)
+{
+    constexpr int NB = D / 64, IT = D / 32;   // 8-column items of a [D][64] fp32 matrix per thread
+    extern __shared__ __align__(128) unsigned char smem_dyn[];
+    GradSmem<D> &sm = *reinterpret_cast<GradSmem<D> *>(smem_dyn);
+    static_assert(sizeof(GradSmem<D>) <= 232448, "shared memory of one block");
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int slot = blockIdx.x / p.H, h = blockIdx.x % p.H;
+    const Where w = locate(p, slot);
+    if (w.c * C >= w.len) return;
+    const int rows = min(C, w.len - w.c * C);
+    const size_t t0 = (size_t)w.tok0 + w.c * C, ch = (size_t)slot * p.H + h;
+    load_tile<NB, D, 256>(smem_u32(sm.dout), p.dout, t0, rows, p.H, h, 0, tid);
+    if (tid < (int)sizeof(Scal) / 16) cp16(smem_u32(&sm.s) + tid * 16, reinterpret_cast<const char *>(p.scal + ch) + tid * 16, true);
+    cp_commit();
+
+    // S_0^T / G_1^T: rows d_v, 64 columns of d_k from 64 hh on
+    float4 ps[IT][2], pg[IT][2];
+    auto fetch = [&](float4 (&pre)[IT][2], const float *src, int hh) {
+#pragma unroll
+        for (int i = 0; i < IT; ++i) {
+            const int e = tid + i * 256, r = e >> 3, c8 = e & 7;
+            const float *x = src + ch * D * D + (size_t)r * D + hh * 64 + c8 * 8;
+            pre[i][0] = load4(x);
+            pre[i][1] = load4(x + 4);
+        }
+    };
+    auto put8 = [&](unsigned char *dst, int plane, uint32_t off, const float4 &a, const float4 &b) {
+        uint32_t hh[4], mm[4], ll[4];
+        split3(a.x, a.y, hh[0], mm[0], ll[0]);
+        split3(a.z, a.w, hh[1], mm[1], ll[1]);
+        split3(b.x, b.y, hh[2], mm[2], ll[2]);
+        split3(b.z, b.w, hh[3], mm[3], ll[3]);
+        *reinterpret_cast<uint4 *>(dst + off) = make_uint4(hh[0], hh[1], hh[2], hh[3]);
+        *reinterpret_cast<uint4 *>(dst + plane + off) = make_uint4(mm[0], mm[1], mm[2], mm[3]);
+        *reinterpret_cast<uint4 *>(dst + 2 * plane + off) = make_uint4(ll[0], ll[1], ll[2], ll[3]);
+    };
+    auto commit = [&](const float4 (&pre)[IT][2]) {
+#pragma unroll
+        for (int i = 0; i < IT; ++i) {
+            const int e = tid + i * 256;
+            put8(sm.sg, D * 128, sw128(e >> 3, e & 7), pre[i][0], pre[i][1]);
+        }
+    };
+
+    // U and lam as operand planes; dbeta_i = (U_i / beta_i) . (lam_i / beta_i)
+    {
+        float4 a[NB * 2][4];
+#pragma unroll
+        for (int i = 0; i < NB * 2; ++i) {
+            const int e = tid + i * 256, r = e / (D / 8), c8 = e % (D / 8);
+            const float *x = p.u + ch * C * D + (size_t)r * D + c8 * 8;
+            const float *y = p.dv + ((t0 + (r < rows ? r : 0)) * p.H + h) * D + c8 * 8;
+            a[i][0] = load4(x);
+            a[i][1] = load4(x + 4);
+            a[i][2] = load4(y);
+            a[i][3] = load4(y + 4);
+        }
+        fetch(ps, p.s0, 0);
+        cp_wait<0>();
+        __syncthreads();   // scalars (and dO) are there
+#pragma unroll
+        for (int i = 0; i < NB * 2; ++i) {
+            const int e = tid + i * 256, r = e / (D / 8), c8 = e % (D / 8);
+            if (r >= rows) a[i][0] = a[i][1] = a[i][2] = a[i][3] = make_float4(0.f, 0.f, 0.f, 0.f);
+            const uint32_t off = (c8 >> 3) * 8192 + sw128(r, c8 & 7);
+            put8(sm.u, NB * 8192, off, a[i][0], a[i][1]);
+            put8(sm.lam, NB * 8192, off, a[i][2], a[i][3]);
+            const float bi = r < rows ? 1.f / sm.s.beta[r] : 0.f;
+            float d = (a[i][0].x * bi) * (a[i][2].x * bi) + (a[i][0].y * bi) * (a[i][2].y * bi) + (a[i][0].z * bi) * (a[i][2].z * bi) +
+                      (a[i][0].w * bi) * (a[i][2].w * bi) + (a[i][1].x * bi) * (a[i][3].x * bi) + (a[i][1].y * bi) * (a[i][3].y * bi) +
+                      (a[i][1].z * bi) * (a[i][3].z * bi) + (a[i][1].w * bi) * (a[i][3].w * bi);
+#pragma unroll
+            for (int o = D / 16; o > 0; o >>= 1) d += __shfl_xor_sync(0xffffffffu, d, o);
+            if (c8 == 0) {
+                const float de = p.coeff_eta ? d : d / sm.s.nrm[r];
+                if (r < rows) p.deta[(t0 + r) * p.H + h] = de;
+                sm.s.dn[r] = p.coeff_eta ? 0.f : -2.f * de * sm.s.beta[r];   // dk_i += this x k_i
+            }
+        }
+    }
+    __syncthreads();
+
+    const int r = lane >> 2, cq = 2 * (lane & 3);
+    auto ratio = [&](int i, int j) { return exp2f((sm.s.g2h[i] - sm.s.g2h[j]) + (sm.s.g2l[i] - sm.s.g2l[j])); };
+    // F = qinv A o (dO U^T) (three terms) and E = -A o (lam U^T) (six), in 16 x 16 blocks on and below the diagonal
+    auto block = [&](bool is_e, int blk) {
+        const int bi = blk < 1 ? 0 : blk < 3 ? 1 : blk < 6 ? 2 : 3, bj = blk - bi * (bi + 1) / 2;
+        float c0[4] = {0.f, 0.f, 0.f, 0.f}, c1[4] = {0.f, 0.f, 0.f, 0.f};
+        const uint32_t at = smem_u32(is_e ? sm.lam : sm.dout), bt = smem_u32(sm.u);
+#pragma unroll 2
+        for (int ks = 0; ks < D / 16; ++ks) {
+            const uint32_t o = (ks >> 2) * 8192;
+            uint32_t a[3][4], b[3][4];
+#pragma unroll
+            for (int pl = 0; pl < 3; ++pl) frag_b(b[pl], bt + pl * NB * 8192 + o, (ks & 3) * 16, bj * 16, lane);
+            frag_a(a[0], at + o, bi * 16, (ks & 3) * 16, lane);
+            if (is_e) {
+                frag_a(a[1], at + NB * 8192 + o, bi * 16, (ks & 3) * 16, lane);
+                frag_a(a[2], at + 2 * NB * 8192 + o, bi * 16, (ks & 3) * 16, lane);
+                mma6(c0, c1, a, b);
+            } else {
+#pragma unroll
+                for (int pl = 0; pl < 3; ++pl) {
+                    mma(c0, a[0], b[pl][0], b[pl][1]);
+                    mma(c1, a[0], b[pl][2], b[pl][3]);
+                }
+            }
+        }
+        unsigned char *dst = is_e ? sm.e : sm.f;
+#pragma unroll
+        for (int t = 0; t < 2; ++t)
+#pragma unroll
+            for (int e = 0; e < 4; e += 2) {
+                const int i = bi * 16 + r + (e >> 1) * 8, j = bj * 16 + t * 8 + cq;
+                const float sc = is_e ? -1.f : sm.s.qinv[i];
+                float x = t ? c1[e] : c0[e], y = t ? c1[e + 1] : c0[e + 1];
+                x = (is_e ? j < i : j <= i) ? sc * ratio(i, j) * x : 0.f;
+                y = (is_e ? j + 1 < i : j + 1 <= i) ? sc * ratio(i, j + 1) * y : 0.f;
+                uint32_t hh, mm, ll;
+                split3(x, y, hh, mm, ll);
+                const uint32_t off = sw128(i, bj * 2 + t) + 4 * (lane & 3);
+                *reinterpret_cast<uint32_t *>(dst + off) = hh;
+                *reinterpret_cast<uint32_t *>(dst + 8192 + off) = mm;
+                *reinterpret_cast<uint32_t *>(dst + 16384 + off) = ll;
+            }
+    };
+    // ten blocks of each, an E block costs two F blocks: warps 0, 1 two of E; 2 .. 5 one of E, two of F; 6, 7 one of each
+    block(true, warp);
+    if (warp < 2) block(true, 8 + warp);
+    else if (warp < 6) {
+        block(false, 2 * (warp - 2));
+        block(false, 2 * (warp - 2) + 1);
+    } else block(false, warp + 2);
+
+    const int mt = warp & 3, nh = warp >> 2, i0 = mt * 16;   // this warp's 16 tokens and 32 of the half's 64 columns
+    const int ia = i0 + r, ib = ia + 8;
+    float gs = 0.f;             // this thread's part of <G_1, S_1>
+    float dga = 0.f, dgb = 0.f; // ... of dg of its two rows
+    const float gama = sm.s.gam[ia], gamb = sm.s.gam[ib], deca = sm.s.dec[ia], decb = sm.s.dec[ib], gc = sm.s.gam[C - 1];
+    const float qia = sm.s.qinv[ia], qib = sm.s.qinv[ib];
+    // products x . y of this lane's elements of the two rows, added to a and b
+    auto dot = [&](const unsigned char *tile, const float (&x)[4][4], float &a, float &b) {
+#pragma unroll
+        for (int t = 0; t < 4; ++t) {
+            const float2 fa = unpack(*reinterpret_cast<const uint32_t *>(tile + sw128(ia, nh * 4 + t) + 4 * (lane & 3)));
+            const float2 fb = unpack(*reinterpret_cast<const uint32_t *>(tile + sw128(ib, nh * 4 + t) + 4 * (lane & 3)));
+            a += fa.x * x[t][0] + fa.y * x[t][1];
+            b += fb.x * x[t][2] + fb.y * x[t][3];
+        }
+    };
+    const uint32_t sg = smem_u32(sm.sg), kt = smem_u32(sm.k), qt = smem_u32(sm.q);
+#pragma unroll 1
+    for (int hh = 0; hh < NB; ++hh) {
+        load_tile<1, D, 256>(kt, p.k, t0, rows, p.H, h, hh * 64, tid);
+        load_tile<1, D, 256>(qt, p.q, t0, rows, p.H, h, hh * 64, tid);
+        cp_commit();
+        commit(ps);
+        fetch(pg, p.g1, hh);
+        cp_wait<0>();
+        __syncthreads();   // S_0 planes, K, Q (and, the first time, E and F)
+        float xq[4][4], xk[4][4];
+#pragma unroll
+        for (int t = 0; t < 4; ++t)
+#pragma unroll
+            for (int e = 0; e < 4; ++e) xq[t][e] = xk[t][e] = 0.f;
+        // dO S_0^T and lam S_0^T
+#pragma unroll 2
+        for (int ks = 0; ks < D / 16; ++ks) {
+            const uint32_t o = (ks >> 2) * 8192;
+            uint32_t a[4], l[3][4];
+            frag_a(a, smem_u32(sm.dout) + o, i0, (ks & 3) * 16, lane);
+#pragma unroll
+            for (int pl = 0; pl < 3; ++pl) frag_a(l[pl], smem_u32(sm.lam) + pl * NB * 8192 + o, i0, (ks & 3) * 16, lane);
+#pragma unroll
+            for (int np = 0; np < 2; ++np) {
+                uint32_t b[3][4];
+#pragma unroll
+                for (int pl = 0; pl < 3; ++pl) frag_bt(b[pl], sg + pl * D * 128, ks * 16, nh * 32 + np * 16, lane);
+#pragma unroll
+                for (int pl = 0; pl < 3; ++pl) {
+                    mma(xq[2 * np], a, b[pl][0], b[pl][1]);
+                    mma(xq[2 * np + 1], a, b[pl][2], b[pl][3]);
+                }
+                mma6(xk[2 * np], xk[2 * np + 1], l, b);
+            }
+        }
+#pragma unroll
+        for (int t = 0; t < 4; ++t) {
+            xq[t][0] *= gama * qia; xq[t][1] *= gama * qia; xq[t][2] *= gamb * qib; xq[t][3] *= gamb * qib;
+            xk[t][0] *= -gama; xk[t][1] *= -gama; xk[t][2] *= -gamb; xk[t][3] *= -gamb;
+        }
+        // += F K and E K
+#pragma unroll 1
+        for (int ks = 0; ks <= mt; ++ks) {
+            uint32_t a[3][4], l[3][4];
+#pragma unroll
+            for (int pl = 0; pl < 3; ++pl) {
+                frag_a(a[pl], smem_u32(sm.f) + pl * 8192, i0, ks * 16, lane);
+                frag_a(l[pl], smem_u32(sm.e) + pl * 8192, i0, ks * 16, lane);
+            }
+#pragma unroll
+            for (int np = 0; np < 2; ++np) {
+                uint32_t b[4];
+                frag_bt(b, kt, ks * 16, nh * 32 + np * 16, lane);
+#pragma unroll
+                for (int pl = 0; pl < 3; ++pl) {
+                    mma(xq[2 * np], a[pl], b[0], b[1]);
+                    mma(xq[2 * np + 1], a[pl], b[2], b[3]);
+                    mma(xk[2 * np], l[pl], b[0], b[1]);
+                    mma(xk[2 * np + 1], l[pl], b[2], b[3]);
+                }
+            }
+        }
+        // dq (with the normalised read-out its projection follows below)
+        const size_t ga = ((t0 + ia) * p.H + h) * D + hh * 64 + nh * 32 + cq, gb = ga + (size_t)8 * p.H * D;
+#pragma unroll
+        for (int t = 0; t < 4; ++t) {
+            if (ia < rows) store2(p.dq + ga + 8 * t, xq[t][0], xq[t][1]);
+            if (ib < rows) store2(p.dq + gb + 8 * t, xq[t][2], xq[t][3]);
+        }
+        dot(sm.q, xq, dga, dgb);
+        dot(sm.k, xk, dga, dgb);
+        __syncthreads();   // the S_0 planes have been read
+#pragma unroll
+        for (int i = 0; i < IT; ++i)
+#pragma unroll
+            for (int u = 0; u < 2; ++u)
+                gs += gc * (ps[i][u].x * pg[i][u].x + ps[i][u].y * pg[i][u].y + ps[i][u].z * pg[i][u].z + ps[i][u].w * pg[i][u].w);
+        commit(pg);
+        if (hh + 1 < NB) fetch(ps, p.s0, hh + 1);
+        __syncthreads();
+        // D U G_1^T
+#pragma unroll
+        for (int t = 0; t < 4; ++t)
+#pragma unroll
+            for (int e = 0; e < 4; ++e) xq[t][e] = 0.f;
+#pragma unroll 2
+        for (int ks = 0; ks < D / 16; ++ks) {
+            uint32_t a[3][4];
+#pragma unroll
+            for (int pl = 0; pl < 3; ++pl) frag_a(a[pl], smem_u32(sm.u) + (pl * NB + (ks >> 2)) * 8192, i0, (ks & 3) * 16, lane);
+#pragma unroll
+            for (int np = 0; np < 2; ++np) {
+                uint32_t b[3][4];
+#pragma unroll
+                for (int pl = 0; pl < 3; ++pl) frag_bt(b[pl], sg + pl * D * 128, ks * 16, nh * 32 + np * 16, lane);
+                mma6(xq[2 * np], xq[2 * np + 1], a, b);
+            }
+        }
+#pragma unroll
+        for (int t = 0; t < 4; ++t) {
+            xq[t][0] *= deca; xq[t][1] *= deca; xq[t][2] *= decb; xq[t][3] *= decb;
+        }
+        dot(sm.k, xq, gs, gs);   // <G_1, S_1> = gC <G_1, S_0> + sum_j k_j . (D U G_1^T)_j
+        // += E^T K + F^T Q: rows of this warp are the columns of E and F
+#pragma unroll 1
+        for (int ks = mt; ks < 4; ++ks) {
+            uint32_t a[3][4], l[3][4];
+#pragma unroll
+            for (int pl = 0; pl < 3; ++pl) {
+                frag_at(a[pl], smem_u32(sm.f) + pl * 8192, i0, ks * 16, lane);
+                frag_at(l[pl], smem_u32(sm.e) + pl * 8192, i0, ks * 16, lane);
+            }
+#pragma unroll
+            for (int np = 0; np < 2; ++np) {
+                uint32_t b[4], b2[4];
+                frag_bt(b, qt, ks * 16, nh * 32 + np * 16, lane);
+                frag_bt(b2, kt, ks * 16, nh * 32 + np * 16, lane);
+#pragma unroll
+                for (int pl = 0; pl < 3; ++pl) {
+                    mma(xq[2 * np], a[pl], b[0], b[1]);
+                    mma(xq[2 * np + 1], a[pl], b[2], b[3]);
+                    mma(xq[2 * np], l[pl], b2[0], b2[1]);
+                    mma(xq[2 * np + 1], l[pl], b2[2], b2[3]);
+                }
+            }
+        }
+        float ca = 0.f, cb = 0.f;
+        dot(sm.k, xq, ca, cb);
+        dga -= ca;
+        dgb -= cb;
+        const float na = sm.s.dn[ia], nb = sm.s.dn[ib];
+#pragma unroll
+        for (int t = 0; t < 4; ++t) {
+            const float2 fa = unpack(*reinterpret_cast<const uint32_t *>(sm.k + sw128(ia, nh * 4 + t) + 4 * (lane & 3)));
+            const float2 fb = unpack(*reinterpret_cast<const uint32_t *>(sm.k + sw128(ib, nh * 4 + t) + 4 * (lane & 3)));
+            if (ia < rows) store2(p.dk + ga + 8 * t, xk[t][0] + xq[t][0] + na * fa.x, xk[t][1] + xq[t][1] + na * fa.y);
+            if (ib < rows) store2(p.dk + gb + 8 * t, xk[t][2] + xq[t][2] + nb * fb.x, xk[t][3] + xq[t][3] + nb * fb.y);
+        }
+        __syncthreads();   // K, Q and the planes may be overwritten
+    }
+
+    // dlog_alpha_t = <G_1, S_1> + sum_{i >= t} dg_i
+    dga += __shfl_xor_sync(0xffffffffu, dga, 1);
+    dgb += __shfl_xor_sync(0xffffffffu, dgb, 1);
+    dga += __shfl_xor_sync(0xffffffffu, dga, 2);
+    dgb += __shfl_xor_sync(0xffffffffu, dgb, 2);
+    if ((lane & 3) == 0) {
+        sm.red[nh][ia] = dga;
+        sm.red[nh][ib] = dgb;
+    }
+    gs = warp_sum(gs);
+    if (lane == 0) sm.gs[warp] = gs;
+    __syncthreads();
+    if (warp == 0) {
+        double tot = 0.0;
+#pragma unroll
+        for (int i = 0; i < 8; ++i) tot += (double)sm.gs[i];
+        const int a = 63 - 2 * lane, b = a - 1;   // lane 0 holds the last two tokens
+        const double x0 = (double)sm.red[0][a] + (double)sm.red[1][a], x1 = (double)sm.red[0][b] + (double)sm.red[1][b];
+        double incl = x0 + x1;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const double y = __shfl_up_sync(0xffffffffu, incl, o);
+            if (lane >= o) incl += y;
+        }
+        if (a < rows) p.dlog_alpha[(t0 + a) * p.H + h] = (float)(tot + incl - x1);
+        if (b < rows) p.dlog_alpha[(t0 + b) * p.H + h] = (float)(tot + incl);
+    } else if (p.qnorm) {
+        // z = dq so far; q^ = q / ||q||: dq = z - q^ (q^ . z), the read-out's projection (the block's own stores, after the barrier)
+        for (int i = warp - 1; i < rows; i += 7) {
+            const size_t g = ((t0 + i) * p.H + h) * D;
+            float z[D / 32], q[D / 32], s = 0.f;
+#pragma unroll
+            for (int j = 0; j < D / 32; ++j) {
+                z[j] = p.dq[g + lane + 32 * j];
+                q[j] = to_f32(p.q[g + lane + 32 * j]) * sm.s.qinv[i];
+                s += q[j] * z[j];
+            }
+            s = warp_sum(s);
+#pragma unroll
+            for (int j = 0; j < D / 32; ++j) p.dq[g + lane + 32 * j] = z[j] - q[j] * s;
+        }
+    }
+}
+
+// ---- host side ------------------------------------------------------------------------------------------------------------
+template <typename K>
+cudaError_t allow_smem(K kern, int bytes)
+{
+    return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+}
+
+template <int D>
+cudaError_t launch_d(const BwdChunkParams &p, cudaStream_t stream)
+{
+    const int smem1 = (int)sizeof(PrepSmem<D>) + 1024, smem2 = (int)sizeof(ChainSmem<D>) + 1024, smem3 = (int)sizeof(GradSmem<D>);
+    cudaError_t e = allow_smem(kla_bwd_prepare_kernel<D>, smem1);
+    if (e == cudaSuccess) e = allow_smem(kla_bwd_chain_kernel<D>, smem2);
+    if (e == cudaSuccess) e = allow_smem(kla_bwd_grad_kernel<D>, smem3);
+    if (e != cudaSuccess) return e;
+    const int units = p.n_seq * p.H * (D / 64);
+    if (units == 0) return cudaSuccess;
+    if (p.n_slots > 0) kla_bwd_prepare_kernel<D><<<p.n_slots * p.H, 256, smem1, stream>>>(p);
+    kla_bwd_chain_kernel<D><<<2 * units, 128, smem2, stream>>>(p, units);   // (empty sequences: dinit)
+    if (p.n_slots > 0) kla_bwd_grad_kernel<D><<<p.n_slots * p.H, 256, smem3, stream>>>(p);
+    count_launch(p.n_slots > 0 ? 3 : 1);
+    return cudaGetLastError();
+}
+
+// Bytes of the workspace areas of one (slot, head), each a multiple of 1024.
+constexpr size_t per_entry(int d) { return (size_t)T_BYTES + 2 * (size_t)d * C * 4 + 2 * (size_t)d * d * 4 + sizeof(Scal); }
+size_t order_area(int n_seq) { return ((size_t)n_seq * 4 + 1023) & ~(size_t)1023; }
+
+}  // namespace
+
+size_t bwd_chunk_workspace_bytes(int n_seq, long long n_tok, int H, int d)
+{
+    return order_area(n_seq) + (size_t)(n_tok / C + n_seq) * H * per_entry(d);
+}
+
+cudaError_t launch_bwd_chunk(const BwdArgs &a, cudaStream_t stream)
+{
+    BwdChunkParams p;
+    p.q = (const __nv_bfloat16 *)a.q; p.k = (const __nv_bfloat16 *)a.k; p.v = (const __nv_bfloat16 *)a.v; p.dout = (const __nv_bfloat16 *)a.dout;
+    p.log_alpha = a.log_alpha; p.eta = a.eta;
+    p.init_state = a.init_state; p.dfinal = a.dfinal;
+    p.dq = a.dq; p.dk = a.dk; p.dv = a.dv; p.dlog_alpha = a.dlog_alpha; p.deta = a.deta; p.dinit = a.dinit;
+    p.cu_seqlens = a.cu_seqlens;
+    p.T = a.T; p.H = a.H; p.n_seq = a.n_seq;
+    p.eps = a.eps;
+    p.coeff_eta = a.coeff_eta; p.qnorm = a.qnorm;
+    p.n_slots = a.cu_seqlens ? (int)(a.n_tok / C) + a.n_seq : a.n_seq * ((a.T + C - 1) / C);
+    p.order = nullptr;
+    if (a.cu_seqlens && a.n_seq > 1 && a.n_seq <= 4096) {   // (the order takes quadratic work)
+        int32_t *order = (int32_t *)a.workspace;
+        const cudaError_t e = launch_seq_order(a.cu_seqlens, a.n_seq, order, stream);
+        if (e != cudaSuccess) return e;
+        p.order = order;
+    }
+    const size_t n = (size_t)p.n_slots * a.H, d = (size_t)a.d;
+    unsigned char *w = (unsigned char *)a.workspace + order_area(a.n_seq);
+    p.tpl = w;
+    w += n * T_BYTES;
+    p.pdo = (float *)w;
+    w += n * d * C * 4;
+    p.u = (float *)w;
+    w += n * d * C * 4;
+    p.s0 = (float *)w;
+    w += n * d * d * 4;
+    p.g1 = (float *)w;
+    w += n * d * d * 4;
+    p.scal = (Scal *)w;
+    return a.d == 128 ? launch_d<128>(p, stream) : launch_d<64>(p, stream);
+}
+
+}  // namespace kla

@@ -1,5 +1,6 @@
 // Reverse-mode derivative of the KLA recurrence (the training pass of Section 5.1; the paper prints no backward, so this
-// is the chain rule over the loop body of Algorithm 1 left with the coefficient of Eq. 3), token by token on CUDA cores.
+// is the chain rule over the loop body of Algorithm 1 left with the coefficient of Eq. 3), token by token on CUDA cores.  Serves
+// fp32 inputs; bf16 inputs go to the chunkwise kernels (bwd_chunk.cu).
 //
 // For a scalar loss with dO_t = dL/do_t and dS_T = dL/dS_T given, one token in reverse order, G = dL/dS_t on entry:
 //
@@ -433,7 +434,7 @@ cudaError_t launch_io(const BwdParams &p, int qnorm, cudaStream_t stream)
 
 }  // namespace
 
-size_t bwd_workspace_bytes(int n_seq, long long n_tok, int H, int d)
+size_t bwd_scan_workspace_bytes(int n_seq, long long n_tok, int H, int d)
 {
     const size_t state = (size_t)d * d * sizeof(float);
     const long long units = (long long)n_seq * H * (d / 64);
@@ -441,35 +442,31 @@ size_t bwd_workspace_bytes(int n_seq, long long n_tok, int H, int d)
     return 256 + (size_t)(n_tok / L + n_seq) * H * state + blocks * L * 64 * d * sizeof(float);   // (256: the unit counter)
 }
 
-cudaError_t launch_bwd_scan(const void *q, const void *k, const void *v, const float *log_alpha, const float *eta,
-                            const float *init_state, const void *dout, const float *dfinal, float *dq, float *dk, float *dv,
-                            float *dlog_alpha, float *deta, float *dinit, void *workspace, const int32_t *cu_seqlens, int T,
-                            long long n_tok, int H, int n_seq, int d, float eps, int coeff_eta, int qnorm, int io_dtype,
-                            cudaStream_t stream)
+cudaError_t launch_bwd_scan(const BwdArgs &a, cudaStream_t stream)
 {
     BwdParams p;
-    p.q = q; p.k = k; p.v = v; p.dout = dout;
-    p.log_alpha = log_alpha; p.eta = eta;
-    p.init_state = init_state; p.dfinal = dfinal;
-    p.dq = dq; p.dk = dk; p.dv = dv; p.dlog_alpha = dlog_alpha; p.deta = deta; p.dinit = dinit;
-    p.next_unit = reinterpret_cast<int32_t *>(workspace);
-    p.stored = reinterpret_cast<float *>(reinterpret_cast<char *>(workspace) + 256);
-    p.scratch = p.stored + (size_t)(n_tok / L + n_seq) * H * d * d;
+    p.q = a.q; p.k = a.k; p.v = a.v; p.dout = a.dout;
+    p.log_alpha = a.log_alpha; p.eta = a.eta;
+    p.init_state = a.init_state; p.dfinal = a.dfinal;
+    p.dq = a.dq; p.dk = a.dk; p.dv = a.dv; p.dlog_alpha = a.dlog_alpha; p.deta = a.deta; p.dinit = a.dinit;
+    p.next_unit = reinterpret_cast<int32_t *>(a.workspace);
+    p.stored = reinterpret_cast<float *>(reinterpret_cast<char *>(a.workspace) + 256);
+    p.scratch = p.stored + (size_t)(a.n_tok / L + a.n_seq) * a.H * a.d * a.d;
     if (cudaMemsetAsync(p.next_unit, 0, sizeof(int32_t), stream) != cudaSuccess) return cudaGetLastError();
-    p.cu_seqlens = cu_seqlens;
-    p.T = T; p.H = H; p.n_seq = n_seq;
-    p.eps = eps;
-    p.coeff_eta = coeff_eta;
-    p.n_units = n_seq * H * (d / 64);
-    if (d == 128) {   // two blocks per head add into the outputs that are sums over columns
-        cudaError_t e = cudaMemsetAsync(dq, 0, (size_t)n_tok * H * d * sizeof(float), stream);
-        if (e == cudaSuccess) e = cudaMemsetAsync(dk, 0, (size_t)n_tok * H * d * sizeof(float), stream);
-        if (e == cudaSuccess) e = cudaMemsetAsync(dlog_alpha, 0, (size_t)n_tok * H * sizeof(float), stream);
-        if (e == cudaSuccess) e = cudaMemsetAsync(deta, 0, (size_t)n_tok * H * sizeof(float), stream);
+    p.cu_seqlens = a.cu_seqlens;
+    p.T = a.T; p.H = a.H; p.n_seq = a.n_seq;
+    p.eps = a.eps;
+    p.coeff_eta = a.coeff_eta;
+    p.n_units = a.n_seq * a.H * (a.d / 64);
+    if (a.d == 128) {   // two blocks per head add into the outputs that are sums over columns
+        cudaError_t e = cudaMemsetAsync(a.dq, 0, (size_t)a.n_tok * a.H * a.d * sizeof(float), stream);
+        if (e == cudaSuccess) e = cudaMemsetAsync(a.dk, 0, (size_t)a.n_tok * a.H * a.d * sizeof(float), stream);
+        if (e == cudaSuccess) e = cudaMemsetAsync(a.dlog_alpha, 0, (size_t)a.n_tok * a.H * sizeof(float), stream);
+        if (e == cudaSuccess) e = cudaMemsetAsync(a.deta, 0, (size_t)a.n_tok * a.H * sizeof(float), stream);
         if (e != cudaSuccess) return e;
-        return io_dtype == KLA_BF16 ? launch_io<128, __nv_bfloat16>(p, qnorm, stream) : launch_io<128, float>(p, qnorm, stream);
+        return launch_io<128, float>(p, a.qnorm, stream);
     }
-    return io_dtype == KLA_BF16 ? launch_io<64, __nv_bfloat16>(p, qnorm, stream) : launch_io<64, float>(p, qnorm, stream);
+    return launch_io<64, float>(p, a.qnorm, stream);
 }
 
 }  // namespace kla

@@ -98,13 +98,26 @@ struct TokenScanParams {
     int32_t diag;               // one decay per row of the state
 };
 cudaError_t launch_token_scan(const TokenScanParams &p, int d, int io_dtype, int out_dtype, cudaStream_t stream);
-// Reverse-mode derivative of the recurrence, token by token on CUDA cores (bwd_scan.cu); gradients in fp32.
-size_t bwd_workspace_bytes(int n_seq, long long n_tok, int H, int d);
-cudaError_t launch_bwd_scan(const void *q, const void *k, const void *v, const float *log_alpha, const float *eta,
-                            const float *init_state, const void *dout, const float *dfinal, float *dq, float *dk, float *dv,
-                            float *dlog_alpha, float *deta, float *dinit, void *workspace, const int32_t *cu_seqlens, int T,
-                            long long n_tok, int H, int n_seq, int d, float eps, int coeff_eta, int qnorm, int io_dtype,
-                            cudaStream_t stream);
+// Reverse-mode derivative of the recurrence; gradients in fp32.  bf16 inputs: chunkwise (bwd_chunk.cu); fp32 inputs: token by
+// token on CUDA cores (bwd_scan.cu).
+struct BwdArgs {
+    const void *q, *k, *v, *dout;
+    const float *log_alpha, *eta;       // [n_tok, H]
+    const float *init_state, *dfinal;   // [n_seq, H, D, D] or null
+    float *dq, *dk, *dv;                // [n_tok, H, D]
+    float *dlog_alpha, *deta;           // [n_tok, H]
+    float *dinit;                       // [n_seq, H, D, D] or null
+    void *workspace;
+    const int32_t *cu_seqlens;          // null: fixed length T
+    int32_t T, H, n_seq, d;
+    long long n_tok;
+    float eps;
+    int32_t coeff_eta, qnorm;
+};
+size_t bwd_scan_workspace_bytes(int n_seq, long long n_tok, int H, int d);
+cudaError_t launch_bwd_scan(const BwdArgs &a, cudaStream_t stream);
+size_t bwd_chunk_workspace_bytes(int n_seq, long long n_tok, int H, int d);
+cudaError_t launch_bwd_chunk(const BwdArgs &a, cudaStream_t stream);
 // True when the tensor-core kernel covers this case.
 bool chunk_tc_supported(int d, int chunk, int io_dtype);
 

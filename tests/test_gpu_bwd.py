@@ -156,3 +156,25 @@ def test_long_context_workload_full_size_every_head():
     w = W.config3()
     g, do, df = _gpu(w)
     _assert_close(g, _ref(w, do, df), TOL_BF16)
+
+
+@pytest.mark.parametrize("d", [64, 128])
+@pytest.mark.parametrize("T", [63, 64, 65, 127, 128, 129])
+def test_chunk_edges(T, d):
+    w = _with_state(W.config2(B=1, H=2, T=T, d=d, seed=930 + T), T)
+    g, do, df = _gpu(w)
+    _assert_close(g, _ref(w, do, df), 1e-4)
+
+
+def test_packed_sequences_ending_on_and_next_to_chunk_edges():
+    w = _with_state(W.config5(H=2, d=128, lengths=[64, 0, 128, 63, 1, 65, 192, 0], seed=931), 932)
+    g, do, df = _gpu(w, cu=w.cu_seqlens)
+    _assert_close(g, _ref(w, do, df), TOL_BF16)
+
+
+def test_tokens_with_eta_zero():
+    # beta = 0: the residual that deta needs cannot be read off the written update
+    w = _with_state(W.config2(B=1, H=2, T=150, d=128, seed=933), 934)
+    w.eta = torch.where(torch.rand(w.eta.shape, generator=torch.Generator().manual_seed(935)) < 0.3, torch.zeros_like(w.eta), w.eta)
+    g, do, df = _gpu(w)
+    _assert_close(g, _ref(w, do, df), 1e-4)
