@@ -653,9 +653,11 @@ __global__ void __launch_bounds__(128, 2) kla_bwd_chain_kernel(BwdChunkParams p,
 }
 
 // ---- 3. gradients ---------------------------------------------------------------------------------------------------------
-// One block of eight warps per (chunk, head).  Output columns (d_k) are taken in halves of 64: the operand planes of S_0, then
-// of G_1, of one half share a buffer.  A warp owns 16 tokens x 32 columns; operands that two products have in common are
+// One block of sixteen warps per (chunk, head).  Output columns (d_k) are taken in halves of 64: the operand planes of S_0, then
+// of G_1, of one half share a buffer.  A warp owns 16 tokens x 16 columns; operands that two products have in common are
 // loaded once for both.  Global loads of the next operand are requested before the products of the one at hand.
+constexpr int GW = 16;         // warps
+constexpr int GT = 32 * GW;
 template <int D>
 struct GradSmem {
     unsigned char dout[D / 64 * 8192];            // [token][d_v]
@@ -665,14 +667,14 @@ struct GradSmem {
     unsigned char sg[3 * D * 128];                // S_0^T or G_1^T, planes, [d_v][64 of d_k]
     unsigned char k[8192], q[8192];               // [token][64 of d_k]
     Scal s;
-    float red[2][64];                             // dg_i, the parts of the two column halves of the warps
-    float gs[8];                                  // <G_1, S_1> of the warps
+    float red[4][64];                             // dg_i, the parts of the four column groups of the warps
 };
 
 template <int D>
-__global__ void __launch_bounds__(256, 1) kla_bwd_grad_kernel(BwdChunkParams p)
+__global__ void __launch_bounds__(GT, 1) kla_bwd_grad_kernel(BwdChunkParams p)
 {
-    constexpr int NB = D / 64, IT = D / 32;   // 8-column items of a [D][64] fp32 matrix per thread
+    constexpr int NB = D / 64, IT = D * 8 / GT;   // 8-column items of a [D][64] fp32 matrix per thread
+    constexpr int UI = C * D / 8 / GT;            // 8-column items of a [64][D] matrix per thread
     extern __shared__ __align__(128) unsigned char smem_dyn[];
     GradSmem<D> &sm = *reinterpret_cast<GradSmem<D> *>(smem_dyn);
     static_assert(sizeof(GradSmem<D>) <= 232448, "shared memory of one block");
@@ -682,7 +684,7 @@ __global__ void __launch_bounds__(256, 1) kla_bwd_grad_kernel(BwdChunkParams p)
     if (w.c * C >= w.len) return;
     const int rows = min(C, w.len - w.c * C);
     const size_t t0 = (size_t)w.tok0 + w.c * C, ch = (size_t)slot * p.H + h;
-    load_tile<NB, D, 256>(smem_u32(sm.dout), p.dout, t0, rows, p.H, h, 0, tid);
+    load_tile<NB, D, GT>(smem_u32(sm.dout), p.dout, t0, rows, p.H, h, 0, tid);
     if (tid < (int)sizeof(Scal) / 16) cp16(smem_u32(&sm.s) + tid * 16, reinterpret_cast<const char *>(p.scal + ch) + tid * 16, true);
     cp_commit();
 
@@ -691,7 +693,7 @@ __global__ void __launch_bounds__(256, 1) kla_bwd_grad_kernel(BwdChunkParams p)
     auto fetch = [&](float4 (&pre)[IT][2], const float *src, int hh) {
 #pragma unroll
         for (int i = 0; i < IT; ++i) {
-            const int e = tid + i * 256, r = e >> 3, c8 = e & 7;
+            const int e = tid + i * GT, r = e >> 3, c8 = e & 7;
             const float *x = src + ch * D * D + (size_t)r * D + hh * 64 + c8 * 8;
             pre[i][0] = load4(x);
             pre[i][1] = load4(x + 4);
@@ -710,17 +712,17 @@ __global__ void __launch_bounds__(256, 1) kla_bwd_grad_kernel(BwdChunkParams p)
     auto commit = [&](const float4 (&pre)[IT][2]) {
 #pragma unroll
         for (int i = 0; i < IT; ++i) {
-            const int e = tid + i * 256;
+            const int e = tid + i * GT;
             put8(sm.sg, D * 128, sw128(e >> 3, e & 7), pre[i][0], pre[i][1]);
         }
     };
 
     // U and lam as operand planes; dbeta_i = (U_i / beta_i) . (lam_i / beta_i)
     {
-        float4 a[NB * 2][4];
+        float4 a[UI][4];
 #pragma unroll
-        for (int i = 0; i < NB * 2; ++i) {
-            const int e = tid + i * 256, r = e / (D / 8), c8 = e % (D / 8);
+        for (int i = 0; i < UI; ++i) {
+            const int e = tid + i * GT, r = e / (D / 8), c8 = e % (D / 8);
             const float *x = p.u + ch * C * D + (size_t)r * D + c8 * 8;
             const float *y = p.dv + ((t0 + (r < rows ? r : 0)) * p.H + h) * D + c8 * 8;
             a[i][0] = load4(x);
@@ -732,8 +734,8 @@ __global__ void __launch_bounds__(256, 1) kla_bwd_grad_kernel(BwdChunkParams p)
         cp_wait<0>();
         __syncthreads();   // scalars (and dO) are there
 #pragma unroll
-        for (int i = 0; i < NB * 2; ++i) {
-            const int e = tid + i * 256, r = e / (D / 8), c8 = e % (D / 8);
+        for (int i = 0; i < UI; ++i) {
+            const int e = tid + i * GT, r = e / (D / 8), c8 = e % (D / 8);
             if (r >= rows) a[i][0] = a[i][1] = a[i][2] = a[i][3] = make_float4(0.f, 0.f, 0.f, 0.f);
             const uint32_t off = (c8 >> 3) * 8192 + sw128(r, c8 & 7);
             put8(sm.u, NB * 8192, off, a[i][0], a[i][1]);
@@ -797,26 +799,23 @@ __global__ void __launch_bounds__(256, 1) kla_bwd_grad_kernel(BwdChunkParams p)
                 *reinterpret_cast<uint32_t *>(dst + 16384 + off) = ll;
             }
     };
-    // ten blocks of each, an E block costs two F blocks: warps 0, 1 two of E; 2 .. 5 one of E, two of F; 6, 7 one of each
-    block(true, warp);
-    if (warp < 2) block(true, 8 + warp);
-    else if (warp < 6) {
-        block(false, 2 * (warp - 2));
-        block(false, 2 * (warp - 2) + 1);
-    } else block(false, warp + 2);
+    // ten blocks of each, an E block costs two F blocks
+    if (warp < 10) block(true, warp);
+    else
+        for (int b = warp - 10; b < 10; b += 6) block(false, b);
 
-    const int mt = warp & 3, nh = warp >> 2, i0 = mt * 16;   // this warp's 16 tokens and 32 of the half's 64 columns
+    const int mt = warp & 3, nh = warp >> 2, i0 = mt * 16;   // this warp's 16 tokens and 16 of the half's 64 columns
     const int ia = i0 + r, ib = ia + 8;
     float gs = 0.f;             // this thread's part of <G_1, S_1>
     float dga = 0.f, dgb = 0.f; // ... of dg of its two rows
     const float gama = sm.s.gam[ia], gamb = sm.s.gam[ib], deca = sm.s.dec[ia], decb = sm.s.dec[ib], gc = sm.s.gam[C - 1];
     const float qia = sm.s.qinv[ia], qib = sm.s.qinv[ib];
     // products x . y of this lane's elements of the two rows, added to a and b
-    auto dot = [&](const unsigned char *tile, const float (&x)[4][4], float &a, float &b) {
+    auto dot = [&](const unsigned char *tile, const float (&x)[2][4], float &a, float &b) {
 #pragma unroll
-        for (int t = 0; t < 4; ++t) {
-            const float2 fa = unpack(*reinterpret_cast<const uint32_t *>(tile + sw128(ia, nh * 4 + t) + 4 * (lane & 3)));
-            const float2 fb = unpack(*reinterpret_cast<const uint32_t *>(tile + sw128(ib, nh * 4 + t) + 4 * (lane & 3)));
+        for (int t = 0; t < 2; ++t) {
+            const float2 fa = unpack(*reinterpret_cast<const uint32_t *>(tile + sw128(ia, nh * 2 + t) + 4 * (lane & 3)));
+            const float2 fb = unpack(*reinterpret_cast<const uint32_t *>(tile + sw128(ib, nh * 2 + t) + 4 * (lane & 3)));
             a += fa.x * x[t][0] + fa.y * x[t][1];
             b += fb.x * x[t][2] + fb.y * x[t][3];
         }
@@ -824,16 +823,16 @@ __global__ void __launch_bounds__(256, 1) kla_bwd_grad_kernel(BwdChunkParams p)
     const uint32_t sg = smem_u32(sm.sg), kt = smem_u32(sm.k), qt = smem_u32(sm.q);
 #pragma unroll 1
     for (int hh = 0; hh < NB; ++hh) {
-        load_tile<1, D, 256>(kt, p.k, t0, rows, p.H, h, hh * 64, tid);
-        load_tile<1, D, 256>(qt, p.q, t0, rows, p.H, h, hh * 64, tid);
+        load_tile<1, D, GT>(kt, p.k, t0, rows, p.H, h, hh * 64, tid);
+        load_tile<1, D, GT>(qt, p.q, t0, rows, p.H, h, hh * 64, tid);
         cp_commit();
         commit(ps);
         fetch(pg, p.g1, hh);
         cp_wait<0>();
         __syncthreads();   // S_0 planes, K, Q (and, the first time, E and F)
-        float xq[4][4], xk[4][4];
+        float xq[2][4], xk[2][4];
 #pragma unroll
-        for (int t = 0; t < 4; ++t)
+        for (int t = 0; t < 2; ++t)
 #pragma unroll
             for (int e = 0; e < 4; ++e) xq[t][e] = xk[t][e] = 0.f;
         // dO S_0^T and lam S_0^T
@@ -844,21 +843,20 @@ __global__ void __launch_bounds__(256, 1) kla_bwd_grad_kernel(BwdChunkParams p)
             frag_a(a, smem_u32(sm.dout) + o, i0, (ks & 3) * 16, lane);
 #pragma unroll
             for (int pl = 0; pl < 3; ++pl) frag_a(l[pl], smem_u32(sm.lam) + pl * NB * 8192 + o, i0, (ks & 3) * 16, lane);
-#pragma unroll
-            for (int np = 0; np < 2; ++np) {
+            {
                 uint32_t b[3][4];
 #pragma unroll
-                for (int pl = 0; pl < 3; ++pl) frag_bt(b[pl], sg + pl * D * 128, ks * 16, nh * 32 + np * 16, lane);
+                for (int pl = 0; pl < 3; ++pl) frag_bt(b[pl], sg + pl * D * 128, ks * 16, nh * 16, lane);
 #pragma unroll
                 for (int pl = 0; pl < 3; ++pl) {
-                    mma(xq[2 * np], a, b[pl][0], b[pl][1]);
-                    mma(xq[2 * np + 1], a, b[pl][2], b[pl][3]);
+                    mma(xq[0], a, b[pl][0], b[pl][1]);
+                    mma(xq[1], a, b[pl][2], b[pl][3]);
                 }
-                mma6(xk[2 * np], xk[2 * np + 1], l, b);
+                mma6(xk[0], xk[1], l, b);
             }
         }
 #pragma unroll
-        for (int t = 0; t < 4; ++t) {
+        for (int t = 0; t < 2; ++t) {
             xq[t][0] *= gama * qia; xq[t][1] *= gama * qia; xq[t][2] *= gamb * qib; xq[t][3] *= gamb * qib;
             xk[t][0] *= -gama; xk[t][1] *= -gama; xk[t][2] *= -gamb; xk[t][3] *= -gamb;
         }
@@ -871,23 +869,22 @@ __global__ void __launch_bounds__(256, 1) kla_bwd_grad_kernel(BwdChunkParams p)
                 frag_a(a[pl], smem_u32(sm.f) + pl * 8192, i0, ks * 16, lane);
                 frag_a(l[pl], smem_u32(sm.e) + pl * 8192, i0, ks * 16, lane);
             }
-#pragma unroll
-            for (int np = 0; np < 2; ++np) {
+            {
                 uint32_t b[4];
-                frag_bt(b, kt, ks * 16, nh * 32 + np * 16, lane);
+                frag_bt(b, kt, ks * 16, nh * 16, lane);
 #pragma unroll
                 for (int pl = 0; pl < 3; ++pl) {
-                    mma(xq[2 * np], a[pl], b[0], b[1]);
-                    mma(xq[2 * np + 1], a[pl], b[2], b[3]);
-                    mma(xk[2 * np], l[pl], b[0], b[1]);
-                    mma(xk[2 * np + 1], l[pl], b[2], b[3]);
+                    mma(xq[0], a[pl], b[0], b[1]);
+                    mma(xq[1], a[pl], b[2], b[3]);
+                    mma(xk[0], l[pl], b[0], b[1]);
+                    mma(xk[1], l[pl], b[2], b[3]);
                 }
             }
         }
         // dq (with the normalised read-out its projection follows below)
-        const size_t ga = ((t0 + ia) * p.H + h) * D + hh * 64 + nh * 32 + cq, gb = ga + (size_t)8 * p.H * D;
+        const size_t ga = ((t0 + ia) * p.H + h) * D + hh * 64 + nh * 16 + cq, gb = ga + (size_t)8 * p.H * D;
 #pragma unroll
-        for (int t = 0; t < 4; ++t) {
+        for (int t = 0; t < 2; ++t) {
             if (ia < rows) store2(p.dq + ga + 8 * t, xq[t][0], xq[t][1]);
             if (ib < rows) store2(p.dq + gb + 8 * t, xq[t][2], xq[t][3]);
         }
@@ -904,7 +901,7 @@ __global__ void __launch_bounds__(256, 1) kla_bwd_grad_kernel(BwdChunkParams p)
         __syncthreads();
         // D U G_1^T
 #pragma unroll
-        for (int t = 0; t < 4; ++t)
+        for (int t = 0; t < 2; ++t)
 #pragma unroll
             for (int e = 0; e < 4; ++e) xq[t][e] = 0.f;
 #pragma unroll 2
@@ -912,16 +909,15 @@ __global__ void __launch_bounds__(256, 1) kla_bwd_grad_kernel(BwdChunkParams p)
             uint32_t a[3][4];
 #pragma unroll
             for (int pl = 0; pl < 3; ++pl) frag_a(a[pl], smem_u32(sm.u) + (pl * NB + (ks >> 2)) * 8192, i0, (ks & 3) * 16, lane);
-#pragma unroll
-            for (int np = 0; np < 2; ++np) {
+            {
                 uint32_t b[3][4];
 #pragma unroll
-                for (int pl = 0; pl < 3; ++pl) frag_bt(b[pl], sg + pl * D * 128, ks * 16, nh * 32 + np * 16, lane);
-                mma6(xq[2 * np], xq[2 * np + 1], a, b);
+                for (int pl = 0; pl < 3; ++pl) frag_bt(b[pl], sg + pl * D * 128, ks * 16, nh * 16, lane);
+                mma6(xq[0], xq[1], a, b);
             }
         }
 #pragma unroll
-        for (int t = 0; t < 4; ++t) {
+        for (int t = 0; t < 2; ++t) {
             xq[t][0] *= deca; xq[t][1] *= deca; xq[t][2] *= decb; xq[t][3] *= decb;
         }
         dot(sm.k, xq, gs, gs);   // <G_1, S_1> = gC <G_1, S_0> + sum_j k_j . (D U G_1^T)_j
@@ -934,17 +930,16 @@ __global__ void __launch_bounds__(256, 1) kla_bwd_grad_kernel(BwdChunkParams p)
                 frag_at(a[pl], smem_u32(sm.f) + pl * 8192, i0, ks * 16, lane);
                 frag_at(l[pl], smem_u32(sm.e) + pl * 8192, i0, ks * 16, lane);
             }
-#pragma unroll
-            for (int np = 0; np < 2; ++np) {
+            {
                 uint32_t b[4], b2[4];
-                frag_bt(b, qt, ks * 16, nh * 32 + np * 16, lane);
-                frag_bt(b2, kt, ks * 16, nh * 32 + np * 16, lane);
+                frag_bt(b, qt, ks * 16, nh * 16, lane);
+                frag_bt(b2, kt, ks * 16, nh * 16, lane);
 #pragma unroll
                 for (int pl = 0; pl < 3; ++pl) {
-                    mma(xq[2 * np], a[pl], b[0], b[1]);
-                    mma(xq[2 * np + 1], a[pl], b[2], b[3]);
-                    mma(xq[2 * np], l[pl], b2[0], b2[1]);
-                    mma(xq[2 * np + 1], l[pl], b2[2], b2[3]);
+                    mma(xq[0], a[pl], b[0], b[1]);
+                    mma(xq[1], a[pl], b[2], b[3]);
+                    mma(xq[0], l[pl], b2[0], b2[1]);
+                    mma(xq[1], l[pl], b2[2], b2[3]);
                 }
             }
         }
@@ -954,9 +949,9 @@ __global__ void __launch_bounds__(256, 1) kla_bwd_grad_kernel(BwdChunkParams p)
         dgb -= cb;
         const float na = sm.s.dn[ia], nb = sm.s.dn[ib];
 #pragma unroll
-        for (int t = 0; t < 4; ++t) {
-            const float2 fa = unpack(*reinterpret_cast<const uint32_t *>(sm.k + sw128(ia, nh * 4 + t) + 4 * (lane & 3)));
-            const float2 fb = unpack(*reinterpret_cast<const uint32_t *>(sm.k + sw128(ib, nh * 4 + t) + 4 * (lane & 3)));
+        for (int t = 0; t < 2; ++t) {
+            const float2 fa = unpack(*reinterpret_cast<const uint32_t *>(sm.k + sw128(ia, nh * 2 + t) + 4 * (lane & 3)));
+            const float2 fb = unpack(*reinterpret_cast<const uint32_t *>(sm.k + sw128(ib, nh * 2 + t) + 4 * (lane & 3)));
             if (ia < rows) store2(p.dk + ga + 8 * t, xk[t][0] + xq[t][0] + na * fa.x, xk[t][1] + xq[t][1] + na * fa.y);
             if (ib < rows) store2(p.dk + gb + 8 * t, xk[t][2] + xq[t][2] + nb * fb.x, xk[t][3] + xq[t][3] + nb * fb.y);
         }
@@ -973,14 +968,15 @@ __global__ void __launch_bounds__(256, 1) kla_bwd_grad_kernel(BwdChunkParams p)
         sm.red[nh][ib] = dgb;
     }
     gs = warp_sum(gs);
-    if (lane == 0) sm.gs[warp] = gs;
+    if (lane == 0) sm.s.nrm[warp] = gs;   // (the norms have been used; no room for an array of its own at d = 128)
     __syncthreads();
     if (warp == 0) {
         double tot = 0.0;
 #pragma unroll
-        for (int i = 0; i < 8; ++i) tot += (double)sm.gs[i];
+        for (int i = 0; i < GW; ++i) tot += (double)sm.s.nrm[i];
+        auto rsum = [&](int i) { return ((double)sm.red[0][i] + (double)sm.red[1][i]) + ((double)sm.red[2][i] + (double)sm.red[3][i]); };
         const int a = 63 - 2 * lane, b = a - 1;   // lane 0 holds the last two tokens
-        const double x0 = (double)sm.red[0][a] + (double)sm.red[1][a], x1 = (double)sm.red[0][b] + (double)sm.red[1][b];
+        const double x0 = rsum(a), x1 = rsum(b);
         double incl = x0 + x1;
 #pragma unroll
         for (int o = 1; o < 32; o <<= 1) {
@@ -991,7 +987,7 @@ __global__ void __launch_bounds__(256, 1) kla_bwd_grad_kernel(BwdChunkParams p)
         if (b < rows) p.dlog_alpha[(t0 + b) * p.H + h] = (float)(tot + incl);
     } else if (p.qnorm) {
         // z = dq so far; q^ = q / ||q||: dq = z - q^ (q^ . z), the read-out's projection (the block's own stores, after the barrier)
-        for (int i = warp - 1; i < rows; i += 7) {
+        for (int i = warp - 1; i < rows; i += GW - 1) {
             const size_t g = ((t0 + i) * p.H + h) * D;
             float z[D / 32], q[D / 32], s = 0.f;
 #pragma unroll
@@ -1026,7 +1022,7 @@ cudaError_t launch_d(const BwdChunkParams &p, cudaStream_t stream)
     if (units == 0) return cudaSuccess;
     if (p.n_slots > 0) kla_bwd_prepare_kernel<D><<<p.n_slots * p.H, 256, smem1, stream>>>(p);
     kla_bwd_chain_kernel<D><<<2 * units, 128, smem2, stream>>>(p, units);   // (empty sequences: dinit)
-    if (p.n_slots > 0) kla_bwd_grad_kernel<D><<<p.n_slots * p.H, 256, smem3, stream>>>(p);
+    if (p.n_slots > 0) kla_bwd_grad_kernel<D><<<p.n_slots * p.H, GT, smem3, stream>>>(p);
     count_launch(p.n_slots > 0 ? 3 : 1);
     return cudaGetLastError();
 }
