@@ -72,11 +72,8 @@ typedef enum { KLA_F32 = 0, KLA_BF16 = 1 } kla_dtype;
  * CTA gives up in an orderly way and KLA_ERR_TIMEOUT appears in *status_word.  Outputs are then undefined; the
  * context stays usable. */
 #define KLA_INTERNAL_FLAG_TEST_TIMEOUT 16
-/* With d_v = 128 the two CTAs that hold the two 64-column slices of a head run as a thread-block cluster and share
- * the work that does not depend on the state (each inverts every other chunk's I + B X and hands the result to its
- * peer through distributed shared memory).  This flag launches them as independent CTAs instead, each doing all of
- * that work itself; the arithmetic is the same, so the results are bit-identical.  Used to cross-check the two
- * launch forms. */
+/* Accepted and without effect: the blocks that hold the 64-column slices of a head always run independently of each other (an
+ * earlier kernel could pair them). */
 #define KLA_FLAG_NO_PAIR 32
 /* Head dimension 128 only (ignored otherwise): run the chunk forward in the WY form of Appendix B (Props. 5-6 and the
  * combined representation U^ = U - W S_0, with W = T B D_gamma K and U = T B V formed on tensor cores off the serial

@@ -245,7 +245,7 @@ static kla_status chunk_fwd_impl(const kla_desc *desc, const void *q, const void
     p.seg_pass = 0; p.seg_G = 0; p.map_state = nullptr;
     p.variant = ((desc->flags & KLA_FLAG_COEFF_ETA) ? VARIANT_COEFF_ETA : 0) | ((desc->flags & KLA_FLAG_QNORM) ? VARIANT_QNORM : 0) |
                 ((desc->flags & KLA_INTERNAL_FLAG_TEST_TIMEOUT) ? VARIANT_TEST_TIMEOUT : 0) |
-                ((desc->flags & KLA_FLAG_NO_PAIR) ? VARIANT_NO_PAIR : 0) | ((desc->flags & KLA_FLAG_WY_FORM) ? VARIANT_WY : 0);
+                ((desc->flags & KLA_FLAG_WY_FORM) ? VARIANT_WY : 0);
     p.B = desc->B; p.T = desc->T; p.H = desc->H; p.n_seq = desc->n_seq;
     p.eps = eps;
     if (desc->T == 0) {
@@ -423,7 +423,7 @@ kla_status kla_chunk_span_map(const kla_desc *desc, const void *k, const void *v
     p.B = desc->B; p.T = desc->T; p.H = desc->H; p.n_seq = desc->B * 2;
     p.eps = eps;
     p.seg_pass = 1; p.seg_G = 2;
-    p.variant = ((desc->flags & KLA_FLAG_COEFF_ETA) ? VARIANT_COEFF_ETA : 0) | ((desc->flags & KLA_FLAG_NO_PAIR) ? VARIANT_NO_PAIR : 0) |
+    p.variant = ((desc->flags & KLA_FLAG_COEFF_ETA) ? VARIANT_COEFF_ETA : 0) |
                 ((desc->flags & KLA_FLAG_WY_FORM) ? VARIANT_WY : 0);
     p.map_state = map;
     if (launch_chunk_tc(p, desc->d_k, desc->io_dtype, KLA_F32, stream) != cudaSuccess) return KLA_ERR_LAUNCH;

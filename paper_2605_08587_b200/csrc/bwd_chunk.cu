@@ -113,7 +113,7 @@ __device__ __forceinline__ void load_tile(uint32_t dst, const __nv_bfloat16 *src
 }
 
 // ---- 1. prepare -----------------------------------------------------------------------------------------------------------
-// One level of the blocked inverse of I + B X (see chunk_tc.cu): for every pair of adjacent inverted BS x BS diagonal blocks the
+// One level of the blocked inverse of I + B X (see chunk_pieces.cuh): for every pair of adjacent inverted BS x BS diagonal blocks the
 // block below the diagonal becomes T_10 = -T_11 (B_1 X_10 T_00).  256 threads, 1 x 4 results each.
 template <int BS>
 __device__ __forceinline__ void merge_level(float *tl, float *mm, const float *bet, int pt)

@@ -1,5 +1,4 @@
-// Pieces shared by the two tensor-core chunk kernels (chunk_tc.cu: one CTA per state slice, W-free form of
-// Algorithm 1 right; chunk_wy.cu: two CTAs per head, WY form): constants, bounded barrier waits, the decay scan, the
+// Pieces of the WY-form chunk kernel (chunk_wy.cu: two CTAs per head): constants, bounded barrier waits, the decay scan, the
 // blocked inverse of I + B X in shared memory, tile helpers and the host side of the tensor maps.
 #pragma once
 #include <cuda.h>

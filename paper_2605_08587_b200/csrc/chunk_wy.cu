@@ -37,8 +37,8 @@
 // (S_0 against Q, T B, P D^-1, D U^) need 16 significand bits and are hi/lo pairs; W S_0 only corrects U by what the
 // incoming state already predicts, and an 11-bit W and S_0 there (fp16, one term) keeps the layer-shaped workloads
 // below 1e-3 in max|err|/rms.  The state and W must stay inside the fp16 range (|x| < 65504); beyond it the result
-// is Inf/NaN, never silently wrong.  Inputs with heavy-tailed key norms want all-16-bit operands: KLA_FLAG_NO_PAIR
-// routes to the kernel of chunk_tc.cu, which has them.
+// is Inf/NaN, never silently wrong.  Inputs with heavy-tailed key norms want all-16-bit operands, which the kernel of
+// chunk_mma.cu has.
 //
 // Every wait on an mbarrier is bounded; when one gives up the CTA raises an abort flag, reports KLA_ERR_TIMEOUT
 // through the status word, releases its TMEM and exits.
@@ -1036,7 +1036,7 @@ cudaError_t launch_v(const ChunkParams &p, cudaStream_t stream)
 
 cudaError_t launch_chunk_wy(const ChunkParams &p, int out_dtype, cudaStream_t stream)
 {
-    const bool var = (p.variant & ~(VARIANT_NO_PAIR | VARIANT_WY)) != 0;
+    const bool var = (p.variant & ~VARIANT_WY) != 0;
     if (out_dtype == KLA_BF16) return var ? launch_v<128, __nv_bfloat16, true>(p, stream) : launch_v<128, __nv_bfloat16, false>(p, stream);
     return var ? launch_v<128, float, true>(p, stream) : launch_v<128, float, false>(p, stream);
 }

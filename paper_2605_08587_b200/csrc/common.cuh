@@ -33,7 +33,7 @@ struct ChunkParams {
     //   seg_pass 6: the plain packed launch, taken only if the pieces' plan word, seq_order[seg_G], is 0.
     //   Passes 1 and 3 return at once when the plan word (cu_seqlens[n_seq + 1]) is 1, passes 4 and 5 when it is not.
     int32_t seg_pass, seg_G;
-    int32_t variant;     // bit 0: beta_t = eta_t instead of Eq. 3; bit 1: read-out divided by ||q_t||; bit 2: test hook; bits 3, 4: see VARIANT_NO_PAIR, VARIANT_WY
+    int32_t variant;     // bit 0: beta_t = eta_t instead of Eq. 3; bit 1: read-out divided by ||q_t||; bit 2: test hook; bit 4: see VARIANT_WY
     union {
         float *map_state;            // segment pass 1
         const int32_t *seq_order;    // packed input, plain launch: block b works on sequence seq_order[b] (longest
@@ -41,7 +41,6 @@ struct ChunkParams {
     };
 };
 constexpr int32_t VARIANT_COEFF_ETA = 1, VARIANT_QNORM = 2, VARIANT_TEST_TIMEOUT = 4;
-constexpr int32_t VARIANT_NO_PAIR = 8;   // host side only: launch the two slices of a head as independent CTAs
 constexpr int32_t VARIANT_WY = 16;       // host side only: head dimension 128 goes to the WY-form kernel (chunk_wy.cu)
 
 struct DecodeParams {
