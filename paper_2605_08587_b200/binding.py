@@ -338,36 +338,12 @@ def kla_bwd(q, k, v, log_alpha, eta, eps, d_out, init_state=None, d_final_state=
     d_final_state = dL/dfinal_state (or None).  Returns a dict of fp32 tensors dq, dk, dv, dlog_alpha, deta and
     dinit_state (None unless asked for).  `workspace`: a uint8 CUDA tensor of at least kla_bwd_workspace_bytes, else
     one is allocated here."""
-    lib = load()
-    B, T, H, d_k = q.shape
-    d_v = v.shape[-1]
-    if tuple(d_out.shape) != (B, T, H, d_v) or d_out.dtype != q.dtype:
-        raise ValueError("d_out must be [B, T, H, d_v] with the dtype of q")
-    n_seq, hs = B, None
-    if cu_seqlens is not None:
-        hs = (cu_seqlens.cpu() if host_seqlens is None else host_seqlens).contiguous()
-        n_seq = cu_seqlens.numel() - 1
-    f32 = dict(device=q.device, dtype=torch.float32)
-    g = dict(dq=torch.empty((B, T, H, d_k), **f32), dk=torch.empty((B, T, H, d_k), **f32), dv=torch.empty((B, T, H, d_v), **f32),
-             dlog_alpha=torch.empty((B, T, H), **f32), deta=torch.empty((B, T, H), **f32),
-             dinit_state=torch.empty((n_seq, H, d_k, d_v), **f32) if want_dinit_state else None)
-    desc = KlaDesc(B=B, T=T, H=H, d_k=d_k, d_v=d_v, n_seq=n_seq, cu_seqlens=_dev(cu_seqlens, "cu_seqlens"),
-                   host_seqlens=hs.data_ptr() if hs is not None else None, io_dtype=_dt(q), out_dtype=KLA_F32, flags=flags,
-                   workspace=None, workspace_bytes=0, status_word=None, stream=_stream(q.device))
-    need = int(lib.kla_bwd_workspace_bytes(ctypes.byref(desc)))
-    if workspace is None and need > 0:
-        workspace = torch.empty(need, device=q.device, dtype=torch.uint8)
-    if workspace is not None:
-        desc.workspace = _dev(workspace, "workspace")
-        desc.workspace_bytes = workspace.numel() * workspace.element_size()
-    with torch.cuda.device(q.device):
-        code = lib.kla_bwd(ctypes.byref(desc), _dev(q, "q"), _dev(k, "k"), _dev(v, "v"), _dev(log_alpha, "log_alpha", torch.float32),
-                           _dev(eta, "eta", torch.float32), float(eps), _dev(init_state, "init_state", torch.float32),
-                           _dev(d_out, "d_out"), _dev(d_final_state, "d_final_state", torch.float32),
-                           _dev(g["dq"], "dq"), _dev(g["dk"], "dk"), _dev(g["dv"], "dv"), _dev(g["dlog_alpha"], "dlog_alpha"),
-                           _dev(g["deta"], "deta"), _dev(g["dinit_state"], "dinit_state"))
-    _check(code)
-    return g
+    if _host is None:
+        load()
+    if cu_seqlens is not None and host_seqlens is None:
+        host_seqlens = cu_seqlens.cpu()
+    return _host.backward(q, k, v, log_alpha, eta, float(eps), d_out, init_state, d_final_state, cu_seqlens, host_seqlens, flags,
+                          want_dinit_state, workspace)
 
 
 def kla_dg_decode_step(q, k, v, log_alpha, eta, eps, state_inout, out=None, out_dtype=None, flags=KLA_FLAG_NONE):

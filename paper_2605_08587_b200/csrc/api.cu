@@ -9,6 +9,14 @@ namespace kla {
 static std::atomic<uint64_t> g_launches{0};
 void count_launch(int n) { g_launches.fetch_add((uint64_t)n, std::memory_order_relaxed); }
 
+int sm_count()
+{
+    int dev = 0, n = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || n <= 0)
+        return 148;
+    return n;
+}
+
 static bool aligned16(const void *p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
 
 static kla_status check_arch()
@@ -80,7 +88,6 @@ struct PackedPlan {
     size_t off_plan = 0, bytes = 0;   // the piece tables follow the longest-first order array in the workspace
 };
 
-static int sm_count();
 
 static PackedPlan plan_packed(const kla_desc *d, int32_t chunk)
 {
@@ -123,14 +130,6 @@ struct SegPlan {
     int seg_len = 0;      // tokens per segment (a multiple of the chunk length)
     size_t off_map = 0, off_local = 0, off_start = 0, bytes = 0;   // workspace layout; cu_seg sits at offset 0
 };
-
-static int sm_count()
-{
-    int dev = 0, n = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || n <= 0)
-        return 148;
-    return n;
-}
 
 // Few long sequences leave most SMs idle (one CTA per sequence x head x slice, each walking its chunks in series).
 // Cutting every sequence into G segments costs about two more passes of state work but runs G times as many CTAs.
@@ -300,7 +299,8 @@ static kla_status chunk_fwd_impl(const kla_desc *desc, const void *q, const void
     }
     if (!(desc->flags & KLA_FLAG_FORCE_SIMT) && chunk_tc_supported(desc->d_k, chunk, desc->io_dtype)) {
         const PackedPlan pp = plan_packed(desc, chunk);
-        if (order_bytes(desc, chunk)) {
+        // (longest first: only where the blocks do not all start at once, or the pieces' plan word is looked up beside it)
+        if (order_bytes(desc, chunk) && (pp.seg_len || (long long)desc->n_seq * desc->H * (desc->d_k / 64) > sm_count())) {
             int32_t *order = (int32_t *)desc->workspace;
             if (launch_seq_order(desc->cu_seqlens, desc->n_seq, order, stream) != cudaSuccess) return KLA_ERR_LAUNCH;
             p.seq_order = order;

@@ -171,9 +171,9 @@ struct PrepSmem {
 template <int D>
 __global__ void __launch_bounds__(256, 2) kla_bwd_prepare_kernel(BwdChunkParams p)
 {
-    extern __shared__ unsigned char smem_dyn[];
+    extern __shared__ __align__(1024) unsigned char smem_dyn[];   // used as declared: rounded up at run time, every access would be generic
     using Smem = PrepSmem<D>;
-    Smem &sm = *reinterpret_cast<Smem *>((reinterpret_cast<uintptr_t>(smem_dyn) + 1023) & ~(uintptr_t)1023);
+    Smem &sm = *reinterpret_cast<Smem *>(smem_dyn);
     constexpr int NB = D / 64;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int slot = blockIdx.x / p.H, h = blockIdx.x % p.H;
@@ -645,8 +645,8 @@ __device__ __forceinline__ void chain(const BwdChunkParams &p, ChainSmem<D> &sm,
 template <int D>
 __global__ void __launch_bounds__(128, 2) kla_bwd_chain_kernel(BwdChunkParams p, int n_units)
 {
-    extern __shared__ unsigned char smem_dyn[];
-    ChainSmem<D> &sm = *reinterpret_cast<ChainSmem<D> *>((reinterpret_cast<uintptr_t>(smem_dyn) + 1023) & ~(uintptr_t)1023);
+    extern __shared__ __align__(1024) unsigned char smem_dyn[];
+    ChainSmem<D> &sm = *reinterpret_cast<ChainSmem<D> *>(smem_dyn);
     // the backward chains, the longer ones, first
     if ((int)blockIdx.x < n_units) chain<D, true>(p, sm, blockIdx.x);
     else chain<D, false>(p, sm, blockIdx.x - n_units);
@@ -1013,7 +1013,7 @@ cudaError_t allow_smem(K kern, int bytes)
 template <int D>
 cudaError_t launch_d(const BwdChunkParams &p, cudaStream_t stream)
 {
-    const int smem1 = (int)sizeof(PrepSmem<D>) + 1024, smem2 = (int)sizeof(ChainSmem<D>) + 1024, smem3 = (int)sizeof(GradSmem<D>);
+    const int smem1 = (int)sizeof(PrepSmem<D>), smem2 = (int)sizeof(ChainSmem<D>), smem3 = (int)sizeof(GradSmem<D>);
     cudaError_t e = allow_smem(kla_bwd_prepare_kernel<D>, smem1);
     if (e == cudaSuccess) e = allow_smem(kla_bwd_chain_kernel<D>, smem2);
     if (e == cudaSuccess) e = allow_smem(kla_bwd_grad_kernel<D>, smem3);
@@ -1051,7 +1051,8 @@ cudaError_t launch_bwd_chunk(const BwdArgs &a, cudaStream_t stream)
     p.coeff_eta = a.coeff_eta; p.qnorm = a.qnorm;
     p.n_slots = a.cu_seqlens ? (int)(a.n_tok / C) + a.n_seq : a.n_seq * ((a.T + C - 1) / C);
     p.order = nullptr;
-    if (a.cu_seqlens && a.n_seq > 1 && a.n_seq <= 4096) {   // (the order takes quadratic work)
+    // longest first only where the chains' blocks do not all start at once (the order takes quadratic work)
+    if (a.cu_seqlens && a.n_seq > 1 && a.n_seq <= 4096 && 2LL * a.n_seq * a.H * (a.d / 64) > sm_count()) {
         int32_t *order = (int32_t *)a.workspace;
         const cudaError_t e = launch_seq_order(a.cu_seqlens, a.n_seq, order, stream);
         if (e != cudaSuccess) return e;

@@ -26,8 +26,8 @@
 //
 // Precision.  q, k, v are exact bf16 operands.  Every derived operand (S, R, X, T, P, U) is a pair of bf16 values hi + lo (16
 // significand bits; one bf16 rounding of any of them costs 1e-2..7e-2 in max|err|/rms, above the 2e-3 bound), a product of two
-// of them hi hi + hi lo + lo hi; U in P U has a third part (tokens with a near-zero key have a huge U, and their rounding is the
-// largest error of all).
+// of them hi hi + hi lo + lo hi.  In a chunk with a near-zero key (beta above HOT_BETA) U has a third part in P U: the rounding of such
+// a token's huge U is the largest error of all.  (In every chunk it would cost 8 %.)
 //
 // Every wait is bounded; when one gives up the block raises an abort flag, reports KLA_ERR_TIMEOUT through the status word,
 // lets its copies and products finish and exits.
@@ -60,6 +60,7 @@ constexpr float LOG2E = 1.4426950408889634f;
 // P, and with the floor neither factor leaves the fp32 / bf16 exponent range however strong the decay.  A floored weight puts at
 // most 1e-35 of a token into the state instead of less.
 constexpr float DEC_FLOOR_LOG2 = 115.f;
+constexpr float HOT_BETA = 4096.f;   // q k beta up to ||q|| sqrt(beta) = 64 ||q||: 2^-18 of that is below the other errors
 constexpr int LDB = 20;       // row stride (floats) of a 16 x 16 block in the solve scratch
 // TMEM columns: [S_hi; S_lo]^T [K; Q]^T (128), [K; Q] K^T (64)
 constexpr uint32_t TM_X = 0, TM_G = 128, TM_COLS = 256;
@@ -79,6 +80,7 @@ struct Slot {
     TriOperand t, p;                            // D T_ii and below them -X D^-1; P D^-1 (rows over ||q|| with the normalised read-out)
     alignas(1024) float ngam[C];                // -exp(g_i)
     float gamq[C];                              // exp(g_i) (over ||q_i||)
+    int hot[2];                                 // some beta above HOT_BETA among tokens 0 .. 31, 32 .. 63
 };
 
 struct PrepScratch {             // of one prepare warp
@@ -146,20 +148,19 @@ __device__ __forceinline__ void mma_first(float2 (&c)[2], const uint32_t (&a)[4]
         : "=f"(c[0].x), "=f"(c[0].y), "=f"(c[1].x), "=f"(c[1].y)
         : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1), "f"(0.f));
 }
-// x as packed bf16 hi and lo parts; returns what the hi part leaves.
-__device__ __forceinline__ float2 split(float2 x, uint32_t &hi, uint32_t &lo)
+// x as packed bf16 hi and lo parts.
+__device__ __forceinline__ void split(float2 x, uint32_t &hi, uint32_t &lo)
 {
     const __nv_bfloat162 h = __floats2bfloat162_rn(x.x, x.y);
     hi = *reinterpret_cast<const uint32_t *>(&h);
     const float2 r = fma2(unpack(hi), f2(-1.f), x);   // exact
     const __nv_bfloat162 l = __floats2bfloat162_rn(r.x, r.y);
     lo = *reinterpret_cast<const uint32_t *>(&l);
-    return r;
 }
 // Register u (0..3) of the left operand made of tiles x, y side by side: x0, x1, y0, y1.
-__device__ __forceinline__ float2 split_left(const float2 (&x)[2], const float2 (&y)[2], int u, uint32_t (&h)[4], uint32_t (&l)[4])
+__device__ __forceinline__ void split_left(const float2 (&x)[2], const float2 (&y)[2], int u, uint32_t (&h)[4], uint32_t (&l)[4])
 {
-    return split(u < 2 ? x[u & 1] : y[u & 1], h[u], l[u]);
+    split(u < 2 ? x[u & 1] : y[u & 1], h[u], l[u]);
 }
 // Tiles x, y as a right operand whose n index is the accumulator's row: x0, y0, x1, y1.
 __device__ __forceinline__ void store_right(TriOperand &o, int b, int lane, const float2 (&x)[2], const float2 (&y)[2])
@@ -384,6 +385,10 @@ __device__ void prepare(const ChunkParams &p, Smem<D> &sm, const Work &wk, int n
                 *reinterpret_cast<float2 *>(td + 8 * LDB + 8) = make_float2(v1 && t2 < g ? ex2_approx(r1 - c1.x) * y[1].x : 0.f, v1 && t2 + 1 < g ? ex2_approx(r1 - c1.y) * y[1].y : 0.f);
             }
             __syncwarp();
+            {
+                const bool hot = __any_sync(0xffffffffu, sc.bet[lane] > HOT_BETA);
+                if (lane == 0) sl.hot[w] = hot;
+            }
             // 8 x 8 diagonal blocks by substitution: lane l solves column l % 8 of block l / 8 of four
             float xs[8];
             {
@@ -561,7 +566,8 @@ __device__ void chain(const ChunkParams &p, Smem<D> &sm, const Work &wk, int nch
             }
         };
         float2 o[8][2];   // Gam Q S, then O
-        uint32_t rh[4], rl[4], uh[2][4], ul[2][4], um[2][4];   // operands R_j; D U_j (hi, lo, and the rest for the outputs)
+        uint32_t rh[4], rl[4], uh[2][4], ul[2][4];   // operands R_j, D U_j
+        const bool hot = HAS_OUT && (sl.hot[0] | sl.hot[1]);
         uint32_t b[2][2][4];
         auto fetch_k = [&](int q) {   // K as right operand: step q = (16 tokens, 32 of d_k)
             const int j = q / (KS / 2), n = 2 * (q % (KS / 2));
@@ -590,14 +596,28 @@ __device__ void chain(const ChunkParams &p, Smem<D> &sm, const Work &wk, int nch
 #pragma unroll
                 for (int i = j; i < 4; ++i) f[i] = sl.p.hi[blk(i, j)][lane];
 #pragma unroll
-                for (int tm = 0; tm < 4; ++tm)
+                for (int tm = 0; tm < 3; ++tm)
 #pragma unroll
                     for (int i = j; i < 4; ++i) {
-                        const uint32_t (&a)[4] = tm == 1 ? ul[j & 1] : tm == 2 ? um[j & 1] : uh[j & 1];
-                        mma(o[2 * i], a, f[i].x, f[i].y);
-                        mma(o[2 * i + 1], a, f[i].z, f[i].w);
-                        if (tm == 2) f[i] = sl.p.lo[blk(i, j)][lane];
+                        mma(o[2 * i], tm == 1 ? ul[j & 1] : uh[j & 1], f[i].x, f[i].y);
+                        mma(o[2 * i + 1], tm == 1 ? ul[j & 1] : uh[j & 1], f[i].z, f[i].w);
+                        if (tm == 1) f[i] = sl.p.lo[blk(i, j)][lane];
                     }
+                if (hot) {   // what hi and lo leave of U_j
+                    uint32_t m[4];
+#pragma unroll
+                    for (int u = 0; u < 4; ++u) {
+                        const float2 r = fma2(unpack(ul[j & 1][u]), f2(-1.f), fma2(unpack(uh[j & 1][u]), f2(-1.f), x[2 * j + (u >> 1)][u & 1]));
+                        const __nv_bfloat162 mm = __floats2bfloat162_rn(r.x, r.y);
+                        m[u] = *reinterpret_cast<const uint32_t *>(&mm);
+                    }
+#pragma unroll
+                    for (int i = j; i < 4; ++i) {
+                        const uint4 ph = sl.p.hi[blk(i, j)][lane];
+                        mma(o[2 * i], m, ph.x, ph.y);
+                        mma(o[2 * i + 1], m, ph.z, ph.w);
+                    }
+                }
             }
         };
         constexpr int QJ = KS / 2, QH = QJ / 2;   // update steps per token block, and half of them
@@ -625,14 +645,7 @@ __device__ void chain(const ChunkParams &p, Smem<D> &sm, const Work &wk, int nch
                 for (int q = 0; q < QH; ++q) update((j - 1) * QJ + q, [] {});
             }
 #pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                const float2 r = split_left(x[2 * j], x[2 * j + 1], u, uh[j & 1], ul[j & 1]);
-                if (HAS_OUT) {
-                    const float2 m = fma2(unpack(ul[j & 1][u]), f2(-1.f), r);
-                    const __nv_bfloat162 mm = __floats2bfloat162_rn(m.x, m.y);
-                    um[j & 1][u] = *reinterpret_cast<const uint32_t *>(&mm);
-                }
-            }
+            for (int u = 0; u < 4; ++u) split_left(x[2 * j], x[2 * j + 1], u, uh[j & 1], ul[j & 1]);
             // R_i -= (X_ij D^-1) (D U_j)
             if (j < 3) {
                 uint4 f[3];

@@ -121,6 +121,7 @@ cudaError_t launch_bwd_chunk(const BwdArgs &a, cudaStream_t stream);
 bool chunk_tc_supported(int d, int chunk, int io_dtype);
 
 void count_launch(int n);
+int sm_count();   // of the current device
 // Host-side validation of a chunk-forward call (api.cu); `check_workspace`: also that desc->workspace is large enough.
 kla_status check_chunk_args(const kla_desc *d, const void *q, const void *k, const void *v, const float *log_alpha, const float *eta,
                             float eps, int32_t chunk, const float *init_state, void *out, float *final_state, bool check_workspace);

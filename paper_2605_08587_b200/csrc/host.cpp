@@ -247,6 +247,82 @@ PyObject *forward(PyObject *, PyObject *const *a, Py_ssize_t n)
     }
 }
 
+// kla_bwd: (q, k, v, log_alpha, eta, eps, d_out, init_state, d_final_state, cu_seqlens, host_seqlens, flags, want_dinit_state,
+// workspace) -> dict
+PyObject *backward(PyObject *, PyObject *const *a, Py_ssize_t n)
+{
+    if (n != 14) {
+        PyErr_SetString(PyExc_TypeError, "backward: 14 arguments");
+        return nullptr;
+    }
+    try {
+        const at::Tensor &q = tensor(a[0], "q"), &k = tensor(a[1], "k"), &v = tensor(a[2], "v");
+        const at::Tensor &la = tensor(a[3], "log_alpha"), &eta = tensor(a[4], "eta"), &d_out = tensor(a[6], "d_out");
+        const float eps = (float)number(a[5]);
+        if (q.dim() != 4 || v.dim() < 1) fail(PyExc_ValueError, "q must be [B, T, H, d_k]");
+        const int64_t B = q.size(0), T = q.size(1), H = q.size(2), d_k = q.size(3), d_v = v.size(-1);
+        if (!has_shape(d_out, {B, T, H, d_v}) || d_out.scalar_type() != q.scalar_type())
+            fail(PyExc_ValueError, "d_out must be [B, T, H, d_v] with the dtype of q");
+        int64_t n_seq = B;
+        const at::Tensor *cu = opt_tensor(a[9], "cu_seqlens"), *init = opt_tensor(a[7], "init_state"), *dfin = opt_tensor(a[8], "d_final_state");
+        const at::Tensor *given = opt_tensor(a[13], "workspace");
+        at::Tensor host;
+        if (cu) {
+            host = tensor(a[10], "host_seqlens");
+            if (!host.is_contiguous()) host = host.contiguous();
+            n_seq = cu->numel() - 1;
+        }
+        void *qa = addr(&q, "q");
+        const c10::cuda::OptionalCUDAGuard guard(q.device());
+        kla_desc d = {};
+        d.B = (int32_t)B;
+        d.T = (int32_t)T;
+        d.H = (int32_t)H;
+        d.d_k = (int32_t)d_k;
+        d.d_v = (int32_t)d_v;
+        d.n_seq = (int32_t)n_seq;
+        d.cu_seqlens = static_cast<const int32_t *>(addr(cu, "cu_seqlens"));
+        d.host_seqlens = cu ? static_cast<const int32_t *>(host.data_ptr()) : nullptr;
+        d.io_dtype = kla_dtype_of(q);
+        d.out_dtype = KLA_F32;
+        d.flags = (int32_t)integer(a[11]);
+        d.stream = c10::cuda::getCurrentCUDAStream(q.device().index()).stream();
+        const auto f32 = q.options().dtype(at::kFloat);
+        const bool want = PyObject_IsTrue(a[12]) == 1;
+        at::Tensor g[6] = {at::empty({B, T, H, d_k}, f32), at::empty({B, T, H, d_k}, f32), at::empty({B, T, H, d_v}, f32),
+                           at::empty({B, T, H}, f32), at::empty({B, T, H}, f32), want ? at::empty({n_seq, H, d_k, d_v}, f32) : at::Tensor()};
+        at::Tensor ws;
+        if (given) ws = *given;
+        else if (const size_t need = kla_bwd_workspace_bytes(&d)) ws = at::empty({(int64_t)need}, q.options().dtype(at::kByte));
+        if (ws.defined()) {
+            d.workspace = addr(&ws, "workspace");
+            d.workspace_bytes = (size_t)ws.numel() * ws.element_size();
+        }
+        void *ka = addr(&k, "k"), *va = addr(&v, "v"), *da = addr(&d_out, "d_out");
+        float *laa = addr_f32(&la, "log_alpha"), *ea = addr_f32(&eta, "eta"), *ia = addr_f32(init, "init_state"), *fa = addr_f32(dfin, "d_final_state");
+        float *ga[6];
+        for (int i = 0; i < 6; ++i) ga[i] = g[i].defined() ? static_cast<float *>(g[i].data_ptr()) : nullptr;
+        kla_status st;
+        Py_BEGIN_ALLOW_THREADS
+        st = kla_bwd(&d, qa, ka, va, laa, ea, eps, ia, da, fa, ga[0], ga[1], ga[2], ga[3], ga[4], ga[5]);
+        Py_END_ALLOW_THREADS
+        check(st);
+        static const char *const names[6] = {"dq", "dk", "dv", "dlog_alpha", "deta", "dinit_state"};
+        PyObject *r = PyDict_New();
+        for (int i = 0; r && i < 6; ++i) {
+            PyObject *o = g[i].defined() ? THPVariable_Wrap(std::move(g[i])) : (Py_INCREF(Py_None), Py_None);
+            if (!o || PyDict_SetItemString(r, names[i], o) != 0) Py_CLEAR(r);
+            Py_XDECREF(o);
+        }
+        return r;
+    } catch (const Failed &) {
+        return nullptr;
+    } catch (const std::exception &e) {
+        PyErr_SetString(PyExc_RuntimeError, e.what());
+        return nullptr;
+    }
+}
+
 PyObject *init(PyObject *, PyObject *const *a, Py_ssize_t n)
 {
     if (n != 2) {
@@ -261,6 +337,7 @@ PyObject *init(PyObject *, PyObject *const *a, Py_ssize_t n)
 PyMethodDef methods[] = {{"init", (PyCFunction)(void (*)())init, METH_FASTCALL, nullptr},
                          {"decode", (PyCFunction)(void (*)())decode, METH_FASTCALL, nullptr},
                          {"forward", (PyCFunction)(void (*)())forward, METH_FASTCALL, nullptr},
+                         {"backward", (PyCFunction)(void (*)())backward, METH_FASTCALL, nullptr},
                          {nullptr, nullptr, 0, nullptr}};
 PyModuleDef module = {PyModuleDef_HEAD_INIT, "_host", nullptr, -1, methods, nullptr, nullptr, nullptr, nullptr};
 
