@@ -21,7 +21,7 @@
 // the schedulers' instruction caches and issues at about one instruction in three cycles (measured on unrolled against rolled
 // copies of the same products).  With all products on mma.sync (504 per chunk and warp at d = 128 instead of 248) a chunk took
 // 8 000 cycles; with all of them on tcgen05, whose every product on the chain ends in a hand-over through tensor memory and shared
-// memory, 7 400; this way 5 300.  mma.sync stands still while a tcgen05 product runs, so the two add up: 570 cycles for the state
+// memory, 7 400; this way 5 100.  mma.sync stands still while a tcgen05 product runs, so the two add up: 570 cycles for the state
 // product, 400 for [K; Q] K^T, 8 per mma.sync.
 //
 // Precision.  q, k, v are exact bf16 operands.  Every derived operand (S, R, X, T, P, U) is a pair of bf16 values hi + lo (16
@@ -93,11 +93,12 @@ enum Bar {
     B_FULL = 0,      // + slot: tiles landed
     B_READY = 3,     // + slot: operands and scalars written
     B_DONE = 6,      // + slot: every chain warp is through with it
-    B_STATE = 9,     // S^T operand of the next chunk written
+    B_STATE = 9,     // S^T operand of the next chunk written ...
+    B_STATE1 = 13,   // ... its second 64 rows of d_k (d = 128)
     B_X = 10,        // [S_hi; S_lo]^T [K; Q]^T complete
     B_G = 11,        // [K; Q] K^T complete
     B_GFREE = 12,    // ... and read
-    B_COUNT = 13
+    B_COUNT = 14
 };
 
 template <int D>
@@ -206,6 +207,42 @@ __device__ __forceinline__ void tmem_sum(uint32_t addr, float2 (&x)[8][2])
         for (int e = 0; e < 2; ++e)
             x[t][e] = add2(make_float2(__uint_as_float(h[4 * t + 2 * e]), __uint_as_float(h[4 * t + 2 * e + 1])),
                            make_float2(__uint_as_float(l[4 * t + 2 * e]), __uint_as_float(l[4 * t + 2 * e + 1])));
+}
+
+// Tiles 0, 1 and tiles 2 .. 7 of the same.
+__device__ __forceinline__ void tmem_sum_first(uint32_t addr, float2 (&x)[8][2])
+{
+    uint32_t h[8], l[8];
+#define R8(a, i) "=r"(a[i]), "=r"(a[i + 1]), "=r"(a[i + 2]), "=r"(a[i + 3]), "=r"(a[i + 4]), "=r"(a[i + 5]), "=r"(a[i + 6]), "=r"(a[i + 7])
+    asm volatile(
+        "tcgen05.ld.sync.aligned.16x256b.x2.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%16];\n\t"
+        "tcgen05.ld.sync.aligned.16x256b.x2.b32 {%8, %9, %10, %11, %12, %13, %14, %15}, [%17];\n\t"
+        "tcgen05.wait::ld.sync.aligned;" : R8(h, 0), R8(l, 0) : "r"(addr), "r"(addr + (16u << 16)) : "memory");
+#pragma unroll
+    for (int t = 0; t < 2; ++t)
+#pragma unroll
+        for (int e = 0; e < 2; ++e)
+            x[t][e] = add2(make_float2(__uint_as_float(h[4 * t + 2 * e]), __uint_as_float(h[4 * t + 2 * e + 1])),
+                           make_float2(__uint_as_float(l[4 * t + 2 * e]), __uint_as_float(l[4 * t + 2 * e + 1])));
+}
+__device__ __forceinline__ void tmem_sum_rest(uint32_t addr, float2 (&x)[8][2])
+{
+    uint32_t h[24], l[24];
+    asm volatile(
+        "tcgen05.ld.sync.aligned.16x256b.x2.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%48];\n\t"
+        "tcgen05.ld.sync.aligned.16x256b.x2.b32 {%24, %25, %26, %27, %28, %29, %30, %31}, [%49];\n\t"
+        "tcgen05.ld.sync.aligned.16x256b.x4.b32 {%8, %9, %10, %11, %12, %13, %14, %15, %16, %17, %18, %19, %20, %21, %22, %23}, [%50];\n\t"
+        "tcgen05.ld.sync.aligned.16x256b.x4.b32 {%32, %33, %34, %35, %36, %37, %38, %39, %40, %41, %42, %43, %44, %45, %46, %47}, [%51];\n\t"
+        "tcgen05.wait::ld.sync.aligned;"
+        : R8(h, 0), R8(h, 8), R8(h, 16), R8(l, 0), R8(l, 8), R8(l, 16)
+        : "r"(addr + 16), "r"(addr + 16 + (16u << 16)), "r"(addr + 32), "r"(addr + 32 + (16u << 16)) : "memory");
+#undef R8
+#pragma unroll
+    for (int t = 0; t < 6; ++t)
+#pragma unroll
+        for (int e = 0; e < 2; ++e)
+            x[t + 2][e] = add2(make_float2(__uint_as_float(h[4 * t + 2 * e]), __uint_as_float(h[4 * t + 2 * e + 1])),
+                               make_float2(__uint_as_float(l[4 * t + 2 * e]), __uint_as_float(l[4 * t + 2 * e + 1])));
 }
 
 // What a block works on; see ChunkParams for the segment passes.
@@ -527,15 +564,17 @@ __device__ void chain(const ChunkParams &p, Smem<D> &sm, const Work &wk, int nch
         asm volatile("stmatrix.sync.aligned.m8n8.x4.shared.b16 [%0], {%1, %2, %3, %4};" ::"r"(a), "r"(h[0]), "r"(h[1]), "r"(h[2]), "r"(h[3]) : "memory");
         asm volatile("stmatrix.sync.aligned.m8n8.x4.shared.b16 [%0], {%1, %2, %3, %4};" ::"r"(a + 2048), "r"(l[0]), "r"(l[1]), "r"(l[2]), "r"(l[3]) : "memory");
     };
-    auto state_written = [&]() {
+    // d = 128: the product over the first 64 rows of d_k starts while the others are being finished (-1.5 %)
+    auto state_written = [&](int part) {
         fence_async_smem();
         tc_fence_before();
         __syncwarp();
-        if (lane == 0) mbar_arrive(&sm.bar[B_STATE]);
+        if (lane == 0) mbar_arrive(&sm.bar[part ? B_STATE1 : B_STATE]);
     };
 #pragma unroll
     for (int ks = 0; ks < KS; ++ks) store_state(ks);
-    state_written();
+    if (D == 128) state_written(1);
+    state_written(0);
 
     const size_t tok_stride = (size_t)p.H * D;
     Elem *out = static_cast<Elem *>(p.out) + ((size_t)wk.tok0 * p.H + wk.h) * D + wk.sl * NS + 16 * w;
@@ -555,7 +594,7 @@ __device__ void chain(const ChunkParams &p, Smem<D> &sm, const Work &wk, int nch
         tc_fence_after();
 
         float2 x[8][2];   // K S, then R, then D U
-        tmem_sum(tx, x);
+        tmem_sum_first(tx, x);
         auto residual = [&](int t) {   // R = V - Gam K S, 8 tokens
             const float2 gm = load2(&sl.ngam[8 * t + t2]);
             x[t][0] = fma2(gm, x[t][0], unpack(vv[t >> 1][2 * (t & 1)]));
@@ -638,6 +677,7 @@ __device__ void chain(const ChunkParams &p, Smem<D> &sm, const Work &wk, int nch
                 mma(x[2 * j + 1], rh, tl.z, tl.w);
             }
             if (j == 0) {
+                tmem_sum_rest(tx, x);
 #pragma unroll
                 for (int t = 2; t < 8; ++t) residual(t);
             } else {
@@ -698,10 +738,11 @@ __device__ void chain(const ChunkParams &p, Smem<D> &sm, const Work &wk, int nch
                     store_state(2 * q - 2);
                     store_state(2 * q - 1);
                 }
+                if (D == 128 && q == QJ / 2 && c + 1 < nchunks) state_written(0);
             });
         store_state(KS - 2);
         store_state(KS - 1);
-        if (c + 1 < nchunks) state_written();
+        if (c + 1 < nchunks) state_written(D == 128);
         if constexpr (HAS_OUT) {
             const int live = c >= wk.first_out ? rows : 0;
             if constexpr (std::is_same<OUT, float>::value) {
@@ -795,7 +836,10 @@ __device__ void issue(const CUtensorMap *tm_q, const CUtensorMap *tm_k, const CU
         if (!wait(B_STATE, c)) return;
         const uint32_t a = desc_lo(smem_desc_sw128(smem_u32(sm.st), 0, 1024)), b = desc_lo(smem_desc_sw128(smem_u32(sm.slot[c % NSLOT].kq), 0, 1024));
 #pragma unroll
-        for (int kb = 0; kb < NB; ++kb) mma4_bf16_lo<2, 2>(sm.tmem + TM_X, a + kb * 1024, b + kb * 1024, idesc_bf16(128, HAS_OUT ? 128 : 64, 0, 0), kb > 0);
+        for (int kb = 0; kb < NB; ++kb) {
+            if (kb == 1 && !wait(B_STATE1, c)) return;
+            mma4_bf16_lo<2, 2>(sm.tmem + TM_X, a + kb * 1024, b + kb * 1024, idesc_bf16(128, HAS_OUT ? 128 : 64, 0, 0), kb > 0);
+        }
         mma_commit(&sm.bar[B_X]);
         if (c + 1 < nchunks) {
             if (!wait(B_FULL + (c + 1) % NSLOT, (c + 1) / NSLOT) || !wait(B_GFREE, c)) return;
@@ -835,6 +879,7 @@ kla_chunk_mma_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_cons
             mbar_init(&sm.bar[B_DONE + s], 4);
         }
         mbar_init(&sm.bar[B_STATE], 4);
+        mbar_init(&sm.bar[B_STATE1], 4);
         mbar_init(&sm.bar[B_X], 1);
         mbar_init(&sm.bar[B_G], 1);
         mbar_init(&sm.bar[B_GFREE], 4);
