@@ -89,6 +89,14 @@ struct PackedPlan {
 };
 
 
+// Time of a launch of the chunk kernel per chunk of a block, in units of a chunk of a block that has its SM to itself (measured: d = 64, B 16, H 16, T 4096, two blocks on an SM 4.5 us a chunk, one 2.75 us).
+static double rounds(int d, long long blocks)
+{
+    const bool two = d == 64 && blocks > sm_count();
+    const int r = two ? 2 * sm_count() : sm_count();
+    return (double)((blocks + r - 1) / r) * (two ? 1.63 : 1.0);
+}
+
 static PackedPlan plan_packed(const kla_desc *d, int32_t chunk)
 {
     PackedPlan pp;
@@ -145,16 +153,15 @@ static SegPlan plan_segments(const kla_desc *d, int32_t chunk)
     if (forced >= 2) {
         best_len = (chunks + forced - 1) / forced;
     } else if (forced == 0) {
-        const int sms = sm_count();
-        auto waves = [&](int ctas) { return (ctas + sms - 1) / sms; };
-        const double plain = (double)waves(units) * chunks;
+        auto waves = [&](long long blocks) { return rounds(d->d_k, blocks); };
+        const double plain = waves(units) * chunks;
         double best = 0.75 * plain;   // only worth it for a clear win
         for (int G = 2; G <= 32 && chunks / G >= 8; ++G) {
             const int len = (chunks + G - 1) / G, Ge = (chunks + len - 1) / len;
             if (Ge < 2) continue;
             // measured on the 65K single-sequence workload (per-pass device times): a chunk of pass 1 (no outputs) takes 0.86 of a
             // main-pass chunk, and chaining the maps costs 2.2 chunk periods per segment
-            const double cost = 0.86 * waves(units * 2 * (Ge - 1)) * len + (double)waves(units * Ge) * len + 2.2 * Ge;
+            const double cost = 0.86 * waves(2LL * units * (Ge - 1)) * len + waves((long long)units * Ge) * len + 2.2 * Ge;
             if (cost < best) {
                 best = cost;
                 best_len = len;
@@ -283,17 +290,17 @@ static kla_status chunk_fwd_impl(const kla_desc *desc, const void *q, const void
         if (launch_seg_combine(init_state, map, local, start, desc->B, desc->H, pl.G, desc->d_k, cu_seg + desc->B * pl.G + 1, stream) != cudaSuccess)
             return KLA_ERR_LAUNCH;
         mark(3);
-        ChunkParams p3 = p;   // pass 3: every segment from its true start state
+        ChunkParams p3 = p;   // pass 3: every segment from its true start state; or pass 4: from a warm-up run
         p3.cu_seqlens = cu_seg; p3.n_seq = desc->B * pl.G;
-        p3.init_state = start;
-        p3.seg_pass = 3; p3.seg_G = pl.G;
-        err = launch_chunk_tc(p3, desc->d_k, desc->io_dtype, desc->out_dtype, stream);
-        if (err == cudaSuccess && try_warm) {
-            ChunkParams p4 = p;   // pass 4: every segment from a warm-up run (the sequence's first from its initial state)
-            p4.cu_seqlens = cu_seg; p4.n_seq = desc->B * pl.G;
-            p4.seg_pass = 4; p4.seg_G = pl.G;
-            err = launch_chunk_tc(p4, desc->d_k, desc->io_dtype, desc->out_dtype, stream);
+        p3.seg_G = pl.G;
+        if (try_warm) {
+            p3.seg_pass = 7;
+            p3.map_state = start;
+        } else {
+            p3.seg_pass = 3;
+            p3.init_state = start;
         }
+        err = launch_chunk_tc(p3, desc->d_k, desc->io_dtype, desc->out_dtype, stream);
         mark(4);
         return err == cudaSuccess ? KLA_OK : KLA_ERR_LAUNCH;
     }

@@ -52,7 +52,6 @@ using namespace umma;
 
 constexpr int C = 64;         // chunk length
 constexpr int NS = 64;        // state columns per block
-constexpr int NSLOT = 3;      // chunk slots
 constexpr int CHAIN_T = 128, PREP_T = 128, NT = CHAIN_T + PREP_T + 128;   // (the last warpgroup: one warp works)
 constexpr long long WAIT_LIMIT = 2000000000LL;   // SM clocks (~1 s) before a wait gives up
 constexpr float LOG2E = 1.4426950408889634f;
@@ -78,14 +77,15 @@ struct Slot {
     alignas(1024) unsigned char kq[NB * 16384];
     alignas(1024) unsigned char v[8192];        // this block's 64 columns; then the outputs on their way out
     TriOperand t, p;                            // D T_ii and below them -X D^-1; P D^-1 (rows over ||q|| with the normalised read-out)
-    alignas(1024) float ngam[C];                // -exp(g_i)
-    float gamq[C];                              // exp(g_i) (over ||q_i||)
-    int hot[2];                                 // some beta above HOT_BETA among tokens 0 .. 31, 32 .. 63
+};
+struct alignas(16) Scalars {     // of one chunk
+    float ngam[C];               // -exp(g_i)
+    float gamq[C];               // exp(g_i) (over ||q_i||)
+    int hot[2];                  // some beta above HOT_BETA among tokens 0 .. 31, 32 .. 63
 };
 
-struct PrepScratch {             // of one prepare warp
-    float td[2][16 * LDB];       // X_ii, then T_ii, of its two row blocks
-    float m[2][8 * LDB];
+struct alignas(16) PrepScratch {             // of one prepare warp
+    float td[2][16 * LDB];       // X_ii, then T_ii, of its two row blocks; the unused upper right 8 x 8 holds an intermediate
     float bet[32];
 };
 
@@ -101,13 +101,17 @@ enum Bar {
     B_COUNT = 14
 };
 
-template <int D>
+// BPS, blocks per SM.  One: three chunk slots, registers for the whole chain.  Two (d = 64, more blocks than SMs): two slots and
+// half the registers each, so that one block's products fill the other's latencies.
+template <int D, int BPS>
 struct Smem {
+    static constexpr int NSLOT = BPS == 1 ? 3 : 2;
     Slot<D> slot[NSLOT];
     // S^T as left operand, per 64 of d_k: 128 rows of 128 bytes; warp w: rows 32 w .. the hi, 32 w + 16 .. the lo parts of its columns
     alignas(1024) unsigned char st[D / 64 * 16384];
+    Scalars scal[NSLOT];
     PrepScratch prep[2];
-    float g2[4][C], g3[4][C];    // log2(e) g_i, max(log2(e) g_C, log2(e) g_i - floor): a copy for each prepare warp
+    float g2[4][C];              // log2(e) g_i, a copy for each prepare warp
     float qinv[C];
     alignas(8) uint64_t bar[B_COUNT];
     uint32_t tmem;
@@ -256,8 +260,17 @@ struct Work {
 };
 // Returns false when there is nothing to do (the other kind of pass does the work, or an empty sequence, done here).
 template <int D>
-__device__ bool find_work(const ChunkParams &p, Work &w)
+__device__ bool find_work(const ChunkParams &params, Work &w)
 {
+    ChunkParams p = params;
+    if (p.seg_pass == 7) {
+        if (p.cu_seqlens[p.n_seq + 1] == 1) {
+            p.seg_pass = 4;
+        } else {
+            p.seg_pass = 3;
+            p.init_state = p.map_state;
+        }
+    }
     constexpr int SLICES = D / NS;
     if (p.seg_pass == 6) {
         if (p.seq_order[p.seg_G] != 0) return false;
@@ -322,17 +335,17 @@ __device__ bool find_work(const ChunkParams &p, Work &w)
 // loop.  T_ii = (I + B X)_ii^-1 B by 8 x 8 substitution (a column per lane) and one merge; the rest of the triangular solve is
 // left to the chain, which takes U block by block: as many products there as with the whole inverse, and the block products of
 // the inverse, longer than everything else here, are not needed.
-template <int D, bool VAR>
-__device__ void prepare(const ChunkParams &p, Smem<D> &sm, const Work &wk, int nchunks)
+template <int D, int BPS, bool VAR>
+__device__ void prepare(const ChunkParams &p, Smem<D, BPS> &sm, const Work &wk, int nchunks)
 {
-    constexpr int NB = D / 64;
+    constexpr int NB = D / 64, NSLOT = Smem<D, BPS>::NSLOT;
     const int lane = threadIdx.x & 31, w = (threadIdx.x >> 5) & 3;
     const int g = lane >> 2, t2 = 2 * (lane & 3);
     const int h = wk.h;
     const bool isx = w < 2;
     const uint32_t tg = sm.tmem + TM_G + ((uint32_t)(32 * w) << 16);
     PrepScratch &sc = sm.prep[w & 1];
-    float *g2 = sm.g2[w], *g3 = sm.g3[w];
+    float *g2 = sm.g2[w];
 
     // log alpha of tokens 2 lane, 2 lane + 1; eta of the warp's token blocks (X warps), tokens g, g + 8 of each: a chunk ahead
     float la[2], et[4];
@@ -366,8 +379,8 @@ __device__ void prepare(const ChunkParams &p, Smem<D> &sm, const Work &wk, int n
         const float gc2 = __shfl_sync(0xffffffffu, incl, 31) * LOG2E, ga2 = (incl - la[1]) * LOG2E, gb2 = incl * LOG2E;
         const float e4[4] = {et[0], et[1], et[2], et[3]};
         *reinterpret_cast<float2 *>(&g2[2 * lane]) = make_float2(ga2, gb2);
-        *reinterpret_cast<float2 *>(&g3[2 * lane]) = make_float2(fmaxf(gc2, ga2 - DEC_FLOOR_LOG2), fmaxf(gc2, gb2 - DEC_FLOOR_LOG2));
         if (c + 1 < nchunks) fetch(c + 1);
+        auto floored = [&](float2 x) { return make_float2(fmaxf(gc2, x.x - DEC_FLOOR_LOG2), fmaxf(gc2, x.y - DEC_FLOOR_LOG2)); };
         const bool qnorm = VAR && (p.variant & VARIANT_QNORM);
         // the product is there: so are the tiles, and the slot's last user is through
         if (!bar_wait(&sm.bar[B_G], c & 1, &sm.abort_flag)) break;
@@ -391,9 +404,9 @@ __device__ void prepare(const ChunkParams &p, Smem<D> &sm, const Work &wk, int n
             }
             if ((lane >> 4) == w - 2) {   // per-token scalars
                 float2 gm = make_float2(ex2_approx(ga2), ex2_approx(gb2));
-                *reinterpret_cast<float2 *>(&sl.ngam[2 * lane]) = make_float2(-gm.x, -gm.y);
+                *reinterpret_cast<float2 *>(&sm.scal[s].ngam[2 * lane]) = make_float2(-gm.x, -gm.y);
                 if (qnorm) gm = mul2(gm, load2(&sm.qinv[2 * lane]));
-                *reinterpret_cast<float2 *>(&sl.gamq[2 * lane]) = gm;
+                *reinterpret_cast<float2 *>(&sm.scal[s].gamq[2 * lane]) = gm;
             }
         }
         __syncwarp();
@@ -424,7 +437,7 @@ __device__ void prepare(const ChunkParams &p, Smem<D> &sm, const Work &wk, int n
             __syncwarp();
             {
                 const bool hot = __any_sync(0xffffffffu, sc.bet[lane] > HOT_BETA);
-                if (lane == 0) sl.hot[w] = hot;
+                if (lane == 0) sm.scal[s].hot[w] = hot;
             }
             // 8 x 8 diagonal blocks by substitution: lane l solves column l % 8 of block l / 8 of four
             float xs[8];
@@ -458,7 +471,7 @@ __device__ void prepare(const ChunkParams &p, Smem<D> &sm, const Work &wk, int n
                 float2 a = f2(0.f);
 #pragma unroll
                 for (int m = 0; m < 8; ++m) a = fma2(f2(f[m]), load2(td + m * LDB + t2), a);
-                *reinterpret_cast<float2 *>(sc.m[rb] + g * LDB + t2) = mul2(f2(-sc.bet[16 * rb + 8 + g]), a);
+                *reinterpret_cast<float2 *>(sc.td[rb] + g * LDB + 8 + t2) = mul2(f2(-sc.bet[16 * rb + 8 + g]), a);
             }
             __syncwarp();
 #pragma unroll
@@ -468,7 +481,7 @@ __device__ void prepare(const ChunkParams &p, Smem<D> &sm, const Work &wk, int n
                 const float f[8] = {f0.x, f0.y, f0.z, f0.w, f1.x, f1.y, f1.z, f1.w};
                 float2 a = f2(0.f);
 #pragma unroll
-                for (int m = 0; m < 8; ++m) a = fma2(f2(f[m]), load2(sc.m[rb] + m * LDB + t2), a);
+                for (int m = 0; m < 8; ++m) a = fma2(f2(f[m]), load2(td + m * LDB + 8 + t2), a);
                 const float2 c0 = load2(&sc.bet[16 * rb + t2]), c1 = load2(&sc.bet[16 * rb + 8 + t2]);
                 const int i0 = 32 * w + 16 * rb + g;
                 const float2 d0 = f2(ex2_approx(fmaxf(gc2 - g2[i0], -DEC_FLOOR_LOG2))), d1 = f2(ex2_approx(fmaxf(gc2 - g2[i0 + 8], -DEC_FLOOR_LOG2)));
@@ -491,7 +504,7 @@ __device__ void prepare(const ChunkParams &p, Smem<D> &sm, const Work &wk, int n
 #pragma unroll 1
             for (int j = 0; j < nb; ++j) {
                 tmem_block(tg + ((uint32_t)(16 * rb) << 16) + 16 * j, x, y);
-                const float2 c0 = load2(&g3[16 * j + t2]), c1 = load2(&g3[16 * j + 8 + t2]);
+                const float2 c0 = floored(load2(&g2[16 * j + t2])), c1 = floored(load2(&g2[16 * j + 8 + t2]));
                 const int lim = j == bi ? g : 16;   // columns up to the row on the diagonal block
                 x[0].x = v0 && t2 <= lim ? f0 * ex2_approx(r0 - c0.x) * x[0].x : 0.f;
                 x[0].y = v0 && t2 < lim ? f0 * ex2_approx(r0 - c0.y) * x[0].y : 0.f;
@@ -525,12 +538,12 @@ __device__ void prepare(const ChunkParams &p, Smem<D> &sm, const Work &wk, int n
 // OUT = void: no outputs (segment pass 1).  A warp has its scheduler almost to itself and issues in order, so what waits for
 // nothing is placed between what does: the state update and the outputs of token block j - 1 cover the solve of block j, and the
 // outputs leave while the next chunk's state product runs.
-template <int D, typename OUT>
-__device__ void chain(const ChunkParams &p, Smem<D> &sm, const Work &wk, int nchunks)
+template <int D, int BPS, typename OUT>
+__device__ void chain(const ChunkParams &p, Smem<D, BPS> &sm, const Work &wk, int nchunks)
 {
     constexpr bool HAS_OUT = !std::is_void<OUT>::value;
     using Elem = typename std::conditional<HAS_OUT, OUT, char>::type;
-    constexpr int KS = D / 16;
+    constexpr int KS = D / 16, NSLOT = Smem<D, BPS>::NSLOT;
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const int g = lane >> 2, t2 = 2 * (lane & 3);
     const int dv = wk.sl * NS + 16 * w + g;   // columns dv, dv + 8 of d_v
@@ -596,7 +609,7 @@ __device__ void chain(const ChunkParams &p, Smem<D> &sm, const Work &wk, int nch
         float2 x[8][2];   // K S, then R, then D U
         tmem_sum_first(tx, x);
         auto residual = [&](int t) {   // R = V - Gam K S, 8 tokens
-            const float2 gm = load2(&sl.ngam[8 * t + t2]);
+            const float2 gm = load2(&sm.scal[s].ngam[8 * t + t2]);
             x[t][0] = fma2(gm, x[t][0], unpack(vv[t >> 1][2 * (t & 1)]));
             x[t][1] = fma2(gm, x[t][1], unpack(vv[t >> 1][2 * (t & 1) + 1]));
             if (rows < C) {   // tokens past the end
@@ -606,7 +619,7 @@ __device__ void chain(const ChunkParams &p, Smem<D> &sm, const Work &wk, int nch
         };
         float2 o[8][2];   // Gam Q S, then O
         uint32_t rh[4], rl[4], uh[2][4], ul[2][4];   // operands R_j, D U_j
-        const bool hot = HAS_OUT && (sl.hot[0] | sl.hot[1]);
+        const bool hot = HAS_OUT && (sm.scal[s].hot[0] | sm.scal[s].hot[1]);
         uint32_t b[2][2][4];
         auto fetch_k = [&](int q) {   // K as right operand: step q = (16 tokens, 32 of d_k)
             const int j = q / (KS / 2), n = 2 * (q % (KS / 2));
@@ -706,7 +719,7 @@ __device__ void chain(const ChunkParams &p, Smem<D> &sm, const Work &wk, int nch
                 }
             }
             if (j == 0) {
-                const float2 gC = f2(-sl.ngam[C - 1]);
+                const float2 gC = f2(-sm.scal[s].ngam[C - 1]);
                 fetch_k(0);
 #pragma unroll
                 for (int t = 0; t < D / 8; ++t) { S[t][0] = mul2(S[t][0], gC); S[t][1] = mul2(S[t][1], gC); }
@@ -714,7 +727,7 @@ __device__ void chain(const ChunkParams &p, Smem<D> &sm, const Work &wk, int nch
                     tmem_sum(tx + 64, o);
 #pragma unroll
                     for (int t = 0; t < 8; ++t) {
-                        const float2 gq = load2(&sl.gamq[8 * t + t2]);
+                        const float2 gq = load2(&sm.scal[s].gamq[8 * t + t2]);
                         o[t][0] = mul2(o[t][0], gq);
                         o[t][1] = mul2(o[t][1], gq);
                     }
@@ -797,11 +810,12 @@ __device__ void chain(const ChunkParams &p, Smem<D> &sm, const Work &wk, int nch
 }
 
 // ---- issue ----------------------------------------------------------------------------------------------------------------
-// One warp in lock step.  In the order the events fall: the state product of chunk c, [K; Q] K^T of chunk c + 1, the loads of c + 2.
-template <int D, bool HAS_OUT>
-__device__ void issue(const CUtensorMap *tm_q, const CUtensorMap *tm_k, const CUtensorMap *tm_v, Smem<D> &sm, const Work &wk, int nchunks)
+// One warp in lock step.  In the order the events fall: the state product of chunk c, [K; Q] K^T of chunk c + 1, the loads of c + 2
+// (with two slots those of c + 1, before its [K; Q] K^T).
+template <int D, int BPS, bool HAS_OUT>
+__device__ void issue(const CUtensorMap *tm_q, const CUtensorMap *tm_k, const CUtensorMap *tm_v, Smem<D, BPS> &sm, const Work &wk, int nchunks)
 {
-    constexpr int NB = D / 64;
+    constexpr int NB = D / 64, NSLOT = Smem<D, BPS>::NSLOT;
     const bool first = (threadIdx.x & 31) == 0;
     auto load = [&](int c) {
         if (first) {
@@ -841,29 +855,35 @@ __device__ void issue(const CUtensorMap *tm_q, const CUtensorMap *tm_k, const CU
             mma4_bf16_lo<2, 2>(sm.tmem + TM_X, a + kb * 1024, b + kb * 1024, idesc_bf16(128, HAS_OUT ? 128 : 64, 0, 0), kb > 0);
         }
         mma_commit(&sm.bar[B_X]);
-        if (c + 1 < nchunks) {
-            if (!wait(B_FULL + (c + 1) % NSLOT, (c + 1) / NSLOT) || !wait(B_GFREE, c)) return;
+        auto next_gram = [&]() {
+            if (c + 1 >= nchunks) return true;
+            if (!wait(B_FULL + (c + 1) % NSLOT, (c + 1) / NSLOT) || !wait(B_GFREE, c)) return false;
             gram(c + 1);
-        }
-        if (c >= 1 && c + 2 < nchunks) {
-            if (!wait(B_DONE + (c + 2) % NSLOT, (c + 2) / NSLOT - 1)) return;
-            load(c + 2);
-        }
+            return true;
+        };
+        auto next_load = [&]() {   // into the slot of chunk c - 1
+            if (c == 0 || c - 1 + NSLOT >= nchunks) return true;
+            if (!wait(B_DONE + (c - 1) % NSLOT, (c - 1) / NSLOT)) return false;
+            load(c - 1 + NSLOT);
+            return true;
+        };
+        if (NSLOT == 3 ? !next_gram() || !next_load() : !next_load() || !next_gram()) return;
     }
 }
 
 // VAR: compiled with the layer-edge variants (beta = eta, read-out over ||q||) and the test hook; the default instantiation
 // carries none of their code.
-template <int D, typename OUT, bool VAR>
-__global__ void __launch_bounds__(NT, 1)
+template <int D, int BPS, typename OUT, bool VAR>
+__global__ void __launch_bounds__(NT, BPS)
 kla_chunk_mma_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k,
                      const __grid_constant__ CUtensorMap tm_v, ChunkParams p)
 {
     // Used as declared, not rounded up at run time: the compiler then knows that it is shared memory (rounded up, every access is
     // a generic one: 12 % slower).  There is no static shared memory, so it starts on such a boundary; checked all the same.
     extern __shared__ __align__(1024) unsigned char smem_dyn[];
-    Smem<D> &sm = *reinterpret_cast<Smem<D> *>(smem_dyn);
-    static_assert(sizeof(Smem<D>) <= 232448, "shared memory of one block");
+    constexpr int NSLOT = Smem<D, BPS>::NSLOT;
+    Smem<D, BPS> &sm = *reinterpret_cast<Smem<D, BPS> *>(smem_dyn);
+    static_assert(sizeof(Smem<D, BPS>) <= (BPS == 1 ? 232448 : 115712), "shared memory of one block");
     if (smem_u32(smem_dyn) & 1023) {
         if (threadIdx.x == 0 && p.status_word) atomicExch(p.status_word, (int)KLA_ERR_ALIGN);
         return;
@@ -893,16 +913,19 @@ kla_chunk_mma_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_cons
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    // 384 threads x 168 registers at launch = 128 x (240 + 200 + 64)
+    // One block per SM: 384 threads x 168 registers at launch = 128 x (240 + 200 + 64).  Two: 384 x 80 = 128 x (152 + 64 + 24).
     if (tid < CHAIN_T) {
-        asm volatile("setmaxnreg.inc.sync.aligned.u32 240;");
-        chain<D, OUT>(p, sm, wk, nchunks);
+        if (BPS == 1) asm volatile("setmaxnreg.inc.sync.aligned.u32 240;");
+        else asm volatile("setmaxnreg.inc.sync.aligned.u32 152;");
+        chain<D, BPS, OUT>(p, sm, wk, nchunks);
     } else if (tid < CHAIN_T + PREP_T) {
-        asm volatile("setmaxnreg.inc.sync.aligned.u32 200;");
-        prepare<D, VAR>(p, sm, wk, nchunks);
+        if (BPS == 1) asm volatile("setmaxnreg.inc.sync.aligned.u32 200;");
+        else asm volatile("setmaxnreg.dec.sync.aligned.u32 64;");
+        prepare<D, BPS, VAR>(p, sm, wk, nchunks);
     } else {
-        asm volatile("setmaxnreg.dec.sync.aligned.u32 64;");
-        if (tid < CHAIN_T + PREP_T + 32) issue<D, !std::is_void<OUT>::value>(&tm_q, &tm_k, &tm_v, sm, wk, nchunks);
+        if (BPS == 1) asm volatile("setmaxnreg.dec.sync.aligned.u32 64;");
+        else asm volatile("setmaxnreg.dec.sync.aligned.u32 24;");
+        if (tid < CHAIN_T + PREP_T + 32) issue<D, BPS, !std::is_void<OUT>::value>(&tm_q, &tm_k, &tm_v, sm, wk, nchunks);
     }
     tc_fence_before();
     __syncthreads();
@@ -949,7 +972,13 @@ bool make_tmap(CUtensorMap *tm, const void *base, uint64_t n_tok, uint64_t row_e
               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-template <int D, typename OUT, bool VAR>
+// segment pass 1: (seg_G - 1) segments per sequence, twice the slices; p.n_seq counts all segments there
+template <int D>
+int blocks_of(const ChunkParams &p)
+{
+    return p.seg_pass == 1 ? (p.n_seq / p.seg_G) * (p.seg_G - 1) * p.H * 2 * (D / NS) : p.n_seq * p.H * (D / NS);
+}
+template <int D, int BPS, typename OUT, bool VAR>
 cudaError_t launch_v(const ChunkParams &p, cudaStream_t stream)
 {
     const uint64_t n_tok = (uint64_t)p.B * p.T;
@@ -957,12 +986,11 @@ cudaError_t launch_v(const ChunkParams &p, cudaStream_t stream)
     if (!make_tmap(&tq, p.q, n_tok, (uint64_t)p.H * D) || !make_tmap(&tk, p.k, n_tok, (uint64_t)p.H * D) ||
         !make_tmap(&tv, p.v, n_tok, (uint64_t)p.H * D))
         return cudaErrorInvalidValue;
-    auto kern = kla_chunk_mma_kernel<D, OUT, VAR>;
-    const int smem = (int)sizeof(Smem<D>);
+    auto kern = kla_chunk_mma_kernel<D, BPS, OUT, VAR>;
+    const int smem = (int)sizeof(Smem<D, BPS>);
     cudaError_t err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (err != cudaSuccess) return err;
-    // segment pass 1: (seg_G - 1) segments per sequence, twice the slices; p.n_seq counts all segments there
-    const int grid = p.seg_pass == 1 ? (p.n_seq / p.seg_G) * (p.seg_G - 1) * p.H * 2 * (D / NS) : p.n_seq * p.H * (D / NS);
+    const int grid = blocks_of<D>(p);
     if (grid == 0) return cudaSuccess;
     kern<<<grid, NT, smem, stream>>>(tq, tk, tv, p);
     count_launch(1);
@@ -971,7 +999,10 @@ cudaError_t launch_v(const ChunkParams &p, cudaStream_t stream)
 template <int D, typename OUT>
 cudaError_t launch_o(const ChunkParams &p, cudaStream_t stream)
 {
-    return (p.variant & ~VARIANT_WY) ? launch_v<D, OUT, true>(p, stream) : launch_v<D, OUT, false>(p, stream);
+    const bool var = (p.variant & ~VARIANT_WY) != 0;
+    if constexpr (D == 64)
+        if (blocks_of<D>(p) > sm_count()) return var ? launch_v<D, 2, OUT, true>(p, stream) : launch_v<D, 2, OUT, false>(p, stream);
+    return var ? launch_v<D, 1, OUT, true>(p, stream) : launch_v<D, 1, OUT, false>(p, stream);
 }
 template <int D>
 cudaError_t launch_d(const ChunkParams &p, int out_dtype, cudaStream_t stream)

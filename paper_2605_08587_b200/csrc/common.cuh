@@ -31,11 +31,12 @@ struct ChunkParams {
     //               pieces; the table after the warm-up lengths (cu_seqlens[n_seq + 2 + n_seq H + u]) names each piece's
     //               sequence and says whether it is the first (initial state) and the last (final state) of it.
     //   seg_pass 6: the plain packed launch, taken only if the pieces' plan word, seq_order[seg_G], is 0.
+    //   seg_pass 7: 4 if the plan word (cu_seqlens[n_seq + 1]) is 1, else 3 with map_state as the start states.
     //   Passes 1 and 3 return at once when the plan word (cu_seqlens[n_seq + 1]) is 1, passes 4 and 5 when it is not.
     int32_t seg_pass, seg_G;
     int32_t variant;     // bit 0: beta_t = eta_t instead of Eq. 3; bit 1: read-out divided by ||q_t||; bit 2: test hook; bit 4: see VARIANT_WY
     union {
-        float *map_state;            // segment pass 1
+        float *map_state;            // segment passes 1 and 7
         const int32_t *seq_order;    // packed input, plain launch: block b works on sequence seq_order[b] (longest
                                      // first, so that the long sequences do not end up in the last wave); may be null
     };
