@@ -31,7 +31,7 @@ UNIT = "Mtok/s"
 WORKLOAD = "cfg2_bf16_B8_H8_T4096_d128_chunk64"   # the same string in both arms
 # dram__bytes_read.sum + dram__bytes_write.sum of one headline launch of the chunk kernel, from the ncu capture
 # summarised under profiles/; None while the kernel has changed since the counters were taken.
-CHUNK_TC_DRAM_BYTES_PER_LAUNCH = 255039232   # 203.86 MB read + 51.18 MB written
+CHUNK_DRAM_BYTES_PER_LAUNCH = 255039232   # 203.86 MB read + 51.18 MB written
 FALLBACK_PEAKS = {"hbm_gbs": 6650.0, "bf16_tflops": 1590.0, "bf16_tflops_sustained": 1400.0}
 
 
@@ -464,11 +464,11 @@ def run_ours(args):
     achieved = nbytes / (ms * 1e-3) / 1e9
     roofline = {"bound": "hbm" if t_hbm >= t_tc else "tensor", "achieved": achieved, "peak": peaks["hbm_gbs"], "unit": "GB/s",
                 "frac": achieved / peaks["hbm_gbs"], "traffic": None, "peak_source": peak_src + " (burst copy)",
-                "kernel": "kla_chunk_tc_kernel",
+                "kernel": "kla_chunk_mma_kernel",
                 "algorithmic_bytes_per_launch": nbytes, "algorithmic_flops_per_launch": flops,
                 "tensor_time_us_at_peak": t_tc * 1e6, "hbm_time_us_at_peak": t_hbm * 1e6,
                 "frac_of_roofline_time": max(t_hbm, t_tc) / (ms * 1e-3)}
-    roofline["traffic"] = CHUNK_TC_DRAM_BYTES_PER_LAUNCH
+    roofline["traffic"] = CHUNK_DRAM_BYTES_PER_LAUNCH
 
     extras = {}
     if args.quick and args.also:
