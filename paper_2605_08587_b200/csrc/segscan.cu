@@ -65,13 +65,22 @@ __global__ void seg_warm_plan_kernel(int32_t *cu_seg, const float *log_alpha, co
     const int start = cu_seg[n];   // first token of the segment (a multiple of 64 tokens into its sequence)
     float acc = 0.f;
     int w = 0;
-    while (w < max_warm && acc > WARM_LOG_DECAY) {
-        ++w;
-        const size_t t = (size_t)(start - w * 64 + 2 * lane);
-        float x = log_alpha[t * H + h] + log_alpha[(t + 1) * H + h];
+    while (w < max_warm && acc > WARM_LOG_DECAY) {   // four chunks' loads at a time (one by one: 7.5 us for 7 chunks)
+        float x[4];
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
-        acc += x;
+        for (int u = 0; u < 4; ++u) {
+            const size_t t = (size_t)(start - (w + u + 1) * 64 + 2 * lane);
+            x[u] = w + u < max_warm ? log_alpha[t * H + h] + log_alpha[(t + 1) * H + h] : 0.f;
+        }
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) x[u] += __shfl_xor_sync(0xffffffffu, x[u], o);
+            if (w < max_warm && acc > WARM_LOG_DECAY) {
+                ++w;
+                acc += x[u];
+            }
+        }
     }
     if (lane == 0) {
         warm[unit] = w;
