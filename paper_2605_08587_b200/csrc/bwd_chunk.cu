@@ -361,9 +361,10 @@ __global__ void __launch_bounds__(256, 3) kla_bwd_prepare_kernel(BwdChunkParams 
         for (int r = 0; r < 8; ++r) sm.tl[(blk * 8 + r) * LDT + blk * 8 + j] = x[r];
     }
     __syncthreads();
-    merge_level<8>(sm.tl, sm.mm, bet, tid);
-    merge_level<16>(sm.tl, sm.mm, bet, tid);
-    merge_level<32>(sm.tl, sm.mm, bet, tid);
+    // (a block whose rows all lie past the end of the sequence is zero as it stands)
+    if (rows > 8) merge_level<8>(sm.tl, sm.mm, bet, tid);
+    if (rows > 16) merge_level<16>(sm.tl, sm.mm, bet, tid);
+    if (rows > 32) merge_level<32>(sm.tl, sm.mm, bet, tid);
     // T as three operand planes: 8 columns per item
     unsigned char *tp = p.tpl + ch * T_BYTES;
 #pragma unroll
@@ -767,6 +768,7 @@ __global__ void __launch_bounds__(GT, 1) kla_bwd_grad_kernel(BwdChunkParams p)
     // F = qinv A o (dO U^T) (three terms) and E = -A o (lam U^T) (six), in 16 x 16 blocks on and below the diagonal
     auto block = [&](bool is_e, int blk) {
         const int bi = blk < 1 ? 0 : blk < 3 ? 1 : blk < 6 ? 2 : 3, bj = blk - bi * (bi + 1) / 2;
+        if (bi * 16 >= rows) return;   // tokens past the end: never read
         float c0[4] = {0.f, 0.f, 0.f, 0.f}, c1[4] = {0.f, 0.f, 0.f, 0.f};
         const uint32_t at = smem_u32(is_e ? sm.lam : sm.dout), bt = smem_u32(sm.u);
 #pragma unroll 2
@@ -813,6 +815,8 @@ __global__ void __launch_bounds__(GT, 1) kla_bwd_grad_kernel(BwdChunkParams p)
 
     const int mt = warp & 3, nh = warp >> 2, i0 = mt * 16;   // this warp's 16 tokens and 16 of the half's 64 columns
     const int ia = i0 + r, ib = ia + 8;
+    const int ks_s = i0 < rows ? D / 16 : 0;      // a warp whose tokens all lie past the end takes no part in the products
+    const int ks_j = (rows + 15) / 16;            // token blocks that hold any
     float gs = 0.f;             // this thread's part of <G_1, S_1>
     float dga = 0.f, dgb = 0.f; // ... of dg of its two rows
     const float gama = sm.s.gam[ia], gamb = sm.s.gam[ib], deca = sm.s.dec[ia], decb = sm.s.dec[ib], gc = sm.s.gam[C - 1];
@@ -844,7 +848,7 @@ __global__ void __launch_bounds__(GT, 1) kla_bwd_grad_kernel(BwdChunkParams p)
             for (int e = 0; e < 4; ++e) xq[t][e] = xk[t][e] = 0.f;
         // dO S_0^T and lam S_0^T
 #pragma unroll 2
-        for (int ks = 0; ks < D / 16; ++ks) {
+        for (int ks = 0; ks < ks_s; ++ks) {
             const uint32_t o = (ks >> 2) * 8192;
             uint32_t a[4], l[3][4];
             frag_a(a, smem_u32(sm.dout) + o, i0, (ks & 3) * 16, lane);
@@ -869,7 +873,7 @@ __global__ void __launch_bounds__(GT, 1) kla_bwd_grad_kernel(BwdChunkParams p)
         }
         // += F K and E K
 #pragma unroll 1
-        for (int ks = 0; ks <= mt; ++ks) {
+        for (int ks = 0; ks <= mt && mt < ks_j; ++ks) {
             uint32_t a[3][4], l[3][4];
 #pragma unroll
             for (int pl = 0; pl < 3; ++pl) {
@@ -912,7 +916,7 @@ __global__ void __launch_bounds__(GT, 1) kla_bwd_grad_kernel(BwdChunkParams p)
 #pragma unroll
             for (int e = 0; e < 4; ++e) xq[t][e] = 0.f;
 #pragma unroll 2
-        for (int ks = 0; ks < D / 16; ++ks) {
+        for (int ks = 0; ks < ks_s; ++ks) {
             uint32_t a[3][4];
 #pragma unroll
             for (int pl = 0; pl < 3; ++pl) frag_a(a[pl], smem_u32(sm.u) + (pl * NB + (ks >> 2)) * 8192, i0, (ks & 3) * 16, lane);
@@ -930,7 +934,7 @@ __global__ void __launch_bounds__(GT, 1) kla_bwd_grad_kernel(BwdChunkParams p)
         dot(sm.k, xq, gs, gs);   // <G_1, S_1> = gC <G_1, S_0> + sum_j k_j . (D U G_1^T)_j
         // += E^T K + F^T Q: rows of this warp are the columns of E and F
 #pragma unroll 1
-        for (int ks = mt; ks < 4; ++ks) {
+        for (int ks = mt; ks < ks_j; ++ks) {
             uint32_t a[3][4], l[3][4];
 #pragma unroll
             for (int pl = 0; pl < 3; ++pl) {
