@@ -4,11 +4,12 @@
 // Nine warps in three roles, connected by a ring of three chunk slots in shared memory (K, Q, V tiles, operands, per-token scalars):
 //
 //   chain (4 warps)       the serial dependency over chunks, 16 columns of the state each:
-//                             U_i = T_ii (R_i - sum_{j<i} X_ij U_j),  R = V - Gam K S     (Eq. 7, by blocks of 16 tokens)
+//                             Y_i = R_i - sum_{j<i} X_ij U_j,  R = V - Gam K S            (Eq. 7, by blocks of 16 tokens)
+//                             U_i = B_i Y_i + N_ii B_i Y_i
 //                             O = Gam Q S + P U                                           (Eq. 8)
 //                             S <- gamma_C S + K^T D U,  D = diag(exp(g_C - g_j))         (Eq. 9)
 //   prepare (4 warps)     what does not depend on the state, a chunk ahead: decay sums, beta (Eq. 3, ||k||^2 from the diagonal
-//                         of K K^T), X = A^- o K K^T, the diagonal blocks T_ii = (I + B X)_ii^-1 B, P = A o Q K^T
+//                         of K K^T), X = A^- o K K^T, N_ii = (I + B X)_ii^-1 - I, P = A o Q K^T
 //   issue (1 warp)        TMA loads and tcgen05 products
 //
 // Products with the whole state go to tcgen05: [S_hi; S_lo]^T [K; Q]^T, one product of 128 rows (hi and lo parts of 64 columns) and
@@ -24,10 +25,13 @@
 // memory, 7 400; this way 5 100.  mma.sync stands still while a tcgen05 product runs, so the two add up: 570 cycles for the state
 // product, 400 for [K; Q] K^T, 8 per mma.sync.
 //
-// Precision.  q, k, v are exact bf16 operands.  Every derived operand (S, R, X, T, P, U) is a pair of bf16 values hi + lo (16
+// Precision.  q, k, v are exact bf16 operands.  Every derived operand (S, Y, X, N, P, U) is a pair of bf16 values hi + lo (16
 // significand bits; one bf16 rounding of any of them costs 1e-2..7e-2 in max|err|/rms, above the 2e-3 bound), a product of two
-// of them hi hi + hi lo + lo hi.  In a chunk with a near-zero key (beta above HOT_BETA) U has a third part in P U: the rounding of such
-// a token's huge U is the largest error of all.  (In every chunk it would cost 8 %.)
+// of them hi hi + hi lo + lo hi.  The rounding of a pair is 2.2e-6 of the operand's norm, and so is the term left out.  The block solve
+// therefore adds N B Y to B Y in fp32 instead of multiplying Y by (I + N) B: with the identity in the operand U carried three such
+// errors of its whole size (2-norm errors of final state and output 5.1e-6 and 6.3e-6; this way 2.5e-6 and 4.5e-6).  In a chunk
+// with a near-zero key (beta above HOT_BETA) U has a third part in P U: the rounding of such a token's huge U is the largest error
+// of all.  (In every chunk it would cost 8 %.)
 //
 // Every wait is bounded; when one gives up the block raises an abort flag, reports KLA_ERR_TIMEOUT through the status word,
 // lets its copies and products finish and exits.
@@ -76,11 +80,12 @@ struct Slot {
     // per 64 columns: 64 tokens of K, then 64 of Q, rows of 128 bytes, 128-byte swizzle
     alignas(1024) unsigned char kq[NB * 16384];
     alignas(1024) unsigned char v[8192];        // this block's 64 columns; then the outputs on their way out
-    TriOperand t, p;                            // D T_ii and below them -X D^-1; P D^-1 (rows over ||q|| with the normalised read-out)
+    TriOperand t, p;                            // D N_ii B and below them -X D^-1; P D^-1 (rows over ||q|| with the normalised read-out)
 };
 struct alignas(16) Scalars {     // of one chunk
     float ngam[C];               // -exp(g_i)
     float gamq[C];               // exp(g_i) (over ||q_i||)
+    float bd[C];                 // beta_i exp(g_C - g_i)
     int hot[2];                  // some beta above HOT_BETA among tokens 0 .. 31, 32 .. 63
 };
 
@@ -98,7 +103,8 @@ enum Bar {
     B_X = 10,        // [S_hi; S_lo]^T [K; Q]^T complete
     B_G = 11,        // [K; Q] K^T complete
     B_GFREE = 12,    // ... and read
-    B_COUNT = 14
+    B_TD = 14,       // diagonal blocks and beta of prepare warp 1 in its scratch
+    B_COUNT = 15
 };
 
 // BPS, blocks per SM.  One: three chunk slots, registers for the whole chain.  Two (d = 64, more blocks than SMs): two slots and
@@ -146,12 +152,6 @@ __device__ __forceinline__ void mma(float2 (&c)[2], const uint32_t (&a)[4], uint
     asm("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, {%0, %1, %2, %3};"
         : "+f"(c[0].x), "+f"(c[0].y), "+f"(c[1].x), "+f"(c[1].y)
         : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
-}
-__device__ __forceinline__ void mma_first(float2 (&c)[2], const uint32_t (&a)[4], uint32_t b0, uint32_t b1)   // c = a b
-{
-    asm("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, {%10, %10, %10, %10};"
-        : "=f"(c[0].x), "=f"(c[0].y), "=f"(c[1].x), "=f"(c[1].y)
-        : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1), "f"(0.f));
 }
 // x as packed bf16 hi and lo parts.
 __device__ __forceinline__ void split(float2 x, uint32_t &hi, uint32_t &lo)
@@ -331,10 +331,11 @@ __device__ bool find_work(const ChunkParams &params, Work &w)
 
 // ---- prepare --------------------------------------------------------------------------------------------------------------
 // [K; Q] K^T lies in TMEM with its rows as lanes, 32 per warp: warps 0 and 1 form X (token blocks 0, 1 and 2, 3) and the diagonal
-// blocks of T, warps 2 and 3 P.  Blocks of 16 x 16 are read, weighted and stored as operands one after the other in a rolled
-// loop.  T_ii = (I + B X)_ii^-1 B by 8 x 8 substitution (a column per lane) and one merge; the rest of the triangular solve is
+// blocks N, warps 2 and 3 P.  Blocks of 16 x 16 are read, weighted and stored as operands one after the other in a rolled
+// loop.  (I + B X)_ii^-1 by 8 x 8 substitution (a column per lane) and one merge; the rest of the triangular solve is
 // left to the chain, which takes U block by block: as many products there as with the whole inverse, and the block products of
-// the inverse, longer than everything else here, are not needed.
+// the inverse, longer than everything else here, are not needed.  Warp 1 has the most blocks and the chain waits for it, so warp 2,
+// which has the fewest, inverts its diagonal blocks for it (32 packed sequences, d 64, two blocks per SM: -3 %).
 template <int D, int BPS, bool VAR>
 __device__ void prepare(const ChunkParams &p, Smem<D, BPS> &sm, const Work &wk, int nchunks)
 {
@@ -439,58 +440,8 @@ __device__ void prepare(const ChunkParams &p, Smem<D, BPS> &sm, const Work &wk, 
                 const bool hot = __any_sync(0xffffffffu, sc.bet[lane] > HOT_BETA);
                 if (lane == 0) sm.scal[s].hot[w] = hot;
             }
-            // 8 x 8 diagonal blocks by substitution: lane l solves column l % 8 of block l / 8 of four
-            float xs[8];
-            {
-                const int b8 = lane >> 3, col = lane & 7;
-                float *td = sc.td[b8 >> 1] + (b8 & 1) * (8 * LDB + 8);
-                const float4 bl = load4(sc.bet + b8 * 8), bh = load4(sc.bet + b8 * 8 + 4);
-                const float bb[8] = {bl.x, bl.y, bl.z, bl.w, bh.x, bh.y, bh.z, bh.w};
-#pragma unroll
-                for (int r = 0; r < 8; ++r) {
-                    float a = 0.f;
-                    if (r > 0) {
-                        const float4 f0 = load4(td + r * LDB), f1 = r > 4 ? load4(td + r * LDB + 4) : make_float4(0.f, 0.f, 0.f, 0.f);
-                        const float f[8] = {f0.x, f0.y, f0.z, f0.w, f1.x, f1.y, f1.z, f1.w};
-#pragma unroll
-                        for (int m = 0; m < r; ++m) a += f[m] * xs[m];
-                    }
-                    xs[r] = r == col ? 1.f : (r > col ? -bb[r] * a : 0.f);
-                }
-                __syncwarp();
-#pragma unroll
-                for (int r = 0; r < 8; ++r) td[r * LDB + col] = xs[r];
-            }
             __syncwarp();
-            // T_10 = -T_11 (B_1 X_10 T_00): row g, columns t2, t2 + 1 of both blocks
-#pragma unroll
-            for (int rb = 0; rb < 2; ++rb) {
-                const float *td = sc.td[rb];
-                const float4 f0 = load4(td + (8 + g) * LDB), f1 = load4(td + (8 + g) * LDB + 4);
-                const float f[8] = {f0.x, f0.y, f0.z, f0.w, f1.x, f1.y, f1.z, f1.w};
-                float2 a = f2(0.f);
-#pragma unroll
-                for (int m = 0; m < 8; ++m) a = fma2(f2(f[m]), load2(td + m * LDB + t2), a);
-                *reinterpret_cast<float2 *>(sc.td[rb] + g * LDB + 8 + t2) = mul2(f2(-sc.bet[16 * rb + 8 + g]), a);
-            }
-            __syncwarp();
-#pragma unroll
-            for (int rb = 0; rb < 2; ++rb) {
-                const float *td = sc.td[rb];
-                const float4 f0 = load4(td + (8 + g) * LDB + 8), f1 = load4(td + (8 + g) * LDB + 12);
-                const float f[8] = {f0.x, f0.y, f0.z, f0.w, f1.x, f1.y, f1.z, f1.w};
-                float2 a = f2(0.f);
-#pragma unroll
-                for (int m = 0; m < 8; ++m) a = fma2(f2(f[m]), load2(td + m * LDB + 8 + t2), a);
-                const float2 c0 = load2(&sc.bet[16 * rb + t2]), c1 = load2(&sc.bet[16 * rb + 8 + t2]);
-                const int i0 = 32 * w + 16 * rb + g;
-                const float2 d0 = f2(ex2_approx(fmaxf(gc2 - g2[i0], -DEC_FLOOR_LOG2))), d1 = f2(ex2_approx(fmaxf(gc2 - g2[i0 + 8], -DEC_FLOOR_LOG2)));
-                x[0] = mul2(mul2(load2(td + g * LDB + t2), c0), d0);
-                x[1] = mul2(mul2(a, c0), d1);
-                y[0] = f2(0.f);
-                y[1] = mul2(mul2(load2(td + (8 + g) * LDB + 8 + t2), c1), d1);
-                store_right(sl.t, blk(2 * w + rb, 2 * w + rb), lane, x, y);
-            }
+            if (w == 1 && lane == 0) mbar_arrive(&sm.bar[B_TD]);
         }
         // -X D^-1 below the diagonal blocks, P D^-1 up to them
         const bool qn = qnorm && !isx;
@@ -517,9 +468,74 @@ __device__ void prepare(const ChunkParams &p, Smem<D, BPS> &sm, const Work &wk, 
                 store_right(isx ? sl.t : sl.p, blk(bi, j), lane, x, y);
             }
         }
+        // the inverses of the diagonal blocks: warp 0 those of its own, warp 2, which has the fewest blocks, those of warp 1
+        if (!(w & 1)) {
+            if (w == 2 && !bar_wait(&sm.bar[B_TD], c & 1, &sm.abort_flag)) break;
+            PrepScratch &si = sm.prep[w >> 1];
+            // 8 x 8 diagonal blocks by substitution: lane l solves column l % 8 of block l / 8 of four
+            float xs[8];
+            {
+                const int b8 = lane >> 3, col = lane & 7;
+                float *td = si.td[b8 >> 1] + (b8 & 1) * (8 * LDB + 8);
+                const float4 bl = load4(si.bet + b8 * 8), bh = load4(si.bet + b8 * 8 + 4);
+                const float bb[8] = {bl.x, bl.y, bl.z, bl.w, bh.x, bh.y, bh.z, bh.w};
+#pragma unroll
+                for (int r = 0; r < 8; ++r) {
+                    float a = 0.f;
+                    if (r > 0) {
+                        const float4 f0 = load4(td + r * LDB), f1 = r > 4 ? load4(td + r * LDB + 4) : make_float4(0.f, 0.f, 0.f, 0.f);
+                        const float f[8] = {f0.x, f0.y, f0.z, f0.w, f1.x, f1.y, f1.z, f1.w};
+#pragma unroll
+                        for (int m = 0; m < r; ++m) a += f[m] * xs[m];
+                    }
+                    xs[r] = r == col ? 1.f : (r > col ? -bb[r] * a : 0.f);
+                }
+                __syncwarp();
+#pragma unroll
+                for (int r = 0; r < 8; ++r) td[r * LDB + col] = xs[r];
+            }
+            __syncwarp();
+            // T_10 = -T_11 (B_1 X_10 T_00): row g, columns t2, t2 + 1 of both blocks
+#pragma unroll 1
+            for (int rb = 0; rb < 2; ++rb) {
+                const float *td = si.td[rb];
+                const float4 f0 = load4(td + (8 + g) * LDB), f1 = load4(td + (8 + g) * LDB + 4);
+                const float f[8] = {f0.x, f0.y, f0.z, f0.w, f1.x, f1.y, f1.z, f1.w};
+                float2 a = f2(0.f);
+#pragma unroll
+                for (int m = 0; m < 8; ++m) a = fma2(f2(f[m]), load2(td + m * LDB + t2), a);
+                *reinterpret_cast<float2 *>(si.td[rb] + g * LDB + 8 + t2) = mul2(f2(-si.bet[16 * rb + 8 + g]), a);
+            }
+            __syncwarp();
+#pragma unroll 1
+            for (int rb = 0; rb < 2; ++rb) {
+                const float *td = si.td[rb];
+                const float4 f0 = load4(td + (8 + g) * LDB + 8), f1 = load4(td + (8 + g) * LDB + 12);
+                const float f[8] = {f0.x, f0.y, f0.z, f0.w, f1.x, f1.y, f1.z, f1.w};
+                float2 a = f2(0.f);
+#pragma unroll
+                for (int m = 0; m < 8; ++m) a = fma2(f2(f[m]), load2(td + m * LDB + 8 + t2), a);
+                const float2 c0 = load2(&si.bet[16 * rb + t2]), c1 = load2(&si.bet[16 * rb + 8 + t2]);
+                const int i0 = 16 * (w + rb) + g;
+                const float2 d0 = f2(ex2_approx(fmaxf(gc2 - g2[i0], -DEC_FLOOR_LOG2))), d1 = f2(ex2_approx(fmaxf(gc2 - g2[i0 + 8], -DEC_FLOOR_LOG2)));
+                x[0] = mul2(mul2(load2(td + g * LDB + t2), c0), d0);
+                x[1] = mul2(mul2(a, c0), d1);
+                y[0] = f2(0.f);
+                y[1] = mul2(mul2(load2(td + (8 + g) * LDB + 8 + t2), c1), d1);
+                // the diagonal, D B, stays in fp32
+                const bool e0 = t2 == g, e1 = t2 + 1 == g;
+                if (e0 || e1) {
+                    sm.scal[s].bd[i0] = e0 ? x[0].x : x[0].y;
+                    sm.scal[s].bd[i0 + 8] = e0 ? y[1].x : y[1].y;
+                }
+                x[0] = make_float2(e0 ? 0.f : x[0].x, e1 ? 0.f : x[0].y);
+                y[1] = make_float2(e0 ? 0.f : y[1].x, e1 ? 0.f : y[1].y);
+                store_right(sl.t, blk(w + rb, w + rb), lane, x, y);
+            }
+        }
         tc_fence_before();
         __syncwarp();
-        if (lane == 0) mbar_arrive(&sm.bar[B_GFREE]);
+        if (lane == 0) mbar_arrive(&sm.bar[B_GFREE]);   // (of warp 2 also: the scratch of warp 1 has been read)
         if (rows < C) {   // K rows past the end of the sequence hold a neighbour's tokens: inert from here on
             for (int e = threadIdx.x & 127; e < (C - rows) * 8; e += PREP_T) {
                 const uint32_t off = sw128(rows + (e >> 3), e & 7);
@@ -606,19 +622,19 @@ __device__ void chain(const ChunkParams &p, Smem<D, BPS> &sm, const Work &wk, in
         if (!bar_wait(&sm.bar[B_X], c & 1, &sm.abort_flag)) break;
         tc_fence_after();
 
-        float2 x[8][2];   // K S, then R, then D U
+        float2 x[8][2];   // K S, then R, then Y, then D U
         tmem_sum_first(tx, x);
         auto residual = [&](int t) {   // R = V - Gam K S, 8 tokens
             const float2 gm = load2(&sm.scal[s].ngam[8 * t + t2]);
             x[t][0] = fma2(gm, x[t][0], unpack(vv[t >> 1][2 * (t & 1)]));
             x[t][1] = fma2(gm, x[t][1], unpack(vv[t >> 1][2 * (t & 1) + 1]));
-            if (rows < C) {   // tokens past the end
-                if (8 * t + t2 >= rows) x[t][0].x = x[t][1].x = 0.f;
-                if (8 * t + t2 + 1 >= rows) x[t][0].y = x[t][1].y = 0.f;
-            }
+        };
+        auto live_only = [&](int t) {   // nothing from tokens past the end
+            if (8 * t + t2 >= rows) x[t][0].x = x[t][1].x = 0.f;
+            if (8 * t + t2 + 1 >= rows) x[t][0].y = x[t][1].y = 0.f;
         };
         float2 o[8][2];   // Gam Q S, then O
-        uint32_t rh[4], rl[4], uh[2][4], ul[2][4];   // operands R_j, D U_j
+        uint32_t rh[4], rl[4], uh[2][4], ul[2][4];   // operands Y_j, D U_j
         const bool hot = HAS_OUT && (sm.scal[s].hot[0] | sm.scal[s].hot[1]);
         uint32_t b[2][2][4];
         auto fetch_k = [&](int q) {   // K as right operand: step q = (16 tokens, 32 of d_k)
@@ -675,15 +691,25 @@ __device__ void chain(const ChunkParams &p, Smem<D, BPS> &sm, const Work &wk, in
         constexpr int QJ = KS / 2, QH = QJ / 2;   // update steps per token block, and half of them
         residual(0);
         residual(1);
+        if (rows < C) {
+            live_only(0);
+            live_only(1);
+        }
 #pragma unroll
         for (int u = 0; u < 4; ++u) split_left(x[0], x[1], u, rh, rl);
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
-            // D U_j = (D T_jj) R_j
+            // D U_j = D B Y_j + (D N_jj B) Y_j
             {
                 const uint4 th = sl.t.hi[blk(j, j)][lane], tl = sl.t.lo[blk(j, j)][lane];
-                mma_first(x[2 * j], rh, th.x, th.y);
-                mma_first(x[2 * j + 1], rh, th.z, th.w);
+#pragma unroll
+                for (int u = 0; u < 2; ++u) {
+                    const float2 bd = load2(&sm.scal[s].bd[16 * j + 8 * u + t2]);
+                    x[2 * j + u][0] = mul2(bd, x[2 * j + u][0]);
+                    x[2 * j + u][1] = mul2(bd, x[2 * j + u][1]);
+                }
+                mma(x[2 * j], rh, th.x, th.y);
+                mma(x[2 * j + 1], rh, th.z, th.w);
                 mma(x[2 * j], rl, th.x, th.y);
                 mma(x[2 * j + 1], rl, th.z, th.w);
                 mma(x[2 * j], rh, tl.x, tl.y);
@@ -693,13 +719,17 @@ __device__ void chain(const ChunkParams &p, Smem<D, BPS> &sm, const Work &wk, in
                 tmem_sum_rest(tx, x);
 #pragma unroll
                 for (int t = 2; t < 8; ++t) residual(t);
+                if (rows < C) {
+#pragma unroll
+                    for (int t = 2; t < 8; ++t) live_only(t);
+                }
             } else {
 #pragma unroll
                 for (int q = 0; q < QH; ++q) update((j - 1) * QJ + q, [] {});
             }
 #pragma unroll
             for (int u = 0; u < 4; ++u) split_left(x[2 * j], x[2 * j + 1], u, uh[j & 1], ul[j & 1]);
-            // R_i -= (X_ij D^-1) (D U_j)
+            // Y_i -= (X_ij D^-1) (D U_j)
             if (j < 3) {
                 uint4 f[3];
 #pragma unroll
@@ -903,6 +933,7 @@ kla_chunk_mma_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_cons
         mbar_init(&sm.bar[B_X], 1);
         mbar_init(&sm.bar[B_G], 1);
         mbar_init(&sm.bar[B_GFREE], 4);
+        mbar_init(&sm.bar[B_TD], 1);
         sm.abort_flag = 0;
         mbar_fence_init();
         tma_prefetch_desc(&tm_q);
