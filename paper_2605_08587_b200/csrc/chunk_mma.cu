@@ -15,8 +15,8 @@
 // Products with the whole state go to tcgen05: [S_hi; S_lo]^T [K; Q]^T, one product of 128 rows (hi and lo parts of 64 columns) and
 // 128 columns (the chunk's keys and queries), and [K; Q] K^T.  The serial part runs on mma.sync inside single warps: everything
 // transposed, an accumulator tile (16 columns of d_v x tokens or d_k) is at the same time a left operand of the next product, so
-// R -> U -> state goes from product to product in registers, without a barrier.  The state itself stays in registers too, as
-// accumulators; once per chunk its hi and lo parts go to shared memory for the tcgen05 product of the next chunk.
+// R -> U -> state goes from product to product in registers, without a barrier.  Once per chunk the hi and lo parts of the new state
+// go to shared memory for the tcgen05 product of the next chunk.
 //
 // What bounds it: the latency of that chain and the number of instructions in it.  Code that runs once per chunk does not stay in
 // the schedulers' instruction caches and issues at about one instruction in three cycles (measured on unrolled against rolled
@@ -32,6 +32,11 @@
 // errors of its whole size (2-norm errors of final state and output 5.1e-6 and 6.3e-6; this way 2.5e-6 and 4.5e-6).  In a chunk
 // with a near-zero key (beta above HOT_BETA) U has a third part in P U: the rounding of such a token's huge U is the largest error
 // of all.  (In every chunk it would cost 8 %.)
+//
+// mma.sync truncates its sums: used as the accumulator, the state would lose a fraction of a unit in the last place, always towards
+// zero, with each of eight products per chunk, which adds up where little is forgotten (log alpha = 0, eta 1e-3, 16 384 tokens: 6e-5
+// of the state's norm, now 1.4e-6).  K^T D U is therefore summed by itself, and gamma_C S + that is one fp32 operation per chunk; the
+// fp32 state waits in tensor memory meanwhile (registers hold one of the two; 2 % at d = 128, -2 % at d = 64 with two blocks per SM).
 //
 // Every wait is bounded; when one gives up the block raises an abort flag, reports KLA_ERR_TIMEOUT through the status word,
 // lets its copies and products finish and exits.
@@ -65,8 +70,8 @@ constexpr float LOG2E = 1.4426950408889634f;
 constexpr float DEC_FLOOR_LOG2 = 115.f;
 constexpr float HOT_BETA = 4096.f;   // q k beta up to ||q|| sqrt(beta) = 64 ||q||: 2^-18 of that is below the other errors
 constexpr int LDB = 20;       // row stride (floats) of a 16 x 16 block in the solve scratch
-// TMEM columns: [S_hi; S_lo]^T [K; Q]^T (128), [K; Q] K^T (64)
-constexpr uint32_t TM_X = 0, TM_G = 128, TM_COLS = 256;
+// TMEM columns: [S_hi; S_lo]^T [K; Q]^T (128), [K; Q] K^T (64), the state in fp32 (D / 2)
+constexpr uint32_t TM_X = 0, TM_G = 128, TM_S = 192, TM_COLS = 256;
 
 // Lower triangle of 16 x 16 blocks, in fragment order: the four registers of a right operand, 16 bytes per lane.
 __device__ __forceinline__ constexpr int blk(int i, int j) { return i * (i + 1) / 2 + j; }
@@ -153,6 +158,12 @@ __device__ __forceinline__ void mma(float2 (&c)[2], const uint32_t (&a)[4], uint
         : "+f"(c[0].x), "+f"(c[0].y), "+f"(c[1].x), "+f"(c[1].y)
         : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
 }
+__device__ __forceinline__ void mma_first(float2 (&c)[2], const uint32_t (&a)[4], uint32_t b0, uint32_t b1)   // c = a b
+{
+    asm("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, {%10, %10, %10, %10};"
+        : "=f"(c[0].x), "=f"(c[0].y), "=f"(c[1].x), "=f"(c[1].y)
+        : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1), "f"(0.f));
+}
 // x as packed bf16 hi and lo parts.
 __device__ __forceinline__ void split(float2 x, uint32_t &hi, uint32_t &lo)
 {
@@ -180,6 +191,19 @@ __device__ __forceinline__ void store_right(TriOperand &o, int b, int lane, cons
 }
 __device__ __forceinline__ float2 load2(const float *p) { return *reinterpret_cast<const float2 *>(p); }
 
+// Four accumulator tiles in sixteen TMEM columns of the warp's lanes, written (there after a wait::st) and read back.
+#define R8(c, x, i) c(x[i][0].x), c(x[i][0].y), c(x[i][1].x), c(x[i][1].y), c(x[i + 1][0].x), c(x[i + 1][0].y), c(x[i + 1][1].x), c(x[i + 1][1].y)
+__device__ __forceinline__ void tmem_keep(uint32_t addr, const float2 (*x)[2])
+{
+    asm volatile("tcgen05.st.sync.aligned.32x32b.x16.b32 [%16], {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15};"
+                 ::R8("f", x, 0), R8("f", x, 2), "r"(addr) : "memory");
+}
+__device__ __forceinline__ void tmem_kept(uint32_t addr, float2 (&x)[4][2])
+{
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];\n\t"
+                 "tcgen05.wait::ld.sync.aligned;" : R8("=f", x, 0), R8("=f", x, 2) : "r"(addr) : "memory");
+}
+#undef R8
 // 16 TMEM lanes x 16 columns as two accumulator tiles side by side.
 __device__ __forceinline__ void tmem_block(uint32_t addr, float2 (&x)[2], float2 (&y)[2])
 {
@@ -563,7 +587,7 @@ __device__ void chain(const ChunkParams &p, Smem<D, BPS> &sm, const Work &wk, in
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const int g = lane >> 2, t2 = 2 * (lane & 3);
     const int dv = wk.sl * NS + 16 * w + g;   // columns dv, dv + 8 of d_v
-    // S[t][e]: rows 8 t + t2, + 1 of d_k, column dv + 8 e
+    // S[t][e]: rows 8 t + t2, + 1 of d_k, column dv + 8 e: the state, during a chunk K^T D U of the tokens so far
     float2 S[D / 8][2];
 #pragma unroll
     for (int t = 0; t < D / 8; ++t)
@@ -602,6 +626,10 @@ __device__ void chain(const ChunkParams &p, Smem<D, BPS> &sm, const Work &wk, in
     };
 #pragma unroll
     for (int ks = 0; ks < KS; ++ks) store_state(ks);
+    const uint32_t ts = sm.tmem + TM_S + ((uint32_t)(32 * w) << 16);
+#pragma unroll
+    for (int ks = 0; ks < KS; ks += 2) tmem_keep(ts + 8 * ks, &S[2 * ks]);
+    asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
     if (D == 128) state_written(1);
     state_written(0);
 
@@ -642,14 +670,19 @@ __device__ void chain(const ChunkParams &p, Smem<D, BPS> &sm, const Work &wk, in
 #pragma unroll
             for (int u = 0; u < 2; ++u) ldsm4t(b[q & 1][u], kt + ktx[(n + u) & 3] + ((n + u) >> 2) * 16384 + j * 2048);
         };
-        // S += (D U_j)^T K_j, 32 rows of d_k; `extra` between the products
+        // += (D U_j)^T K_j, 32 rows of d_k; `extra` between the products
         auto update = [&](int q, auto &&extra) {
             const int j = q / (KS / 2), n = 2 * (q % (KS / 2));
             if (q + 1 < 2 * KS) fetch_k(q + 1);
 #pragma unroll
             for (int u = 0; u < 2; ++u) {
-                mma(S[2 * (n + u)], uh[j & 1], b[q & 1][u][0], b[q & 1][u][1]);
-                mma(S[2 * (n + u) + 1], uh[j & 1], b[q & 1][u][2], b[q & 1][u][3]);
+                if (j == 0) {
+                    mma_first(S[2 * (n + u)], uh[0], b[q & 1][u][0], b[q & 1][u][1]);
+                    mma_first(S[2 * (n + u) + 1], uh[0], b[q & 1][u][2], b[q & 1][u][3]);
+                } else {
+                    mma(S[2 * (n + u)], uh[j & 1], b[q & 1][u][0], b[q & 1][u][1]);
+                    mma(S[2 * (n + u) + 1], uh[j & 1], b[q & 1][u][2], b[q & 1][u][3]);
+                }
             }
             extra();
 #pragma unroll
@@ -749,10 +782,7 @@ __device__ void chain(const ChunkParams &p, Smem<D, BPS> &sm, const Work &wk, in
                 }
             }
             if (j == 0) {
-                const float2 gC = f2(-sm.scal[s].ngam[C - 1]);
                 fetch_k(0);
-#pragma unroll
-                for (int t = 0; t < D / 8; ++t) { S[t][0] = mul2(S[t][0], gC); S[t][1] = mul2(S[t][1], gC); }
                 if (HAS_OUT) {
                     tmem_sum(tx + 64, o);
 #pragma unroll
@@ -773,18 +803,27 @@ __device__ void chain(const ChunkParams &p, Smem<D, BPS> &sm, const Work &wk, in
             }
         }
         outputs(3);
-        // the last token block, and the finished rows of the state on their way to the next product
+        // the last token block, and the finished rows of the state, gC S + K^T D U, on their way to the next product
+        const float2 gC = f2(-sm.scal[s].ngam[C - 1]);
+        auto finish = [&](int q) {   // 32 rows
+            float2 kept[4][2];
+            tmem_kept(ts + 16 * q, kept);
+#pragma unroll
+            for (int t = 0; t < 4; ++t)
+#pragma unroll
+                for (int e = 0; e < 2; ++e) S[4 * q + t][e] = fma2(gC, kept[t][e], S[4 * q + t][e]);
+            tmem_keep(ts + 16 * q, &S[4 * q]);
+            store_state(2 * q);
+            store_state(2 * q + 1);
+        };
 #pragma unroll
         for (int q = 0; q < QJ; ++q)
             update(3 * QJ + q, [&] {
-                if (q > 0) {
-                    store_state(2 * q - 2);
-                    store_state(2 * q - 1);
-                }
+                if (q > 0) finish(q - 1);
                 if (D == 128 && q == QJ / 2 && c + 1 < nchunks) state_written(0);
             });
-        store_state(KS - 2);
-        store_state(KS - 1);
+        finish(QJ - 1);
+        asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
         if (c + 1 < nchunks) state_written(D == 128);
         if constexpr (HAS_OUT) {
             const int live = c >= wk.first_out ? rows : 0;

@@ -36,3 +36,16 @@ def test_forward(kind):
     ro, rf = oracle_chunk(w)[:2]
     assert _norm_err(out.reshape(ro.shape), ro) <= 1.15 * 4 ** 0.5 * PAIR
     assert _norm_err(fin, rf) <= 1.15 * 1.5 ** 0.5 * PAIR
+
+
+@pytest.mark.parametrize("d", [64, 128])
+def test_forward_that_forgets_little(d):
+    """No decay and small steps: what a chunk adds is a small part of the state, so anything lost from the whole state at every chunk
+    would add up over the 64 chunks.  Same bounds as above: the pairs are roundings of the parts added, not of the sum."""
+    w = W.config3(B=1, H=2, T=4096, d=d, seed=1410 + d)
+    w.log_alpha = torch.zeros_like(w.log_alpha)
+    w.eta = w.eta * 1e-3
+    out, fin = gpu_chunk(w, out_dtype=torch.float32)
+    ro, rf = oracle_chunk(w)[:2]
+    assert _norm_err(out, ro) <= 1.15 * 4 ** 0.5 * PAIR
+    assert _norm_err(fin, rf) <= 1.15 * 1.5 ** 0.5 * PAIR
