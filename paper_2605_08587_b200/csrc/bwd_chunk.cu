@@ -20,6 +20,13 @@
 //   3. gradients one block per (chunk, head): everything that is left, in parallel over chunks.
 // Token by token on CUDA cores (bwd_scan.cu, which stays for fp32 inputs) the layer shape took 8.1 ms.
 //
+// Precision.  mma.sync truncates its fp32 sums (mma_pieces.cuh), so how often a sum is truncated at its full size decides how exact it is.
+// The products of the first planes, the size of the result, are therefore summed apart from the terms of the lower planes (2^-8 of it
+// and less), in runs of at most eight, and everything else is added in fp32: the states to what a chunk adds to them, the two halves
+// of a long sum, the parts of a gradient.  2-norm errors against fp64, B 8, H 8, T 4096, d 128: dq 1.4e-7, dk 1.5e-7, dv 1.5e-7,
+// dlog_alpha 4e-7, deta 1.9e-7, dinit 1.5e-7, as those of the token-by-token kernel (1.8e-7, 1.9e-7, 1.9e-7, 2.9e-7, 2.0e-7, 1.9e-7);
+// with all terms in one accumulator they were 4e-7 .. 1.1e-6.  Cost: 1.50 -> 1.62 ms.
+//
 // beta = 0 (eta = 0) would make U = B (...) carry no trace of the residual e = U / beta that dbeta needs; such a beta is taken
 // as 1e-30, where every gradient has its limit to the last bit.
 #include "common.cuh"
@@ -319,11 +326,11 @@ __global__ void __launch_bounds__(256, 3) kla_bwd_prepare_kernel(BwdChunkParams 
             for (int e = 0; e < 4; ++e) o[t][e] = 0.f;
         const uint32_t at = smem_u32(sm.dout) + (warp >> 2) * 8192, bt = smem_u32(sm.p);
 #pragma unroll
-        for (int ks = 0; ks < 4; ++ks) {
-            uint32_t a[4];
-            frag_at(a, at, (warp & 3) * 16, ks * 16, lane);
+        for (int pl = 2; pl >= 0; --pl)
 #pragma unroll
-            for (int pl = 0; pl < 3; ++pl)
+            for (int ks = 0; ks < 4; ++ks) {
+                uint32_t a[4];
+                frag_at(a, at, (warp & 3) * 16, ks * 16, lane);
 #pragma unroll
                 for (int np = 0; np <= ks; ++np) {
                     uint32_t b[4];
@@ -331,7 +338,7 @@ __global__ void __launch_bounds__(256, 3) kla_bwd_prepare_kernel(BwdChunkParams 
                     mma(o[2 * np], a, b[0], b[1]);
                     mma(o[2 * np + 1], a, b[2], b[3]);
                 }
-        }
+            }
         float *dst = p.pdo + ch * D * C + (size_t)(warp * 16 + (lane >> 2)) * C + cq;
 #pragma unroll
         for (int t = 0; t < 8; ++t) {
@@ -395,53 +402,67 @@ struct ChainSmem {
     Scal s[2];
 };
 
-// acc[token tile] = (16 x D state) (64 x D tile)^T: columns are tokens
-template <int D>
-__device__ __forceinline__ void state_times_tile(float (&acc)[8][4], const float (&S)[D / 8][4], uint32_t kt, int lane)
+// acc[token tile] = (16 x D state) (64 x D tile)^T: columns are tokens.  `late`: called before the last products
+template <int D, typename F>
+__device__ __forceinline__ void state_times_tile(float (&acc)[8][4], const float (&S)[D / 8][4], uint32_t kt, int lane, F &&late)
 {
+    float low[8][4];
 #pragma unroll
     for (int t = 0; t < 8; ++t)
 #pragma unroll
-        for (int e = 0; e < 4; ++e) acc[t][e] = 0.f;
+        for (int e = 0; e < 4; ++e) acc[t][e] = low[t][e] = 0.f;
 #pragma unroll
     for (int ks = 0; ks < D / 16; ++ks) {
-        uint32_t a[3][4], b[4][4];
+        if (ks == D / 16 - 2) late();
+        uint32_t a[3][4];
         split_a(S[2 * ks], S[2 * ks + 1], a[0], a[1], a[2]);
+        uint32_t b[4][4];
 #pragma unroll
         for (int np = 0; np < 4; ++np) frag_b(b[np], kt + (ks >> 2) * 8192, (ks & 3) * 16, np * 16, lane);
 #pragma unroll
         for (int pl = 0; pl < 3; ++pl)
 #pragma unroll
             for (int np = 0; np < 4; ++np) {
-                mma(acc[2 * np], a[pl], b[np][0], b[np][1]);
-                mma(acc[2 * np + 1], a[pl], b[np][2], b[np][3]);
+                mma(pl ? low[2 * np] : acc[2 * np], a[pl], b[np][0], b[np][1]);
+                mma(pl ? low[2 * np + 1] : acc[2 * np + 1], a[pl], b[np][2], b[np][3]);
             }
     }
+#pragma unroll
+    for (int t = 0; t < 8; ++t)
+#pragma unroll
+        for (int e = 0; e < 4; ++e) acc[t][e] += low[t][e];
 }
-// S += (16 tokens of a 16 x 64 factor, three planes) (tile)[those tokens][D]
+// S = gc S + (64 tokens of a 16 x 64 factor, three planes) (tile)[those tokens][D]
 template <int D>
-__device__ __forceinline__ void state_update(float (&S)[D / 8][4], const uint32_t (&a)[3][4], uint32_t tile, int ks, int lane)
+__device__ __forceinline__ void state_update(float (&S)[D / 8][4], float gc, const uint32_t (&a)[4][3][4], uint32_t tile, int lane)
 {
 #pragma unroll
-    for (int np = 0; np < D / 16; np += 2) {
-        uint32_t b[2][4];
-        frag_bt(b[0], tile + (np >> 2) * 8192, ks * 16, (np & 3) * 16, lane);
-        frag_bt(b[1], tile + (np >> 2) * 8192, ks * 16, (np & 3) * 16 + 16, lane);
+    for (int np = 0; np < D / 16; ++np) {
+        uint32_t b[4][4];
+        float d[2][4];
 #pragma unroll
-        for (int pl = 0; pl < 3; ++pl)
+        for (int e = 0; e < 4; ++e) d[0][e] = d[1][e] = 0.f;
 #pragma unroll
-            for (int u = 0; u < 2; ++u) {
-                mma(S[2 * (np + u)], a[pl], b[u][0], b[u][1]);
-                mma(S[2 * (np + u) + 1], a[pl], b[u][2], b[u][3]);
+        for (int ks = 0; ks < 4; ++ks) frag_bt(b[ks], tile + (np >> 2) * 8192, ks * 16, (np & 3) * 16, lane);
+#pragma unroll
+        for (int pl = 2; pl >= 0; --pl)
+#pragma unroll
+            for (int ks = 0; ks < 4; ++ks) {
+                mma(d[0], a[ks][pl], b[ks][0], b[ks][1]);
+                mma(d[1], a[ks][pl], b[ks][2], b[ks][3]);
             }
+#pragma unroll
+        for (int t = 0; t < 2; ++t)
+#pragma unroll
+            for (int e = 0; e < 4; ++e) S[2 * np + t][e] = gc * S[2 * np + t][e] + d[t][e];
     }
 }
-// three-plane x three-plane product on two tiles, terms down to 2^-24
-__device__ __forceinline__ void mma6(float (&c0)[4], float (&c1)[4], const uint32_t (&a)[3][4], const uint32_t (&b)[3][4])
+// three-plane x three-plane product on two tiles, terms down to 2^-24: all but the first
+__device__ __forceinline__ void mma5(float (&c0)[4], float (&c1)[4], const uint32_t (&a)[3][4], const uint32_t (&b)[3][4])
 {
-    constexpr int PA[6] = {0, 0, 1, 0, 2, 1}, PB[6] = {0, 1, 0, 2, 0, 1};
+    constexpr int PA[5] = {1, 2, 0, 1, 0}, PB[5] = {1, 0, 2, 0, 1};
 #pragma unroll
-    for (int t = 0; t < 6; ++t) {
+    for (int t = 0; t < 5; ++t) {
         mma(c0, a[PA[t]], b[PB[t]][0], b[PB[t]][1]);
         mma(c1, a[PA[t]], b[PB[t]][2], b[PB[t]][3]);
     }
@@ -521,16 +542,17 @@ __device__ __forceinline__ void chain(const BwdChunkParams &p, ChainSmem<D> &sm,
             }
         }
         float2 pd[BWD ? 8 : 1][2];
-        if constexpr (BWD) {
-            const float *src = p.pdo + ch * D * C + (size_t)col * C + cq;
-#pragma unroll
-            for (int t = 0; t < 8; ++t) {
-                pd[t][0] = *reinterpret_cast<const float2 *>(src + 8 * t);
-                pd[t][1] = *reinterpret_cast<const float2 *>(src + 8 * C + 8 * t);
-            }
-        }
         float x[8][4], y[8][4];
-        state_times_tile<D>(x, S, kt, lane);   // (K S_0)^T or (K G_1)^T
+        state_times_tile<D>(x, S, kt, lane, [&] {   // (K S_0)^T or (K G_1)^T
+            if constexpr (BWD) {
+                const float *src = p.pdo + ch * D * C + (size_t)col * C + cq;
+#pragma unroll
+                for (int t = 0; t < 8; ++t) {
+                    pd[t][0] = *reinterpret_cast<const float2 *>(src + 8 * t);
+                    pd[t][1] = *reinterpret_cast<const float2 *>(src + 8 * C + 8 * t);
+                }
+            }
+        });
         if constexpr (BWD) {   // dU = D K G_1 + P^T dO
 #pragma unroll
             for (int t = 0; t < 8; ++t) {
@@ -562,10 +584,13 @@ __device__ __forceinline__ void chain(const BwdChunkParams &p, ChainSmem<D> &sm,
         for (int t = 0; t < 8; ++t)
 #pragma unroll
             for (int e = 0; e < 4; ++e) y[t][e] = 0.f;
+        uint32_t xh[4][4];
 #pragma unroll
         for (int ks = 0; ks < 4; ++ks) {
             uint32_t a[3][4];
             split_a(x[2 * ks], x[2 * ks + 1], a[0], a[1], a[2]);
+#pragma unroll
+            for (int e = 0; e < 4; ++e) xh[ks][e] = a[0][e];
 #pragma unroll
             for (int np = BWD ? 0 : ks; np <= (BWD ? ks : 3); ++np) {
                 uint32_t b[3][4];
@@ -574,9 +599,30 @@ __device__ __forceinline__ void chain(const BwdChunkParams &p, ChainSmem<D> &sm,
                     if (BWD) frag_bt(b[pl], tt + pl * 8192, ks * 16, np * 16, lane);
                     else frag_b(b[pl], tt + pl * 8192, ks * 16, np * 16, lane);
                 }
-                mma6(y[2 * np], y[2 * np + 1], a, b);
+                mma5(y[2 * np], y[2 * np + 1], a, b);
             }
         }
+        // the first planes, 32 tokens at a time, added in fp32
+#pragma unroll
+        for (int half = 0; half < 2; ++half)
+#pragma unroll
+            for (int np = 0; np < 4; ++np) {
+                if (BWD ? np > 2 * half + 1 : np < 2 * half) continue;
+                float d[2][4];
+#pragma unroll
+                for (int e = 0; e < 4; ++e) d[0][e] = d[1][e] = 0.f;
+#pragma unroll
+                for (int ks = 2 * half; ks < 2 * half + 2; ++ks) {
+                    if (BWD ? np > ks : np < ks) continue;
+                    uint32_t b[4];
+                    if (BWD) frag_bt(b, tt, ks * 16, np * 16, lane);
+                    else frag_b(b, tt, ks * 16, np * 16, lane);
+                    mma(d[0], xh[ks], b[0], b[1]);
+                    mma(d[1], xh[ks], b[2], b[3]);
+                }
+#pragma unroll
+                for (int e = 0; e < 4; ++e) y[2 * np][e] += d[0][e], y[2 * np + 1][e] += d[1][e];
+            }
         if (BWD) cp_wait<1>();   // Q and dO have landed
         __syncthreads();         // every warp is done with T (and V)
         if (it + 1 < nc) {
@@ -615,30 +661,24 @@ __device__ __forceinline__ void chain(const BwdChunkParams &p, ChainSmem<D> &sm,
                 y[t][0] *= d.x; y[t][1] *= d.y; y[t][2] *= d.x; y[t][3] *= d.y;
             }
         }
+        uint32_t a[4][3][4];
 #pragma unroll
-        for (int t = 0; t < D / 8; ++t)
+        for (int ks = 0; ks < 4; ++ks) split_a(y[2 * ks], y[2 * ks + 1], a[ks][0], a[ks][1], a[ks][2]);
+        state_update<D>(S, gc, a, kt, lane);   // += (D U)^T K, or -= (Gam lam)^T K
+        if constexpr (BWD) {   // += dO^T (Gam Q): the decay goes with dO, in registers
 #pragma unroll
-            for (int e = 0; e < 4; ++e) S[t][e] *= gc;
-#pragma unroll
-        for (int ks = 0; ks < 4; ++ks) {   // += (D U)^T K, or -= (Gam lam)^T K
-            uint32_t a[3][4];
-            split_a(y[2 * ks], y[2 * ks + 1], a[0], a[1], a[2]);
-            state_update<D>(S, a, kt, ks, lane);
-        }
-        if constexpr (BWD) {
-#pragma unroll
-            for (int ks = 0; ks < 4; ++ks) {   // += dO^T (Gam Q): the decay goes with dO, in registers
-                uint32_t d[4], a[3][4];
+            for (int ks = 0; ks < 4; ++ks) {
+                uint32_t d[4];
                 frag_at(d, smem_u32(sm.vd), warp * 16, ks * 16, lane);
                 // registers: (row r, tokens cq, cq + 1), (row r + 8, ...), then tokens + 8
 #pragma unroll
                 for (int e = 0; e < 4; ++e) {
                     const int tk = ks * 16 + cq + (e >> 1) * 8;
                     const float2 f = unpack(d[e]), g = *reinterpret_cast<const float2 *>(&s.gam[tk]), qi = *reinterpret_cast<const float2 *>(&s.qinv[tk]);
-                    split3(f.x * (g.x * qi.x), f.y * (g.y * qi.y), a[0][e], a[1][e], a[2][e]);
+                    split3(f.x * (g.x * qi.x), f.y * (g.y * qi.y), a[ks][0][e], a[ks][1][e], a[ks][2][e]);
                 }
-                state_update<D>(S, a, smem_u32(sm.q), ks, lane);
             }
+            state_update<D>(S, 1.f, a, smem_u32(sm.q), lane);
         }
     }
     if (BWD && p.dinit) {
@@ -765,31 +805,45 @@ __global__ void __launch_bounds__(GT, 1) kla_bwd_grad_kernel(BwdChunkParams p)
 
     const int r = lane >> 2, cq = 2 * (lane & 3);
     auto ratio = [&](int i, int j) { return exp2f((sm.s.g2h[i] - sm.s.g2h[j]) + (sm.s.g2l[i] - sm.s.g2l[j])); };
-    // F = qinv A o (dO U^T) (three terms) and E = -A o (lam U^T) (six), in 16 x 16 blocks on and below the diagonal
+    // F = qinv A o (dO U^T) (three terms) and E = -A o (lam U^T) (six), in 16 x 16 blocks on and below the diagonal; their planes hold what
+    // lies below it
     auto block = [&](bool is_e, int blk) {
         const int bi = blk < 1 ? 0 : blk < 3 ? 1 : blk < 6 ? 2 : 3, bj = blk - bi * (bi + 1) / 2;
         if (bi * 16 >= rows) return;   // tokens past the end: never read
-        float c0[4] = {0.f, 0.f, 0.f, 0.f}, c1[4] = {0.f, 0.f, 0.f, 0.f};
+        float c0[4], c1[4], l0[4], l1[4];
+#pragma unroll
+        for (int e = 0; e < 4; ++e) c0[e] = c1[e] = l0[e] = l1[e] = 0.f;
         const uint32_t at = smem_u32(is_e ? sm.lam : sm.dout), bt = smem_u32(sm.u);
+#pragma unroll 1
+        for (int half = 0; half < 2; ++half) {   // the first planes: half of d_v at a time, added in fp32
+            float h0[4] = {0.f, 0.f, 0.f, 0.f}, h1[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll 2
-        for (int ks = 0; ks < D / 16; ++ks) {
-            const uint32_t o = (ks >> 2) * 8192;
-            uint32_t a[3][4], b[3][4];
+            for (int kk = 0; kk < D / 32; ++kk) {
+                const int ks = half * (D / 32) + kk;
+                const uint32_t o = (ks >> 2) * 8192;
+                uint32_t a[3][4], b[3][4];
 #pragma unroll
-            for (int pl = 0; pl < 3; ++pl) frag_b(b[pl], bt + pl * NB * 8192 + o, (ks & 3) * 16, bj * 16, lane);
-            frag_a(a[0], at + o, bi * 16, (ks & 3) * 16, lane);
-            if (is_e) {
-                frag_a(a[1], at + NB * 8192 + o, bi * 16, (ks & 3) * 16, lane);
-                frag_a(a[2], at + 2 * NB * 8192 + o, bi * 16, (ks & 3) * 16, lane);
-                mma6(c0, c1, a, b);
-            } else {
+                for (int pl = 0; pl < 3; ++pl) frag_b(b[pl], bt + pl * NB * 8192 + o, (ks & 3) * 16, bj * 16, lane);
+                frag_a(a[0], at + o, bi * 16, (ks & 3) * 16, lane);
+                mma(h0, a[0], b[0][0], b[0][1]);
+                mma(h1, a[0], b[0][2], b[0][3]);
+                if (is_e) {
+                    frag_a(a[1], at + NB * 8192 + o, bi * 16, (ks & 3) * 16, lane);
+                    frag_a(a[2], at + 2 * NB * 8192 + o, bi * 16, (ks & 3) * 16, lane);
+                    mma5(l0, l1, a, b);
+                } else {
 #pragma unroll
-                for (int pl = 0; pl < 3; ++pl) {
-                    mma(c0, a[0], b[pl][0], b[pl][1]);
-                    mma(c1, a[0], b[pl][2], b[pl][3]);
+                    for (int pl = 2; pl > 0; --pl) {
+                        mma(l0, a[0], b[pl][0], b[pl][1]);
+                        mma(l1, a[0], b[pl][2], b[pl][3]);
+                    }
                 }
             }
+#pragma unroll
+            for (int e = 0; e < 4; ++e) c0[e] += h0[e], c1[e] += h1[e];
         }
+#pragma unroll
+        for (int e = 0; e < 4; ++e) c0[e] += l0[e], c1[e] += l1[e];
         unsigned char *dst = is_e ? sm.e : sm.f;
 #pragma unroll
         for (int t = 0; t < 2; ++t)
@@ -798,8 +852,9 @@ __global__ void __launch_bounds__(GT, 1) kla_bwd_grad_kernel(BwdChunkParams p)
                 const int i = bi * 16 + r + (e >> 1) * 8, j = bj * 16 + t * 8 + cq;
                 const float sc = is_e ? -1.f : sm.s.qinv[i];
                 float x = t ? c1[e] : c0[e], y = t ? c1[e + 1] : c0[e + 1];
-                x = (is_e ? j < i : j <= i) ? sc * ratio(i, j) * x : 0.f;
-                y = (is_e ? j + 1 < i : j + 1 <= i) ? sc * ratio(i, j + 1) * y : 0.f;
+                if (!is_e && j == (i & ~1)) sm.s.beta[i] = sc * (j == i ? x : y);   // the diagonal of F (the betas have been used)
+                x = j < i ? sc * ratio(i, j) * x : 0.f;
+                y = j + 1 < i ? sc * ratio(i, j + 1) * y : 0.f;
                 uint32_t hh, mm, ll;
                 split3(x, y, hh, mm, ll);
                 const uint32_t off = sw128(i, bj * 2 + t) + 4 * (lane & 3);
@@ -817,16 +872,17 @@ __global__ void __launch_bounds__(GT, 1) kla_bwd_grad_kernel(BwdChunkParams p)
     const int ia = i0 + r, ib = ia + 8;
     const int ks_s = i0 < rows ? D / 16 : 0;      // a warp whose tokens all lie past the end takes no part in the products
     const int ks_j = (rows + 15) / 16;            // token blocks that hold any
-    float gs = 0.f;             // this thread's part of <G_1, S_1>
-    float dga = 0.f, dgb = 0.f; // ... of dg of its two rows
+    float gs = 0.f;             // this thread's part of gC <G_1, S_0>
+    float dga = 0.f, dgb = 0.f; // ... of dg of its two rows, without
+    float cja = 0.f, cjb = 0.f; // ... what they have in common with <G_1, S_1>
     const float gama = sm.s.gam[ia], gamb = sm.s.gam[ib], deca = sm.s.dec[ia], decb = sm.s.dec[ib], gc = sm.s.gam[C - 1];
     const float qia = sm.s.qinv[ia], qib = sm.s.qinv[ib];
+    auto pair = [&](const unsigned char *tile, int i, int t) { return unpack(*reinterpret_cast<const uint32_t *>(tile + sw128(i, nh * 2 + t) + 4 * (lane & 3))); };
     // products x . y of this lane's elements of the two rows, added to a and b
     auto dot = [&](const unsigned char *tile, const float (&x)[2][4], float &a, float &b) {
 #pragma unroll
         for (int t = 0; t < 2; ++t) {
-            const float2 fa = unpack(*reinterpret_cast<const uint32_t *>(tile + sw128(ia, nh * 2 + t) + 4 * (lane & 3)));
-            const float2 fb = unpack(*reinterpret_cast<const uint32_t *>(tile + sw128(ib, nh * 2 + t) + 4 * (lane & 3)));
+            const float2 fa = pair(tile, ia, t), fb = pair(tile, ib, t);
             a += fa.x * x[t][0] + fa.y * x[t][1];
             b += fb.x * x[t][2] + fb.y * x[t][3];
         }
@@ -841,31 +897,40 @@ __global__ void __launch_bounds__(GT, 1) kla_bwd_grad_kernel(BwdChunkParams p)
         fetch(pg, p.g1, hh);
         cp_wait<0>();
         __syncthreads();   // S_0 planes, K, Q (and, the first time, E and F)
-        float xq[2][4], xk[2][4];
+        float xq[2][4], xk[2][4], yq[2][4], yk[2][4];   // y: the lower planes' part
 #pragma unroll
         for (int t = 0; t < 2; ++t)
 #pragma unroll
-            for (int e = 0; e < 4; ++e) xq[t][e] = xk[t][e] = 0.f;
+            for (int e = 0; e < 4; ++e) xq[t][e] = xk[t][e] = yq[t][e] = yk[t][e] = 0.f;
         // dO S_0^T and lam S_0^T
 #pragma unroll 2
         for (int ks = 0; ks < ks_s; ++ks) {
             const uint32_t o = (ks >> 2) * 8192;
-            uint32_t a[4], l[3][4];
+            uint32_t a[4], l[3][4], b[3][4];
             frag_a(a, smem_u32(sm.dout) + o, i0, (ks & 3) * 16, lane);
 #pragma unroll
             for (int pl = 0; pl < 3; ++pl) frag_a(l[pl], smem_u32(sm.lam) + pl * NB * 8192 + o, i0, (ks & 3) * 16, lane);
-            {
-                uint32_t b[3][4];
 #pragma unroll
-                for (int pl = 0; pl < 3; ++pl) frag_bt(b[pl], sg + pl * D * 128, ks * 16, nh * 16, lane);
+            for (int pl = 0; pl < 3; ++pl) frag_bt(b[pl], sg + pl * D * 128, ks * 16, nh * 16, lane);
+            mma(xq[0], a, b[0][0], b[0][1]);
+            mma(xq[1], a, b[0][2], b[0][3]);
+            mma(xk[0], l[0], b[0][0], b[0][1]);
+            mma(xk[1], l[0], b[0][2], b[0][3]);
 #pragma unroll
-                for (int pl = 0; pl < 3; ++pl) {
-                    mma(xq[0], a, b[pl][0], b[pl][1]);
-                    mma(xq[1], a, b[pl][2], b[pl][3]);
-                }
-                mma6(xk[0], xk[1], l, b);
+            for (int pl = 2; pl > 0; --pl) {
+                mma(yq[0], a, b[pl][0], b[pl][1]);
+                mma(yq[1], a, b[pl][2], b[pl][3]);
             }
+            mma5(yk[0], yk[1], l, b);
         }
+#pragma unroll
+        for (int t = 0; t < 2; ++t)
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                xq[t][e] += yq[t][e];
+                xk[t][e] += yk[t][e];
+                yq[t][e] = yk[t][e] = 0.f;
+            }
 #pragma unroll
         for (int t = 0; t < 2; ++t) {
             xq[t][0] *= gama * qia; xq[t][1] *= gama * qia; xq[t][2] *= gamb * qib; xq[t][3] *= gamb * qib;
@@ -874,33 +939,57 @@ __global__ void __launch_bounds__(GT, 1) kla_bwd_grad_kernel(BwdChunkParams p)
         // += F K and E K
 #pragma unroll 1
         for (int ks = 0; ks <= mt && mt < ks_j; ++ks) {
-            uint32_t a[3][4], l[3][4];
+            uint32_t a[3][4], l[3][4], b[4];
+            float hq[2][4], hk[2][4];
+#pragma unroll
+            for (int t = 0; t < 2; ++t)
+#pragma unroll
+                for (int e = 0; e < 4; ++e) hq[t][e] = hk[t][e] = 0.f;
 #pragma unroll
             for (int pl = 0; pl < 3; ++pl) {
                 frag_a(a[pl], smem_u32(sm.f) + pl * 8192, i0, ks * 16, lane);
                 frag_a(l[pl], smem_u32(sm.e) + pl * 8192, i0, ks * 16, lane);
             }
-            {
-                uint32_t b[4];
-                frag_bt(b, kt, ks * 16, nh * 16, lane);
+            frag_bt(b, kt, ks * 16, nh * 16, lane);
+            mma(hq[0], a[0], b[0], b[1]);
+            mma(hq[1], a[0], b[2], b[3]);
+            mma(hk[0], l[0], b[0], b[1]);
+            mma(hk[1], l[0], b[2], b[3]);
 #pragma unroll
-                for (int pl = 0; pl < 3; ++pl) {
-                    mma(xq[0], a[pl], b[0], b[1]);
-                    mma(xq[1], a[pl], b[2], b[3]);
-                    mma(xk[0], l[pl], b[0], b[1]);
-                    mma(xk[1], l[pl], b[2], b[3]);
-                }
+            for (int pl = 2; pl > 0; --pl) {
+                mma(yq[0], a[pl], b[0], b[1]);
+                mma(yq[1], a[pl], b[2], b[3]);
+                mma(yk[0], l[pl], b[0], b[1]);
+                mma(yk[1], l[pl], b[2], b[3]);
             }
+#pragma unroll
+            for (int t = 0; t < 2; ++t)
+#pragma unroll
+                for (int e = 0; e < 4; ++e) {
+                    xq[t][e] += hq[t][e];
+                    xk[t][e] += hk[t][e];
+                }
         }
+#pragma unroll
+        for (int t = 0; t < 2; ++t)
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                xq[t][e] += yq[t][e];
+                xk[t][e] += yk[t][e];
+            }
+        // dg from dq and dk without the diagonal of F: no decay acts on it, and its shares of q . dq and k . dk, which under strong decay
+        // are nearly all of both, would have to cancel
+        dot(sm.q, xq, dga, dgb);
+        dot(sm.k, xk, dga, dgb);
         // dq (with the normalised read-out its projection follows below)
+        const float fda = sm.s.beta[ia], fdb = sm.s.beta[ib];
         const size_t ga = ((t0 + ia) * p.H + h) * D + hh * 64 + nh * 16 + cq, gb = ga + (size_t)8 * p.H * D;
 #pragma unroll
         for (int t = 0; t < 2; ++t) {
-            if (ia < rows) store2(p.dq + ga + 8 * t, xq[t][0], xq[t][1]);
-            if (ib < rows) store2(p.dq + gb + 8 * t, xq[t][2], xq[t][3]);
+            const float2 ka = pair(sm.k, ia, t), kb = pair(sm.k, ib, t);
+            if (ia < rows) store2(p.dq + ga + 8 * t, xq[t][0] + fda * ka.x, xq[t][1] + fda * ka.y);
+            if (ib < rows) store2(p.dq + gb + 8 * t, xq[t][2] + fdb * kb.x, xq[t][3] + fdb * kb.y);
         }
-        dot(sm.q, xq, dga, dgb);
-        dot(sm.k, xk, dga, dgb);
         __syncthreads();   // the S_0 planes have been read
 #pragma unroll
         for (int i = 0; i < IT; ++i)
@@ -914,69 +1003,102 @@ __global__ void __launch_bounds__(GT, 1) kla_bwd_grad_kernel(BwdChunkParams p)
 #pragma unroll
         for (int t = 0; t < 2; ++t)
 #pragma unroll
-            for (int e = 0; e < 4; ++e) xq[t][e] = 0.f;
+            for (int e = 0; e < 4; ++e) xq[t][e] = yq[t][e] = 0.f;
 #pragma unroll 2
         for (int ks = 0; ks < ks_s; ++ks) {
-            uint32_t a[3][4];
+            uint32_t a[3][4], b[3][4];
 #pragma unroll
             for (int pl = 0; pl < 3; ++pl) frag_a(a[pl], smem_u32(sm.u) + (pl * NB + (ks >> 2)) * 8192, i0, (ks & 3) * 16, lane);
-            {
-                uint32_t b[3][4];
 #pragma unroll
-                for (int pl = 0; pl < 3; ++pl) frag_bt(b[pl], sg + pl * D * 128, ks * 16, nh * 16, lane);
-                mma6(xq[0], xq[1], a, b);
-            }
+            for (int pl = 0; pl < 3; ++pl) frag_bt(b[pl], sg + pl * D * 128, ks * 16, nh * 16, lane);
+            mma(xq[0], a[0], b[0][0], b[0][1]);
+            mma(xq[1], a[0], b[0][2], b[0][3]);
+            mma5(yq[0], yq[1], a, b);
         }
+#pragma unroll
+        for (int t = 0; t < 2; ++t)
+#pragma unroll
+            for (int e = 0; e < 4; ++e) xq[t][e] += yq[t][e];
 #pragma unroll
         for (int t = 0; t < 2; ++t) {
             xq[t][0] *= deca; xq[t][1] *= deca; xq[t][2] *= decb; xq[t][3] *= decb;
         }
-        dot(sm.k, xq, gs, gs);   // <G_1, S_1> = gC <G_1, S_0> + sum_j k_j . (D U G_1^T)_j
+        dot(sm.k, xq, cja, cjb);   // <G_1, S_1> = gC <G_1, S_0> + sum_j k_j . (D U G_1^T)_j
         // += E^T K + F^T Q: rows of this warp are the columns of E and F
-#pragma unroll 1
-        for (int ks = mt; ks < ks_j; ++ks) {
-            uint32_t a[3][4], l[3][4];
+        {
+            float y[2][4], z[2][4];
 #pragma unroll
-            for (int pl = 0; pl < 3; ++pl) {
-                frag_at(a[pl], smem_u32(sm.f) + pl * 8192, i0, ks * 16, lane);
-                frag_at(l[pl], smem_u32(sm.e) + pl * 8192, i0, ks * 16, lane);
-            }
-            {
-                uint32_t b[4], b2[4];
-                frag_bt(b, qt, ks * 16, nh * 16, lane);
-                frag_bt(b2, kt, ks * 16, nh * 16, lane);
+            for (int t = 0; t < 2; ++t)
+#pragma unroll
+                for (int e = 0; e < 4; ++e) y[t][e] = z[t][e] = 0.f;
+#pragma unroll 1
+            for (int ks = mt; ks < ks_j; ++ks) {
+                uint32_t a[3][4], l[3][4], b[4], b2[4];
+                float h[2][4];
+#pragma unroll
+                for (int e = 0; e < 4; ++e) h[0][e] = h[1][e] = 0.f;
 #pragma unroll
                 for (int pl = 0; pl < 3; ++pl) {
-                    mma(xq[0], a[pl], b[0], b[1]);
-                    mma(xq[1], a[pl], b[2], b[3]);
-                    mma(xq[0], l[pl], b2[0], b2[1]);
-                    mma(xq[1], l[pl], b2[2], b2[3]);
+                    frag_at(a[pl], smem_u32(sm.f) + pl * 8192, i0, ks * 16, lane);
+                    frag_at(l[pl], smem_u32(sm.e) + pl * 8192, i0, ks * 16, lane);
                 }
+                frag_bt(b, qt, ks * 16, nh * 16, lane);
+                frag_bt(b2, kt, ks * 16, nh * 16, lane);
+                mma(h[0], a[0], b[0], b[1]);
+                mma(h[1], a[0], b[2], b[3]);
+                mma(h[0], l[0], b2[0], b2[1]);
+                mma(h[1], l[0], b2[2], b2[3]);
+#pragma unroll
+                for (int pl = 2; pl > 0; --pl) {
+                    mma(y[0], a[pl], b[0], b[1]);
+                    mma(y[1], a[pl], b[2], b[3]);
+                    mma(y[0], l[pl], b2[0], b2[1]);
+                    mma(y[1], l[pl], b2[2], b2[3]);
+                }
+#pragma unroll
+                for (int t = 0; t < 2; ++t)
+#pragma unroll
+                    for (int e = 0; e < 4; ++e) z[t][e] += h[t][e];
             }
+#pragma unroll
+            for (int t = 0; t < 2; ++t)
+#pragma unroll
+                for (int e = 0; e < 4; ++e) z[t][e] += y[t][e];
+            float ca = 0.f, cb = 0.f;
+            dot(sm.k, z, ca, cb);
+            dga -= ca;
+            dgb -= cb;
+#pragma unroll
+            for (int t = 0; t < 2; ++t)
+#pragma unroll
+                for (int e = 0; e < 4; ++e) xq[t][e] += z[t][e];
         }
-        float ca = 0.f, cb = 0.f;
-        dot(sm.k, xq, ca, cb);
-        dga -= ca;
-        dgb -= cb;
         const float na = sm.s.dn[ia], nb = sm.s.dn[ib];
 #pragma unroll
         for (int t = 0; t < 2; ++t) {
-            const float2 fa = unpack(*reinterpret_cast<const uint32_t *>(sm.k + sw128(ia, nh * 2 + t) + 4 * (lane & 3)));
-            const float2 fb = unpack(*reinterpret_cast<const uint32_t *>(sm.k + sw128(ib, nh * 2 + t) + 4 * (lane & 3)));
-            if (ia < rows) store2(p.dk + ga + 8 * t, xk[t][0] + xq[t][0] + na * fa.x, xk[t][1] + xq[t][1] + na * fa.y);
-            if (ib < rows) store2(p.dk + gb + 8 * t, xk[t][2] + xq[t][2] + nb * fb.x, xk[t][3] + xq[t][3] + nb * fb.y);
+            const float2 ka = pair(sm.k, ia, t), kb = pair(sm.k, ib, t), qa = pair(sm.q, ia, t), qb = pair(sm.q, ib, t);
+            if (ia < rows) store2(p.dk + ga + 8 * t, (xk[t][0] + xq[t][0]) + (na * ka.x + fda * qa.x), (xk[t][1] + xq[t][1]) + (na * ka.y + fda * qa.y));
+            if (ib < rows) store2(p.dk + gb + 8 * t, (xk[t][2] + xq[t][2]) + (nb * kb.x + fdb * qb.x), (xk[t][3] + xq[t][3]) + (nb * kb.y + fdb * qb.y));
         }
         __syncthreads();   // K, Q and the planes may be overwritten
     }
 
-    // dlog_alpha_t = <G_1, S_1> + sum_{i >= t} dg_i
-    dga += __shfl_xor_sync(0xffffffffu, dga, 1);
-    dgb += __shfl_xor_sync(0xffffffffu, dgb, 1);
-    dga += __shfl_xor_sync(0xffffffffu, dga, 2);
-    dgb += __shfl_xor_sync(0xffffffffu, dgb, 2);
+    // dlog_alpha_t = <G_1, S_1> + sum_{i >= t} dg_i; the write of token j is in the first with c_j = k_j . (D U G_1^T)_j and in dg_j with -c_j,
+    // the same fp32 value, so that what no decay has touched cancels exactly
+    float (*cj)[64] = reinterpret_cast<float (*)[64]>(sm.f);   // (F has been used)
+    auto quad = [](float x) {
+        x += __shfl_xor_sync(0xffffffffu, x, 1);
+        return x + __shfl_xor_sync(0xffffffffu, x, 2);
+    };
+    dga = quad(dga);
+    dgb = quad(dgb);
+    cja = quad(cja);
+    cjb = quad(cjb);
     if ((lane & 3) == 0) {
         sm.red[nh][ia] = dga;
         sm.red[nh][ib] = dgb;
+        cj[nh][ia] = cja;
+        cj[nh][ib] = cjb;
     }
     gs = warp_sum(gs);
     if (lane == 0) sm.s.nrm[warp] = gs;   // (the norms have been used; no room for an array of its own at d = 128)
@@ -985,9 +1107,14 @@ __global__ void __launch_bounds__(GT, 1) kla_bwd_grad_kernel(BwdChunkParams p)
         double tot = 0.0;
 #pragma unroll
         for (int i = 0; i < GW; ++i) tot += (double)sm.s.nrm[i];
-        auto rsum = [&](int i) { return ((double)sm.red[0][i] + (double)sm.red[1][i]) + ((double)sm.red[2][i] + (double)sm.red[3][i]); };
+        auto rsum = [](const float (*r)[64], int i) { return ((double)r[0][i] + (double)r[1][i]) + ((double)r[2][i] + (double)r[3][i]); };
         const int a = 63 - 2 * lane, b = a - 1;   // lane 0 holds the last two tokens
-        const double x0 = rsum(a), x1 = rsum(b);
+        const double c0 = rsum(cj, a), c1 = rsum(cj, b);
+        double c = c0 + c1;
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) c += __shfl_xor_sync(0xffffffffu, c, o);
+        tot += c;
+        const double x0 = rsum(sm.red, a) - c0, x1 = rsum(sm.red, b) - c1;
         double incl = x0 + x1;
 #pragma unroll
         for (int o = 1; o < 32; o <<= 1) {

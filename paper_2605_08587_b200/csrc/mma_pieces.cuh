@@ -3,8 +3,13 @@
 //
 // Precision.  q, k, v, dO are exact bf16 operands.  A derived fp32 value x is split into h + m + l, each the bf16 rounding of
 // what the ones before it leave: 24 significand bits, as many as x has.  A product of an exact with a derived operand is then
-// three instructions, one of two derived operands six (the terms below 2^-24 are dropped), so results are those of fp32
-// arithmetic up to the order of the sums.
+// three instructions, one of two derived operands six (the terms below 2^-24 are dropped).
+//
+// The sums inside an instruction are truncated, not rounded: 1 + 0.75 ulp gives 1, 1 - 0.25 ulp gives 1 - 0.5 ulp, and sixteen
+// addends of 2^-26 leave 1 as it is (measured; two bits below the last place of the largest addend are kept).  On random data an
+// instruction that adds to a sum of its own size is off by 0.27 ulp towards zero in the mean; errors of one sign add up over a
+// long sum.  So the terms of the lower planes have accumulators of their own, and where a result is added to something larger
+// or is a long sum itself, the parts are added in fp32.
 //
 // Why mma.sync and not tcgen05 here: its operands and accumulators live in registers, so a chain of products needs no round
 // trip through tensor memory, no shared-memory operand tiles for the derived factor and no barrier between the warps of a

@@ -8,11 +8,13 @@ import numpy as np
 import pytest
 import torch
 
+import oracle
 from helpers import gpu_chunk, np64, oracle_chunk
-from paper_2605_08587_b200 import workloads as W
+from paper_2605_08587_b200 import kla_bwd, workloads as W
 
 pytestmark = pytest.mark.gpu
 PAIR = 2.2e-6
+SUM = 8 * 0.4 * 0.72 * 2.0 ** -23 / 2
 
 
 def _norm_err(got, ref):
@@ -49,3 +51,43 @@ def test_forward_that_forgets_little(d):
     ro, rf = oracle_chunk(w)[:2]
     assert _norm_err(out, ro) <= 1.15 * 4 ** 0.5 * PAIR
     assert _norm_err(fin, rf) <= 1.15 * 1.5 ** 0.5 * PAIR
+
+
+def _backward_errors(w, seed):
+    H, d = w.q.shape[2:]
+    w.init_state = (0.02 * torch.randn(w.n_seq, H, d, d, generator=torch.Generator().manual_seed(seed))).float()
+    do, df = W.upstream_grads(w)
+    dev = "cuda:0"
+    cu = w.cu_seqlens
+    g = kla_bwd(*[x.to(dev) for x in (w.q, w.k, w.v, w.log_alpha, w.eta)], w.eps, do.to(dev), init_state=w.init_state.to(dev),
+                d_final_state=df.to(dev), cu_seqlens=None if cu is None else cu.to(dev), host_seqlens=cu)
+    ins = [np64(x) for x in (w.q, w.k, w.v, w.log_alpha, w.eta)]
+    if cu is None:
+        r = oracle.backward(*ins, w.eps, np64(do), np64(w.init_state), np64(df))
+    else:
+        r = oracle.backward_packed(*[x[0] for x in ins], w.eps, cu.numpy(), np64(do)[0], np64(w.init_state), np64(df))
+    r["dinit_state"] = r["dinit"]
+    return {n: _norm_err(g[n].reshape(r[n].shape), r[n]) for n in ("dq", "dk", "dv", "dlog_alpha", "deta", "dinit_state")}
+
+
+def _check_backward(w, seed, times=1.0):
+    for name, err in _backward_errors(w, seed).items():
+        # five products in succession (P^T dO or K S_0, U or w, E or F, and two of the gradient) in quadrature; dlog_alpha is a sum of
+        # differences of such gradients, twice the size of what is left
+        bound = times * 5 ** 0.5 * SUM * (2.0 if name == "dlog_alpha" else 1.0)
+        assert err <= bound, "%s: %.2e > %.2e" % (name, err, bound)
+
+
+@pytest.mark.parametrize("kind", ["d64", "d128", "packed"])
+def test_backward(kind):
+    _check_backward(_workload(kind), 1420)
+
+
+@pytest.mark.parametrize("d", [64, 128])
+def test_backward_that_forgets_little(d):
+    """As for the forward.  What each of 64 chunks adds has such an error of its own; they are of both signs, and a state keeps what
+    d / eta tokens, here all of them, have added: twice the bound for the states' part."""
+    w = W.config2(B=1, H=2, T=4096, d=d, seed=1430 + d)
+    w.log_alpha = torch.zeros_like(w.log_alpha)
+    w.eta = w.eta * 1e-3
+    _check_backward(w, 1431, times=2.0)
