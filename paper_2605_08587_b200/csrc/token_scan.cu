@@ -13,11 +13,14 @@
 //     S_4 = A_4 o S_0 + sum_s (beta_s k_s o A_4/A_s) e_s                          one update of the state for all four
 //
 // where Lk_ts = beta_s k_t . (A_t/A_s o k_s) and Lq likewise with q_t.  All decay ratios are products of alphas (never a
-// quotient), so nothing overflows however strong the decay.  What depends on the head only -- the decayed vectors, the
+// quotient), so nothing overflows however strong the decay.  A_4 itself, which the state meets with every block, is applied with its
+// rounding error (expm1 of the sum of log alpha where it is near 1): an error of 2^-25 in a decay near 1 is the same for the whole
+// state and, of one sign as those of expf are, adds up over all that is remembered (log alpha / 100, eta / 10, 4 096 tokens, fp32: final
+// state off by 5.8e-6 of its norm with A_4 as a product of four expf, 4e-7 this way).  What depends on the head only -- the decayed vectors, the
 // triangles, beta -- is prepared once per block of tokens by one warp and read by every warp from shared memory.
 //
-// What bounds it: the fp32 pipe.  A token costs 3.25 d^2 multiply-adds per head (2 d^2 in the sweep, d^2 in the update, a
-// quarter for the decay), fewer than the chunk algebra on the same cores (4 C d + 6 d^2 flops, half as multiply-adds, plus
+// What bounds it: the fp32 pipe.  A token costs 3.5 d^2 multiply-adds per head (2 d^2 in the sweep, d^2 in the update, half
+// for the decay and its rounding error), fewer than the chunk algebra on the same cores (4 C d + 6 d^2 flops, half as multiply-adds, plus
 // the triangular solve), and the four-token block divides the latency of the reductions by four (one token at a time, the
 // scan of a layer with diagonal gates, B8 H8 T4096 d128, took 2.94 ms: 1 370 cycles per token for 340 cycles of arithmetic; the
 // chunk algebra on CUDA cores took 102 us for the 256 tokens of the small fp32 configuration, this scan 33 us).
@@ -28,7 +31,7 @@
 // fp32 multiply-adds without duplicating an operand, and leaves only three butterfly stages for the sums over rows.
 // CPL: a float4 from shared memory costs four cycles of the load pipe even when it is a broadcast, and feeds 2 CPL packed
 // multiply-adds (four SM cycles at CPL = 4): with CPL = 2 the scan of a layer was bound by those loads (436 wavefronts per
-// token, load pipe 75 % busy, 1.40 ms; with CPL = 4 and both sweeps in one loop 1.00 ms, bound by the latency of one scanning
+// token, load pipe 75 % busy, 1.40 ms; with CPL = 4 and both sweeps in one loop 1.00 ms (1.06 with the decay's rounding error), bound by the latency of one scanning
 // warp per scheduler, fp32 pipe 53 % busy).  CPL = 2 stays where there are too few (sequence, head) pairs to give every SM more than
 // two warps of 16 columns: twice the warps then halve the latency.
 #include "common.cuh"
@@ -42,11 +45,12 @@ constexpr int BT = 4;     // tokens per block
 constexpr int NW = 4;     // scanning warps per thread block, and as many preparing ones: one of each per scheduler
 
 // One block of BT tokens as the scan reads it.
-template <int D, int CPL>
+template <int D, int CPL, bool DIAG>
 struct Block {
     float k[BT][D], q[BT][D];    // A_t o k_t, A_t o q_t
     float b[BT][D];              // beta_s k_s o A_4 / A_s
-    float decay[D];              // A_4
+    float decay[DIAG ? D : 4];      // A_4 rounded (without diagonal gates one number, [0])
+    float decay_lo[DIAG ? D : 4];   // what the rounding left out
     float tri[BT][BT];           // [t][s], s <= t: Lq_ts;  [s][t], s < t: Lk_ts
     float v[BT][NW * 4 * CPL];   // the thread block's columns
 };
@@ -54,7 +58,7 @@ struct Block {
 template <int D, int CPL, typename IO, typename OUT, bool DIAG>
 __global__ void __launch_bounds__(64 * NW, 1) kla_token_scan_kernel(TokenScanParams p)
 {
-    using Blk = Block<D, CPL>;
+    using Blk = Block<D, CPL, DIAG>;
     constexpr int WCOLS = 4 * CPL, COLS = NW * WCOLS, GROUPS = D / COLS;   // columns per warp, per thread block
     constexpr int VL = CPL / 2;                                            // sums per lane after the butterflies
     constexpr int VC = COLS / 8;                                           // columns of v per lane in the preparation
@@ -194,7 +198,27 @@ __global__ void __launch_bounds__(64 * NW, 1) kla_token_scan_kernel(TokenScanPar
             put(bl.k[t], y);
             put(bl.q[t], z);
         }
-        put(bl.decay, A);
+        float lo[JD];
+#pragma unroll
+        for (int j = 0; j < JD; ++j) {
+            float sum = 0.f;
+#pragma unroll
+            for (int t = 0; t < BT; ++t) {
+                const float la = DIAG ? r.la[DIAG ? t : 0][DIAG ? j : 0] : __shfl_sync(0xffffffffu, r.la_s, t);
+                sum += t0 + t < len ? la : 0.f;
+            }
+            const float m = expm1f(sum), hi = 1.f + m;
+            lo[j] = A[j] > 0.5f ? (1.f - hi) + m : 0.f;
+            if (A[j] > 0.5f) A[j] = hi;
+            if (!DIAG) break;   // one number for all rows
+        }
+        if constexpr (DIAG) {
+            put(bl.decay, A);
+            put(bl.decay_lo, lo);
+        } else if (lane == 0) {
+            bl.decay[0] = A[0];
+            bl.decay_lo[0] = lo[0];
+        }
 #pragma unroll
         for (int j = 0; j < JD; ++j) A[j] = 1.f;
 #pragma unroll
@@ -252,6 +276,7 @@ __global__ void __launch_bounds__(64 * NW, 1) kla_token_scan_kernel(TokenScanPar
             }
 
     auto process = [&](const Blk &bl, int t0) {
+        const float d0 = bl.decay[0], d1 = bl.decay_lo[0];
         // one sweep over the state for k and q of all four tokens
         float2 au[BT][CPL], aw[BT][CPL];
 #pragma unroll
@@ -320,11 +345,12 @@ __global__ void __launch_bounds__(64 * NW, 1) kla_token_scan_kernel(TokenScanPar
         // state first (the next block waits for it), then this lane's outputs
 #pragma unroll
         for (int i = 0; i < NI; ++i) {
-            const float4 dd = DIAG ? load4(&bl.decay[4 * (rg + 8 * i)]) : make_float4(bl.decay[0], bl.decay[0], bl.decay[0], bl.decay[0]);
+            const float4 dd = DIAG ? load4(&bl.decay[4 * (rg + 8 * i)]) : make_float4(d0, d0, d0, d0);
+            const float4 dl = DIAG ? load4(&bl.decay_lo[4 * (rg + 8 * i)]) : make_float4(d1, d1, d1, d1);
 #pragma unroll
             for (int c = 0; c < CPL; ++c) {
-                S[i][0][c] = mul2(f2(dd.x, dd.y), S[i][0][c]);
-                S[i][1][c] = mul2(f2(dd.z, dd.w), S[i][1][c]);
+                S[i][0][c] = fma2(f2(dd.x, dd.y), S[i][0][c], mul2(f2(dl.x, dl.y), S[i][0][c]));
+                S[i][1][c] = fma2(f2(dd.z, dd.w), S[i][1][c], mul2(f2(dl.z, dl.w), S[i][1][c]));
             }
 #pragma unroll
             for (int s = 0; s < BT; ++s) {
@@ -376,7 +402,7 @@ template <int D, int CPL, typename IO, typename OUT, bool DIAG>
 cudaError_t launch_k(const TokenScanParams &p, cudaStream_t stream)
 {
     auto kern = kla_token_scan_kernel<D, CPL, IO, OUT, DIAG>;
-    constexpr int smem = 2 * NW * (int)sizeof(Block<D, CPL>);
+    constexpr int smem = 2 * NW * (int)sizeof(Block<D, CPL, DIAG>);
     if (smem > 48 * 1024) {
         cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
         if (e != cudaSuccess) return e;
@@ -391,7 +417,7 @@ cudaError_t launch_t(const TokenScanParams &p, cudaStream_t stream)
 {
     if (p.n_seq * p.H == 0) return cudaSuccess;
     // 16 columns per warp as soon as that gives every SM more than two scanning warps (see the head of the file)
-    if ((long long)p.n_seq * p.H * (D / 16) > 2 * 148) return launch_k<D, 4, IO, OUT, DIAG>(p, stream);
+    if ((long long)p.n_seq * p.H * (D / 16) > 2LL * sm_count()) return launch_k<D, 4, IO, OUT, DIAG>(p, stream);
     return launch_k<D, 2, IO, OUT, DIAG>(p, stream);
 }
 

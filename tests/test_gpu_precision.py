@@ -10,7 +10,7 @@ import torch
 
 import oracle
 from helpers import gpu_chunk, np64, oracle_chunk
-from paper_2605_08587_b200 import kla_bwd, workloads as W
+from paper_2605_08587_b200 import kla_bwd, kla_chunk_fwd, kla_dg_fwd, workloads as W
 
 pytestmark = pytest.mark.gpu
 PAIR = 2.2e-6
@@ -91,3 +91,45 @@ def test_backward_that_forgets_little(d):
     w.log_alpha = torch.zeros_like(w.log_alpha)
     w.eta = w.eta * 1e-3
     _check_backward(w, 1431, times=2.0)
+
+
+@pytest.mark.parametrize("diag", [False, True])
+@pytest.mark.parametrize("d", [64, 128])
+def test_recurrence_with_weak_decay(d, diag):
+    """fp32 scan, log alpha / 100, eta / 10.  The state is rounded five times in four tokens, each time by a uniform error within half
+    a unit in the last place, a unit being 0.72 * 2^-23 of a value in the mean, independently; what it remembers, and the errors with it, decays over
+    half of d / eta < 4 000 tokens for errors added in quadrature.  An error in the decay, one for the whole state, would add up."""
+    steps = 5 * 4000 / 2 / 4
+    bound = steps ** 0.5 * 2.0 ** -24 * 0.72 / 3 ** 0.5
+    if diag:
+        w = W.config_dg(B=1, H=2, T=4096, d=d, seed=1440 + d, dtype=torch.float32)
+    else:
+        w = W.config2(B=1, H=2, T=4096, d=d, seed=1440 + d)
+        w.q, w.k, w.v = w.q.float(), w.k.float(), w.v.float()
+    w.log_alpha, w.eta = w.log_alpha * 1e-2, w.eta * 0.1
+    a = [x.to("cuda:0") for x in (w.q, w.k, w.v, w.log_alpha, w.eta)]
+    s0 = None if w.init_state is None else w.init_state.to("cuda:0")
+    out, fin = (kla_dg_fwd if diag else kla_chunk_fwd)(*a, w.eps, init_state=s0, out_dtype=torch.float32)
+    ro, rf, _ = oracle.forward(*[np64(x) for x in (w.q, w.k, w.v, w.log_alpha, w.eta)], w.eps, None if s0 is None else np64(s0), diagonal_gates=diag)
+    assert _norm_err(out, ro) <= bound
+    assert _norm_err(fin, rf) <= bound
+
+
+@pytest.mark.parametrize("diag", [False, True])
+def test_recurrence_with_decays_on_both_sides_of_one_half(diag):
+    """Decays of a block of four tokens from 1 down to 0, no writes: the state keeps the product of them."""
+    B, T, H, d = 1, 64, 2, 64
+    g = torch.Generator().manual_seed(1450)
+    q, k, v = (torch.randn(B, T, H, d, generator=g) for _ in range(3))
+    la = -torch.logspace(-6, 0.5, T).reshape(1, T, 1).expand(B, T, H).contiguous() * torch.tensor([1.0, 30.0])   # head 1: down to nothing
+    la[:, 0] = 0.0
+    s0 = torch.randn(B, H, d, d, generator=g)
+    eta = torch.zeros(B, T, H)
+    if diag:
+        la = (la.unsqueeze(-1) * torch.linspace(0.0, 2.0, d)).contiguous()
+    a = [x.to("cuda:0") for x in (q, k, v, la, eta)]
+    _, fin = (kla_dg_fwd if diag else kla_chunk_fwd)(*a, 1e-6, init_state=s0.to("cuda:0"), out_dtype=torch.float32)
+    ref = s0.double() * torch.exp(la.double().sum(1)).reshape(B, H, d if diag else 1, 1)
+    err = ((fin.cpu().double() - ref).abs() / ref.abs().clamp_min(1e-30)).max()
+    # 16 blocks: a rounding of the state each, and a decay that is a product of four expf (2 ulp each) where it is below one half
+    assert float(err) <= 16 * (1 + 4 * 3) * 2.0 ** -24
