@@ -353,7 +353,7 @@ def test_variants_fp32_and_segments():
 
 
 # ---- the bounded-wait error path (no fault, no hang: a wait runs out by design and the kernel reports it) -------------
-@pytest.mark.parametrize("no_pair", [0, 32])   # paired CTAs (a cluster per head) and independent CTAs
+@pytest.mark.parametrize("no_pair", [0, 32])   # (KLA_FLAG_NO_PAIR: without effect)
 def test_bounded_wait_reports_timeout_and_context_stays_usable(no_pair):
     from paper_2605_08587_b200 import binding
     w = W.config2(B=1, H=2, T=200, seed=501)
@@ -391,14 +391,13 @@ def test_timeout_without_a_caller_status_word_is_raised_by_check():
     assert rel_err(np64(out), ro) <= TOL_BF16 and rel_err(np64(fin), rf) <= TOL_BF16
 
 
-# ---- d_v = 128: the two slices of a head as a cluster that shares the solve (default) or as independent CTAs ----------
+# ---- KLA_FLAG_NO_PAIR is accepted and changes nothing (blocks never work in pairs); repeated launches are bit-identical ----------
 from paper_2605_08587_b200 import KLA_FLAG_NO_PAIR  # noqa: E402
 
 
 @pytest.mark.parametrize("T", [1, 64, 65, 129, 1000, 2048 + 17])
-def test_independent_ctas_match_oracle_and_paired_launch_bitwise(T):
-    """Both launch forms do the same arithmetic on the same operands: the results must be identical, and the
-    unpaired form is checked against the oracle by itself."""
+def test_no_pair_flag_matches_oracle_and_default_bitwise(T):
+    """The flag selects the same kernel: identical results, checked against the oracle."""
     w = W.config3(B=2, H=2, T=T, seed=300 + T)
     out_u, fin_u = _check_fixed(w, TOL_BF16, flags=KLA_FLAG_NO_PAIR)
     out_p, fin_p = gpu_chunk(w)
@@ -406,7 +405,7 @@ def test_independent_ctas_match_oracle_and_paired_launch_bitwise(T):
     assert torch.equal(fin_p, fin_u)
 
 
-def test_paired_segments_and_packed_input_bitwise():
+def test_no_pair_flag_with_segments_and_packed_input_bitwise():
     w = W.config3(B=1, H=3, T=1536 + 40, seed=311)
     o_p, f_p = gpu_chunk(w, flags=KLA_FLAG_SEGMENTS(3))
     o_u, f_u = gpu_chunk(w, flags=KLA_FLAG_SEGMENTS(3) | KLA_FLAG_NO_PAIR)
@@ -417,15 +416,15 @@ def test_paired_segments_and_packed_input_bitwise():
     assert torch.equal(o_p, o_u) and torch.equal(f_p, f_u)
 
 
-def test_paired_launch_is_repeatable_over_several_waves():
-    """More clusters than the GPU holds at once, many launches: every launch must reproduce the independent-CTA result
-    bit for bit (a hand-over between the CTAs of a pair that relied on timing would show up here)."""
-    w = W.config2(B=24, H=8, T=640, seed=321)          # 384 CTAs of one CTA per SM
+def test_launches_are_repeatable_over_several_waves():
+    """More blocks than the GPU holds at once, many launches: every launch must reproduce the first bit for bit (a hand-over between
+    the warps of a block that relied on timing would show up here)."""
+    w = W.config2(B=24, H=8, T=640, seed=321)          # 384 blocks, one per SM
     o_u, f_u = gpu_chunk(w, flags=KLA_FLAG_NO_PAIR)
     for _ in range(12):
         o_p, f_p = gpu_chunk(w)
         assert torch.equal(o_p, o_u) and torch.equal(f_p, f_u)
-    wl = W.config3()                                    # one long sequence: segment passes of 256 and 144 CTAs
+    wl = W.config3()                                    # one long sequence: 144 blocks that start from warm-up runs
     o_u, f_u = gpu_chunk(wl, flags=KLA_FLAG_NO_PAIR)
     for _ in range(12):
         o_p, f_p = gpu_chunk(wl)

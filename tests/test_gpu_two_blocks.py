@@ -2,8 +2,9 @@
 import pytest
 import torch
 
-from helpers import TOL_BF16, gpu_chunk, np64, oracle_chunk, rel_err
-from paper_2605_08587_b200 import workloads as W
+import oracle
+from helpers import TOL_BF16, assert_bf16_out_close, gpu_chunk, np64, oracle_chunk, rel_err
+from paper_2605_08587_b200 import KLA_FLAG_COEFF_ETA, KLA_FLAG_QNORM, workloads as W
 
 pytestmark = pytest.mark.gpu
 
@@ -28,3 +29,22 @@ def test_both_forms_agree_bit_for_bit():
         setattr(part, name, getattr(w, name)[:4].contiguous())
     o, f = gpu_chunk(part, out_dtype=torch.float32)
     assert torch.equal(out[:4], o) and torch.equal(fin[:4], f)
+
+
+@pytest.mark.parametrize("out_dtype", [torch.float32, torch.bfloat16])
+@pytest.mark.parametrize("variant", [(True, False), (False, True), (True, True)])
+@pytest.mark.parametrize("B", [2, 20])   # 32 blocks: one on an SM; 320: two
+def test_layer_edge_variants(B, variant, out_dtype):
+    coeff_eta, qnorm = variant
+    w = W.config3(B=B, H=16, T=200, d=64, seed=1310 + 2 * coeff_eta + qnorm)   # three chunks and a ragged one: every slot is used again
+    if coeff_eta:   # beta = eta is a contraction only on unit keys
+        k = w.k.float()
+        w.k = (k / k.norm(dim=-1, keepdim=True)).to(w.k.dtype)
+    out, fin = gpu_chunk(w, out_dtype=out_dtype, flags=(KLA_FLAG_COEFF_ETA if coeff_eta else 0) | (KLA_FLAG_QNORM if qnorm else 0))
+    with oracle.variant(coeff_eta=coeff_eta, qnorm=qnorm):
+        ro, rf = oracle_chunk(w)[:2]
+    if out_dtype == torch.bfloat16:
+        assert_bf16_out_close(out, ro)
+    else:
+        assert rel_err(np64(out), ro) <= TOL_BF16
+    assert rel_err(np64(fin), rf) <= TOL_BF16
