@@ -160,6 +160,19 @@ def _stream(dev):
     return torch.cuda.current_stream(dev).cuda_stream
 
 
+def _sequence_shapes(q, k, v, log_alpha, eta):
+    """B, T, H, d_k, d_v of a call that does not go through the native half, which checks the same (csrc/host.cpp)."""
+    B, T, H, d_k = q.shape
+    d_v = v.shape[-1]
+    if tuple(k.shape) != (B, T, H, d_k) or tuple(v.shape) != (B, T, H, d_v):
+        raise ValueError("q, k, v shapes disagree")
+    if tuple(log_alpha.shape) != (B, T, H) or tuple(eta.shape) != (B, T, H):
+        raise ValueError("log_alpha, eta must be [B, T, H]")
+    if k.dtype != q.dtype or v.dtype != q.dtype:
+        raise TypeError("q, k, v must share one dtype")
+    return B, T, H, d_k, d_v
+
+
 def kla_chunk_fwd(q, k, v, log_alpha, eta, eps, chunk=64, init_state=None, out=None, final_state=None,
                   cu_seqlens=None, host_seqlens=None, out_dtype=None, flags=KLA_FLAG_NONE,
                   want_final_state=True, status_word=None, pass_ms=None, plan_word=None):
@@ -182,14 +195,7 @@ def kla_chunk_fwd(q, k, v, log_alpha, eta, eps, chunk=64, init_state=None, out=N
             host_seqlens = cu_seqlens.cpu()
         return _host.forward(q, k, v, log_alpha, eta, eps, chunk, init_state, out, final_state, cu_seqlens, host_seqlens, out_dtype,
                              flags, want_final_state, status_word, 0)
-    B, T, H, d_k = q.shape
-    d_v = v.shape[-1]
-    if tuple(k.shape) != (B, T, H, d_k) or tuple(v.shape) != (B, T, H, d_v):
-        raise ValueError("q, k, v shapes disagree")
-    if tuple(log_alpha.shape) != (B, T, H) or tuple(eta.shape) != (B, T, H):
-        raise ValueError("log_alpha, eta must be [B, T, H]")
-    if k.dtype != q.dtype or v.dtype != q.dtype:
-        raise TypeError("q, k, v must share one dtype")
+    B, T, H, d_k, d_v = _sequence_shapes(q, k, v, log_alpha, eta)
     n_seq = B
     hs = None
     if cu_seqlens is not None:
@@ -245,12 +251,9 @@ def kla_chunk_fwd_static_scratch(q, k, v, log_alpha, eta, eps, out, final_state=
     be passed in, and for packed input both `cu_seqlens` (CUDA int32) and `host_seqlens` (CPU int32 copy).  Shapes whose
     scratch would exceed STATIC_SCRATCH_BYTES raise KlaError (workspace).  Calls must not overlap on the GPU."""
     lib = load()
-    B, T, H, d_k = q.shape
-    d_v = v.shape[-1]
-    if tuple(k.shape) != (B, T, H, d_k) or tuple(v.shape) != (B, T, H, d_v) or tuple(out.shape) != (B, T, H, d_v):
+    B, T, H, d_k, d_v = _sequence_shapes(q, k, v, log_alpha, eta)
+    if tuple(out.shape) != (B, T, H, d_v):
         raise ValueError("q, k, v, out shapes disagree")
-    if tuple(log_alpha.shape) != (B, T, H) or tuple(eta.shape) != (B, T, H):
-        raise ValueError("log_alpha, eta must be [B, T, H]")
     n_seq = B
     if cu_seqlens is not None:
         if host_seqlens is None or host_seqlens.is_cuda or host_seqlens.dtype != torch.int32 or cu_seqlens.dtype != torch.int32:

@@ -128,6 +128,11 @@ kla_status check_chunk_args(const kla_desc *d, const void *q, const void *k, con
                             float eps, int32_t chunk, const float *init_state, void *out, float *final_state, bool check_workspace);
 
 // ---- device helpers -------------------------------------------------------------------------
+__device__ __forceinline__ uint32_t smem_u32(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
+// Byte offset of 16-byte piece `c` (0..7) of row `r` in a tile with 128-byte rows (the layout TMA writes with SWIZZLE_128B and the
+// descriptors of tcgen05.mma read; eight rows of an ldmatrix fall into different banks).
+__device__ __forceinline__ uint32_t sw128(int r, int c) { return (uint32_t)(r * 128 + ((c ^ (r & 7)) << 4)); }
+
 __device__ __forceinline__ float to_f32(float x) { return x; }
 __device__ __forceinline__ float to_f32(__nv_bfloat16 x) { return __bfloat162float(x); }
 

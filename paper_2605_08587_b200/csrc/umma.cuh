@@ -4,10 +4,10 @@
 #include <cuda_bf16.h>
 #include <stdint.h>
 
+#include "common.cuh"
+
 namespace kla {
 namespace umma {
-
-__device__ __forceinline__ uint32_t smem_u32(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
 
 // ---- mbarrier ------------------------------------------------------------------------------------
 __device__ __forceinline__ void mbar_init(uint64_t *bar, uint32_t count)
@@ -323,10 +323,6 @@ __device__ __forceinline__ void split2(float a, float b, uint32_t &hi, uint32_t 
     hi = *reinterpret_cast<uint32_t *>(&h);
     lo = *reinterpret_cast<uint32_t *>(&l);
 }
-
-// Byte offset of 16-byte chunk `c` (0..7) of row `r` in a 128-byte-swizzled tile with 128-byte rows
-// (the layout TMA writes with SWIZZLE_128B and the MMA descriptors above read).
-__device__ __forceinline__ uint32_t sw128(int r, int c) { return (uint32_t)(r * 128 + ((c ^ (r & 7)) << 4)); }
 
 }  // namespace umma
 }  // namespace kla
