@@ -89,12 +89,13 @@ struct PackedPlan {
 };
 
 
-// Time of a launch of the chunk kernel per chunk of a block, in units of a chunk of a block that has its SM to itself (measured: d = 64, B 16, H 16, T 4096, two blocks on an SM 4.5 us a chunk, one 2.75 us).
+// Time of a launch of the chunk kernel per chunk of a block, in units of a chunk of a block that has its SM to itself (measured:
+// d = 64, H 16, T 4096: two blocks on an SM (B 16) 4.58 us a chunk, one (B 8) 2.70 us).
 static double rounds(int d, long long blocks)
 {
     const bool two = d == 64 && blocks > sm_count();
     const int r = two ? 2 * sm_count() : sm_count();
-    return (double)((blocks + r - 1) / r) * (two ? 1.63 : 1.0);
+    return (double)((blocks + r - 1) / r) * (two ? 1.70 : 1.0);
 }
 
 static PackedPlan plan_packed(const kla_desc *d, int32_t chunk)
@@ -116,7 +117,9 @@ static PackedPlan plan_packed(const kla_desc *d, int32_t chunk)
     if (forced >= 2) {
         seg_chunks = (longest + forced - 1) / forced;
     } else {
-        // chunks per SM if the work were spread evenly; a sequence well beyond that sets the length of the launch
+        // chunks per SM if the work were spread evenly; a sequence well beyond that sets the length of the launch (at d = 64, where
+        // two blocks share an SM, it does so from 1.7 times fewer chunks on; the line is drawn as for one block, on the safe side:
+        // pieces cost their warm-up)
         const long long even = total * d->H * (d->d_k / 64) / sm_count();
         const int target = even > 32 ? (int)even : 32;
         if (longest >= target + target / 4 + 8) seg_chunks = target;
@@ -139,8 +142,10 @@ struct SegPlan {
     size_t off_map = 0, off_local = 0, off_start = 0, bytes = 0;   // workspace layout; cu_seg sits at offset 0
 };
 
-// Few long sequences leave most SMs idle (one CTA per sequence x head x slice, each walking its chunks in series).
-// Cutting every sequence into G segments costs about two more passes of state work but runs G times as many CTAs.
+// Few long sequences leave most SMs idle (one block per sequence x head x slice, each walking its chunks in series).
+// Cutting every sequence into G segments runs G times as many blocks.  The rule prices the transition maps, about two more passes of
+// state work: the form that any input can take.  Decaying input takes the warm-up form instead (decided on the device), which costs
+// less; shapes where only that form would pay are not cut, because the decay is not known here.
 static SegPlan plan_segments(const kla_desc *d, int32_t chunk)
 {
     SegPlan pl;
