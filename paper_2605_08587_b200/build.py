@@ -10,7 +10,7 @@ CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libkla_b200.so")
 HOST = os.path.join(HERE, "_host.so")   # native half of the Python binding (csrc/host.cpp)
 SOURCES = ["api.cu", "decode.cu", "chunk_mma.cu", "chunk_wy.cu", "segscan.cu", "static_scratch.cu", "token_scan.cu", "bwd_scan.cu", "bwd_chunk.cu"]
-HEADERS = [os.path.join(CSRC, "common.cuh"), os.path.join(CSRC, "umma.cuh"), os.path.join(CSRC, "chunk_pieces.cuh"), os.path.join(CSRC, "scan_pieces.cuh"), os.path.join(CSRC, "mma_pieces.cuh"), os.path.join(ROOT, "include", "kla.h")]
+HEADERS = [os.path.join(CSRC, "common.cuh"), os.path.join(CSRC, "umma.cuh"), os.path.join(CSRC, "chunk_pieces.cuh"), os.path.join(CSRC, "scan_pieces.cuh"), os.path.join(CSRC, "solve_pieces.cuh"), os.path.join(CSRC, "mma_pieces.cuh"), os.path.join(ROOT, "include", "kla.h")]
 NVCC_FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
               "-Xcompiler", "-fPIC", "-I" + os.path.join(ROOT, "include"), "-I" + CSRC]
 

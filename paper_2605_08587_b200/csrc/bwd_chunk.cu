@@ -32,6 +32,7 @@
 #include "common.cuh"
 #include "mma_pieces.cuh"
 #include "scan_pieces.cuh"
+#include "solve_pieces.cuh"
 
 namespace kla {
 
@@ -40,8 +41,6 @@ namespace {
 using namespace wmm;
 
 constexpr int C = 64;        // chunk length
-constexpr int LDT = 68;      // row stride (floats) of the fp32 solve matrix
-constexpr int LDM = 40;      // row stride of the solve scratch
 constexpr int T_BYTES = 3 * 8192;   // three planes of a 64 x 64 operand
 
 // Per-token scalars of one chunk, as the kernels hand them on.
@@ -120,51 +119,6 @@ __device__ __forceinline__ void load_tile(uint32_t dst, const __nv_bfloat16 *src
 }
 
 // ---- 1. prepare -----------------------------------------------------------------------------------------------------------
-// One level of the blocked inverse of I + B X (see chunk_pieces.cuh): for every pair of adjacent inverted BS x BS diagonal blocks the
-// block below the diagonal becomes T_10 = -T_11 (B_1 X_10 T_00).  256 threads, 1 x 4 results each.
-template <int BS>
-__device__ __forceinline__ void merge_level(float *tl, float *mm, const float *bet, int pt)
-{
-    constexpr int QPR = BS / 4;
-    const bool act = pt < 8 * BS;
-    const int R = pt / QPR, c4 = (pt % QPR) * 4;
-    const int pr = R / BS, r = R % BS;
-    const int rb = (2 * pr + 1) * BS, cb = 2 * pr * BS;
-    if (act) {
-        const float *Ap = tl + (rb + r) * LDT + cb, *Bp = tl + cb * LDT + cb + c4;
-        float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
-#pragma unroll 2
-        for (int k = 0; k < BS; k += 4) {
-            const float4 a = load4(Ap + k);
-            const float av[4] = {a.x, a.y, a.z, a.w};
-#pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                const float4 b = load4(Bp + (k + u) * LDT);
-                acc.x += av[u] * b.x; acc.y += av[u] * b.y; acc.z += av[u] * b.z; acc.w += av[u] * b.w;
-            }
-        }
-        const float s = bet[rb + r];
-        store4(&mm[R * LDM + c4], make_float4(s * acc.x, s * acc.y, s * acc.z, s * acc.w));
-    }
-    __syncthreads();
-    if (act) {
-        const float *Ap = tl + (rb + r) * LDT + rb, *Bp = mm + (pr * BS) * LDM + c4;
-        float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
-#pragma unroll 2
-        for (int k = 0; k <= r; k += 4) {   // T_11 is lower triangular
-            const float4 a = load4(Ap + k);
-            const float av[4] = {a.x, a.y, a.z, a.w};
-#pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                const float4 b = load4(Bp + (k + u) * LDM);
-                acc.x += av[u] * b.x; acc.y += av[u] * b.y; acc.z += av[u] * b.z; acc.w += av[u] * b.w;
-            }
-        }
-        store4(&tl[(rb + r) * LDT + cb + c4], make_float4(-acc.x, -acc.y, -acc.z, -acc.w));
-    }
-    __syncthreads();
-}
-
 template <int D>
 struct PrepSmem {
     union {
@@ -369,9 +323,9 @@ __global__ void __launch_bounds__(256, 3) kla_bwd_prepare_kernel(BwdChunkParams 
     }
     __syncthreads();
     // (a block whose rows all lie past the end of the sequence is zero as it stands)
-    if (rows > 8) merge_level<8>(sm.tl, sm.mm, bet, tid);
-    if (rows > 16) merge_level<16>(sm.tl, sm.mm, bet, tid);
-    if (rows > 32) merge_level<32>(sm.tl, sm.mm, bet, tid);
+    if (rows > 8) merge_level<8, LDM, false>(sm.tl, sm.mm, bet, tid, [] { __syncthreads(); });
+    if (rows > 16) merge_level<16, LDM, false>(sm.tl, sm.mm, bet, tid, [] { __syncthreads(); });
+    if (rows > 32) merge_level<32, LDM, false>(sm.tl, sm.mm, bet, tid, [] { __syncthreads(); });
     // T as three operand planes: 8 columns per item
     unsigned char *tp = p.tpl + ch * T_BYTES;
 #pragma unroll

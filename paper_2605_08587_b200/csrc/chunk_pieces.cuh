@@ -1,11 +1,12 @@
-// Pieces of the WY-form chunk kernel (chunk_wy.cu: two CTAs per head): constants, bounded barrier waits, the decay scan, the
-// blocked inverse of I + B X in shared memory, tile helpers and the host side of the tensor maps.
+// Pieces of the WY-form chunk kernel (chunk_wy.cu: two CTAs per head): constants, bounded barrier waits, the decay scan,
+// tile helpers and the host side of the tensor maps.
 #pragma once
 #include <cuda.h>
 
 #include <mutex>
 
 #include "common.cuh"
+#include "solve_pieces.cuh"
 #include "umma.cuh"
 
 namespace kla {
@@ -23,8 +24,6 @@ constexpr float LOG2E = 1.4426950408889634f;
 // floored weight puts at most 1e-35 of a token into the state instead of less.
 constexpr float DEC_FLOOR_LOG2 = 115.f;
 
-constexpr int LDT = 68;  // row stride (floats) of the fp32 solve matrix
-constexpr int LDM = 40;  // row stride of the solve scratch
 
 // Bounded wait on an mbarrier phase that also leaves when another role has aborted.  Every lane of the
 // calling warp polls: letting one lane poll and broadcasting the result splits the warp, and each later
@@ -89,60 +88,6 @@ __device__ __forceinline__ void quad_transpose(uint32_t (&v)[4], int t)
     x = __shfl_xor_sync(0xffffffffu, x, 2);
     y = __shfl_xor_sync(0xffffffffu, y, 2);
     if (o2) { v[0] = x; v[1] = y; } else { v[2] = x; v[3] = y; }
-}
-
-// One level of the blocked inverse of I + B X (X strictly lower triangular, 64 x 64, in `tl`): for every pair
-// of adjacent BS x BS diagonal blocks (T_00, T_11 already inverted) the block below the diagonal becomes
-//   T_10 = -T_11 (B_1 X_10 T_00).
-// All pairs of the level are done at once by the 256 threads of the pre group: 32 result rows x BS columns,
-// one 1 x 4 tile per thread; `mm` (row stride ldm) holds the intermediate product.  Trip counts are warp-uniform.
-template <int BS>
-__device__ __forceinline__ void merge_level(float *tl, float *mm, int ldm, const float *bet, int pt)
-{
-    constexpr int QPR = BS / 4;                 // column quads per row
-    constexpr int RMASK = 128 / BS - 1;         // a warp covers 128 / BS consecutive rows
-    const bool act = pt < 8 * BS;
-    const int R = pt / QPR, c4 = (pt % QPR) * 4;
-    const int pr = R / BS, r = R % BS;          // pair, row inside the block
-    const int rb = (2 * pr + 1) * BS, cb = 2 * pr * BS;
-    if (act) {
-        // M = B_1 X_10 T_00
-        const float *Ap = tl + (rb + r) * LDT + cb;
-        const float *Bp = tl + cb * LDT + cb + c4;
-        float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
-#pragma unroll 2
-        for (int k = 0; k < BS; k += 4) {
-            const float4 a = *reinterpret_cast<const float4 *>(Ap + k);
-            const float av[4] = {a.x, a.y, a.z, a.w};
-#pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                const float4 b = *reinterpret_cast<const float4 *>(Bp + (k + u) * LDT);
-                acc.x += av[u] * b.x; acc.y += av[u] * b.y; acc.z += av[u] * b.z; acc.w += av[u] * b.w;
-            }
-        }
-        const float s = bet[rb + r];
-        *reinterpret_cast<float4 *>(&mm[R * ldm + c4]) = make_float4(s * acc.x, s * acc.y, s * acc.z, s * acc.w);
-    }
-    pg_sync();
-    if (act) {
-        // T_10 = -T_11 M; T_11 is lower triangular: columns k > r of its row r are zero
-        const float *Ap = tl + (rb + r) * LDT + rb;
-        const float *Bp = mm + (pr * BS) * ldm + c4;
-        const int kend = min(BS, (r | RMASK) + 1);
-        float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
-#pragma unroll 2
-        for (int k = 0; k < kend; k += 4) {
-            const float4 a = *reinterpret_cast<const float4 *>(Ap + k);
-            const float av[4] = {a.x, a.y, a.z, a.w};
-#pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                const float4 b = *reinterpret_cast<const float4 *>(Bp + (k + u) * ldm);
-                acc.x += av[u] * b.x; acc.y += av[u] * b.y; acc.z += av[u] * b.z; acc.w += av[u] * b.w;
-            }
-        }
-        *reinterpret_cast<float4 *>(&tl[(rb + r) * LDT + cb + c4]) = make_float4(-acc.x, -acc.y, -acc.z, -acc.w);
-    }
-    pg_sync();
 }
 
 // Decay scan of one chunk by one warp (lane l holds log alpha of tokens 2l, 2l + 1): log2(e) g_i, gamma_i = exp(g_i),

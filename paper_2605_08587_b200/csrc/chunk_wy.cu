@@ -791,9 +791,9 @@ kla_chunk_wy_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
             // (CUDA-core FMAs: block products on the warp-level tensor instruction, mma.sync with bf16 hi/lo register fragments,
             // were measured too -- they slow every tcgen05 product of the CTA down, 272 -> 420 us when tried in the default
             // kernel, so the two tensor paths are not mixed)
-            merge_level<8>(sm.tl, mm, LDT, bet, pt);
-            merge_level<16>(sm.tl, mm, LDT, bet, pt);
-            merge_level<32>(sm.tl, mm, LDT, bet, pt);
+            merge_level<8, LDT, true>(sm.tl, mm, bet, pt, [] { pg_sync(); });
+            merge_level<16, LDT, true>(sm.tl, mm, bet, pt, [] { pg_sync(); });
+            merge_level<32, LDT, true>(sm.tl, mm, bet, pt, [] { pg_sync(); });
             // ---- T B D_gamma tiles (this CTA only); the W product of this CTA's previous chunk has read the old ones -----------
             bool okd = true;
             if (o > 0 && pt >= PG_T - 32) okd = wait(B_W_DONE, (uint32_t)((o - 1) & 1));
