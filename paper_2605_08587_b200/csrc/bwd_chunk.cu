@@ -23,8 +23,8 @@
 // Precision.  mma.sync truncates its fp32 sums (mma_pieces.cuh), so how often a sum is truncated at its full size decides how exact it is.
 // The products of the first planes, the size of the result, are therefore summed apart from the terms of the lower planes (2^-8 of it
 // and less), in runs of at most eight, and everything else is added in fp32: the states to what a chunk adds to them, the two halves
-// of a long sum, the parts of a gradient.  2-norm errors against fp64, B 8, H 8, T 4096, d 128: dq 1.4e-7, dk 1.5e-7, dv 1.5e-7,
-// dlog_alpha 4e-7, deta 1.9e-7, dinit 1.5e-7, as those of the token-by-token kernel (1.8e-7, 1.9e-7, 1.9e-7, 2.9e-7, 2.0e-7, 1.9e-7);
+// of a long sum, the parts of a gradient.  2-norm errors against fp64, B 8, H 8, T 4096, d 128: dq 1.4e-7, dk 1.5e-7, dv 1.4e-7,
+// dlog_alpha 3.4e-7, deta 1.9e-7, dinit 1.5e-7, as those of the token-by-token kernel (1.8e-7, 1.9e-7, 1.9e-7, 2.9e-7, 2.0e-7, 1.9e-7);
 // with all terms in one accumulator they were 4e-7 .. 1.1e-6.  Cost: 1.50 -> 1.62 ms.
 //
 // beta = 0 (eta = 0) would make U = B (...) carry no trace of the residual e = U / beta that dbeta needs; such a beta is taken

@@ -789,8 +789,8 @@ kla_chunk_wy_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_const
             if (pt < 64) substitute_diag_blocks(sm.tl, bet, pt);
             pg_sync();
             // (CUDA-core FMAs: block products on the warp-level tensor instruction, mma.sync with bf16 hi/lo register fragments,
-            // were measured too -- they slow every tcgen05 product of the CTA down, 272 -> 420 us when tried in the default
-            // kernel, so the two tensor paths are not mixed)
+            // were measured too -- mma.sync stands still while a tcgen05 product runs and slows it down: 382 us for 320.  This kernel keeps
+            // all its products on tcgen05)
             merge_level<8, LDT, true>(sm.tl, mm, bet, pt, [] { pg_sync(); });
             merge_level<16, LDT, true>(sm.tl, mm, bet, pt, [] { pg_sync(); });
             merge_level<32, LDT, true>(sm.tl, mm, bet, pt, [] { pg_sync(); });

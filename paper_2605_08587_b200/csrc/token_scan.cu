@@ -16,8 +16,8 @@
 // quotient), so nothing overflows however strong the decay.  A_4 itself, which the state meets with every block, is applied with its
 // rounding error (expm1 of the sum of log alpha where it is near 1): an error of 2^-25 in a decay near 1 is the same for the whole
 // state and, of one sign as those of expf are, adds up over all that is remembered (log alpha / 100, eta / 10, 4 096 tokens, fp32: final
-// state off by 5.8e-6 of its norm with A_4 as a product of four expf, 4e-7 this way).  What depends on the head only -- the decayed vectors, the
-// triangles, beta -- is prepared once per block of tokens by one warp and read by every warp from shared memory.
+// state off by 5.9e-6 of its norm with A_4 as a product of four expf, 4.7e-7 this way).  What depends on the head only -- the decayed
+// vectors, the triangles, beta -- is prepared once per block of tokens by one warp and read by every warp from shared memory.
 //
 // What bounds it: the fp32 pipe.  A token costs 3.5 d^2 multiply-adds per head (2 d^2 in the sweep, d^2 in the update, half
 // for the decay and its rounding error), fewer than the chunk algebra on the same cores (4 C d + 6 d^2 flops, half as multiply-adds, plus
@@ -30,9 +30,9 @@
 // columns, in registers.  That layout reads every operand as float4 without bank conflicts, pairs adjacent rows into packed
 // fp32 multiply-adds without duplicating an operand, and leaves only three butterfly stages for the sums over rows.
 // CPL: a float4 from shared memory costs four cycles of the load pipe even when it is a broadcast, and feeds 2 CPL packed
-// multiply-adds (four SM cycles at CPL = 4): with CPL = 2 the scan of a layer was bound by those loads (436 wavefronts per
-// token, load pipe 75 % busy, 1.40 ms; with CPL = 4 and both sweeps in one loop 1.00 ms (1.06 with the decay's rounding error), bound by the latency of one scanning
-// warp per scheduler, fp32 pipe 53 % busy).  CPL = 2 stays where there are too few (sequence, head) pairs to give every SM more than
+// multiply-adds (four SM cycles at CPL = 4): with CPL = 2 the scan of a layer was bound by those loads (1.40 ms; with
+// CPL = 4 and both sweeps in one loop 1.00 ms, 1.06 with the decay's rounding error, bound by the latency of one scanning warp per
+// scheduler: fp32 pipe 56 % busy, load pipe 25 %, schedulers 50 %).  CPL = 2 stays where there are too few (sequence, head) pairs to give every SM more than
 // two warps of 16 columns: twice the warps then halve the latency.
 #include "common.cuh"
 #include "scan_pieces.cuh"
