@@ -22,8 +22,10 @@
 // the schedulers' instruction caches and issues at about one instruction in three cycles (measured on unrolled against rolled
 // copies of the same products).  With all products on mma.sync (504 per chunk and warp at d = 128 instead of 248) a chunk took
 // 8 000 cycles; with all of them on tcgen05, whose every product on the chain ends in a hand-over through tensor memory and shared
-// memory, 7 400; this way 5 900 (2.99 us, B 8, H 8, d 128, between T 4096 and 8192).  mma.sync stands still while a tcgen05 product runs, so the two add up: 570 cycles for the state
-// product, 400 for [K; Q] K^T, 8 per mma.sync.
+// memory, 7 400; this way 5 400 (2.85 us, B 8, H 8, d 128, T 4096).  mma.sync stands still while a tcgen05 product
+// runs, so the two add up: 400 cycles for [K; Q] K^T, 8 per mma.sync.  [S_hi; S_lo]^T is a left operand in tensor memory: from shared
+// memory the state product was bound by the fetch of both operands (8 KB for each 32 cycles of products: 570 cycles), and its
+// operand took a proxy fence (headline shape 200.6 -> 194.7 us, 32 packed sequences at d 64 487 -> 472).
 //
 // Precision.  q, k, v are exact bf16 operands.  Every derived operand (S, Y, X, N, P, U) is a pair of bf16 values hi + lo (16
 // significand bits; one bf16 rounding of any of them costs 1e-2..7e-2 in max|err|/rms, above the 2e-3 bound), a product of two
@@ -70,8 +72,13 @@ constexpr float LOG2E = 1.4426950408889634f;
 constexpr float DEC_FLOOR_LOG2 = 115.f;
 constexpr float HOT_BETA = 4096.f;   // q k beta up to ||q|| sqrt(beta) = 64 ||q||: 2^-18 of that is below the other errors
 constexpr int LDB = 20;       // row stride (floats) of a 16 x 16 block in the solve scratch
-// TMEM columns: [S_hi; S_lo]^T [K; Q]^T (128), [K; Q] K^T (64), the state in fp32 (D / 2)
-constexpr uint32_t TM_X = 0, TM_G = 128, TM_S = 192, TM_COLS = 256;
+// TMEM columns: [S_hi; S_lo]^T [K; Q]^T (128), [K; Q] K^T (64), the state in fp32 (D / 2), [S_hi; S_lo]^T as left operand (D / 2):
+// warp w: lanes 32 w .. the hi, 32 w + 16 .. the lo parts of its columns of d_v, a column for two of d_k.
+constexpr uint32_t TM_X = 0, TM_G = 128, TM_S = 192;
+template <int D>
+constexpr uint32_t TM_A = TM_S + D / 2;
+template <int D>
+constexpr uint32_t TM_COLS = D == 64 ? 256 : 512;
 
 // Lower triangle of 16 x 16 blocks, in fragment order: the four registers of a right operand, 16 bytes per lane.
 __device__ __forceinline__ constexpr int blk(int i, int j) { return i * (i + 1) / 2 + j; }
@@ -118,8 +125,6 @@ template <int D, int BPS>
 struct Smem {
     static constexpr int NSLOT = BPS == 1 ? 3 : 2;
     Slot<D> slot[NSLOT];
-    // S^T as left operand, per 64 of d_k: 128 rows of 128 bytes; warp w: rows 32 w .. the hi, 32 w + 16 .. the lo parts of its columns
-    alignas(1024) unsigned char st[D / 64 * 16384];
     Scalars scal[NSLOT];
     PrepScratch prep[2];
     float g2[4][C];              // log2(e) g_i, a copy for each prepare warp
@@ -204,6 +209,12 @@ __device__ __forceinline__ void tmem_kept(uint32_t addr, float2 (&x)[4][2])
                  "tcgen05.wait::ld.sync.aligned;" : R8("=f", x, 0), R8("=f", x, 2) : "r"(addr) : "memory");
 }
 #undef R8
+// Two left operands side by side (16 rows, 32 of the contraction) in sixteen TMEM columns of sixteen lanes.
+__device__ __forceinline__ void tmem_left(uint32_t addr, const uint32_t (&a)[2][4])
+{
+    asm volatile("tcgen05.st.sync.aligned.16x128b.x4.b32 [%8], {%0, %1, %2, %3, %4, %5, %6, %7};"
+                 ::"r"(a[0][0]), "r"(a[0][1]), "r"(a[0][2]), "r"(a[0][3]), "r"(a[1][0]), "r"(a[1][1]), "r"(a[1][2]), "r"(a[1][3]), "r"(addr) : "memory");
+}
 // 16 TMEM lanes x 16 columns as two accumulator tiles side by side.
 __device__ __forceinline__ void tmem_block(uint32_t addr, float2 (&x)[2], float2 (&y)[2])
 {
@@ -598,38 +609,34 @@ __device__ void chain(const ChunkParams &p, Smem<D, BPS> &sm, const Work &wk, in
                               : make_float2(wk.ident && r == cc ? 1.f : 0.f, wk.ident && r + 1 == cc ? 1.f : 0.f);
         }
     const uint32_t tx = sm.tmem + TM_X + ((uint32_t)(32 * w) << 16);
-    // per-lane parts of the tile addresses: rows of S^T written by stmatrix; right operands K (16 tokens x 16 of d_k); V
-    const int sr = 32 * w + (lane & 15), sp = lane >> 4;
-    const uint32_t st0 = smem_u32(sm.st) + sr * 128;
-    uint32_t stx[4], ktx[4];
+    // per-lane parts of the tile addresses: right operands K (16 tokens x 16 of d_k); V
+    uint32_t ktx[4];
 #pragma unroll
-    for (int u = 0; u < 4; ++u) {
-        stx[u] = (uint32_t)((2 * u + sp) ^ (sr & 7)) << 4;
-        ktx[u] = sw128(lane & 15, 2 * u + (lane >> 4));
-    }
+    for (int u = 0; u < 4; ++u) ktx[u] = sw128(lane & 15, 2 * u + (lane >> 4));
     const uint32_t vtx = sw128((lane & 7) + (lane >> 4) * 8, 2 * w + ((lane >> 3) & 1));
 
-    auto store_state = [&](int ks) {   // rows 16 ks .. of d_k
-        uint32_t h[4], l[4];
+    const uint32_t ta = sm.tmem + TM_A<D> + ((uint32_t)(32 * w) << 16);
+    auto store_state = [&](int q) {   // rows 32 q .. of d_k
+        uint32_t h[2][4], l[2][4];
 #pragma unroll
-        for (int u = 0; u < 4; ++u) split_left(S[2 * ks], S[2 * ks + 1], u, h, l);
-        const uint32_t a = st0 + (ks >> 2) * 16384 + stx[ks & 3];
-        asm volatile("stmatrix.sync.aligned.m8n8.x4.shared.b16 [%0], {%1, %2, %3, %4};" ::"r"(a), "r"(h[0]), "r"(h[1]), "r"(h[2]), "r"(h[3]) : "memory");
-        asm volatile("stmatrix.sync.aligned.m8n8.x4.shared.b16 [%0], {%1, %2, %3, %4};" ::"r"(a + 2048), "r"(l[0]), "r"(l[1]), "r"(l[2]), "r"(l[3]) : "memory");
+        for (int v = 0; v < 2; ++v)
+#pragma unroll
+            for (int u = 0; u < 4; ++u) split_left(S[4 * q + 2 * v], S[4 * q + 2 * v + 1], u, h[v], l[v]);
+        tmem_left(ta + 16 * q, h);
+        tmem_left(ta + 16 * q + (16u << 16), l);
     };
     // d = 128: the product over the first 64 rows of d_k starts while the others are being finished (-1.5 %)
     auto state_written = [&](int part) {
-        fence_async_smem();
+        asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
         tc_fence_before();
         __syncwarp();
         if (lane == 0) mbar_arrive(&sm.bar[part ? B_STATE1 : B_STATE]);
     };
 #pragma unroll
-    for (int ks = 0; ks < KS; ++ks) store_state(ks);
+    for (int q = 0; q < KS / 2; ++q) store_state(q);
     const uint32_t ts = sm.tmem + TM_S + ((uint32_t)(32 * w) << 16);
 #pragma unroll
     for (int ks = 0; ks < KS; ks += 2) tmem_keep(ts + 8 * ks, &S[2 * ks]);
-    asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
     if (D == 128) state_written(1);
     state_written(0);
 
@@ -813,8 +820,7 @@ __device__ void chain(const ChunkParams &p, Smem<D, BPS> &sm, const Work &wk, in
 #pragma unroll
                 for (int e = 0; e < 2; ++e) S[4 * q + t][e] = fma2(gC, kept[t][e], S[4 * q + t][e]);
             tmem_keep(ts + 16 * q, &S[4 * q]);
-            store_state(2 * q);
-            store_state(2 * q + 1);
+            store_state(q);
         };
 #pragma unroll
         for (int q = 0; q < QJ; ++q)
@@ -823,7 +829,6 @@ __device__ void chain(const ChunkParams &p, Smem<D, BPS> &sm, const Work &wk, in
                 if (D == 128 && q == QJ / 2 && c + 1 < nchunks) state_written(0);
             });
         finish(QJ - 1);
-        asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
         if (c + 1 < nchunks) state_written(D == 128);
         if constexpr (HAS_OUT) {
             const int live = c >= wk.first_out ? rows : 0;
@@ -917,11 +922,11 @@ __device__ void issue(const CUtensorMap *tm_q, const CUtensorMap *tm_k, const CU
     gram(0);
     for (int c = 0; c < nchunks; ++c) {
         if (!wait(B_STATE, c)) return;
-        const uint32_t a = desc_lo(smem_desc_sw128(smem_u32(sm.st), 0, 1024)), b = desc_lo(smem_desc_sw128(smem_u32(sm.slot[c % NSLOT].kq), 0, 1024));
+        const uint32_t b = desc_lo(smem_desc_sw128(smem_u32(sm.slot[c % NSLOT].kq), 0, 1024));
 #pragma unroll
         for (int kb = 0; kb < NB; ++kb) {
             if (kb == 1 && !wait(B_STATE1, c)) return;
-            mma4_bf16_lo<2, 2>(sm.tmem + TM_X, a + kb * 1024, b + kb * 1024, idesc_bf16(128, HAS_OUT ? 128 : 64, 0, 0), kb > 0);
+            mma4_bf16_ta<2>(sm.tmem + TM_X, sm.tmem + TM_A<D> + kb * 32, b + kb * 1024, idesc_bf16(128, HAS_OUT ? 128 : 64, 0, 0), kb > 0);
         }
         mma_commit(&sm.bar[B_X]);
         auto next_gram = [&]() {
@@ -979,7 +984,7 @@ kla_chunk_mma_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_cons
         tma_prefetch_desc(&tm_k);
         tma_prefetch_desc(&tm_v);
     }
-    if (tid < 32) tmem_alloc(&sm.tmem, TM_COLS);
+    if (tid < 32) tmem_alloc(&sm.tmem, TM_COLS<D>);
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
@@ -1005,7 +1010,7 @@ kla_chunk_mma_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_cons
     }
     if (tid < 32) {
         tc_fence_after();
-        tmem_dealloc(sm.tmem, TM_COLS);
+        tmem_dealloc(sm.tmem, TM_COLS<D>);
     }
 }
 

@@ -206,6 +206,27 @@ __device__ __forceinline__ void mma4_bf16_lo(uint32_t tmem_d, uint32_t a_lo, uin
         ::"r"(tmem_d), "r"(a_lo), "r"(b_lo), "r"(idesc), "r"(accumulate), "n"(DESC_HI_SW128_SBO1024), "n"(ASTEP), "n"(BSTEP)
         : "memory");
 }
+// The same with A in tensor memory (row = lane, eight columns of packed pairs per k step): B alone is fetched from shared memory.
+template <uint32_t BSTEP>
+__device__ __forceinline__ void mma4_bf16_ta(uint32_t tmem_d, uint32_t tmem_a, uint32_t b_lo, uint32_t idesc, uint32_t accumulate)
+{
+    asm volatile(
+        "{\n\t.reg .pred p, e;\n\t.reg .b64 db;\n\t.reg .b32 ra, rb;\n\t"
+        "setp.ne.b32 p, %4, 0;\n\t"
+        "elect.sync _|e, 0xffffffff;\n\t"
+        "@!e bra MMA4TA_DONE;\n\t"
+        "mov.b64 db, {%2, %5};\n\t"
+        "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], db, %3, p;\n\t"
+        "add.u32 ra, %1, 8;\n\tadd.u32 rb, %2, %6;\n\tmov.b64 db, {rb, %5};\n\t"
+        "tcgen05.mma.cta_group::1.kind::f16 [%0], [ra], db, %3, 1;\n\t"
+        "add.u32 ra, ra, 8;\n\tadd.u32 rb, rb, %6;\n\tmov.b64 db, {rb, %5};\n\t"
+        "tcgen05.mma.cta_group::1.kind::f16 [%0], [ra], db, %3, 1;\n\t"
+        "add.u32 ra, ra, 8;\n\tadd.u32 rb, rb, %6;\n\tmov.b64 db, {rb, %5};\n\t"
+        "tcgen05.mma.cta_group::1.kind::f16 [%0], [ra], db, %3, 1;\n\t"
+        "MMA4TA_DONE:\n\t}"
+        ::"r"(tmem_d), "r"(tmem_a), "r"(b_lo), "r"(idesc), "r"(accumulate), "n"(DESC_HI_SW128_SBO1024), "n"(BSTEP)
+        : "memory");
+}
 // Arrive on an mbarrier once all MMAs issued so far by this warp's elected lane have completed
 // (same calling convention: converged warp, one elected lane issues).
 __device__ __forceinline__ void mma_commit(uint64_t *bar)
