@@ -22,10 +22,13 @@
 // the schedulers' instruction caches and issues at about one instruction in three cycles (measured on unrolled against rolled
 // copies of the same products).  With all products on mma.sync (504 per chunk and warp at d = 128 instead of 248) a chunk took
 // 8 000 cycles; with all of them on tcgen05, whose every product on the chain ends in a hand-over through tensor memory and shared
-// memory, 7 400; this way 5 400 (2.85 us, B 8, H 8, d 128, T 4096).  mma.sync stands still while a tcgen05 product
+// memory, 7 400; this way 5 200 (2.75 us, B 8, H 8, d 128, T 4096).  mma.sync stands still while a tcgen05 product
 // runs, so the two add up: 400 cycles for [K; Q] K^T, 8 per mma.sync.  [S_hi; S_lo]^T is a left operand in tensor memory: from shared
 // memory the state product was bound by the fetch of both operands (8 KB for each 32 cycles of products: 570 cycles), and its
-// operand took a proxy fence (headline shape 200.6 -> 194.7 us, 32 packed sequences at d 64 487 -> 472).
+// operand took a proxy fence (headline shape 200.6 -> 194.7 us, 32 packed sequences at d 64 487 -> 472).  The outputs are transposed through
+// a buffer that TMA never touches: in the V tile they took such a fence too, in which the warp stood (194.7 -> 188, 472 -> 462).
+// The outputs on four warps of their own cost more than they took off the chain: 246 us against 201 (82 KB of code instead of 70,
+// fetched by all SMs at once, and the Gram product then falls into the block solve).
 //
 // Precision.  q, k, v are exact bf16 operands.  Every derived operand (S, Y, X, N, P, U) is a pair of bf16 values hi + lo (16
 // significand bits; one bf16 rounding of any of them costs 1e-2..7e-2 in max|err|/rms, above the 2e-3 bound), a product of two
@@ -91,7 +94,7 @@ struct Slot {
     static constexpr int NB = D / 64;
     // per 64 columns: 64 tokens of K, then 64 of Q, rows of 128 bytes, 128-byte swizzle
     alignas(1024) unsigned char kq[NB * 16384];
-    alignas(1024) unsigned char v[8192];        // this block's 64 columns; then the outputs on their way out
+    alignas(1024) unsigned char v[8192];        // this block's 64 columns
     TriOperand t, p;                            // D N_ii B and below them -X D^-1; P D^-1 (rows over ||q|| with the normalised read-out)
 };
 struct alignas(16) Scalars {     // of one chunk
@@ -126,6 +129,7 @@ struct Smem {
     static constexpr int NSLOT = BPS == 1 ? 3 : 2;
     Slot<D> slot[NSLOT];
     Scalars scal[NSLOT];
+    alignas(16) unsigned char outb[4][C * 32];   // a chain warp's 16 columns of the outputs (bf16) on their way out
     PrepScratch prep[2];
     float g2[4][C];              // log2(e) g_i, a copy for each prepare warp
     float qinv[C];
@@ -613,6 +617,7 @@ __device__ void chain(const ChunkParams &p, Smem<D, BPS> &sm, const Work &wk, in
     uint32_t ktx[4];
 #pragma unroll
     for (int u = 0; u < 4; ++u) ktx[u] = sw128(lane & 15, 2 * u + (lane >> 4));
+    const uint32_t ob = smem_u32(sm.outb[w]) + ((lane & 7) + (lane >> 4) * 8) * 32 + ((((lane >> 3) & 1) ^ ((lane >> 2) & 1)) << 4);
     const uint32_t vtx = sw128((lane & 7) + (lane >> 4) * 8, 2 * w + ((lane >> 3) & 1));
 
     const uint32_t ta = sm.tmem + TM_A<D> + ((uint32_t)(32 * w) << 16);
@@ -830,6 +835,8 @@ __device__ void chain(const ChunkParams &p, Smem<D, BPS> &sm, const Work &wk, in
             });
         finish(QJ - 1);
         if (c + 1 < nchunks) state_written(D == 128);
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&sm.bar[B_DONE + s]);
         if constexpr (HAS_OUT) {
             const int live = c >= wk.first_out ? rows : 0;
             if constexpr (std::is_same<OUT, float>::value) {
@@ -842,7 +849,8 @@ __device__ void chain(const ChunkParams &p, Smem<D, BPS> &sm, const Work &wk, in
                         if (8 * t + t2 + 1 < live) d[tok_stride] = o[t][e].y;
                     }
             } else {
-                // transposed through the warp's own columns of the V tile, so that a store is 16 bytes of one token
+                // transposed through shared memory, so that a store is 16 bytes of one token (a buffer of its own: in a tile that
+                // TMA refills it takes a proxy fence, on which the warp then stands)
 #pragma unroll
                 for (int t = 0; t < 8; t += 2) {
                     uint32_t r[4];
@@ -852,24 +860,21 @@ __device__ void chain(const ChunkParams &p, Smem<D, BPS> &sm, const Work &wk, in
                         r[u] = *reinterpret_cast<const uint32_t *>(&hh);
                     }
                     asm volatile("stmatrix.sync.aligned.m8n8.x4.trans.shared.b16 [%0], {%1, %2, %3, %4};"
-                                 ::"r"(vt + t * 1024), "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]) : "memory");
+                                 ::"r"(ob + t * 256), "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]) : "memory");
                 }
                 __syncwarp();
                 const int r0 = lane >> 1, ch = lane & 1;
-                const unsigned char *src = sl.v + sw128(r0, 2 * w + ch);
+                const unsigned char *src = sm.outb[w] + r0 * 32 + ((ch ^ ((r0 >> 2) & 1)) << 4);
                 Elem *d = out + r0 * tok_stride + ch * 8;
                 uint4 r[4];
 #pragma unroll
-                for (int e = 0; e < 4; ++e) r[e] = *reinterpret_cast<const uint4 *>(src + e * 2048);
+                for (int e = 0; e < 4; ++e) r[e] = *reinterpret_cast<const uint4 *>(src + e * 512);
 #pragma unroll
                 for (int e = 0; e < 4; ++e)
                     if (16 * e + r0 < live) *reinterpret_cast<uint4 *>(d + 16 * e * tok_stride) = r[e];
-                fence_async_smem();   // (the slot is refilled by TMA)
             }
             out += C * tok_stride;
         }
-        __syncwarp();
-        if (lane == 0) mbar_arrive(&sm.bar[B_DONE + s]);
     }
     if (wk.fin && !sm.abort_flag) {
 #pragma unroll
