@@ -672,8 +672,36 @@ struct GradSmem {
     float red[4][64];                             // dg_i, the parts of the four column groups of the warps
 };
 
+// Asks for what block `b` of the gradients reads to be brought into L2; nothing is waited for.
 template <int D>
-__global__ void __launch_bounds__(GT, 1) kla_bwd_grad_kernel(BwdChunkParams p)
+__device__ __forceinline__ void prefetch_block(const BwdChunkParams &p, int b, int tid)
+{
+    const int slot = b / p.H, h = b % p.H;
+    const Where w = locate(p, slot);
+    if (w.c * C >= w.len) return;
+    const int rows = min(C, w.len - w.c * C);
+    const size_t t0 = (size_t)w.tok0 + w.c * C, ch = (size_t)slot * p.H + h;
+    if (tid == 0) {
+        auto bulk = [](const void *x, int bytes) { asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(x), "r"(bytes) : "memory"); };
+        bulk(p.u + ch * C * D, C * D * 4);
+        bulk(p.s0 + ch * D * D, D * D * 4);
+        bulk(p.g1 + ch * D * D, D * D * 4);
+    }
+    auto line = [](const void *x) { asm volatile("prefetch.global.L2 [%0];" ::"l"(x)); };
+    constexpr int LF = D / 32, LB = D / 64;   // 128-byte lines of a row of floats, of bf16
+    for (int e = tid; e < rows * (LF + 3 * LB); e += GT) {
+        const int r = e / (LF + 3 * LB), i = e % (LF + 3 * LB);
+        const size_t row = ((t0 + r) * p.H + h) * D;
+        if (i < LF) line(p.dv + row + 32 * i);
+        else {
+            const int a = (i - LF) / LB, o = 64 * ((i - LF) % LB);
+            line((a == 0 ? p.dout : a == 1 ? p.k : p.q) + row + o);
+        }
+    }
+}
+
+template <int D>
+__global__ void __launch_bounds__(GT, 1) kla_bwd_grad_kernel(BwdChunkParams p, int ahead)
 {
     constexpr int NB = D / 64, IT = D * 8 / GT;   // 8-column items of a [D][64] fp32 matrix per thread
     constexpr int UI = C * D / 8 / GT;            // 8-column items of a [64][D] matrix per thread
@@ -733,6 +761,7 @@ __global__ void __launch_bounds__(GT, 1) kla_bwd_grad_kernel(BwdChunkParams p)
             a[i][3] = load4(y + 4);
         }
         fetch(ps, p.s0, 0);
+        if ((int)blockIdx.x + ahead < (int)gridDim.x) prefetch_block<D>(p, blockIdx.x + ahead, tid);
         cp_wait<0>();
         __syncthreads();   // scalars (and dO) are there
 #pragma unroll
@@ -1114,7 +1143,7 @@ cudaError_t launch_d(const BwdChunkParams &p, cudaStream_t stream)
     if (units == 0) return cudaSuccess;
     if (p.n_slots > 0) kla_bwd_prepare_kernel<D><<<p.n_slots * p.H, 256, smem1, stream>>>(p);
     kla_bwd_chain_kernel<D><<<2 * units, 128, smem2, stream>>>(p, units);   // (empty sequences: dinit)
-    if (p.n_slots > 0) kla_bwd_grad_kernel<D><<<p.n_slots * p.H, GT, smem3, stream>>>(p);
+    if (p.n_slots > 0) kla_bwd_grad_kernel<D><<<p.n_slots * p.H, GT, smem3, stream>>>(p, sm_count());
     count_launch(p.n_slots > 0 ? 3 : 1);
     return cudaGetLastError();
 }
