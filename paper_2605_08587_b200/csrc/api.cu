@@ -592,6 +592,7 @@ kla_status kla_bwd(const kla_desc *desc, const void *q, const void *k, const voi
     a.eps = eps;
     a.coeff_eta = (desc->flags & KLA_FLAG_COEFF_ETA) ? 1 : 0;
     a.qnorm = (desc->flags & KLA_FLAG_QNORM) ? 1 : 0;
+    a.status_word = desc->status_word;
     const cudaError_t err = desc->io_dtype == KLA_BF16 ? launch_bwd_chunk(a, stream) : launch_bwd_scan(a, stream);
     return err == cudaSuccess ? KLA_OK : KLA_ERR_LAUNCH;
 }

@@ -29,10 +29,13 @@
 //
 // beta = 0 (eta = 0) would make U = B (...) carry no trace of the residual e = U / beta that dbeta needs; such a beta is taken
 // as 1e-30, where every gradient has its limit to the last bit.
+#include <cuda.h>
+
 #include "common.cuh"
 #include "mma_pieces.cuh"
 #include "scan_pieces.cuh"
 #include "solve_pieces.cuh"
+#include "umma.cuh"
 
 namespace kla {
 
@@ -66,11 +69,17 @@ struct BwdChunkParams {
     int32_t coeff_eta, qnorm;
     // workspace, one entry per (slot, head); a slot is a chunk: n ceil(T / 64) + c, packed tok0 / 64 + n + c
     unsigned char *tpl;   // T as three operand planes, 64 x 64 each, sw128 layout
-    float *pdo;           // (P^T dO)^T  [D][64]
+    // As accumulator tiles: 16 rows x 8 columns, a lane's four values side by side, so that a warp writes and reads 512 bytes in a row
+    // (row by row, 8 lines to an instruction, the chains stood in their stores: 2 000 - 3 000 cycles of a chunk's 12 000 - 17 000)
+    float *pdo;           // (P^T dO)^T  [D / 16][8] tiles
+    float *s0, *g1;       // S_0^T, G_1^T  [d_v / 16][d_k / 8] tiles
     float *u;             // U           [64][D]
-    float *s0, *g1;       // S_0^T, G_1^T  [d_v][d_k]
     Scal *scal;
     int32_t n_slots;
+    int32_t *status_word;
+};
+struct TileMaps {
+    CUtensorMap q, k, v, dout;   // 64 tokens x 64 columns
 };
 
 struct Where {
@@ -293,12 +302,9 @@ __global__ void __launch_bounds__(256, 3) kla_bwd_prepare_kernel(BwdChunkParams 
                     mma(o[2 * np + 1], a, b[2], b[3]);
                 }
             }
-        float *dst = p.pdo + ch * D * C + (size_t)(warp * 16 + (lane >> 2)) * C + cq;
+        float *dst = p.pdo + ch * D * C + warp * 16 * C + lane * 4;
 #pragma unroll
-        for (int t = 0; t < 8; ++t) {
-            store2(dst + 8 * t, o[t][0], o[t][1]);
-            store2(dst + 8 * C + 8 * t, o[t][2], o[t][3]);
-        }
+        for (int t = 0; t < 8; ++t) store4(dst + 128 * t, make_float4(o[t][0], o[t][1], o[t][2], o[t][3]));
     }
 
     // T = (I + B X)^-1: 8 x 8 diagonal blocks by substitution (column tid % 8 of block tid / 8), then block merges
@@ -344,7 +350,9 @@ __global__ void __launch_bounds__(256, 3) kla_bwd_prepare_kernel(BwdChunkParams 
 // ---- 2. chains ------------------------------------------------------------------------------------------------------------
 // Four warps, 16 columns of d_v each; the transposed state (16 x D) stays in registers as accumulator tiles, is split into
 // operand planes on the fly and never leaves the warp.  K is fetched a chunk ahead into the other of two buffers; what a chunk
-// uses last (T, V, respectively T, Q, dO) has one buffer and is fetched as soon as every warp has passed it.
+// uses last (T, V, respectively T, Q, dO) has one buffer and is fetched as soon as every warp has passed it.  One thread fetches
+// by TMA: as asynchronous copies of 16 bytes the 33 of a thread and chunk, a dozen instructions each that run once and come from
+// beyond the instruction caches, took 2 900 (backward) and 1 200 (forward) cycles of a chunk's 16 300 and 13 000.
 // What bounds it: the warp-level tensor pipe, 504 (forward) and 696 (backward) instructions per chunk and warp at D = 128.
 // Both directions are one launch so that an SM holds a block of each and one fills the other's latencies.
 template <int D>
@@ -354,7 +362,20 @@ struct ChainSmem {
     alignas(1024) unsigned char vd[8192];            // V (forward), dO (backward): this block's 64 columns
     alignas(1024) unsigned char q[D / 64 * 8192];    // backward only
     Scal s[2];
+    alignas(8) uint64_t bar[2];                      // K, scalars, T (and V) of a chunk; Q and dO of it
 };
+constexpr long long CHAIN_WAIT_LIMIT = 2000000000LL;   // SM clocks (~1 s) before a wait gives up
+
+// Rows from `rows` on of NB 64 x 64 tiles, which hold what follows the sequence, become zero.
+template <int NB>
+__device__ __forceinline__ void zero_rows(unsigned char *tile, int rows, int tid)
+{
+#pragma unroll 1
+    for (int e = tid; e < (C - rows) * 8 * NB; e += 128) {
+        const int r = rows + e / (8 * NB), ch = e % (8 * NB);
+        *reinterpret_cast<uint4 *>(tile + (ch >> 3) * 8192 + sw128(r, ch & 7)) = make_uint4(0, 0, 0, 0);
+    }
+}
 
 // acc[token tile] = (16 x D state) (64 x D tile)^T: columns are tokens.  `late`: called before the last products
 template <int D, typename F>
@@ -423,7 +444,7 @@ __device__ __forceinline__ void mma5(float (&c0)[4], float (&c1)[4], const uint3
 }
 
 template <int D, bool BWD>
-__device__ __forceinline__ void chain(const BwdChunkParams &p, ChainSmem<D> &sm, int unit)
+__device__ __forceinline__ void chain(const BwdChunkParams &p, const TileMaps &tm, ChainSmem<D> &sm, int unit)
 {
     constexpr int NB = D / 64;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -453,68 +474,76 @@ __device__ __forceinline__ void chain(const BwdChunkParams &p, ChainSmem<D> &sm,
     }
     const size_t ch0 = (size_t)slot_of(p, n, tok0, 0) * p.H + h;   // chunk c: + c H
     auto rows_of = [&](int c) { return min(C, len - c * C); };
+    // (one thread)
     auto load_k = [&](int c) {
-        load_tile<NB, D, 128>(smem_u32(sm.k[c & 1]), p.k, (size_t)tok0 + c * C, rows_of(c), p.H, h, 0, tid);
-        cp16(smem_u32(&sm.s[c & 1]) + tid * 16, reinterpret_cast<const char *>(p.scal + ch0 + (size_t)c * p.H) + tid * 16, true);
-    };
-    auto load_t = [&](int c) {
-        const unsigned char *src = p.tpl + (ch0 + (size_t)c * p.H) * T_BYTES;
+        umma::mbar_expect_tx(&sm.bar[0], NB * 8192 + sizeof(Scal) + T_BYTES + (BWD ? 0 : 8192));
 #pragma unroll
-        for (int e = tid; e < T_BYTES / 16; e += 128) cp16(smem_u32(sm.t) + e * 16, src + e * 16, true);
+        for (int b = 0; b < NB; ++b) umma::tma_load_2d(sm.k[c & 1] + b * 8192, &tm.k, h * D + b * 64, tok0 + c * C, &sm.bar[0]);
+        umma::bulk_load(&sm.s[c & 1], p.scal + ch0 + (size_t)c * p.H, sizeof(Scal), &sm.bar[0]);
     };
-    auto load_vd = [&](int c) {
-        load_tile<1, D, 128>(smem_u32(sm.vd), BWD ? p.dout : p.v, (size_t)tok0 + c * C, rows_of(c), p.H, h, sl * 64, tid);
+    auto load_t = [&](int c) {   // counted with K
+        umma::bulk_load(sm.t, p.tpl + (ch0 + (size_t)c * p.H) * T_BYTES, T_BYTES, &sm.bar[0]);
+        if (!BWD) umma::tma_load_2d(sm.vd, &tm.v, h * D + sl * 64, tok0 + c * C, &sm.bar[0]);
     };
+    auto load_q = [&](int c) {
+        umma::mbar_expect_tx(&sm.bar[1], (NB + 1) * 8192);
+        umma::tma_load_2d(sm.vd, &tm.dout, h * D + sl * 64, tok0 + c * C, &sm.bar[1]);
+#pragma unroll
+        for (int b = 0; b < NB; ++b) umma::tma_load_2d(sm.q + b * 8192, &tm.q, h * D + b * 64, tok0 + c * C, &sm.bar[1]);
+    };
+    if (tid == 0) {
+        umma::mbar_init(&sm.bar[0], 1);
+        umma::mbar_init(&sm.bar[1], 1);
+        umma::mbar_fence_init();
+    }
+    __syncthreads();
+    bool late = false;   // a wait ran out (for the whole block)
     const int step = BWD ? -1 : 1;
     int c = BWD ? nc - 1 : 0;
-    if (nc > 0) {
+    if (nc > 0 && tid == 0) {
         load_k(c);
         load_t(c);
-        if (!BWD) load_vd(c);
-        cp_commit();
     }
     for (int it = 0; it < nc; ++it, c += step) {
         const Scal &s = sm.s[c & 1];
         const size_t ch = ch0 + (size_t)c * p.H;
         const uint32_t kt = smem_u32(sm.k[c & 1]), tt = smem_u32(sm.t);
-        cp_wait<0>();
-        __syncthreads();
-        if (BWD) {
-            load_vd(c);
-            load_tile<NB, D, 128>(smem_u32(sm.q), p.q, (size_t)tok0 + c * C, rows_of(c), p.H, h, 0, tid);
-            cp_commit();
+        const int rows = rows_of(c);
+        late = __syncthreads_or(!umma::mbar_wait(&sm.bar[0], it & 1, CHAIN_WAIT_LIMIT));
+        if (late) break;
+        if (rows < C) {
+            zero_rows<NB>(sm.k[c & 1], rows, tid);
+            if (!BWD) zero_rows<1>(sm.vd, rows, tid);
+            umma::fence_async_smem();
+            __syncthreads();
         }
-        if (it + 1 < nc) load_k(c + step);
-        cp_commit();
+        if (tid == 0) {
+            if (BWD) load_q(c);
+            if (it + 1 < nc) load_k(c + step);
+        }
         // the state at this end of the chunk, transposed
         {
-            float *dst = (BWD ? p.g1 : p.s0) + ch * D * D + (size_t)col * D + cq;
+            float *dst = (BWD ? p.g1 : p.s0) + ch * D * D + (sl * 4 + warp) * 16 * D + lane * 4;
 #pragma unroll
-            for (int t = 0; t < D / 8; ++t) {
-                store2(dst + 8 * t, S[t][0], S[t][1]);
-                store2(dst + 8 * D + 8 * t, S[t][2], S[t][3]);
-            }
+            for (int t = 0; t < D / 8; ++t) store4(dst + 128 * t, make_float4(S[t][0], S[t][1], S[t][2], S[t][3]));
         }
-        float2 pd[BWD ? 8 : 1][2];
+        float4 pd[BWD ? 8 : 1];
         float x[8][4], y[8][4];
         state_times_tile<D>(x, S, kt, lane, [&] {   // (K S_0)^T or (K G_1)^T
             if constexpr (BWD) {
-                const float *src = p.pdo + ch * D * C + (size_t)col * C + cq;
+                const float *src = p.pdo + ch * D * C + (sl * 4 + warp) * 16 * C + lane * 4;
 #pragma unroll
-                for (int t = 0; t < 8; ++t) {
-                    pd[t][0] = *reinterpret_cast<const float2 *>(src + 8 * t);
-                    pd[t][1] = *reinterpret_cast<const float2 *>(src + 8 * C + 8 * t);
-                }
+                for (int t = 0; t < 8; ++t) pd[t] = load4(src + 128 * t);
             }
         });
         if constexpr (BWD) {   // dU = D K G_1 + P^T dO
 #pragma unroll
             for (int t = 0; t < 8; ++t) {
                 const float2 d = *reinterpret_cast<const float2 *>(&s.dec[8 * t + cq]);
-                x[t][0] = d.x * x[t][0] + pd[t][0].x;
-                x[t][1] = d.y * x[t][1] + pd[t][0].y;
-                x[t][2] = d.x * x[t][2] + pd[t][1].x;
-                x[t][3] = d.y * x[t][3] + pd[t][1].y;
+                x[t][0] = d.x * x[t][0] + pd[t].x;
+                x[t][1] = d.y * x[t][1] + pd[t].y;
+                x[t][2] = d.x * x[t][2] + pd[t].z;
+                x[t][3] = d.y * x[t][3] + pd[t].w;
             }
         } else {   // B (V - Gam K S_0)
 #pragma unroll
@@ -577,14 +606,16 @@ __device__ __forceinline__ void chain(const BwdChunkParams &p, ChainSmem<D> &sm,
 #pragma unroll
                 for (int e = 0; e < 4; ++e) y[2 * np][e] += d[0][e], y[2 * np + 1][e] += d[1][e];
             }
-        if (BWD) cp_wait<1>();   // Q and dO have landed
-        __syncthreads();         // every warp is done with T (and V)
-        if (it + 1 < nc) {
-            load_t(c + step);
-            if (!BWD) load_vd(c + step);
+        // every warp is done with T (and V); Q and dO have landed
+        late = __syncthreads_or(BWD && !umma::mbar_wait(&sm.bar[1], it & 1, CHAIN_WAIT_LIMIT));
+        if (late) break;
+        if (BWD && rows < C) {
+            zero_rows<NB>(sm.q, rows, tid);
+            zero_rows<1>(sm.vd, rows, tid);
+            umma::fence_async_smem();
+            __syncthreads();
         }
-        cp_commit();
-        const int rows = rows_of(c);
+        if (tid == 0 && it + 1 < nc) load_t(c + step);
         const float gc = s.gam[C - 1];
         if constexpr (BWD) {   // lam = B w
             float *dst = p.dv + (((size_t)tok0 + c * C + cq) * p.H + h) * D + col;
@@ -635,6 +666,11 @@ __device__ __forceinline__ void chain(const BwdChunkParams &p, ChainSmem<D> &sm,
             state_update<D>(S, 1.f, a, smem_u32(sm.q), lane);
         }
     }
+    if (late) {   // copies issued just before a wait gave up finish first
+        for (int i = 0; i < 32; ++i) __nanosleep(1000);
+        if (tid == 0 && p.status_word) atomicExch(p.status_word, (int)KLA_ERR_TIMEOUT);
+        return;
+    }
     if (BWD && p.dinit) {
         float *dst = p.dinit + ((size_t)n * p.H + h) * D * D + col;
 #pragma unroll
@@ -645,13 +681,13 @@ __device__ __forceinline__ void chain(const BwdChunkParams &p, ChainSmem<D> &sm,
 }
 
 template <int D>
-__global__ void __launch_bounds__(128, 2) kla_bwd_chain_kernel(BwdChunkParams p, int n_units)
+__global__ void __launch_bounds__(128, 2) kla_bwd_chain_kernel(const __grid_constant__ TileMaps tm, BwdChunkParams p, int n_units)
 {
     extern __shared__ __align__(1024) unsigned char smem_dyn[];
     ChainSmem<D> &sm = *reinterpret_cast<ChainSmem<D> *>(smem_dyn);
     // the backward chains, the longer ones, first
-    if ((int)blockIdx.x < n_units) chain<D, true>(p, sm, blockIdx.x);
-    else chain<D, false>(p, sm, blockIdx.x - n_units);
+    if ((int)blockIdx.x < n_units) chain<D, true>(p, tm, sm, blockIdx.x);
+    else chain<D, false>(p, tm, sm, blockIdx.x - n_units);
 }
 
 // ---- 3. gradients ---------------------------------------------------------------------------------------------------------
@@ -703,7 +739,7 @@ __device__ __forceinline__ void prefetch_block(const BwdChunkParams &p, int b, i
 template <int D>
 __global__ void __launch_bounds__(GT, 1) kla_bwd_grad_kernel(BwdChunkParams p, int ahead)
 {
-    constexpr int NB = D / 64, IT = D * 8 / GT;   // 8-column items of a [D][64] fp32 matrix per thread
+    constexpr int NB = D / 64, IT = D / 2 / GW;   // tiles of half a state per warp
     constexpr int UI = C * D / 8 / GT;            // 8-column items of a [64][D] matrix per thread
     extern __shared__ __align__(128) unsigned char smem_dyn[];
     GradSmem<D> &sm = *reinterpret_cast<GradSmem<D> *>(smem_dyn);
@@ -718,16 +754,13 @@ __global__ void __launch_bounds__(GT, 1) kla_bwd_grad_kernel(BwdChunkParams p, i
     if (tid < (int)sizeof(Scal) / 16) cp16(smem_u32(&sm.s) + tid * 16, reinterpret_cast<const char *>(p.scal + ch) + tid * 16, true);
     cp_commit();
 
-    // S_0^T / G_1^T: rows d_v, 64 columns of d_k from 64 hh on
-    float4 ps[IT][2], pg[IT][2];
-    auto fetch = [&](float4 (&pre)[IT][2], const float *src, int hh) {
+    // S_0^T / G_1^T, 64 columns of d_k from 64 hh on: tile tt of the 16 rows of d_v from 16 tg on
+    auto tg = [&](int i) { return (warp * IT + i) / 8; };
+    auto tt = [&](int i) { return (warp * IT + i) % 8; };
+    float4 ps[IT], pg[IT];
+    auto fetch = [&](float4 (&pre)[IT], const float *src, int hh) {
 #pragma unroll
-        for (int i = 0; i < IT; ++i) {
-            const int e = tid + i * GT, r = e >> 3, c8 = e & 7;
-            const float *x = src + ch * D * D + (size_t)r * D + hh * 64 + c8 * 8;
-            pre[i][0] = load4(x);
-            pre[i][1] = load4(x + 4);
-        }
+        for (int i = 0; i < IT; ++i) pre[i] = load4(src + ch * D * D + tg(i) * 16 * D + (8 * hh + tt(i)) * 128 + lane * 4);
     };
     auto put8 = [&](unsigned char *dst, int plane, uint32_t off, const float4 &a, const float4 &b) {
         uint32_t hh[4], mm[4], ll[4];
@@ -739,12 +772,18 @@ __global__ void __launch_bounds__(GT, 1) kla_bwd_grad_kernel(BwdChunkParams p, i
         *reinterpret_cast<uint4 *>(dst + plane + off) = make_uint4(mm[0], mm[1], mm[2], mm[3]);
         *reinterpret_cast<uint4 *>(dst + 2 * plane + off) = make_uint4(ll[0], ll[1], ll[2], ll[3]);
     };
-    auto commit = [&](const float4 (&pre)[IT][2]) {
+    auto commit = [&](const float4 (&pre)[IT]) {
 #pragma unroll
-        for (int i = 0; i < IT; ++i) {
-            const int e = tid + i * GT;
-            put8(sm.sg, D * 128, sw128(e >> 3, e & 7), pre[i][0], pre[i][1]);
-        }
+        for (int i = 0; i < IT; ++i)
+#pragma unroll
+            for (int u = 0; u < 2; ++u) {
+                uint32_t hh, mm, ll;
+                split3(u ? pre[i].z : pre[i].x, u ? pre[i].w : pre[i].y, hh, mm, ll);
+                const uint32_t off = sw128(tg(i) * 16 + u * 8 + (lane >> 2), tt(i)) + 4 * (lane & 3);
+                *reinterpret_cast<uint32_t *>(sm.sg + off) = hh;
+                *reinterpret_cast<uint32_t *>(sm.sg + D * 128 + off) = mm;
+                *reinterpret_cast<uint32_t *>(sm.sg + 2 * D * 128 + off) = ll;
+            }
     };
 
     // U and lam as operand planes; dbeta_i = (U_i / beta_i) . (lam_i / beta_i)
@@ -975,10 +1014,7 @@ __global__ void __launch_bounds__(GT, 1) kla_bwd_grad_kernel(BwdChunkParams p, i
         }
         __syncthreads();   // the S_0 planes have been read
 #pragma unroll
-        for (int i = 0; i < IT; ++i)
-#pragma unroll
-            for (int u = 0; u < 2; ++u)
-                gs += gc * (ps[i][u].x * pg[i][u].x + ps[i][u].y * pg[i][u].y + ps[i][u].z * pg[i][u].z + ps[i][u].w * pg[i][u].w);
+        for (int i = 0; i < IT; ++i) gs += gc * (ps[i].x * pg[i].x + ps[i].y * pg[i].y + ps[i].z * pg[i].z + ps[i].w * pg[i].w);
         commit(pg);
         if (hh + 1 < NB) fetch(ps, p.s0, hh + 1);
         __syncthreads();
@@ -1132,7 +1168,7 @@ cudaError_t allow_smem(K kern, int bytes)
 }
 
 template <int D>
-cudaError_t launch_d(const BwdChunkParams &p, cudaStream_t stream)
+cudaError_t launch_d(const BwdChunkParams &p, uint64_t n_tok, cudaStream_t stream)
 {
     const int smem1 = (int)sizeof(PrepSmem<D>), smem2 = (int)sizeof(ChainSmem<D>), smem3 = (int)sizeof(GradSmem<D>);
     cudaError_t e = allow_smem(kla_bwd_prepare_kernel<D>, smem1);
@@ -1141,8 +1177,13 @@ cudaError_t launch_d(const BwdChunkParams &p, cudaStream_t stream)
     if (e != cudaSuccess) return e;
     const int units = p.n_seq * p.H * (D / 64);
     if (units == 0) return cudaSuccess;
+    TileMaps tm = {};
+    const uint64_t row = (uint64_t)p.H * D;
+    if (n_tok > 0 && (!make_tile_map(&tm.q, p.q, n_tok, row) || !make_tile_map(&tm.k, p.k, n_tok, row) ||
+                      !make_tile_map(&tm.v, p.v, n_tok, row) || !make_tile_map(&tm.dout, p.dout, n_tok, row)))
+        return cudaErrorInvalidValue;
     if (p.n_slots > 0) kla_bwd_prepare_kernel<D><<<p.n_slots * p.H, 256, smem1, stream>>>(p);
-    kla_bwd_chain_kernel<D><<<2 * units, 128, smem2, stream>>>(p, units);   // (empty sequences: dinit)
+    kla_bwd_chain_kernel<D><<<2 * units, 128, smem2, stream>>>(tm, p, units);   // (empty sequences: dinit)
     if (p.n_slots > 0) kla_bwd_grad_kernel<D><<<p.n_slots * p.H, GT, smem3, stream>>>(p, sm_count());
     count_launch(p.n_slots > 0 ? 3 : 1);
     return cudaGetLastError();
@@ -1192,7 +1233,8 @@ cudaError_t launch_bwd_chunk(const BwdArgs &a, cudaStream_t stream)
     p.g1 = (float *)w;
     w += n * d * d * 4;
     p.scal = (Scal *)w;
-    return a.d == 128 ? launch_d<128>(p, stream) : launch_d<64>(p, stream);
+    p.status_word = a.status_word;
+    return a.d == 128 ? launch_d<128>(p, (uint64_t)a.n_tok, stream) : launch_d<64>(p, (uint64_t)a.n_tok, stream);
 }
 
 }  // namespace kla

@@ -1038,20 +1038,6 @@ EncodeTiledFn get_encode_fn()
     return fn;
 }
 
-// 2-D view [rows = tokens][cols = H * d] of a bf16 [*, T, H, d] array; box = 64 tokens x 64 columns.
-bool make_tmap(CUtensorMap *tm, const void *base, uint64_t n_tok, uint64_t row_elems)
-{
-    EncodeTiledFn fn = get_encode_fn();
-    if (!fn) return false;
-    cuuint64_t dims[2] = {row_elems, n_tok};
-    cuuint64_t strides[1] = {row_elems * 2};
-    cuuint32_t box[2] = {64, 64};
-    cuuint32_t estr[2] = {1, 1};
-    return fn(tm, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void *>(base), dims, strides, box, estr,
-              CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
-              CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
-}
-
 // segment pass 1: (seg_G - 1) segments per sequence, twice the slices; p.n_seq counts all segments there
 template <int D>
 int blocks_of(const ChunkParams &p)
@@ -1063,8 +1049,8 @@ cudaError_t launch_v(const ChunkParams &p, cudaStream_t stream)
 {
     const uint64_t n_tok = (uint64_t)p.B * p.T;
     CUtensorMap tq, tk, tv;
-    if (!make_tmap(&tq, p.q, n_tok, (uint64_t)p.H * D) || !make_tmap(&tk, p.k, n_tok, (uint64_t)p.H * D) ||
-        !make_tmap(&tv, p.v, n_tok, (uint64_t)p.H * D))
+    if (!make_tile_map(&tq, p.q, n_tok, (uint64_t)p.H * D) || !make_tile_map(&tk, p.k, n_tok, (uint64_t)p.H * D) ||
+        !make_tile_map(&tv, p.v, n_tok, (uint64_t)p.H * D))
         return cudaErrorInvalidValue;
     auto kern = kla_chunk_mma_kernel<D, BPS, OUT, VAR>;
     const int smem = (int)sizeof(Smem<D, BPS>);
@@ -1092,6 +1078,19 @@ cudaError_t launch_d(const ChunkParams &p, int out_dtype, cudaStream_t stream)
 }
 
 }  // namespace
+
+bool make_tile_map(void *map, const void *base, uint64_t rows, uint64_t row_elems)
+{
+    EncodeTiledFn fn = get_encode_fn();
+    if (!fn) return false;
+    cuuint64_t dims[2] = {row_elems, rows};
+    cuuint64_t strides[1] = {row_elems * 2};
+    cuuint32_t box[2] = {64, 64};
+    cuuint32_t estr[2] = {1, 1};
+    return fn(static_cast<CUtensorMap *>(map), CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void *>(base), dims, strides, box, estr,
+              CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B,
+              CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
 
 bool chunk_tc_supported(int d, int chunk, int io_dtype)
 {

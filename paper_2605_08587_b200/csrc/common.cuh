@@ -113,11 +113,14 @@ struct BwdArgs {
     long long n_tok;
     float eps;
     int32_t coeff_eta, qnorm;
+    int32_t *status_word;               // or null
 };
 size_t bwd_scan_workspace_bytes(int n_seq, long long n_tok, int H, int d);
 cudaError_t launch_bwd_scan(const BwdArgs &a, cudaStream_t stream);
 size_t bwd_chunk_workspace_bytes(int n_seq, long long n_tok, int H, int d);
 cudaError_t launch_bwd_chunk(const BwdArgs &a, cudaStream_t stream);
+// Tensor map (a CUtensorMap) of a bf16 [rows][row_elems] array, boxes of 64 rows x 64 elements, 128-byte swizzle.
+bool make_tile_map(void *map, const void *base, uint64_t rows, uint64_t row_elems);
 // True when the tensor-core kernel covers this case.
 bool chunk_tc_supported(int d, int chunk, int io_dtype);
 
