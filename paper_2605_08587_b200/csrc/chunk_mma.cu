@@ -27,6 +27,8 @@
 // memory the state product was bound by the fetch of both operands (8 KB for each 32 cycles of products: 570 cycles), and its
 // operand took a proxy fence (headline shape 200.6 -> 194.7 us, 32 packed sequences at d 64 487 -> 472).  The outputs are transposed through
 // a buffer that TMA never touches: in the V tile they took such a fence too, in which the warp stood (194.7 -> 188, 472 -> 462).
+// The size of the code counts, all the more the more SMs run it: at 70 KB two KB less in the waits alone (one short loop each instead
+// of two) were worth 2 % of the headline shape and of 65 536 tokens, two KB more cost 10 %.
 // The outputs on four warps of their own cost more than they took off the chain: 246 us against 201 (82 KB of code instead of 70,
 // fetched by all SMs at once, and the Gram product then falls into the block solve).
 //
@@ -67,7 +69,7 @@ using namespace umma;
 constexpr int C = 64;         // chunk length
 constexpr int NS = 64;        // state columns per block
 constexpr int CHAIN_T = 128, PREP_T = 128, NT = CHAIN_T + PREP_T + 128;   // (the last warpgroup: one warp works)
-constexpr long long WAIT_LIMIT = 2000000000LL;   // SM clocks (~1 s) before a wait gives up
+constexpr uint32_t WAIT_LIMIT = 2000000000u;   // SM clocks (~1 s) before a wait gives up
 constexpr float LOG2E = 1.4426950408889634f;
 // The write weights exp(g_C - g_j) are kept above 2^-DEC_FLOOR_LOG2 (~1e-35): U is carried as D U throughout, with D^-1 in X and
 // P, and with the floor neither factor leaves the fp32 / bf16 exponent range however strong the decay.  A floored weight puts at
@@ -138,24 +140,23 @@ struct Smem {
     volatile int abort_flag;
 };
 
+__device__ __forceinline__ uint32_t clock_lo()
+{
+    uint32_t t;
+    asm volatile("mov.u32 %0, %%clock;" : "=r"(t));
+    return t;
+}
 // Every lane polls; the warp leaves together.
 __device__ __forceinline__ bool bar_wait(uint64_t *bar, uint32_t parity, volatile int *abort_flag)
 {
     bool ok = mbar_try_wait(bar, parity);
     if (!ok) {
-        const long long t0 = clock64();
-        while (true) {
+        const uint32_t t0 = clock_lo();
 #pragma unroll 1
-            for (int i = 0; i < 64 && !ok; ++i) {
-                ok = mbar_try_wait(bar, parity);
-                if (!ok) __nanosleep(20);
-            }
-            if (ok || *abort_flag) break;
-            if (clock64() - t0 > WAIT_LIMIT) {
-                *abort_flag = 1;
-                break;
-            }
-        }
+        do {
+            ok = mbar_try_wait(bar, parity);
+        } while (!ok && !*abort_flag && clock_lo() - t0 < WAIT_LIMIT);
+        if (!ok) *abort_flag = 1;
     }
     return __all_sync(0xffffffffu, ok);
 }
