@@ -135,10 +135,10 @@ struct PrepSmem {
             alignas(1024) unsigned char k[D / 64 * 8192], q[D / 64 * 8192];
         };
         alignas(1024) unsigned char p[T_BYTES];   // P, three planes, once K and Q have been read
+        alignas(16) float mm[32 * LDM];           // scratch of the inverse, once P^T dO is done
     };
     alignas(1024) unsigned char dout[D / 64 * 8192];
     alignas(16) float tl[C * LDT];            // X, overwritten by T
-    alignas(16) float mm[32 * LDM];
     Scal s;
     float eta[C];
 };
@@ -146,7 +146,7 @@ struct PrepSmem {
 // What bounds it: the latency of its phases (the levels of the inverse, each behind barriers), so blocks per SM: P over K and Q
 // gives room for a third one (B 8, H 8, T 4096, d 128: 198 -> 168 us; 16 packed sequences, d 64: 369 -> 305 us).
 template <int D>
-__global__ void __launch_bounds__(256, 3) kla_bwd_prepare_kernel(BwdChunkParams p)
+__global__ void __launch_bounds__(256, D == 64 ? 4 : 3) kla_bwd_prepare_kernel(BwdChunkParams p)
 {
     extern __shared__ __align__(1024) unsigned char smem_dyn[];   // used as declared: rounded up at run time, every access would be generic
     using Smem = PrepSmem<D>;
