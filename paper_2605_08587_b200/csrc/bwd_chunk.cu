@@ -114,6 +114,12 @@ __device__ __forceinline__ Where locate(const BwdChunkParams &p, int slot)
     return w;
 }
 
+// `bytes` (a multiple of 16, from a 16-byte boundary) on their way into L2.
+__device__ __forceinline__ void prefetch_l2(const void *x, int bytes)
+{
+    asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(x), "r"(bytes) : "memory");
+}
+
 // Rows t0 .. t0 + 63 (of which `rows` exist, the others become zero) of a [token][H][D] array, columns col .. col + 64 NB - 1
 // of head h, into NB consecutive 64 x 64 tiles; all NTH threads.
 template <int NB, int D, int NTH>
@@ -520,7 +526,10 @@ __device__ __forceinline__ void chain(const BwdChunkParams &p, const TileMaps &t
         }
         if (tid == 0) {
             if (BWD) load_q(c);
-            if (it + 1 < nc) load_k(c + step);
+            if (it + 1 < nc) {
+                load_k(c + step);
+                if (BWD) prefetch_l2(p.pdo + (ch0 + (size_t)(c + step) * p.H) * D * C + sl * 64 * C, 64 * C * 4);
+            }
         }
         // the state at this end of the chunk, transposed
         {
@@ -720,10 +729,9 @@ __device__ __forceinline__ void prefetch_block(const BwdChunkParams &p, int b, i
     const int rows = min(C, w.len - w.c * C);
     const size_t t0 = (size_t)w.tok0 + w.c * C, ch = (size_t)slot * p.H + h;
     if (tid == 0) {
-        auto bulk = [](const void *x, int bytes) { asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(x), "r"(bytes) : "memory"); };
-        bulk(p.u + ch * C * D, C * D * 4);
-        bulk(p.s0 + ch * D * D, D * D * 4);
-        bulk(p.g1 + ch * D * D, D * D * 4);
+        prefetch_l2(p.u + ch * C * D, C * D * 4);
+        prefetch_l2(p.s0 + ch * D * D, D * D * 4);
+        prefetch_l2(p.g1 + ch * D * D, D * D * 4);
     }
     auto line = [](const void *x) { asm volatile("prefetch.global.L2 [%0];" ::"l"(x)); };
     constexpr int LF = D / 32, LB = D / 64;   // 128-byte lines of a row of floats, of bf16
