@@ -22,7 +22,7 @@
 // the schedulers' instruction caches and issues at about one instruction in three cycles (measured on unrolled against rolled
 // copies of the same products).  With all products on mma.sync (504 per chunk and warp at d = 128 instead of 248) a chunk took
 // 8 000 cycles; with all of them on tcgen05, whose every product on the chain ends in a hand-over through tensor memory and shared
-// memory, 7 400; this way 5 200 (2.75 us, B 8, H 8, d 128, T 4096).  mma.sync stands still while a tcgen05 product
+// memory, 7 400; this way 5 400 (2.73 us, B 8, H 8, d 128, between T 4096 and 8192).  mma.sync stands still while a tcgen05 product
 // runs, so the two add up: 400 cycles for [K; Q] K^T, 8 per mma.sync.  [S_hi; S_lo]^T is a left operand in tensor memory: from shared
 // memory the state product was bound by the fetch of both operands (8 KB for each 32 cycles of products: 570 cycles), and its
 // operand took a proxy fence (headline shape 200.6 -> 194.7 us, 32 packed sequences at d 64 487 -> 472).  The outputs are transposed through
