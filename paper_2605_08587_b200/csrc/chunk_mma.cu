@@ -16,7 +16,7 @@
 // 128 columns (the chunk's keys and queries), and [K; Q] K^T.  The serial part runs on mma.sync inside single warps: everything
 // transposed, an accumulator tile (16 columns of d_v x tokens or d_k) is at the same time a left operand of the next product, so
 // R -> U -> state goes from product to product in registers, without a barrier.  Once per chunk the hi and lo parts of the new state
-// go to shared memory for the tcgen05 product of the next chunk.
+// go to tensor memory as left operand of the tcgen05 product of the next chunk.
 //
 // What bounds it: the latency of that chain and the number of instructions in it.  Code that runs once per chunk does not stay in
 // the schedulers' instruction caches and issues at about one instruction in three cycles (measured on unrolled against rolled
