@@ -633,7 +633,7 @@ __device__ void chain(const ChunkParams &p, Smem<D, BPS> &sm, const Work &wk, in
     };
     // d = 128: the product over the first 64 rows of d_k starts while the others are being finished (-1.5 %)
     auto state_written = [&](int part) {
-        asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
+        tmem_wait_stores();
         tc_fence_before();
         __syncwarp();
         if (lane == 0) mbar_arrive(&sm.bar[part ? B_STATE1 : B_STATE]);
@@ -877,6 +877,8 @@ __device__ void chain(const ChunkParams &p, Smem<D, BPS> &sm, const Work &wk, in
             out += C * tok_stride;
         }
     }
+    // The last chunk stores its state to tensor memory like any other, and nobody waits for it: the columns are given back next.
+    tmem_wait_stores();
     if (wk.fin && !sm.abort_flag) {
 #pragma unroll
         for (int t = 0; t < D / 8; ++t)
