@@ -67,10 +67,10 @@ typedef enum { KLA_F32 = 0, KLA_BF16 = 1 } kla_dtype;
 #define KLA_FLAG_COEFF_ETA 4              /* beta_t = eta_t: the gated-delta-rule baseline coefficient of Section 2,
                                              without the key-norm division of Eq. 3 (eps is then unused)          */
 #define KLA_FLAG_QNORM 8                  /* o_t = S_t^T q_t / ||q_t||: the read-out as Algorithm 1 (left) prints it */
-/* Not part of the supported flag set: used by the library's own tests of the error path.  The tensor-core kernel
- * withholds one internal completion signal, so that a bounded device-side wait runs out (about one second), every
- * CTA gives up in an orderly way and KLA_ERR_TIMEOUT appears in *status_word.  Outputs are then undefined; the
- * context stays usable. */
+/* Not part of the supported flag set: used by the library's own tests of the error path.  The tensor-core kernels (kla_chunk_fwd,
+ * kla_chunk_span_map, and kla_bwd with bf16 inputs) withhold one internal completion signal, so that a bounded device-side wait
+ * runs out (about one second), every CTA gives up in an orderly way and KLA_ERR_TIMEOUT appears in *status_word.  Outputs are
+ * then undefined; the context stays usable. */
 #define KLA_INTERNAL_FLAG_TEST_TIMEOUT 16
 /* Accepted and without effect: the blocks that hold the 64-column slices of a head always run independently of each other (an
  * earlier kernel could pair them). */
@@ -121,7 +121,9 @@ typedef struct {
     void *workspace;           /* DEVICE scratch of at least kla_chunk_fwd_workspace_bytes()    */
     size_t workspace_bytes;
     int32_t *status_word;      /* optional DEVICE int32, zeroed by the caller; a kernel whose
-                                  bounded wait expires stores KLA_ERR_TIMEOUT there and exits  */
+                                  bounded wait expires stores KLA_ERR_TIMEOUT there and exits
+                                  (kla_chunk_fwd and its variants, kla_chunk_span_map, kla_bwd): the
+                                  call has then returned KLA_OK, and its outputs are undefined */
     void *stream;              /* cudaStream_t (NULL = default stream)                          */
 } kla_desc;
 
@@ -218,6 +220,7 @@ kla_status kla_chunk_fwd_timed(const kla_desc *desc, const void *q, const void *
  *   phi_out [B, H, d_k, d_k] fp32: the state reached from the identity with v = 0 (S_end = phi_out . S_start + n_out)
  *   n_out   [B, H, d_k, d_v] fp32: the state reached from zero
  *   desc->workspace: at least kla_chunk_span_map_workspace_bytes(desc) bytes.
+ *   desc->status_word as for kla_chunk_fwd: a map formed by a kernel that gave up must not be exchanged.
  *
  * kla_state_chain: start states of R consecutive spans from their maps, in fp32:
  *   start[b, 0] = init_state[b] (or 0);  start[b, r + 1] = phi[b, r] . start[b, r] + n[b, r]
@@ -295,7 +298,8 @@ kla_status kla_dg_decode_step(const kla_desc *desc, const void *q, const void *k
  *   (B T / 64 + n_seq) x H x (24 KB + 512 d_k + 8 d_k d_v + 2 KB) plus 4 bytes per sequence (bf16), and
  *   (B T / 16 + n_seq) x H x d_k x d_v fp32, 16 x 64 x d_k fp32 per resident thread block (at most one per SM), 256 bytes (fp32)
  * (host function; it reads the current device's SM count when a device is present; 0 for an invalid descriptor).  Errors as
- * kla_chunk_fwd.
+ * kla_chunk_fwd.  bf16 inputs: the kernels wait (bounded) for their copies; desc->status_word receives KLA_ERR_TIMEOUT if such a wait
+ * runs out, and every gradient of the call is then undefined, although kla_bwd itself has returned KLA_OK.  fp32 inputs: no waits.
  */
 size_t kla_bwd_workspace_bytes(const kla_desc *desc);
 kla_status kla_bwd(const kla_desc *desc, const void *q, const void *k, const void *v,

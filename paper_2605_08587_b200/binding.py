@@ -143,8 +143,8 @@ def _status_for(dev):
 
 
 def check(device=None):
-    """Reads (and clears) the status word the binding passes to kla_chunk_fwd when the caller gives none: raises KlaError
-    if a kernel on `device` (default: the current one) gave up on a bounded wait since the last check -- its outputs are
+    """Reads (and clears) the status word the binding passes to kla_chunk_fwd, kla_chunk_span_map and kla_bwd when the caller gives none:
+    raises KlaError if a kernel on `device` (default: the current one) gave up on a bounded wait since the last check -- its outputs are
     then undefined.  Waits for the device; meant for the end of a step, not for the hot path."""
     i = torch.cuda.current_device() if device is None else torch.device(device).index
     word = _own_status.get(i)
@@ -272,15 +272,19 @@ def kla_chunk_fwd_static_scratch(q, k, v, log_alpha, eta, eps, out, final_state=
     return out, final_state
 
 
-def kla_chunk_span_map(k, v, log_alpha, eta, eps, flags=KLA_FLAG_NONE):
+def kla_chunk_span_map(k, v, log_alpha, eta, eps, flags=KLA_FLAG_NONE, status_word=None):
     """Transition map of a span of tokens (include/kla.h: kla_chunk_span_map): S_end = phi . S_start + n.
-    k [B, T, H, d]; v [B, T, H, d]; log_alpha, eta [B, T, H]; bf16 inputs.  Returns (phi, n), both [B, H, d, d] fp32."""
+    k [B, T, H, d]; v [B, T, H, d]; log_alpha, eta [B, T, H]; bf16 inputs.  Returns (phi, n), both [B, H, d, d] fp32.
+    `status_word` as for kla_chunk_fwd."""
     lib = load()
     B, T, H, d = k.shape
     phi = torch.empty((B, H, d, d), device=k.device, dtype=torch.float32)
     n = torch.empty((B, H, d, d), device=k.device, dtype=torch.float32)
+    if status_word is None:
+        status_word = _status_for(k.device)
     desc = KlaDesc(B=B, T=T, H=H, d_k=d, d_v=v.shape[-1], n_seq=B, cu_seqlens=None, host_seqlens=None, io_dtype=_dt(k),
-                   out_dtype=KLA_F32, flags=flags, workspace=None, workspace_bytes=0, status_word=None, stream=_stream(k.device))
+                   out_dtype=KLA_F32, flags=flags, workspace=None, workspace_bytes=0,
+                   status_word=_dev(status_word, "status_word", torch.int32), stream=_stream(k.device))
     need = lib.kla_chunk_span_map_workspace_bytes(ctypes.byref(desc))
     ws = torch.empty(max(need, 16), device=k.device, dtype=torch.uint8)
     desc.workspace, desc.workspace_bytes = ws.data_ptr(), need
@@ -336,17 +340,18 @@ def kla_dg_fwd(q, k, v, log_alpha, eta, eps, init_state=None, out=None, final_st
 
 
 def kla_bwd(q, k, v, log_alpha, eta, eps, d_out, init_state=None, d_final_state=None, cu_seqlens=None, host_seqlens=None,
-            flags=KLA_FLAG_NONE, want_dinit_state=True, workspace=None):
+            flags=KLA_FLAG_NONE, want_dinit_state=True, workspace=None, status_word=None):
     """Backward pass (include/kla.h: kla_bwd): gradients of a scalar loss given d_out = dL/dout (dtype of q) and
     d_final_state = dL/dfinal_state (or None).  Returns a dict of fp32 tensors dq, dk, dv, dlog_alpha, deta and
     dinit_state (None unless asked for).  `workspace`: a uint8 CUDA tensor of at least kla_bwd_workspace_bytes, else
-    one is allocated here."""
+    one is allocated here.  `status_word` as for kla_chunk_fwd: the gradients are undefined once it holds KLA_ERR_TIMEOUT (bf16 inputs;
+    the kernel of fp32 inputs waits for nothing)."""
     if _host is None:
         load()
     if cu_seqlens is not None and host_seqlens is None:
         host_seqlens = cu_seqlens.cpu()
     return _host.backward(q, k, v, log_alpha, eta, float(eps), d_out, init_state, d_final_state, cu_seqlens, host_seqlens, flags,
-                          want_dinit_state, workspace)
+                          want_dinit_state, workspace, status_word)
 
 
 def kla_dg_decode_step(q, k, v, log_alpha, eta, eps, state_inout, out=None, out_dtype=None, flags=KLA_FLAG_NONE):

@@ -436,6 +436,7 @@ kla_status kla_chunk_span_map(const kla_desc *desc, const void *k, const void *v
     p.eps = eps;
     p.seg_pass = 1; p.seg_G = 2;
     p.variant = ((desc->flags & KLA_FLAG_COEFF_ETA) ? VARIANT_COEFF_ETA : 0) |
+                ((desc->flags & KLA_INTERNAL_FLAG_TEST_TIMEOUT) ? VARIANT_TEST_TIMEOUT : 0) |
                 ((desc->flags & KLA_FLAG_WY_FORM) ? VARIANT_WY : 0);
     p.map_state = map;
     if (launch_chunk_tc(p, desc->d_k, desc->io_dtype, KLA_F32, stream) != cudaSuccess) return KLA_ERR_LAUNCH;
@@ -592,6 +593,7 @@ kla_status kla_bwd(const kla_desc *desc, const void *q, const void *k, const voi
     a.eps = eps;
     a.coeff_eta = (desc->flags & KLA_FLAG_COEFF_ETA) ? 1 : 0;
     a.qnorm = (desc->flags & KLA_FLAG_QNORM) ? 1 : 0;
+    a.test_timeout = (desc->flags & KLA_INTERNAL_FLAG_TEST_TIMEOUT) ? 1 : 0;
     a.status_word = desc->status_word;
     const cudaError_t err = desc->io_dtype == KLA_BF16 ? launch_bwd_chunk(a, stream) : launch_bwd_scan(a, stream);
     return err == cudaSuccess ? KLA_OK : KLA_ERR_LAUNCH;

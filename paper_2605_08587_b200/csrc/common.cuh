@@ -113,6 +113,7 @@ struct BwdArgs {
     long long n_tok;
     float eps;
     int32_t coeff_eta, qnorm;
+    int32_t test_timeout;               // test hook: the chains' bounded waits run out (bf16 inputs)
     int32_t *status_word;               // or null
 };
 size_t bwd_scan_workspace_bytes(int n_seq, long long n_tok, int H, int d);

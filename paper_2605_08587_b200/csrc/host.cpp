@@ -82,6 +82,23 @@ long integer(PyObject *o)
 }
 bool has_shape(const at::Tensor &t, at::IntArrayRef shape) { return t.sizes() == shape; }
 
+// The status word of a call: the caller's, else the binding's own of the device (kept alive by the binding).
+int32_t *status_word(PyObject *given, c10::Device device)
+{
+    PyObject *o = given;   // borrowed
+    if (o == Py_None) {
+        PyObject *dev = PyLong_FromLong(device.index());
+        o = dev ? PyObject_CallOneArg(g_status_for, dev) : nullptr;
+        Py_XDECREF(dev);
+        if (!o) throw Failed();
+        Py_DECREF(o);
+    }
+    const at::Tensor &t = tensor(o, "status_word");
+    void *p = addr(&t, "status_word");
+    if (t.scalar_type() != at::kInt) fail(PyExc_TypeError, "must be torch.int32", "status_word");
+    return static_cast<int32_t *>(p);
+}
+
 void check(kla_status st)
 {
     if (st == KLA_OK) return;
@@ -186,14 +203,6 @@ PyObject *forward(PyObject *, PyObject *const *a, Py_ssize_t n)
         if (fin_given) fin = *fin_given;
         else if (integer(a[14])) fin = at::empty({n_seq, H, d_k, d_v}, q.options().dtype(at::kFloat));
         if (init && !has_shape(*init, {n_seq, H, d_k, d_v})) fail(PyExc_ValueError, "init_state must be [n_seq, H, d_k, d_v]");
-        PyObject *status = a[15];   // borrowed, or the binding's own word of this device (kept alive by the binding)
-        if (status == Py_None && !dg) {
-            PyObject *dev = PyLong_FromLong(q.device().index());
-            status = dev ? PyObject_CallOneArg(g_status_for, dev) : nullptr;
-            Py_XDECREF(dev);
-            if (!status) throw Failed();
-            Py_DECREF(status);
-        }
         kla_desc d = {};
         d.B = (int32_t)B;
         d.T = (int32_t)T;
@@ -207,9 +216,7 @@ PyObject *forward(PyObject *, PyObject *const *a, Py_ssize_t n)
         d.out_dtype = kla_dtype_of(out);
         d.flags = (int32_t)integer(a[13]);
         d.stream = c10::cuda::getCurrentCUDAStream(q.device().index()).stream();
-        const at::Tensor *word = opt_tensor(status, "status_word");
-        d.status_word = static_cast<int32_t *>(addr(word, "status_word"));
-        if (word && word->scalar_type() != at::kInt) fail(PyExc_TypeError, "must be torch.int32", "status_word");
+        if (!dg) d.status_word = status_word(a[15], q.device());   // (kernels of diagonal gates wait for nothing)
         if (!dg) {
             if (const size_t need = kla_chunk_fwd_workspace_bytes(&d, chunk)) {
                 ws = at::empty({(int64_t)need}, q.options().dtype(at::kByte));
@@ -248,11 +255,11 @@ PyObject *forward(PyObject *, PyObject *const *a, Py_ssize_t n)
 }
 
 // kla_bwd: (q, k, v, log_alpha, eta, eps, d_out, init_state, d_final_state, cu_seqlens, host_seqlens, flags, want_dinit_state,
-// workspace) -> dict
+// workspace, status_word) -> dict
 PyObject *backward(PyObject *, PyObject *const *a, Py_ssize_t n)
 {
-    if (n != 14) {
-        PyErr_SetString(PyExc_TypeError, "backward: 14 arguments");
+    if (n != 15) {
+        PyErr_SetString(PyExc_TypeError, "backward: 15 arguments");
         return nullptr;
     }
     try {
@@ -287,6 +294,7 @@ PyObject *backward(PyObject *, PyObject *const *a, Py_ssize_t n)
         d.out_dtype = KLA_F32;
         d.flags = (int32_t)integer(a[11]);
         d.stream = c10::cuda::getCurrentCUDAStream(q.device().index()).stream();
+        d.status_word = status_word(a[14], q.device());
         const auto f32 = q.options().dtype(at::kFloat);
         const bool want = PyObject_IsTrue(a[12]) == 1;
         at::Tensor g[6] = {at::empty({B, T, H, d_k}, f32), at::empty({B, T, H, d_k}, f32), at::empty({B, T, H, d_v}, f32),
