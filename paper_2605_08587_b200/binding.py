@@ -138,7 +138,7 @@ def _status_for(dev):
     i = dev if isinstance(dev, int) else torch.device(dev).index
     i = torch.cuda.current_device() if i is None else i
     if i not in _own_status:
-        _own_status[i] = torch.zeros(1, dtype=torch.int32, device="cuda:%d" % i)
+        _own_status.setdefault(i, _host.new_status_word(i))   # (one word, whichever thread comes first)
     return _own_status[i]
 
 

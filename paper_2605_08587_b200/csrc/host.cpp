@@ -10,6 +10,9 @@
 
 #include <ATen/core/Tensor.h>
 #include <ATen/ops/empty.h>
+#include <ATen/ops/zeros.h>
+#include <c10/cuda/CUDAException.h>
+#include <c10/cuda/CUDAGraphsC10Utils.h>
 #include <c10/cuda/CUDAGuard.h>
 #include <c10/cuda/CUDAStream.h>
 #include <torch/csrc/Dtype.h>
@@ -331,6 +334,32 @@ PyObject *backward(PyObject *, PyObject *const *a, Py_ssize_t n)
     }
 }
 
+// new_status_word(device index) -> int32[1], zero.  Made on a stream of its own and complete on return: on the current stream, if that is
+// being captured, the word would belong to the graph, whose every replay would clear it.
+PyObject *new_status_word(PyObject *, PyObject *index)
+{
+    try {
+        const c10::Device device(c10::kCUDA, (c10::DeviceIndex)integer(index));
+        const c10::cuda::CUDAGuard guard(device);
+        const c10::cuda::CUDAStreamCaptureModeGuard relaxed(cudaStreamCaptureModeRelaxed);   // (of this thread, for a moment)
+        cudaStream_t own;
+        C10_CUDA_CHECK(cudaStreamCreateWithFlags(&own, cudaStreamNonBlocking));
+        at::Tensor word;
+        {
+            const c10::cuda::CUDAStreamGuard on(c10::cuda::getStreamFromExternal(own, device.index()));
+            word = at::zeros({1}, at::TensorOptions().device(device).dtype(at::kInt));
+        }
+        C10_CUDA_CHECK(cudaStreamSynchronize(own));
+        C10_CUDA_CHECK(cudaStreamDestroy(own));
+        return THPVariable_Wrap(std::move(word));
+    } catch (const Failed &) {
+        return nullptr;
+    } catch (const std::exception &e) {
+        PyErr_SetString(PyExc_RuntimeError, e.what());
+        return nullptr;
+    }
+}
+
 PyObject *init(PyObject *, PyObject *const *a, Py_ssize_t n)
 {
     if (n != 2) {
@@ -345,6 +374,7 @@ PyObject *init(PyObject *, PyObject *const *a, Py_ssize_t n)
 PyMethodDef methods[] = {{"init", (PyCFunction)(void (*)())init, METH_FASTCALL, nullptr},
                          {"decode", (PyCFunction)(void (*)())decode, METH_FASTCALL, nullptr},
                          {"forward", (PyCFunction)(void (*)())forward, METH_FASTCALL, nullptr},
+                         {"new_status_word", new_status_word, METH_O, nullptr},
                          {"backward", (PyCFunction)(void (*)())backward, METH_FASTCALL, nullptr},
                          {nullptr, nullptr, 0, nullptr}};
 PyModuleDef module = {PyModuleDef_HEAD_INIT, "_host", nullptr, -1, methods, nullptr, nullptr, nullptr, nullptr};

@@ -73,3 +73,30 @@ def test_span_map_reports_a_wait_that_ran_out(flags):
     zero = torch.zeros(1, 2, 128, 128, dtype=torch.float64)
     _, fin, _ = oracle.forward(*(np64(x) for x in (w.q, w.k, w.v, w.log_alpha, w.eta)), w.eps, zero.numpy())
     assert rel_err(np64(n), fin) <= TOL_BF16
+
+
+def test_replaying_a_graph_does_not_clear_what_other_calls_reported(monkeypatch):
+    """The first call of all may be a captured one: the binding's status word must not become part of that graph."""
+    from paper_2605_08587_b200 import kla_chunk_fwd
+    w = W.config2(B=1, H=2, T=130, seed=540)
+    do, _ = W.upstream_grads(w)
+    a, do = _args(w), do.to(DEV)
+    kla_bwd(*a, w.eps, do)                      # (what is loaded on first use is loaded)
+    kla_chunk_fwd(*a, w.eps)
+    eager = kla_bwd(*a, w.eps, do)
+    torch.cuda.synchronize()
+    monkeypatch.setattr(binding, "_own_status", {})
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        g = kla_bwd(*a, w.eps, do)
+        out, fin = kla_chunk_fwd(*a, w.eps)
+    check(DEV)                                  # captured, not run: nothing to report
+    kla_bwd(*a, w.eps, do, flags=RUN_OUT)
+    graph.replay()
+    torch.cuda.synchronize()
+    with pytest.raises(KlaError) as e:
+        check(DEV)
+    assert e.value.code == TIMEOUT
+    assert all(torch.equal(g[x], eager[x]) for x in g if g[x] is not None)
+    graph.replay()
+    check(DEV)
