@@ -121,7 +121,8 @@ typedef struct {
     void *workspace;           /* DEVICE scratch of at least kla_chunk_fwd_workspace_bytes()    */
     size_t workspace_bytes;
     int32_t *status_word;      /* optional DEVICE int32, zeroed by the caller; a kernel whose
-                                  bounded wait expires stores KLA_ERR_TIMEOUT there and exits
+                                  bounded wait expires stores KLA_ERR_TIMEOUT there and exits, one
+                                  that finds its shared memory misplaced KLA_ERR_ALIGN
                                   (kla_chunk_fwd and its variants, kla_chunk_span_map, kla_bwd): the
                                   call has then returned KLA_OK, and its outputs are undefined */
     void *stream;              /* cudaStream_t (NULL = default stream)                          */

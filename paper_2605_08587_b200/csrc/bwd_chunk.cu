@@ -697,6 +697,12 @@ __global__ void __launch_bounds__(128, 2) kla_bwd_chain_kernel(const __grid_cons
 {
     extern __shared__ __align__(1024) unsigned char smem_dyn[];
     ChainSmem<D> &sm = *reinterpret_cast<ChainSmem<D> *>(smem_dyn);
+    // TMA permutes the pieces of a row by their address, ldmatrix here by their place in the tile: the same from a 1024-byte boundary on.
+    // There is no static shared memory, so the tiles start on one; checked all the same.
+    if (smem_u32(smem_dyn) & 1023) {
+        if (threadIdx.x == 0 && p.status_word) atomicExch(p.status_word, (int)KLA_ERR_ALIGN);
+        return;
+    }
     // the backward chains, the longer ones, first
     if ((int)blockIdx.x < n_units) chain<D, true>(p, tm, sm, blockIdx.x);
     else chain<D, false>(p, tm, sm, blockIdx.x - n_units);
