@@ -69,16 +69,24 @@ struct BwdChunkParams {
     int32_t coeff_eta, qnorm;
     // workspace, one entry per (slot, head); a slot is a chunk: n ceil(T / 64) + c, packed tok0 / 64 + n + c
     unsigned char *tpl;   // T as three operand planes, 64 x 64 each, sw128 layout
-    // As accumulator tiles: 16 rows x 8 columns, a lane's four values side by side, so that a warp writes and reads 512 bytes in a row
-    // (row by row, 8 lines to an instruction, the chains stood in their stores: 2 000 - 3 000 cycles of a chunk's 12 000 - 17 000)
-    float *pdo;           // (P^T dO)^T  [D / 16][8] tiles
-    float *s0, *g1;       // S_0^T, G_1^T  [d_v / 16][d_k / 8] tiles
+    float *pdo;           // (P^T dO)^T  [D / 16][8] accumulator tiles
+    float *s0, *g1;       // S_0^T, G_1^T  d 64: [d_v / 16][d_k / 8] accumulator tiles; d 128: [d_v][d_k]
     float *u;             // U           [64][D]
     Scal *scal;
     int32_t n_slots;
     int32_t test_timeout;
     int32_t *status_word;
 };
+// How states and P^T dO cross the workspace.  An accumulator tile is 16 rows x 8 columns with a lane's four values side by side: a warp
+// of the chains then writes and reads 512 bytes in a row, where rows take 8 lines to an instruction.  The gradients' planes are rows,
+// and from tiles a thread has two neighbours to write to them (4-byte stores), from rows eight (16 bytes).  Measured, us:
+//                                       chains    gradients   the call
+//     d 64, 16 packed sequences         406 -> 354   778 -> 778   1433 -> 1379    states as rows -> as tiles
+//     d 128, B 8, H 8, T 4096           563 -> 566   813 -> 835   1498 -> 1527
+// so the states are tiles at d 64 alone (at d 128 a chunk has more products to cover its stores with, and the gradients spill registers
+// with tiles, 20 bytes each way, where with rows they do not).  P^T dO, which only the chains read, is tiles at both (1443 -> 1433, 1513 -> 1498).
+template <int D>
+constexpr bool STATE_TILES = D == 64;
 struct TileMaps {
     CUtensorMap q, k, v, dout;   // 64 tokens x 64 columns
 };
@@ -535,9 +543,19 @@ __device__ __forceinline__ void chain(const BwdChunkParams &p, const TileMaps &t
         }
         // the state at this end of the chunk, transposed
         {
-            float *dst = (BWD ? p.g1 : p.s0) + ch * D * D + (sl * 4 + warp) * 16 * D + lane * 4;
+            float *dst = (BWD ? p.g1 : p.s0) + ch * D * D;
+            if constexpr (STATE_TILES<D>) {
+                dst += (sl * 4 + warp) * 16 * D + lane * 4;
 #pragma unroll
-            for (int t = 0; t < D / 8; ++t) store4(dst + 128 * t, make_float4(S[t][0], S[t][1], S[t][2], S[t][3]));
+                for (int t = 0; t < D / 8; ++t) store4(dst + 128 * t, make_float4(S[t][0], S[t][1], S[t][2], S[t][3]));
+            } else {
+                dst += (size_t)col * D + cq;
+#pragma unroll
+                for (int t = 0; t < D / 8; ++t) {
+                    store2(dst + 8 * t, S[t][0], S[t][1]);
+                    store2(dst + 8 * D + 8 * t, S[t][2], S[t][3]);
+                }
+            }
         }
         float4 pd[BWD ? 8 : 1];
         float x[8][4], y[8][4];
@@ -757,7 +775,7 @@ __device__ __forceinline__ void prefetch_block(const BwdChunkParams &p, int b, i
 template <int D>
 __global__ void __launch_bounds__(GT, 1) kla_bwd_grad_kernel(BwdChunkParams p, int ahead)
 {
-    constexpr int NB = D / 64, IT = D / 2 / GW;   // tiles of half a state per warp
+    constexpr int NB = D / 64, NV = D / 32;       // float4 of half a state per thread
     constexpr int UI = C * D / 8 / GT;            // 8-column items of a [64][D] matrix per thread
     extern __shared__ __align__(128) unsigned char smem_dyn[];
     GradSmem<D> &sm = *reinterpret_cast<GradSmem<D> *>(smem_dyn);
@@ -772,13 +790,24 @@ __global__ void __launch_bounds__(GT, 1) kla_bwd_grad_kernel(BwdChunkParams p, i
     if (tid < (int)sizeof(Scal) / 16) cp16(smem_u32(&sm.s) + tid * 16, reinterpret_cast<const char *>(p.scal + ch) + tid * 16, true);
     cp_commit();
 
-    // S_0^T / G_1^T, 64 columns of d_k from 64 hh on: tile tt of the 16 rows of d_v from 16 tg on
-    auto tg = [&](int i) { return (warp * IT + i) / 8; };
-    auto tt = [&](int i) { return (warp * IT + i) % 8; };
-    float4 ps[IT], pg[IT];
-    auto fetch = [&](float4 (&pre)[IT], const float *src, int hh) {
+    // S_0^T / G_1^T, 64 columns of d_k from 64 hh on: tile tt of the 16 rows of d_v from 16 tg on, respectively 8 columns of a row to
+    // two float4
+    auto tg = [&](int i) { return (warp * NV + i) / 8; };
+    auto tt = [&](int i) { return (warp * NV + i) % 8; };
+    float4 ps[NV], pg[NV];
+    auto fetch = [&](float4 (&pre)[NV], const float *src, int hh) {
+        if constexpr (STATE_TILES<D>) {
 #pragma unroll
-        for (int i = 0; i < IT; ++i) pre[i] = load4(src + ch * D * D + tg(i) * 16 * D + (8 * hh + tt(i)) * 128 + lane * 4);
+            for (int i = 0; i < NV; ++i) pre[i] = load4(src + ch * D * D + tg(i) * 16 * D + (8 * hh + tt(i)) * 128 + lane * 4);
+        } else {
+#pragma unroll
+            for (int i = 0; i < NV; i += 2) {
+                const int e = tid + i / 2 * GT;
+                const float *x = src + ch * D * D + (size_t)(e >> 3) * D + hh * 64 + (e & 7) * 8;
+                pre[i] = load4(x);
+                pre[i + 1] = load4(x + 4);
+            }
+        }
     };
     auto put8 = [&](unsigned char *dst, int plane, uint32_t off, const float4 &a, const float4 &b) {
         uint32_t hh[4], mm[4], ll[4];
@@ -790,18 +819,26 @@ __global__ void __launch_bounds__(GT, 1) kla_bwd_grad_kernel(BwdChunkParams p, i
         *reinterpret_cast<uint4 *>(dst + plane + off) = make_uint4(mm[0], mm[1], mm[2], mm[3]);
         *reinterpret_cast<uint4 *>(dst + 2 * plane + off) = make_uint4(ll[0], ll[1], ll[2], ll[3]);
     };
-    auto commit = [&](const float4 (&pre)[IT]) {
+    auto commit = [&](const float4 (&pre)[NV]) {
+        if constexpr (STATE_TILES<D>) {
 #pragma unroll
-        for (int i = 0; i < IT; ++i)
+            for (int i = 0; i < NV; ++i)
 #pragma unroll
-            for (int u = 0; u < 2; ++u) {
-                uint32_t hh, mm, ll;
-                split3(u ? pre[i].z : pre[i].x, u ? pre[i].w : pre[i].y, hh, mm, ll);
-                const uint32_t off = sw128(tg(i) * 16 + u * 8 + (lane >> 2), tt(i)) + 4 * (lane & 3);
-                *reinterpret_cast<uint32_t *>(sm.sg + off) = hh;
-                *reinterpret_cast<uint32_t *>(sm.sg + D * 128 + off) = mm;
-                *reinterpret_cast<uint32_t *>(sm.sg + 2 * D * 128 + off) = ll;
+                for (int u = 0; u < 2; ++u) {
+                    uint32_t hh, mm, ll;
+                    split3(u ? pre[i].z : pre[i].x, u ? pre[i].w : pre[i].y, hh, mm, ll);
+                    const uint32_t off = sw128(tg(i) * 16 + u * 8 + (lane >> 2), tt(i)) + 4 * (lane & 3);
+                    *reinterpret_cast<uint32_t *>(sm.sg + off) = hh;
+                    *reinterpret_cast<uint32_t *>(sm.sg + D * 128 + off) = mm;
+                    *reinterpret_cast<uint32_t *>(sm.sg + 2 * D * 128 + off) = ll;
+                }
+        } else {
+#pragma unroll
+            for (int i = 0; i < NV; i += 2) {
+                const int e = tid + i / 2 * GT;
+                put8(sm.sg, D * 128, sw128(e >> 3, e & 7), pre[i], pre[i + 1]);
             }
+        }
     };
 
     // U and lam as operand planes; dbeta_i = (U_i / beta_i) . (lam_i / beta_i)
@@ -1032,7 +1069,7 @@ __global__ void __launch_bounds__(GT, 1) kla_bwd_grad_kernel(BwdChunkParams p, i
         }
         __syncthreads();   // the S_0 planes have been read
 #pragma unroll
-        for (int i = 0; i < IT; ++i) gs += gc * (ps[i].x * pg[i].x + ps[i].y * pg[i].y + ps[i].z * pg[i].z + ps[i].w * pg[i].w);
+        for (int i = 0; i < NV; ++i) gs += gc * (ps[i].x * pg[i].x + ps[i].y * pg[i].y + ps[i].z * pg[i].z + ps[i].w * pg[i].w);
         commit(pg);
         if (hh + 1 < NB) fetch(ps, p.s0, hh + 1);
         __syncthreads();
