@@ -119,9 +119,12 @@ def _dt(t: torch.Tensor) -> int:
     raise TypeError("q, k, v, out must be float32 or bfloat16, got %s" % t.dtype)
 
 
-def _dev(t, name, dtype=None):
+def _dev(t, name, dtype=None, n=0):
+    """Device address of a contiguous CUDA tensor of `dtype` (if given) and at least n elements; None for None."""
     if t is None:
         return None
+    if isinstance(t, torch.Tensor) and t.numel() < n:
+        raise ValueError("%s holds fewer elements than the call takes" % name)
     if not (isinstance(t, torch.Tensor) and t.is_cuda and t.is_contiguous()):
         raise ValueError("%s must be a contiguous CUDA tensor" % name)
     if dtype is not None and t.dtype != dtype:
@@ -205,6 +208,8 @@ def kla_chunk_fwd(q, k, v, log_alpha, eta, eps, chunk=64, init_state=None, out=N
         if hs.dtype != torch.int32 or hs.is_cuda:
             raise TypeError("host_seqlens must be a CPU int32 tensor")
         n_seq = cu_seqlens.numel() - 1
+        if hs.numel() < n_seq + 1:
+            raise ValueError("host_seqlens holds fewer elements than the call takes")
     if out is None:
         out = torch.empty((B, T, H, d_v), device=q.device, dtype=out_dtype or q.dtype)
     if final_state is None and want_final_state:
@@ -225,7 +230,7 @@ def kla_chunk_fwd(q, k, v, log_alpha, eta, eps, chunk=64, init_state=None, out=N
     args = (ctypes.byref(desc), _dev(q, "q"), _dev(k, "k"), _dev(v, "v"),
             _dev(log_alpha, "log_alpha", torch.float32), _dev(eta, "eta", torch.float32),
             float(eps), int(chunk), _dev(init_state, "init_state", torch.float32),
-            _dev(out, "out"), _dev(final_state, "final_state", torch.float32))
+            _dev(out, "out", n=v.numel()), _dev(final_state, "final_state", torch.float32, n_seq * H * d_k * d_v))
     with torch.cuda.device(q.device):
         if pass_ms is None:
             code = lib.kla_chunk_fwd(*args)
@@ -259,6 +264,8 @@ def kla_chunk_fwd_static_scratch(q, k, v, log_alpha, eta, eps, out, final_state=
         if host_seqlens is None or host_seqlens.is_cuda or host_seqlens.dtype != torch.int32 or cu_seqlens.dtype != torch.int32:
             raise TypeError("packed input needs cu_seqlens (CUDA int32) and host_seqlens (CPU int32)")
         n_seq = cu_seqlens.numel() - 1
+        if host_seqlens.numel() < n_seq + 1:
+            raise ValueError("host_seqlens holds fewer elements than the call takes")
     desc = KlaDesc(B=B, T=T, H=H, d_k=d_k, d_v=d_v, n_seq=n_seq, cu_seqlens=_dev(cu_seqlens, "cu_seqlens"),
                    host_seqlens=host_seqlens.data_ptr() if host_seqlens is not None else None,
                    io_dtype=_dt(q), out_dtype=_dt(out), flags=flags, workspace=None, workspace_bytes=0,
@@ -266,8 +273,8 @@ def kla_chunk_fwd_static_scratch(q, k, v, log_alpha, eta, eps, out, final_state=
     with torch.cuda.device(q.device):
         code = lib.kla_chunk_fwd_static_scratch(
             ctypes.byref(desc), _dev(q, "q"), _dev(k, "k"), _dev(v, "v"), _dev(log_alpha, "log_alpha", torch.float32),
-            _dev(eta, "eta", torch.float32), float(eps), int(chunk), _dev(init_state, "init_state", torch.float32),
-            _dev(out, "out"), _dev(final_state, "final_state", torch.float32))
+            _dev(eta, "eta", torch.float32), float(eps), int(chunk), _dev(init_state, "init_state", torch.float32, n_seq * H * d_k * d_v),
+            _dev(out, "out"), _dev(final_state, "final_state", torch.float32, n_seq * H * d_k * d_v))
     _check(code)
     return out, final_state
 
@@ -289,8 +296,9 @@ def kla_chunk_span_map(k, v, log_alpha, eta, eps, flags=KLA_FLAG_NONE, status_wo
     ws = torch.empty(max(need, 16), device=k.device, dtype=torch.uint8)
     desc.workspace, desc.workspace_bytes = ws.data_ptr(), need
     with torch.cuda.device(k.device):
-        code = lib.kla_chunk_span_map(ctypes.byref(desc), _dev(k, "k"), _dev(v, "v"), _dev(log_alpha, "log_alpha", torch.float32),
-                                      _dev(eta, "eta", torch.float32), float(eps), phi.data_ptr(), n.data_ptr())
+        code = lib.kla_chunk_span_map(ctypes.byref(desc), _dev(k, "k"), _dev(v, "v", n=k.numel()),
+                                      _dev(log_alpha, "log_alpha", torch.float32, B * T * H), _dev(eta, "eta", torch.float32, B * T * H),
+                                      float(eps), phi.data_ptr(), n.data_ptr())
     _check(code)
     return phi, n
 
@@ -305,8 +313,8 @@ def kla_state_chain(phi, n, init_state=None):
     desc = KlaDesc(B=B, T=1, H=H, d_k=d, d_v=d, n_seq=B, cu_seqlens=None, host_seqlens=None, io_dtype=KLA_BF16, out_dtype=KLA_F32,
                    flags=0, workspace=None, workspace_bytes=0, status_word=None, stream=_stream(phi.device))
     with torch.cuda.device(phi.device):
-        code = lib.kla_state_chain(ctypes.byref(desc), R, _dev(init_state, "init_state", torch.float32), _dev(phi, "phi", torch.float32),
-                                   _dev(n, "n", torch.float32), start.data_ptr())
+        code = lib.kla_state_chain(ctypes.byref(desc), R, _dev(init_state, "init_state", torch.float32, B * H * d * d),
+                                   _dev(phi, "phi", torch.float32), _dev(n, "n", torch.float32, phi.numel()), start.data_ptr())
     _check(code)
     return start
 

@@ -83,6 +83,25 @@ long integer(PyObject *o)
     if (x == -1 && PyErr_Occurred()) throw Failed();
     return x;
 }
+// Larger buffers than a call needs are the caller's business; smaller ones would be read or written past their end.
+void holds(const at::Tensor *t, int64_t n, const char *name)
+{
+    if (t && t->numel() < n) fail(PyExc_ValueError, "holds fewer elements than the call takes", name);
+}
+void one_dtype(const at::Tensor &q, const at::Tensor &k, const at::Tensor &v)
+{
+    if (k.scalar_type() != q.scalar_type() || v.scalar_type() != q.scalar_type()) fail(PyExc_TypeError, "q, k, v must share one dtype");
+}
+// Packed input: the host copy of the offsets, contiguous, and the number of sequences.
+at::Tensor offsets(const at::Tensor &cu, PyObject *host_seqlens, int64_t *n_seq)
+{
+    if (cu.scalar_type() != at::kInt) fail(PyExc_TypeError, "cu_seqlens must be int32");
+    const at::Tensor &host = tensor(host_seqlens, "host_seqlens");
+    if (host.is_cuda() || host.scalar_type() != at::kInt) fail(PyExc_TypeError, "host_seqlens must be a CPU int32 tensor");
+    *n_seq = cu.numel() - 1;
+    holds(&host, *n_seq + 1, "host_seqlens");
+    return host.contiguous();
+}
 bool has_shape(const at::Tensor &t, at::IntArrayRef shape) { return t.sizes() == shape; }
 
 // The status word of a call: the caller's, else the binding's own of the device (kept alive by the binding).
@@ -128,10 +147,18 @@ PyObject *decode(PyObject *, PyObject *const *a, Py_ssize_t n)
         const long kind = integer(a[10]);
         const int lead = kind == 1 ? 1 : 0;
         if (q.dim() != 3 + lead || v.dim() < 1) fail(PyExc_ValueError, lead ? "q must be [n, B, H, d_k]" : "q must be [B, H, d_k]");
-        const int64_t steps = lead ? q.size(0) : 1, B = q.size(lead), H = q.size(lead + 1), d_v = v.size(-1);
+        const int64_t steps = lead ? q.size(0) : 1, B = q.size(lead), H = q.size(lead + 1), d_k = q.size(-1), d_v = v.size(-1);
+        const at::Tensor *given = opt_tensor(a[7], "out");
+        one_dtype(q, k, v);
+        const int64_t units = steps * B * H;
+        holds(&k, units * d_k, "k");
+        holds(&v, units * d_v, "v");
+        holds(&la, kind == 2 ? units * d_k : units, "log_alpha");
+        holds(&eta, units, "eta");
+        holds(&state, B * H * d_k * d_v, "state_inout");
+        holds(given, units * d_v, "out");
         void *qa = addr(&q, "q");
         const c10::cuda::OptionalCUDAGuard guard(q.device());
-        const at::Tensor *given = opt_tensor(a[7], "out");
         at::Tensor out;
         if (given) out = *given;
         else if (lead) out = at::empty({steps, B, H, d_v}, q.options().dtype(dtype_arg(a[8], q)));
@@ -140,7 +167,7 @@ PyObject *decode(PyObject *, PyObject *const *a, Py_ssize_t n)
         d.B = d.n_seq = (int32_t)B;
         d.T = 1;
         d.H = (int32_t)H;
-        d.d_k = (int32_t)q.size(-1);
+        d.d_k = (int32_t)d_k;
         d.d_v = (int32_t)d_v;
         d.io_dtype = kla_dtype_of(q);
         d.out_dtype = kla_dtype_of(out);
@@ -186,20 +213,16 @@ PyObject *forward(PyObject *, PyObject *const *a, Py_ssize_t n)
         if (!has_shape(k, q.sizes()) || !has_shape(v, {B, T, H, d_v})) fail(PyExc_ValueError, "q, k, v shapes disagree");
         if (!has_shape(eta, {B, T, H}) || !(dg ? has_shape(la, {B, T, H, d_k}) : has_shape(la, {B, T, H})))
             fail(PyExc_ValueError, dg ? "log_alpha must be [B, T, H, d_k] and eta [B, T, H]" : "log_alpha, eta must be [B, T, H]");
-        if (k.scalar_type() != q.scalar_type() || v.scalar_type() != q.scalar_type()) fail(PyExc_TypeError, "q, k, v must share one dtype");
+        one_dtype(q, k, v);
         int64_t n_seq = B;
         const at::Tensor *cu = opt_tensor(a[10], "cu_seqlens");
         at::Tensor host;
-        if (cu) {
-            if (cu->scalar_type() != at::kInt) fail(PyExc_TypeError, "cu_seqlens must be int32");
-            host = tensor(a[11], "host_seqlens");
-            if (host.is_cuda() || host.scalar_type() != at::kInt) fail(PyExc_TypeError, "host_seqlens must be a CPU int32 tensor");
-            if (!host.is_contiguous()) host = host.contiguous();
-            n_seq = cu->numel() - 1;
-        }
+        if (cu) host = offsets(*cu, a[11], &n_seq);
+        const at::Tensor *out_given = opt_tensor(a[8], "out"), *fin_given = opt_tensor(a[9], "final_state"), *init = opt_tensor(a[7], "init_state");
+        holds(out_given, B * T * H * d_v, "out");
+        holds(fin_given, n_seq * H * d_k * d_v, "final_state");
         void *qa = addr(&q, "q");
         const c10::cuda::OptionalCUDAGuard guard(q.device());
-        const at::Tensor *out_given = opt_tensor(a[8], "out"), *fin_given = opt_tensor(a[9], "final_state"), *init = opt_tensor(a[7], "init_state");
         at::Tensor out, fin, ws;
         if (out_given) out = *out_given;
         else out = at::empty({B, T, H, d_v}, q.options().dtype(dtype_arg(a[12], q)));
@@ -273,15 +296,18 @@ PyObject *backward(PyObject *, PyObject *const *a, Py_ssize_t n)
         const int64_t B = q.size(0), T = q.size(1), H = q.size(2), d_k = q.size(3), d_v = v.size(-1);
         if (!has_shape(d_out, {B, T, H, d_v}) || d_out.scalar_type() != q.scalar_type())
             fail(PyExc_ValueError, "d_out must be [B, T, H, d_v] with the dtype of q");
+        one_dtype(q, k, v);
         int64_t n_seq = B;
         const at::Tensor *cu = opt_tensor(a[9], "cu_seqlens"), *init = opt_tensor(a[7], "init_state"), *dfin = opt_tensor(a[8], "d_final_state");
         const at::Tensor *given = opt_tensor(a[13], "workspace");
         at::Tensor host;
-        if (cu) {
-            host = tensor(a[10], "host_seqlens");
-            if (!host.is_contiguous()) host = host.contiguous();
-            n_seq = cu->numel() - 1;
-        }
+        if (cu) host = offsets(*cu, a[10], &n_seq);
+        holds(&k, q.numel(), "k");
+        holds(&v, B * T * H * d_v, "v");
+        holds(&la, B * T * H, "log_alpha");
+        holds(&eta, B * T * H, "eta");
+        holds(init, n_seq * H * d_k * d_v, "init_state");
+        holds(dfin, n_seq * H * d_k * d_v, "d_final_state");
         void *qa = addr(&q, "q");
         const c10::cuda::OptionalCUDAGuard guard(q.device());
         kla_desc d = {};
