@@ -146,9 +146,9 @@ def _status_for(dev):
 
 
 def check(device=None):
-    """Reads (and clears) the status word the binding passes to kla_chunk_fwd, kla_chunk_span_map and kla_bwd when the caller gives none:
-    raises KlaError if a kernel on `device` (default: the current one) gave up on a bounded wait since the last check -- its outputs are
-    then undefined.  Waits for the device; meant for the end of a step, not for the hot path."""
+    """Reads (and clears) the status word the binding passes to kla_chunk_fwd, kla_chunk_fwd_static_scratch, kla_chunk_span_map and kla_bwd
+    when the caller gives none: raises KlaError if a kernel on `device` (default: the current one) gave up on a bounded wait since the
+    last check -- its outputs are then undefined.  Waits for the device; meant for the end of a step, not for the hot path."""
     i = torch.cuda.current_device() if device is None else torch.device(device).index
     word = _own_status.get(i)
     if word is None:
@@ -254,7 +254,8 @@ def kla_chunk_fwd_static_scratch(q, k, v, log_alpha, eta, eps, out, final_state=
     kla_chunk_fwd_static_scratch).  The scratch (segment-parallel scan; longest-first order of packed sequences) is a
     fixed array inside the library, so this wrapper allocates nothing either: `out` (and `final_state`, if wanted) must
     be passed in, and for packed input both `cu_seqlens` (CUDA int32) and `host_seqlens` (CPU int32 copy).  Shapes whose
-    scratch would exceed STATIC_SCRATCH_BYTES raise KlaError (workspace).  Calls must not overlap on the GPU."""
+    scratch would exceed STATIC_SCRATCH_BYTES raise KlaError (workspace).  Calls must not overlap on the GPU.  `status_word` as for
+    kla_chunk_fwd; the binding's own is made on a device's first call of any function, unless the caller passes one."""
     lib = load()
     B, T, H, d_k, d_v = _sequence_shapes(q, k, v, log_alpha, eta)
     if tuple(out.shape) != (B, T, H, d_v):
@@ -266,6 +267,8 @@ def kla_chunk_fwd_static_scratch(q, k, v, log_alpha, eta, eps, out, final_state=
         n_seq = cu_seqlens.numel() - 1
         if host_seqlens.numel() < n_seq + 1:
             raise ValueError("host_seqlens holds fewer elements than the call takes")
+    if status_word is None:
+        status_word = _status_for(q.device)
     desc = KlaDesc(B=B, T=T, H=H, d_k=d_k, d_v=d_v, n_seq=n_seq, cu_seqlens=_dev(cu_seqlens, "cu_seqlens"),
                    host_seqlens=host_seqlens.data_ptr() if host_seqlens is not None else None,
                    io_dtype=_dt(q), out_dtype=_dt(out), flags=flags, workspace=None, workspace_bytes=0,

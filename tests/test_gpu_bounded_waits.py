@@ -1,12 +1,13 @@
-"""Bounded waits of the backward pass and of the span map: a wait made to run out (a copy that is never asked for; nothing faults or
-hangs) is heard of by a caller who passes a status word and by one who does not, and the context stays usable."""
+"""Bounded waits of the backward pass, the span map and the forward on static scratch: a wait made to run out (a copy or a
+signal that never comes; nothing faults or hangs) is heard of by a caller who passes a status word and by one who does not, and the context stays usable."""
 import numpy as np
 import pytest
 import torch
 
 import oracle
 from helpers import TOL_BF16, np64, rel_err
-from paper_2605_08587_b200 import KLA_FLAG_WY_FORM, KlaError, binding, check, kla_bwd, kla_chunk_span_map, workloads as W
+from paper_2605_08587_b200 import (KLA_FLAG_WY_FORM, KlaError, binding, check, kla_bwd, kla_chunk_fwd, kla_chunk_fwd_static_scratch,
+                                   kla_chunk_span_map, workloads as W)
 
 pytestmark = pytest.mark.gpu
 DEV = "cuda:0"
@@ -75,9 +76,23 @@ def test_span_map_reports_a_wait_that_ran_out(flags):
     assert rel_err(np64(n), fin) <= TOL_BF16
 
 
+def test_static_scratch_reports_a_wait_that_ran_out():
+    w = W.config2(B=1, H=2, T=130, seed=535)
+    a = _args(w)
+    want, _ = kla_chunk_fwd(*a, w.eps)
+    out = torch.empty_like(want)
+    check(DEV)
+    kla_chunk_fwd_static_scratch(*a, w.eps, out, flags=RUN_OUT)
+    with pytest.raises(KlaError) as e:
+        check(DEV)
+    assert e.value.code == TIMEOUT
+    kla_chunk_fwd_static_scratch(*a, w.eps, out)
+    check(DEV)
+    assert torch.equal(out, want)
+
+
 def test_replaying_a_graph_does_not_clear_what_other_calls_reported(monkeypatch):
     """The first call of all may be a captured one: the binding's status word must not become part of that graph."""
-    from paper_2605_08587_b200 import kla_chunk_fwd
     w = W.config2(B=1, H=2, T=130, seed=540)
     do, _ = W.upstream_grads(w)
     a, do = _args(w), do.to(DEV)
