@@ -316,7 +316,7 @@ def dg_leg(dev, steps, warmup, peaks):
 
 
 def bwd_leg(w, dev, steps, warmup, peaks, cpu_baseline):
-    """Backward pass (training, Section 5.1) on the headline shape: reverse sweep over recomputed states, fp32 on CUDA cores."""
+    """Backward pass (training, Section 5.1) of workload w: the derivative of the chunk algebra on tensor cores (bf16 inputs)."""
     import torch
     from paper_2605_08587_b200 import binding, kla_bwd, workloads as W
     do, df = W.upstream_grads(w)

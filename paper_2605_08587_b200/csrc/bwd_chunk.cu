@@ -369,7 +369,8 @@ __global__ void __launch_bounds__(256, D == 64 ? 4 : 3) kla_bwd_prepare_kernel(B
 // uses last (T, V, respectively T, Q, dO) has one buffer and is fetched as soon as every warp has passed it.  One thread fetches
 // by TMA: as asynchronous copies of 16 bytes the 33 of a thread and chunk, a dozen instructions each that run once and come from
 // beyond the instruction caches, took 2 900 (backward) and 1 200 (forward) cycles of a chunk's 16 300 and 13 000.
-// What bounds it: the warp-level tensor pipe, 504 (forward) and 696 (backward) instructions per chunk and warp at D = 128.
+// What bounds it: the latency of one warp per scheduler and block, which issues in order.  Its 504 (forward) and 696 (backward)
+// instructions of the warp-level tensor pipe per chunk at D = 128 keep that pipe busy for 56 % of the cycles.
 // Both directions are one launch so that an SM holds a block of each and one fills the other's latencies.
 template <int D>
 struct ChainSmem {

@@ -27,8 +27,9 @@
 // memory the state product was bound by the fetch of both operands (8 KB for each 32 cycles of products: 570 cycles), and its
 // operand took a proxy fence (headline shape 200.6 -> 194.7 us, 32 packed sequences at d 64 487 -> 472).  The outputs are transposed through
 // a buffer that TMA never touches: in the V tile they took such a fence too, in which the warp stood (194.7 -> 188, 472 -> 462).
-// The size of the code counts, all the more the more SMs run it: at 70 KB two KB less in the waits alone (one short loop each instead
-// of two) were worth 2 % of the headline shape and of 65 536 tokens, two KB more cost 10 %.
+// The size of the code counts, all the more the more SMs run it: of 70 KB, the two that one short loop to a wait instead of two took out
+// were worth 2 % of the headline shape and of 65 536 tokens; two KB more, for tiles of four chunks and two Gram products, gave the
+// headline shape 1.6 % (186 -> 183) and cost 65 536 tokens 2.5 % (366 -> 375).
 // The outputs on four warps of their own cost more than they took off the chain: 246 us against 201 (82 KB of code instead of 70,
 // fetched by all SMs at once, and the Gram product then falls into the block solve).
 //
@@ -78,7 +79,9 @@ constexpr float DEC_FLOOR_LOG2 = 115.f;
 constexpr float HOT_BETA = 4096.f;   // q k beta up to ||q|| sqrt(beta) = 64 ||q||: 2^-18 of that is below the other errors
 constexpr int LDB = 20;       // row stride (floats) of a 16 x 16 block in the solve scratch
 // TMEM columns: [S_hi; S_lo]^T [K; Q]^T (128), [K; Q] K^T (64), the state in fp32 (D / 2), [S_hi; S_lo]^T as left operand (D / 2):
-// warp w: lanes 32 w .. the hi, 32 w + 16 .. the lo parts of its columns of d_v, a column for two of d_k.
+// warp w: lanes 32 w .. the hi, 32 w + 16 .. the lo parts of its columns of d_v, a column for two of d_k.  d 128 uses 320 columns and,
+// as they are given in powers of two, holds all 512: no other block with tensor memory runs beside it on an SM (another one of this
+// library would not find the shared memory either).
 constexpr uint32_t TM_X = 0, TM_G = 128, TM_S = 192;
 template <int D>
 constexpr uint32_t TM_A = TM_S + D / 2;
@@ -878,6 +881,8 @@ __device__ void chain(const ChunkParams &p, Smem<D, BPS> &sm, const Work &wk, in
         }
     }
     // The last chunk stores its state to tensor memory like any other, and nobody waits for it: the columns are given back next.
+    // (Left out in the last chunk instead, the stores stand behind a branch in every one: headline shape 184.7 -> 190.8 us, 65 536 tokens
+    // 362.6 -> 379.9.)
     tmem_wait_stores();
     if (wk.fin && !sm.abort_flag) {
 #pragma unroll
